@@ -373,6 +373,100 @@ __device__ __forceinline__ bool grid_allreduce_sym(double (&v)[NV], double *part
     return ok;
 }
 
+// Totals over the warp of one or two doubles per lane, with half the adds of
+// two butterflies: the two values are folded onto the warp's halves first.
+// Lanes 0..15 return the total of v[0], lanes 16..31 that of v[NV - 1].
+// (FP64 adds issue at 1/64 of the FP32 rate on GB300: 16 cycles per warp.)
+template <int NV>
+__device__ __forceinline__ double warp_fold(const double (&v)[NV]) {
+    static_assert(NV == 1 || NV == 2, "one or two values");
+    const bool up = (threadIdx.x & 16) != 0;
+    const double send = NV == 2 && !up ? v[NV - 1] : v[0];
+    double keep = NV == 2 && up ? v[NV - 1] : v[0];
+    keep += __shfl_xor_sync(0xffffffffu, send, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) keep += __shfl_xor_sync(0xffffffffu, keep, o);
+    return keep;
+}
+
+// grid_allreduce_sym for kernels of few warps per CTA: v holds every thread's
+// own partials (at most 16 warps per CTA), the arrivals are spread over
+// AR_SUB counters on lines of their own as in grid_allreduce_df, and warp 0
+// alone adds the CTAs' partials (each lane's loads issued together), so that
+// an exchange costs two warp-wide folds of FP64 adds instead of two per warp.
+// Same bits in every CTA: fixed orders for a given launch shape.  `bar` holds
+// AR_SUB * 32 words, zero at launch; totals in every thread on return; false
+// on timeout.
+constexpr int AR_SUB = 16;
+template <int NV>
+__device__ __forceinline__ bool grid_allreduce_w0(double (&v)[NV], double *part, unsigned gen, unsigned *bar,
+                                                  int *err, long long limit_cycles) {
+    __shared__ double s_w[NV * 16];
+    __shared__ double s_tot[NV];
+    __shared__ int s_ok;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    double2 *half = reinterpret_cast<double2 *>(part + (size_t)(gen & 1u) * gridDim.x * AR_NV_MAX);
+    {
+        const double t = warp_fold<NV>(v);
+        if (lane == 0) s_w[w] = t;
+        if (NV == 2 && lane == 16) s_w[16 * (NV - 1) + w] = t;
+    }
+    __syncthreads();
+    if (w == 0) {
+        const int l = lane & 15;
+        double t = l < nw ? s_w[(NV == 2 ? lane & 16 : 0) + l] : 0.0;
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1)
+            if (o < nw) t += __shfl_xor_sync(0xffffffffu, t, o);
+        const double t1 = __shfl_sync(0xffffffffu, t, 16);
+        if (lane == 0) {
+            __stcg(half + blockIdx.x, make_double2(t, t1));
+            red_add_release(bar + 32 * (blockIdx.x % AR_SUB), 1u);
+        }
+        int lane_ok = 1;
+        if (lane < AR_SUB) {
+            const unsigned per = gridDim.x / AR_SUB + ((unsigned)lane < gridDim.x % AR_SUB ? 1u : 0u);
+            const unsigned target = (gen + 1u) * per;
+            const long long t0 = clock64();
+            while (ld_acquire(bar + 32 * lane) < target) {
+                if (clock64() - t0 > limit_cycles || *(volatile int *)err == (int)BA_ERR_TIMEOUT) {
+                    lane_ok = 0;
+                    break;
+                }
+            }
+        }
+        const bool ok = __all_sync(0xffffffffu, lane_ok) != 0;  // orders the other lanes' partial reads too
+        double acc[NV];
+#pragma unroll
+        for (int k = 0; k < NV; ++k) acc[k] = 0.0;
+        if (ok) {
+            for (unsigned b0 = lane; b0 < gridDim.x; b0 += 160) {
+                double2 u[5];
+#pragma unroll
+                for (int q = 0; q < 5; ++q)
+                    u[q] = b0 + 32 * q < gridDim.x ? __ldcg(half + b0 + 32 * q) : make_double2(0.0, 0.0);
+#pragma unroll
+                for (int q = 0; q < 5; ++q) {
+                    acc[0] += u[q].x;
+                    if (NV == 2) acc[NV - 1] += u[q].y;
+                }
+            }
+        }
+        __syncwarp();
+        const double tot = warp_fold<NV>(acc);
+        if (lane == 0) {
+            s_tot[0] = tot;
+            s_ok = ok ? 1 : 0;
+            if (!ok) atomicExch(err, (int)BA_ERR_TIMEOUT);
+        }
+        if (NV == 2 && lane == 16) s_tot[NV - 1] = tot;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < NV; ++k) v[k] = s_tot[k];
+    return s_ok != 0;
+}
+
 // ---- 6x6 block SpMV helpers (BSMC and the full-block formats) ----
 
 // One 6x6 block (16-byte aligned) into registers, read-only path.
@@ -536,7 +630,6 @@ __device__ __forceinline__ void block_sum_df(df32 (&v)[NV], float2 *sh) {
 // before arriving is visible to it) right after issuing its partial reads;
 // meant for asynchronous copies that overlap the rest.  On return the
 // totals are valid in thread 0 only (as double-floats); false on timeout.
-constexpr int AR_SUB = 16;
 template <int NV, class F>
 __device__ __forceinline__ bool grid_allreduce_df(df32 (&v)[NV], double *part, unsigned gen, unsigned *bar,
                                                   int *err, long long limit_cycles, df32 (&tot)[NV], float2 *sh,

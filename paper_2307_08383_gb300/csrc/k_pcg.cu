@@ -40,6 +40,31 @@ __device__ __forceinline__ void gather_x(const TV *__restrict__ xz, const TV *__
     }
 }
 
+// Sums of six values over the warp by recursive halving (eight adds per lane
+// instead of thirty: the adds of an FP64 row sum took as long as a quarter of
+// its products).  Lane l ends with the total of component fold6_comp(l); the
+// additions pair the lanes as the xor butterfly 16, 8, 4, 2, 1 does, so the
+// totals are its bits.
+__device__ __forceinline__ int fold6_comp(int lane) {
+    return ((lane & 16) ? 3 : 0) + ((lane & 8) ? 2 : ((lane & 4) ? 1 : 0));
+}
+__device__ __forceinline__ bool fold6_owner(int lane) { return (lane & 3) == 0 && (lane & 12) != 12; }
+template <typename TV>
+__device__ __forceinline__ TV warp_fold6(const TV (&a)[6], int lane) {
+    const unsigned M = 0xffffffffu;
+    const bool b16 = lane & 16, b8 = lane & 8, b4 = lane & 4;
+    TV k[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) k[c] = (b16 ? a[3 + c] : a[c]) + __shfl_xor_sync(M, b16 ? a[c] : a[3 + c], 16);
+    const TV r0 = __shfl_xor_sync(M, b8 ? k[0] : k[2], 8), r1 = __shfl_xor_sync(M, k[1], 8);
+    const TV u = (b8 ? k[2] : k[0]) + r0, v = k[1] + r1;
+    TV t = (b8 || !b4) ? u : v;
+    t += __shfl_xor_sync(M, (b8 || b4) ? u : v, 4);
+    t += __shfl_xor_sync(M, t, 2);
+    t += __shfl_xor_sync(M, t, 1);
+    return t;
+}
+
 // q = S x over BSMC without atomics: a warp per block row i walks the row's
 // two-sided entry list - the stored blocks (i, j >= i), applied as S_ij x_j,
 // then the blocks (j < i, i) of column i, applied as S_ji^T x_j - so q_i is
@@ -49,11 +74,12 @@ __device__ __forceinline__ void gather_x(const TV *__restrict__ xz, const TV *__
 // any arithmetic, so one L2 round trip covers ~64 blocks of the row.
 // PCG variant: x_j = z_j + beta d_old_j, the row owner stores d_new_i, and the
 // function returns this thread's share of d^T S d = sum_i d_i^T q_i.
+// Returns component fold6_comp(lane) of the row's sum.
 template <typename TS, typename TV, class GX>
-__device__ __forceinline__ void spmv_row(int i, int lane, const int *__restrict__ tw_ptr,
-                                         const int2 *__restrict__ tw_ent, const TS *__restrict__ S, GX gx,
-                                         TV (&acc)[6]) {
+__device__ __forceinline__ TV spmv_row(int i, int lane, const int *__restrict__ tw_ptr,
+                                         const int2 *__restrict__ tw_ent, const TS *__restrict__ S, GX gx) {
     const int tb = __ldg(tw_ptr + i), te = __ldg(tw_ptr + i + 1);
+    TV acc[6];
 #pragma unroll
     for (int c = 0; c < 6; ++c) acc[c] = TV(0);
     for (int t0 = tb + lane; t0 < te; t0 += 64) {
@@ -69,8 +95,7 @@ __device__ __forceinline__ void spmv_row(int i, int lane, const int *__restrict_
         block_apply<TV>(Sa, xa, ea.x < 0, acc);
         if (has1) block_apply<TV>(Sb, xb, eb.x < 0, acc);
     }
-#pragma unroll
-    for (int r = 0; r < 6; ++r) acc[r] = warp_sum(acc[r]);
+    return warp_fold6(acc, lane);
 }
 
 template <typename TS, typename TV, bool PCG>
@@ -78,27 +103,22 @@ __device__ __forceinline__ double spmv_rows(int n, const int *__restrict__ tw_pt
                                             const TS *__restrict__ S, const TV *__restrict__ xz,
                                             const TV *__restrict__ dold, TV *__restrict__ dnew, TV *__restrict__ q,
                                             TV beta) {
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, c = fold6_comp(lane);
+    const bool owner = fold6_owner(lane);  // one lane per component
     const int warp = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
     const int nw = (int)(((int64_t)gridDim.x * blockDim.x) >> 5);
     TV pap = TV(0);
     for (int i = warp; i < n; i += nw) {
-        TV di[6];
-        gather_x<TV, PCG>(xz, dold, beta, i, di);
-        if (PCG) {
-#pragma unroll
-            for (int c = 0; c < 6; ++c)
-                if (lane == c) dnew[6 * i + c] = di[c];
+        TV di = TV(0);
+        if (PCG && owner) {
+            di = __ldcg(xz + 6 * i + c) + beta * __ldcg(dold + 6 * i + c);
+            dnew[6 * i + c] = di;
         }
-        TV acc[6];
-        spmv_row<TS, TV>(i, lane, tw_ptr, tw_ent, S,
-                         [&](int j, TV(&x)[6]) { gather_x<TV, PCG>(xz, dold, beta, j, x); }, acc);
-#pragma unroll
-        for (int c = 0; c < 6; ++c)
-            if (lane == c) q[6 * i + c] = acc[c];
-        if (PCG && lane == 0) {
-#pragma unroll
-            for (int c = 0; c < 6; ++c) pap += di[c] * acc[c];
+        const TV qc = spmv_row<TS, TV>(i, lane, tw_ptr, tw_ent, S,
+                                       [&](int j, TV(&x)[6]) { gather_x<TV, PCG>(xz, dold, beta, j, x); });
+        if (owner) {
+            q[6 * i + c] = qc;
+            if (PCG) pap += di * qc;
         }
     }
     return (double)pap;
@@ -322,7 +342,6 @@ __global__ void __launch_bounds__(256) k_pcg_persist(int n, const int *__restric
                                                      const T *__restrict__ S, const T *__restrict__ Minv, T *y, T *r0,
                                                      T *r1, T *z, T *d0, T *d1, T *q0, T *q1, DevScalars *sc,
                                                      double *red, unsigned *bar, long long limit_cycles) {
-    __shared__ double sh[40];
     if (sc->done) return;
     double rz = sc->rz;
     const double rr0 = sc->rr0, tol2 = sc->tol2;
@@ -330,7 +349,9 @@ __global__ void __launch_bounds__(256) k_pcg_persist(int n, const int *__restric
     double beta = 0.0;
     int it = 0;
     unsigned gen = 0;
-    const int ne = 6 * n;
+    // this CTA's vector entries in the update phase: an equal stretch each
+    const int per = (6 * n + gridDim.x - 1) / gridDim.x;
+    const int eb = min(6 * n, (int)blockIdx.x * per), ee = min(6 * n, eb + per);
     for (;;) {
         const bool odd = it & 1;
         T *dold = odd ? d1 : d0, *dnew = odd ? d0 : d1;
@@ -342,8 +363,7 @@ __global__ void __launch_bounds__(256) k_pcg_persist(int n, const int *__restric
             v1[0] = spmv_rows_once(n, row_ptr, col, S, z, dold, dnew, q, (float)beta);
         else
             v1[0] = spmv_rows<T, T, true>(n, tw_ptr, tw_ent, S, z, dold, dnew, q, (T)beta);
-        block_sum<1>(v1, sh);
-        if (!grid_allreduce_sym<1>(v1, red, gen++, bar, &sc->err, limit_cycles)) return;
+        if (!grid_allreduce_w0<1>(v1, red, gen++, bar, &sc->err, limit_cycles)) return;
         const double pAp = v1[0];
         if (!(pAp > 0.0)) {
             if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -356,7 +376,7 @@ __global__ void __launch_bounds__(256) k_pcg_persist(int n, const int *__restric
         const T alpha = (T)(rz / pAp);
         // update phase: y += alpha d, r -= alpha q, z = M^-1 r, r^T z, r^T r
         T rz_p = T(0), rr_p = T(0);
-        for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < ne; e += gridDim.x * blockDim.x) {
+        for (int e = eb + threadIdx.x; e < ee; e += blockDim.x) {
             const int i = e / 6, a = e - 6 * i;
             T ri[6], qi[6];
             load6(rc + 6 * i, ri);
@@ -379,8 +399,7 @@ __global__ void __launch_bounds__(256) k_pcg_persist(int n, const int *__restric
             rr_p += ra * ra;
         }
         double v2[2] = {(double)rz_p, (double)rr_p};
-        block_sum<2>(v2, sh);
-        if (!grid_allreduce_sym<2>(v2, red, gen++, bar, &sc->err, limit_cycles)) return;
+        if (!grid_allreduce_w0<2>(v2, red, gen++, bar, &sc->err, limit_cycles)) return;
         const double rz_new = v2[0], rr = v2[1];
         ++it;
         if (rr <= tol2 * rr0 || it >= max_iters) {
@@ -1149,22 +1168,41 @@ cudaError_t launch_pcg_init(ba_problem *p, const void *rhs, double tol, int max_
 // two-sided product, whose second read hits L2.
 constexpr int64_t ONCE_MIN_BYTES = 64ll << 20;
 
+// arrival counters of the PCG kernels' all-reduces, one per 128-byte line
+static cudaError_t ensure_ar_bar(ba_problem *p) {
+    if (p->ar_bar) return cudaSuccess;
+    void *v = nullptr;
+    const cudaError_t e = cudaMalloc(&v, AR_SUB * 32 * sizeof(unsigned));
+    if (e != cudaSuccess) return e;
+    p->ar_bar = (unsigned *)v;
+    p->allocs.push_back(v);
+    p->dev_bytes += AR_SUB * 32 * sizeof(unsigned);
+    return cudaSuccess;
+}
+
 template <typename T, bool ONCE>
 static cudaError_t pcg_loop_T(ba_problem *p) {
+    // Warps per CTA: the rows are spread over every SM first, then over the
+    // warps of one (one row per warp until eight warps on every SM are in
+    // use).  An FP64 row costs about 100 FP64 warp instructions, which an SM
+    // issues at one per 16 cycles (measured; one per 64 for a single warp), so
+    // eight rows on one SM take 6 us while the next SMs idle.  With the
+    // cheaper sums below: 24.8 -> 14 us per iteration at 200 cameras, 22 -> 12
+    // at 50 (FP64).
     int blocks_per_sm = 0, n_sm = 0;
     cudaError_t e;
     if ((e = occupancy((const void *)k_pcg_persist<T, ONCE>, 256, 0, &blocks_per_sm, &n_sm)) != cudaSuccess) return e;
     if (blocks_per_sm > 2) blocks_per_sm = 2;
     if (blocks_per_sm < 1) return cudaErrorCooperativeLaunchTooLarge;
-    // enough warps for one block row each, at most what is co-resident
-    int64_t want = ((int64_t)p->n * 32 + 255) / 256;
-    int grid = (int)std::min<int64_t>(std::max<int64_t>(want, 1), (int64_t)blocks_per_sm * n_sm);
-    // armed test of the timeout path: the counter starts at -1 (one arrival short)
+    const int warps = std::max(1, std::min(8, (p->n + n_sm - 1) / n_sm));
+    const int grid = std::min((p->n + warps - 1) / warps, blocks_per_sm * n_sm);
+    // armed test of the timeout path: every counter starts at -1, one arrival short
     const long long test_limit = p->test_wait_limit;
     p->test_wait_limit = 0;
-    if ((e = cudaMemsetAsync(p->counters + 14, test_limit > 0 ? 0xFF : 0, sizeof(unsigned), p->st)) != cudaSuccess)
+    if ((e = ensure_ar_bar(p)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(p->ar_bar, test_limit > 0 ? 0xFF : 0, AR_SUB * 32 * sizeof(unsigned), p->st)) !=
+        cudaSuccess)
         return e;
-    if ((e = cudaMemsetAsync(p->counters + 15, 0, sizeof(unsigned), p->st)) != cudaSuccess) return e;
     int n = p->n;
     const int *twp = p->tw_ptr, *rp = p->row_ptr, *cl = p->col;
     const int2 *twe = p->tw_ent;
@@ -1173,10 +1211,10 @@ static cudaError_t pcg_loop_T(ba_problem *p) {
     T *q = (T *)p->sv.pv[5], *r1 = (T *)p->sv.pv[6], *q1 = (T *)p->sv.pv[7];
     DevScalars *sc = p->sc;
     double *red = p->red;
-    unsigned *bar = p->counters + 14;
+    unsigned *bar = p->ar_bar;
     long long limit = test_limit > 0 ? test_limit : 4000000000LL;  // ~2 s of SM clock per barrier wait
     void *args[] = {&n, &twp, &twe, &rp, &cl, &S, &Mi, &y, &r, &r1, &z, &d0, &d1, &q, &q1, &sc, &red, &bar, &limit};
-    return cudaLaunchCooperativeKernel((const void *)k_pcg_persist<T, ONCE>, dim3(grid), dim3(256), args, 0, p->st);
+    return cudaLaunchCooperativeKernel((const void *)k_pcg_persist<T, ONCE>, dim3(grid), dim3(32 * warps), args, 0, p->st);
 }
 
 cudaError_t launch_pcg_loop(ba_problem *p) {
@@ -1540,13 +1578,7 @@ cudaError_t launch_split_init(ba_problem *p, const float *rhs, double tol, int m
 cudaError_t launch_pcg_split(ba_problem *p) {
     cudaEvent_t ev;
     cudaError_t e = cudaSuccess;
-    if (!p->ar_bar) {
-        void *v = nullptr;
-        if ((e = cudaMalloc(&v, AR_SUB * 32 * sizeof(unsigned))) != cudaSuccess) return e;
-        p->ar_bar = (unsigned *)v;
-        p->allocs.push_back(v);
-        p->dev_bytes += AR_SUB * 32 * sizeof(unsigned);
-    }
+    if ((e = ensure_ar_bar(p)) != cudaSuccess) return e;
     ktimer_begin(p, K_PCG_LOOP, &ev);
     // armed test of the timeout path: every counter starts at -1, so each one
     // ends a call one arrival short of its target and the wait runs out

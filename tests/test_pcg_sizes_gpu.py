@@ -1,0 +1,81 @@
+"""Block-Jacobi PCG over the launch shapes its kernels choose by size.
+
+A given system (``Problem.from_rcs``) with seeded SPD values, at camera counts
+on both sides of the lines where the kernels change the warps per CTA, the
+warps per row or the grid.  The reference is the recurrence of Sec. 3.2 in
+numpy FP64.  Tolerances: the solve stops at ||r|| <= 1e-10 ||b|| by its own
+recurrence, whose residual and the true one differ by rounding of the iterates
+(n_iter * 2^-53 * cond, below 1e-13 for these diagonally dominant systems), so
+||b - S x|| <= 1.01e-10 ||b||; iteration counts agree within one; two iterates
+with residuals of 1e-10 differ by at most 2e-10 cond(S), and block dominance
+bounds cond(S) by the ratio of the largest to the smallest diagonal block
+eigenvalue times (1 + s) / (1 - s), s < 1 / 2 the share of a row's norm sum in
+its diagonal: 1e-8 covers the ratios these seeds have (below 50)."""
+import numpy as np
+import pytest
+
+import scenes
+
+pytestmark = pytest.mark.gpu
+
+
+def banded_pattern(n, half):
+    """Every row coupled to four fifths of the next ``half`` cameras."""
+    row_ptr, col = [0], []
+    for i in range(n):
+        c = [i] + [j for j in range(i + 1, min(n, i + half + 1)) if (i * 7 + j) % 5]
+        col += c
+        row_ptr.append(len(col))
+    return np.array(row_ptr, np.int32), np.array(col, np.int32)
+
+
+def system(n, half, seed):
+    row_ptr, col = banded_pattern(n, half)
+    val, _ = scenes.random_block_spd(row_ptr, col, np.full(n, 6, np.int32), seed)
+    b = np.random.default_rng(seed + 1).standard_normal((n, 6))
+    return row_ptr, col, val.reshape(-1, 6, 6), b
+
+
+def product(row_ptr, col, val, x):
+    row = np.repeat(np.arange(len(row_ptr) - 1), np.diff(row_ptr))
+    y = np.zeros_like(x)
+    np.add.at(y, row, np.einsum("kab,kb->ka", val, x[col]))
+    off = row != col
+    np.add.at(y, col[off], np.einsum("kba,kb->ka", val[off], x[row[off]]))
+    return y
+
+
+def pcg(row_ptr, col, val, b, tol):
+    Minv = np.linalg.inv(val[row_ptr[:-1]])
+    x, r = np.zeros_like(b), b.copy()
+    z = np.einsum("nab,nb->na", Minv, r)
+    d, rz, r0 = z, float((r * z).sum()), np.linalg.norm(b)
+    for it in range(1, 10000):
+        q = product(row_ptr, col, val, d)
+        a = rz / float((d * q).sum())
+        x, r = x + a * d, r - a * q
+        if np.linalg.norm(r) <= tol * r0:
+            return x, it
+        z = np.einsum("nab,nb->na", Minv, r)
+        new = float((r * z).sum())
+        d, rz = z + new / rz * d, new
+    raise AssertionError("no convergence")
+
+
+@pytest.mark.parametrize("n,half", [(1, 1), (2, 1), (3, 2), (40, 39), (152, 9), (153, 20), (305, 45), (609, 12),
+                                    (1217, 6), (2500, 4), (130, 129)])
+def test_fp64_pcg_over_launch_shapes(n, half):
+    from paper_2307_08383_gb300.build import build
+    build()
+    import paper_2307_08383_gb300 as B
+    row_ptr, col, val, b = system(n, half, 9100 + n)
+    tol = 1e-10
+    ref, its = pcg(row_ptr, col, val, b, tol)
+    g = B.Problem.from_rcs(row_ptr, col, val, b, precision=B.BA_FP64, pcg_rel_tol=tol)
+    for _ in range(2):  # a second solve finds nothing of the first
+        info, conv = g.solve_rcs()
+        assert conv and abs(info["pcg_iters"] - its) <= 1, (info["pcg_iters"], its)
+        x = g.step()[0].reshape(n, 6)
+        assert np.linalg.norm(b - product(row_ptr, col, val, x)) <= 1.01 * tol * np.linalg.norm(b)
+        assert np.linalg.norm(x - ref) <= 1e-8 * np.linalg.norm(ref)
+    g.close()
