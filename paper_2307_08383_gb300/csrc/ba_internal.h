@@ -82,6 +82,7 @@ struct HostSetup {
     std::vector<int32_t> ct_row;     // ... and their rows j
     std::vector<int32_t> tw_ptr;     // n + 1: entries of row i for the SpMV ...
     std::vector<int2> tw_ent;        // ... {block id | transposed << 31, column j}: row blocks, then column blocks
+    int32_t max_row_ent = 0;         // the longest of those lists
     std::vector<GroupDesc> groups;
     std::vector<ItemDesc> items;
     std::vector<int32_t> lb_gblk;    // global block of each partial

@@ -90,14 +90,15 @@ void build_twosided(HostSetup &hs, int32_t n) {
     // two-sided SpMV entries of row i: (i, j >= i) as stored, then (j < i, i) transposed
     hs.tw_ptr.assign(n + 1, 0);
     hs.tw_ent.clear();
+    hs.max_row_ent = 0;
     hs.tw_ent.reserve(2 * hs.col.size());
     for (int32_t i = 0; i < n; ++i) {
         for (int32_t b = hs.row_ptr[i]; b < hs.row_ptr[i + 1]; ++b) hs.tw_ent.push_back(make_int2(b, hs.col[b]));
         for (int32_t q = hs.ct_ptr[i]; q < hs.ct_ptr[i + 1]; ++q)
             hs.tw_ent.push_back(make_int2((int32_t)((uint32_t)hs.ct_blk[q] | 0x80000000u), hs.ct_row[q]));
         hs.tw_ptr[i + 1] = (int32_t)hs.tw_ent.size();
+        hs.max_row_ent = std::max(hs.max_row_ent, hs.tw_ptr[i + 1] - hs.tw_ptr[i]);
     }
-
 }
 
 // A work item of the RCS formation: products [cbeg, cbeg + cnt) of the

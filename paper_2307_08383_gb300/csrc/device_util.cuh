@@ -389,15 +389,75 @@ __device__ __forceinline__ double warp_fold(const double (&v)[NV]) {
     return keep;
 }
 
-// grid_allreduce_sym for kernels of few warps per CTA: v holds every thread's
-// own partials (at most 16 warps per CTA), the arrivals are spread over
-// AR_SUB counters on lines of their own as in grid_allreduce_df, and warp 0
-// alone adds the CTAs' partials (each lane's loads issued together), so that
-// an exchange costs two warp-wide folds of FP64 adds instead of two per warp.
-// Same bits in every CTA: fixed orders for a given launch shape.  `bar` holds
-// AR_SUB * 32 words, zero at launch; totals in every thread on return; false
-// on timeout.
+// The exchange of a grid all-reduce, run by one warp per CTA of a cooperative
+// launch: v holds the CTA's partials in lane 0; they are published, the CTA
+// announces itself (arrivals spread over AR_SUB counters on lines of their own
+// as in grid_allreduce_df, the wait bounded), and the warp adds all CTAs'
+// partials, each lane's loads issued together.  after_wait() runs once every
+// CTA has arrived, behind those loads.  Totals in every lane, the same bits in
+// every CTA; false on timeout (the error word is set).  `bar` holds
+// AR_SUB * 32 words, zero at launch; `gen` numbers the launch's calls.
 constexpr int AR_SUB = 16;
+template <int NV, class F>
+__device__ __forceinline__ bool grid_exchange(double (&v)[NV], double *part, unsigned gen, unsigned *bar, int *err,
+                                              long long limit_cycles, F &&after_wait) {
+    const int lane = threadIdx.x & 31;
+    double2 *half = reinterpret_cast<double2 *>(part + (size_t)(gen & 1u) * gridDim.x * AR_NV_MAX);
+    if (lane == 0) {
+        __stcg(half + blockIdx.x, make_double2(v[0], v[NV - 1]));
+        red_add_release(bar + 32 * (blockIdx.x % AR_SUB), 1u);
+    }
+    int lane_ok = 1;
+    if (lane < AR_SUB) {
+        const unsigned per = gridDim.x / AR_SUB + ((unsigned)lane < gridDim.x % AR_SUB ? 1u : 0u);
+        const unsigned target = (gen + 1u) * per;
+        const long long t0 = clock64();
+        while (ld_acquire(bar + 32 * lane) < target) {
+            if (clock64() - t0 > limit_cycles || *(volatile int *)err == (int)BA_ERR_TIMEOUT) {
+                lane_ok = 0;
+                break;
+            }
+        }
+    }
+    const bool ok = __all_sync(0xffffffffu, lane_ok) != 0;  // orders the other lanes' partial reads too
+    __syncwarp();
+    double acc[NV];
+#pragma unroll
+    for (int k = 0; k < NV; ++k) acc[k] = 0.0;
+    if (ok) {
+        double2 u[5];
+#pragma unroll
+        for (int q = 0; q < 5; ++q)
+            u[q] = lane + 32 * q < (int)gridDim.x ? __ldcg(half + lane + 32 * q) : make_double2(0.0, 0.0);
+        after_wait();
+#pragma unroll
+        for (int q = 0; q < 5; ++q) {
+            acc[0] += u[q].x;
+            if (NV == 2) acc[NV - 1] += u[q].y;
+        }
+        for (unsigned b0 = lane + 160; b0 < gridDim.x; b0 += 160) {
+#pragma unroll
+            for (int q = 0; q < 5; ++q)
+                u[q] = b0 + 32 * q < gridDim.x ? __ldcg(half + b0 + 32 * q) : make_double2(0.0, 0.0);
+#pragma unroll
+            for (int q = 0; q < 5; ++q) {
+                acc[0] += u[q].x;
+                if (NV == 2) acc[NV - 1] += u[q].y;
+            }
+        }
+    } else if (lane == 0) {
+        atomicExch(err, (int)BA_ERR_TIMEOUT);
+    }
+    const double tot = warp_fold<NV>(acc);
+    v[0] = __shfl_sync(0xffffffffu, tot, 0);
+    if (NV == 2) v[NV - 1] = __shfl_sync(0xffffffffu, tot, 16);
+    return ok;
+}
+
+// grid_allreduce_sym for kernels of few warps per CTA: v holds every thread's
+// own partials (at most 16 warps per CTA), and warp 0 alone runs the exchange,
+// so that a call costs two warp-wide folds of FP64 adds instead of two per
+// warp.  Totals in every thread; false on timeout.
 template <int NV>
 __device__ __forceinline__ bool grid_allreduce_w0(double (&v)[NV], double *part, unsigned gen, unsigned *bar,
                                                   int *err, long long limit_cycles) {
@@ -405,7 +465,6 @@ __device__ __forceinline__ bool grid_allreduce_w0(double (&v)[NV], double *part,
     __shared__ double s_tot[NV];
     __shared__ int s_ok;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    double2 *half = reinterpret_cast<double2 *>(part + (size_t)(gen & 1u) * gridDim.x * AR_NV_MAX);
     {
         const double t = warp_fold<NV>(v);
         if (lane == 0) s_w[w] = t;
@@ -418,48 +477,15 @@ __device__ __forceinline__ bool grid_allreduce_w0(double (&v)[NV], double *part,
 #pragma unroll
         for (int o = 8; o > 0; o >>= 1)
             if (o < nw) t += __shfl_xor_sync(0xffffffffu, t, o);
-        const double t1 = __shfl_sync(0xffffffffu, t, 16);
+        double x[NV];
+        x[NV - 1] = __shfl_sync(0xffffffffu, t, 16);
+        x[0] = t;
+        const bool ok = grid_exchange<NV>(x, part, gen, bar, err, limit_cycles, []() {});
         if (lane == 0) {
-            __stcg(half + blockIdx.x, make_double2(t, t1));
-            red_add_release(bar + 32 * (blockIdx.x % AR_SUB), 1u);
-        }
-        int lane_ok = 1;
-        if (lane < AR_SUB) {
-            const unsigned per = gridDim.x / AR_SUB + ((unsigned)lane < gridDim.x % AR_SUB ? 1u : 0u);
-            const unsigned target = (gen + 1u) * per;
-            const long long t0 = clock64();
-            while (ld_acquire(bar + 32 * lane) < target) {
-                if (clock64() - t0 > limit_cycles || *(volatile int *)err == (int)BA_ERR_TIMEOUT) {
-                    lane_ok = 0;
-                    break;
-                }
-            }
-        }
-        const bool ok = __all_sync(0xffffffffu, lane_ok) != 0;  // orders the other lanes' partial reads too
-        double acc[NV];
 #pragma unroll
-        for (int k = 0; k < NV; ++k) acc[k] = 0.0;
-        if (ok) {
-            for (unsigned b0 = lane; b0 < gridDim.x; b0 += 160) {
-                double2 u[5];
-#pragma unroll
-                for (int q = 0; q < 5; ++q)
-                    u[q] = b0 + 32 * q < gridDim.x ? __ldcg(half + b0 + 32 * q) : make_double2(0.0, 0.0);
-#pragma unroll
-                for (int q = 0; q < 5; ++q) {
-                    acc[0] += u[q].x;
-                    if (NV == 2) acc[NV - 1] += u[q].y;
-                }
-            }
-        }
-        __syncwarp();
-        const double tot = warp_fold<NV>(acc);
-        if (lane == 0) {
-            s_tot[0] = tot;
+            for (int k = 0; k < NV; ++k) s_tot[k] = x[k];
             s_ok = ok ? 1 : 0;
-            if (!ok) atomicExch(err, (int)BA_ERR_TIMEOUT);
         }
-        if (NV == 2 && lane == 16) s_tot[NV - 1] = tot;
     }
     __syncthreads();
 #pragma unroll
@@ -511,7 +537,15 @@ __device__ __forceinline__ void load6(const double *p, double (&v)[6]) {
 
 template <typename TV>
 __device__ __forceinline__ void block_apply(const TV (&Sv)[36], const TV (&x)[6], bool transposed, TV (&acc)[6]) {
-    if (!transposed) {
+    if constexpr (sizeof(TV) == 8) {
+        // a warp whose lanes hold entries of both forms runs one product, not
+        // two (36 FP64 instructions of 16-64 cycles against selects on the
+        // integer pipe); same sums in the same order
+#pragma unroll
+        for (int r = 0; r < 6; ++r)
+#pragma unroll
+            for (int c = 0; c < 6; ++c) acc[r] += (transposed ? Sv[6 * c + r] : Sv[6 * r + c]) * x[c];
+    } else if (!transposed) {
 #pragma unroll
         for (int r = 0; r < 6; ++r)
 #pragma unroll

@@ -416,6 +416,164 @@ __global__ void __launch_bounds__(256) k_pcg_persist(int n, const int *__restric
     }
 }
 
+// The same recurrence for FP64 systems of few cameras, S held in registers.
+// CTA c owns rows c R .. c R + R - 1 (R <= RES64_ROWS), `wpr` warps to a row, one
+// two-sided entry to a lane (already transposed where the entry asks for it,
+// so that no warp runs both forms of the product); lane 6 lr + a of warp 0
+// keeps y, r, d and a row of M^-1 of entry (lr, a) for the whole solve.  Only
+// z and d pass through memory (the neighbours' gather), and warp 0 alone runs
+// the two exchanges of an iteration; the gathers are issued as soon as the
+// second has seen every CTA arrive.
+// What bounds it: FP64 warp instructions of 64 cycles each for one warp (16
+// with all four of an SM's schedulers busy) - 50 per row half, about 60 in the
+// scalar chain - and two grid exchanges of about 1.2 us.  Against
+// k_pcg_persist (which re-reads S and passes r and q through L2 each
+// iteration): 14 -> 9.2 us per iteration at 200 cameras, 12 -> 7.1 at 50.
+constexpr int RES64_ROWS = 5;   // 6 R owner lanes in one warp
+constexpr int RES64_WARPS = 8;  // warps per CTA at most
+__global__ void __launch_bounds__(32 * RES64_WARPS, 1)
+    k_pcg64_res(int n, int rows, int wpr, const int *__restrict__ tw_ptr, const int2 *__restrict__ tw_ent,
+                const double *__restrict__ S, const double *__restrict__ Minv, double *__restrict__ y,
+                const double *__restrict__ r0, double *z, double *d0, double *d1, DevScalars *sc, double *red,
+                unsigned *bar, long long limit_cycles) {
+    __shared__ double s_part[RES64_WARPS][6];
+    __shared__ double s_beta;
+    __shared__ int s_ctl;  // 0 go on, 1 leave
+    if (sc->done) return;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int comp = fold6_comp(lane);
+    const bool writes = fold6_owner(lane);
+    // this lane's entry
+    const int lrow = w / wpr, irow = blockIdx.x * rows + lrow;
+    int j = 0;
+    double Sv[36];
+#pragma unroll
+    for (int q = 0; q < 36; ++q) Sv[q] = 0.0;
+    if (lrow < rows && irow < n) {
+        const int t = __ldg(tw_ptr + irow) + 32 * (w - lrow * wpr) + lane;
+        if (t < __ldg(tw_ptr + irow + 1)) {
+            const int2 e = __ldg(tw_ent + t);
+            double B[36];
+            load_block<double, double>(S + (int64_t)(e.x & 0x7fffffff) * BW, B);
+            j = e.y;
+#pragma unroll
+            for (int r = 0; r < 6; ++r)
+#pragma unroll
+                for (int c = 0; c < 6; ++c) Sv[6 * r + c] = e.x < 0 ? B[6 * c + r] : B[6 * r + c];
+        }
+    }
+    // warp 0: lane o owns entry (o / 6, o % 6) of the CTA's rows
+    const int ol = lane / 6, oc = lane - 6 * ol, oi = blockIdx.x * rows + ol;
+    const bool own = w == 0 && lane < 6 * rows && oi < n;
+    double rv = 0.0, yv = 0.0, zv = 0.0, dv = 0.0, Mr[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    if (own) {
+        rv = r0[6 * oi + oc];
+        zv = __ldcg(z + 6 * oi + oc);
+#pragma unroll
+        for (int c = 0; c < 6; ++c) Mr[c] = __ldg(Minv + 36 * (int64_t)oi + 6 * oc + c);
+    }
+    double rz = sc->rz, beta = 0.0;
+    const double thr = sc->tol2 * sc->rr0;
+    const int max_iters = sc->max_iters;
+    unsigned gen = 0;
+    double zj[6], dj[6];
+    load6(z + 6 * j, zj);
+    load6(d0 + 6 * j, dj);
+    for (int it = 0;;) {
+        double *dnew = (it & 1) ? d0 : d1;
+        double x[6], acc[6];
+#pragma unroll
+        for (int c = 0; c < 6; ++c) x[c] = zj[c] + beta * dj[c];
+#pragma unroll
+        for (int r = 0; r < 6; ++r) {
+            acc[r] = Sv[6 * r] * x[0];
+#pragma unroll
+            for (int c = 1; c < 6; ++c) acc[r] += Sv[6 * r + c] * x[c];
+        }
+        const double pr = warp_fold6(acc, lane);
+        if (writes) s_part[w][comp] = pr;
+        __syncthreads();
+        if (w == 0) {
+            double q = 0.0, v1[1] = {0.0};
+            if (own) {
+                q = s_part[ol * wpr][oc];
+                for (int p = 1; p < wpr; ++p) q += s_part[ol * wpr + p][oc];
+                dv = zv + beta * dv;
+                dnew[6 * oi + oc] = dv;
+                v1[0] = dv * q;
+            }
+            v1[0] = warp_fold<1>(v1);
+            bool ok = grid_exchange<1>(v1, red, gen++, bar, &sc->err, limit_cycles, []() {});
+            const double pAp = v1[0];
+            int ctl = 0;
+            if (!ok || !(pAp > 0.0)) {
+                ctl = 1;
+                if (ok && blockIdx.x == 0 && lane == 0) {
+                    sc->err = (int)BA_ERR_NOT_SPD;
+                    sc->done = 1;
+                    sc->iters = it;
+                }
+            }
+            if (ctl == 0) {
+                const double alpha = rz / pAp;
+                rv -= alpha * q;
+                yv += alpha * dv;
+                double zn = 0.0;
+                const int l6 = lane < 30 ? 6 * ol : 0;
+#pragma unroll
+                for (int c = 0; c < 6; ++c) zn += Mr[c] * __shfl_sync(0xffffffffu, rv, l6 + c);
+                zv = zn;
+                if (own) z[6 * oi + oc] = zv;
+                double v2[2] = {rv * zv, rv * rv};
+                const double f = warp_fold<2>(v2);
+                v2[0] = f;
+                v2[1] = __shfl_sync(0xffffffffu, f, 16);
+                if (lane == 0) s_ctl = 0;
+                ok = grid_exchange<2>(v2, red, gen++, bar, &sc->err, limit_cycles, [&]() {
+                    __syncthreads();  // the other warps' gathers start here
+                    load6(z + 6 * j, zj);
+                    load6(dnew + 6 * j, dj);
+                });
+                ++it;
+                if (!ok) {
+                    ctl = 2;  // the others still wait at the first barrier
+                } else if (v2[1] <= thr || it >= max_iters) {
+                    ctl = 1;
+                    if (blockIdx.x == 0 && lane == 0) {
+                        sc->iters = it;
+                        sc->rr = v2[1];
+                        sc->rz = v2[0];
+                        sc->done = 1;
+                    }
+                } else {
+                    beta = v2[0] / rz;
+                    rz = v2[0];
+                }
+                if (lane == 0) {
+                    s_ctl = ctl;
+                    s_beta = beta;
+                }
+                if (ctl == 2) __syncthreads();
+                __syncthreads();
+                if (ctl) break;
+                continue;
+            }
+            if (lane == 0) s_ctl = 1;
+            __syncthreads();
+            __syncthreads();
+            break;
+        }
+        __syncthreads();
+        load6(z + 6 * j, zj);
+        load6(dnew + 6 * j, dj);
+        __syncthreads();
+        if (s_ctl) break;
+        beta = s_beta;
+        ++it;
+    }
+    if (own) y[6 * oi + oc] = yv;
+}
+
 // r64 = b - q64 (q64 = S x64 from the FP64 SpMV), q64 reset; ||r64||^2, ||b||^2.
 template <typename T>
 __global__ void __launch_bounds__(256) k_resid_fin(int n, const T *__restrict__ b, double *q64, double *r64, DevScalars *sc,
@@ -1180,6 +1338,28 @@ static cudaError_t ensure_ar_bar(ba_problem *p) {
     return cudaSuccess;
 }
 
+// The register-resident FP64 loop, where its CTAs cover the system: at most
+// RES64_ROWS rows per SM, one lane per entry of the longest row.
+static int res64_wpr(const ba_problem *p) { return (p->hs.max_row_ent + 31) / 32; }
+static bool res64_fits(const ba_problem *p, int n_sm) {
+    const int rows = (p->n + n_sm - 1) / n_sm;
+    return p->hs.max_row_ent > 0 && rows <= RES64_ROWS && rows * res64_wpr(p) <= RES64_WARPS;
+}
+static cudaError_t launch_res64(ba_problem *p, int n_sm, long long limit) {
+    int n = p->n, rows = (n + n_sm - 1) / n_sm, wpr = res64_wpr(p);
+    const int grid = (n + rows - 1) / rows;
+    const int *twp = p->tw_ptr;
+    const int2 *twe = p->tw_ent;
+    const double *S = (const double *)p->sv.S, *Mi = (const double *)p->sv.Minv, *r = (const double *)p->sv.pv[1];
+    double *y = (double *)p->sv.pv[0], *z = (double *)p->sv.pv[2], *d0 = (double *)p->sv.pv[3],
+           *d1 = (double *)p->sv.pv[4];
+    DevScalars *sc = p->sc;
+    double *red = p->red;
+    unsigned *bar = p->ar_bar;
+    void *args[] = {&n, &rows, &wpr, &twp, &twe, &S, &Mi, &y, &r, &z, &d0, &d1, &sc, &red, &bar, &limit};
+    return cudaLaunchCooperativeKernel((const void *)k_pcg64_res, dim3(grid), dim3(32 * rows * wpr), args, 0, p->st);
+}
+
 template <typename T, bool ONCE>
 static cudaError_t pcg_loop_T(ba_problem *p) {
     // Warps per CTA: the rows are spread over every SM first, then over the
@@ -1203,6 +1383,8 @@ static cudaError_t pcg_loop_T(ba_problem *p) {
     if ((e = cudaMemsetAsync(p->ar_bar, test_limit > 0 ? 0xFF : 0, AR_SUB * 32 * sizeof(unsigned), p->st)) !=
         cudaSuccess)
         return e;
+    const long long limit_cycles = test_limit > 0 ? test_limit : 4000000000LL;  // ~2 s of SM clock per wait
+    if (sizeof(T) == 8 && res64_fits(p, n_sm)) return launch_res64(p, n_sm, limit_cycles);
     int n = p->n;
     const int *twp = p->tw_ptr, *rp = p->row_ptr, *cl = p->col;
     const int2 *twe = p->tw_ent;
@@ -1212,7 +1394,7 @@ static cudaError_t pcg_loop_T(ba_problem *p) {
     DevScalars *sc = p->sc;
     double *red = p->red;
     unsigned *bar = p->ar_bar;
-    long long limit = test_limit > 0 ? test_limit : 4000000000LL;  // ~2 s of SM clock per barrier wait
+    long long limit = limit_cycles;
     void *args[] = {&n, &twp, &twe, &rp, &cl, &S, &Mi, &y, &r, &r1, &z, &d0, &d1, &q, &q1, &sc, &red, &bar, &limit};
     return cudaLaunchCooperativeKernel((const void *)k_pcg_persist<T, ONCE>, dim3(grid), dim3(32 * warps), args, 0, p->st);
 }
