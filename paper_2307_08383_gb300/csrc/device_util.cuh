@@ -454,33 +454,37 @@ __device__ __forceinline__ bool grid_exchange(double (&v)[NV], double *part, uns
     return ok;
 }
 
-// grid_allreduce_sym for kernels of few warps per CTA: v holds every thread's
-// own partials (at most 16 warps per CTA), and warp 0 alone runs the exchange,
-// so that a call costs two warp-wide folds of FP64 adds instead of two per
-// warp.  Totals in every thread; false on timeout.
-template <int NV>
+// grid_allreduce_sym for kernels of few warps per CTA: v holds the own
+// partials of every thread of the first nwv warps (at most 16 warps per CTA),
+// and warp 0 alone runs the exchange, so that a call costs one warp-wide fold
+// of FP64 adds per such warp and two in warp 0.  Warp 0 then runs
+// fin(totals, ok) (for what only one warp needs to compute) before the CTA's
+// other warps go on.  Totals in every thread; false on timeout.
+template <int NV, class F>
 __device__ __forceinline__ bool grid_allreduce_w0(double (&v)[NV], double *part, unsigned gen, unsigned *bar,
-                                                  int *err, long long limit_cycles) {
+                                                  int *err, long long limit_cycles, int nwv, F &&fin) {
     __shared__ double s_w[NV * 16];
     __shared__ double s_tot[NV];
     __shared__ int s_ok;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (w < nwv) {
         const double t = warp_fold<NV>(v);
         if (lane == 0) s_w[w] = t;
         if (NV == 2 && lane == 16) s_w[16 * (NV - 1) + w] = t;
     }
-    __syncthreads();
+    if (nwv > 1) __syncthreads();
+    else __syncwarp();
     if (w == 0) {
         const int l = lane & 15;
-        double t = l < nw ? s_w[(NV == 2 ? lane & 16 : 0) + l] : 0.0;
+        double t = l < nwv ? s_w[(NV == 2 ? lane & 16 : 0) + l] : 0.0;
 #pragma unroll
         for (int o = 8; o > 0; o >>= 1)
-            if (o < nw) t += __shfl_xor_sync(0xffffffffu, t, o);
+            if (o < nwv) t += __shfl_xor_sync(0xffffffffu, t, o);
         double x[NV];
         x[NV - 1] = __shfl_sync(0xffffffffu, t, 16);
-        x[0] = t;
+        x[0] = __shfl_sync(0xffffffffu, t, 0);
         const bool ok = grid_exchange<NV>(x, part, gen, bar, err, limit_cycles, []() {});
+        fin(x, ok);
         if (lane == 0) {
 #pragma unroll
             for (int k = 0; k < NV; ++k) s_tot[k] = x[k];
@@ -491,6 +495,12 @@ __device__ __forceinline__ bool grid_allreduce_w0(double (&v)[NV], double *part,
 #pragma unroll
     for (int k = 0; k < NV; ++k) v[k] = s_tot[k];
     return s_ok != 0;
+}
+template <int NV>
+__device__ __forceinline__ bool grid_allreduce_w0(double (&v)[NV], double *part, unsigned gen, unsigned *bar,
+                                                  int *err, long long limit_cycles) {
+    return grid_allreduce_w0<NV>(v, part, gen, bar, err, limit_cycles, (int)(blockDim.x >> 5),
+                                 [](const double (&)[NV], bool) {});
 }
 
 // ---- 6x6 block SpMV helpers (BSMC and the full-block formats) ----

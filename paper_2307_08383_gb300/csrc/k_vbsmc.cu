@@ -15,6 +15,7 @@
 #include <cmath>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "device_util.cuh"
@@ -22,102 +23,489 @@
 
 namespace ba {
 
-// Warp-per-row product: lane a + 16 h (a < 16 the output component, h the
-// parity of the entries it takes) sums S_ij x_j over its entries; the halves
-// are joined by one shuffle.  Each two-sided entry is one 16-byte record
-// (value offset lo / hi, vector offset of j, c_j << 1 | transposed), and a
-// lane loads its whole block row (or column) and the c_j values of x with
-// independent predicated loads before the FMAs, so an entry costs two
-// dependent memory round trips, not one per column.  (Staging each block in
-// shared memory with coalesced loads first measured 1.9x slower: the copy,
-// the warp barrier and the shared reads chain per entry.)  gx(idx) returns x
-// at vector index idx; lanes a < c_i of half 0 call out(idx, (S x)_idx).
-template <typename T, class GX, class OUT>
-__device__ __forceinline__ void vb_row(int i, const int *__restrict__ cdim, const int *__restrict__ off,
-                                       const int *__restrict__ tw_ptr, const int4 *__restrict__ tw_info,
-                                       const T *__restrict__ val, GX gx, OUT out) {
-    const int lane = threadIdx.x & 31, a = lane & 15, h = lane >> 4;
-    const int ci = __ldg(cdim + i);
+// One part of a row's product.  The warp's lanes form G = min(32 / c_i, 5)
+// groups of c_i lanes; group g takes entries e0 + g, e0 + g + step, ... below
+// e1, its lane a component a of the row.  The group stages the entry's c_j
+// values of x (each formed once, gx(index)) in the warp's shared memory sx and
+// holds the lane's row (or column) of the block in registers, so an entry
+// costs c_j multiply-adds per lane and one evaluation of x per value.  An
+// entry's record rec[e] is (value offset lo / hi, vector offset of j,
+// c_j << 1 | transposed).  PACKED: every block lies in shared memory stored by
+// columns of this row's form (element (a, c) at offset + c c_i + a).
+// Lanes 0 .. c_i - 1 return the part's sum.
+// (The first version gave every entry 16 lanes, evaluated x in each of them
+// and ran 16 columns whatever c_j: in FP64, where a warp instruction takes 16
+// cycles of its SM, 32 per pair of entries instead of 12 at c = 11.)
+constexpr int VB_GROUPS = 5;
+// One entry's row (or column) of values in registers, zero beyond c_j.
+template <typename T>
+__device__ __forceinline__ void vb_load(int ci, int a, const int4 in, const T *__restrict__ val, T (&bv)[BA_VB_CMAX]) {
+    const int cj = in.w >> 1;
+    const T *Bp = val + ((int64_t)(uint32_t)in.x | ((int64_t)in.y << 32)) + ((in.w & 1) ? a : a * cj);
+    const int stride = (in.w & 1) ? ci : 1;
+#pragma unroll
+    for (int c = 0; c < BA_VB_CMAX; ++c) {
+        bv[c] = T(0);
+        if (c < cj) bv[c] = __ldg(Bp + c * stride);
+    }
+}
+// The groups' sums joined: lanes 0 .. c_i - 1 return the part's sum.
+template <typename T>
+__device__ __forceinline__ T vb_join(T acc, int ci, int G, int a) {
+    T tot = acc;
+    for (int h = 1; h < G; ++h) tot += __shfl_sync(0xffffffffu, acc, (a + h * ci) & 31);
+    return tot;
+}
+template <typename T, class GX>
+__device__ __forceinline__ T vb_part(int ci, int e0, int e1, int step, const int4 *__restrict__ rec,
+                                     const T *__restrict__ val, T *sx, GX gx) {
+    const int lane = threadIdx.x & 31;
+    const int G = min(32 / ci, VB_GROUPS), g = lane / ci, a = lane - g * ci;
     T acc = T(0);
-    const int e1 = __ldg(tw_ptr + i + 1);
-    for (int e = __ldg(tw_ptr + i) + h; e < e1; e += 2) {
-        const int4 in = __ldg(tw_info + e);
-        const int64_t vo = (int64_t)(uint32_t)in.x | ((int64_t)in.y << 32);
-        const int oj = in.z, cj = in.w >> 1;
-        const T *B = val + vo;
-        // element (a, c) of this row's block: B[c * ci + a] if transposed, else B[a * cj + c]
-        const int stride = (in.w & 1) ? ci : 1, base = (in.w & 1) ? a : a * cj;
-        T bv[BA_VB_CMAX], xv[BA_VB_CMAX];
+    for (int t = e0; t < e1; t += step) {
+        const int e = t + g;
+        int4 in = make_int4(0, 0, 0, 0);
+        if (g < G && e < e1) in = __ldg(rec + e);
+        const int cj = in.w >> 1;
+        T bv[BA_VB_CMAX];
+        vb_load<T>(ci, a, in, val, bv);
+        for (int c = a; c < cj; c += ci) sx[BA_VB_CMAX * g + c] = gx(in.z + c);
+        const int cm = (int)__reduce_max_sync(0xffffffffu, (unsigned)cj);
+        __syncwarp();
 #pragma unroll
         for (int c = 0; c < BA_VB_CMAX; ++c) {
-            const bool on = c < cj && a < ci;
-            bv[c] = on ? __ldg(B + base + c * stride) : T(0);
-            xv[c] = c < cj ? gx(oj + c) : T(0);
+            if (c >= cm) break;
+            acc = fma(bv[c], c < cj ? sx[BA_VB_CMAX * g + c] : T(0), acc);
         }
-#pragma unroll
-        for (int c = 0; c < BA_VB_CMAX; ++c) acc += bv[c] * xv[c];
+        __syncwarp();
     }
-    acc += __shfl_xor_sync(0xffffffffu, acc, 16);
-    if (h == 0 && a < ci) out(__ldg(off + i) + a, acc);
+    return vb_join<T>(acc, ci, G, a);
+}
+// The same with every entry's x already in shared memory (sx, 16 values per
+// entry).  PACKED: the values too, each block by columns of this row's form
+// (element (a, c) at in.x + c c_i + a); otherwise the next pass's values are
+// loaded while this one's are used.
+template <typename T, bool PACKED>
+__device__ __forceinline__ T vb_own_part(int ci, int e0, int e1, int step, const int4 *rec, const T *val,
+                                         const T *sx) {
+    const int lane = threadIdx.x & 31;
+    const int G = min(32 / ci, VB_GROUPS), g = lane / ci, a = lane - g * ci;
+    T acc = T(0);
+    // all of a pass's loads are issued before its multiply-adds (columns beyond
+    // c_j read as zeros; FP32 multiplies them, FP64 stops at the warp's
+    // largest c_j)
+    auto apply = [&](const T(&bv)[BA_VB_CMAX], const T(&xv)[BA_VB_CMAX], int cj) {
+        if constexpr (sizeof(T) == 8) {
+            const int cm = (int)__reduce_max_sync(0xffffffffu, (unsigned)cj);
+#pragma unroll
+            for (int c = 0; c < BA_VB_CMAX; ++c) {
+                if (c >= cm) break;
+                acc = fma(bv[c], xv[c], acc);
+            }
+        } else {
+#pragma unroll
+            for (int c = 0; c < BA_VB_CMAX; ++c) acc = fma(bv[c], xv[c], acc);
+        }
+    };
+    auto load_x = [&](bool on, int e, T(&xv)[BA_VB_CMAX]) {
+        using V = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
+        constexpr int N = 16 / (int)sizeof(T);
+        const V *xp = reinterpret_cast<const V *>(sx + BA_VB_CMAX * e);
+#pragma unroll
+        for (int k = 0; k < BA_VB_CMAX / N; ++k) {
+            V v;
+            memset(&v, 0, sizeof(V));
+            if (on) v = xp[k];
+            memcpy(&xv[N * k], &v, sizeof(V));
+        }
+    };
+    if (PACKED) {
+        for (int t = e0; t < e1; t += step) {
+            const int e = t + g;
+            const bool on = g < G && e < e1;
+            int4 in = make_int4(0, 0, 0, 0);
+            if (on) in = rec[e];
+            const int cj = in.w >> 1;
+            const T *Bp = val + in.x + a;
+            T bv[BA_VB_CMAX], xv[BA_VB_CMAX];
+#pragma unroll
+            for (int c = 0; c < BA_VB_CMAX; ++c) {
+                bv[c] = T(0);
+                if (c < cj) bv[c] = Bp[c * ci];
+            }
+            load_x(on, e, xv);
+            apply(bv, xv, cj);
+        }
+    } else {
+        T bn[BA_VB_CMAX];
+        int4 in = make_int4(0, 0, 0, 0);
+        if (g < G && e0 + g < e1) in = rec[e0 + g];
+        vb_load<T>(ci, a, in, val, bn);
+        for (int t = e0; t < e1; t += step) {
+            T bv[BA_VB_CMAX], xv[BA_VB_CMAX];
+#pragma unroll
+            for (int c = 0; c < BA_VB_CMAX; ++c) bv[c] = bn[c];
+            const int cj = in.w >> 1;
+            const bool on = g < G && t + g < e1;
+            in = make_int4(0, 0, 0, 0);
+            if (g < G && t + step + g < e1) in = rec[t + step + g];
+            vb_load<T>(ci, a, in, val, bn);
+            load_x(on, t + g, xv);
+            apply(bv, xv, cj);
+        }
+    }
+    return vb_join<T>(acc, ci, G, a);
 }
 
+// y = S x: `wpr` warps of the CTA's eight to a row, so that systems of few
+// rows still fill the SMs with loads in flight; the parts of a row are added
+// in order.
 template <typename T>
-__global__ void __launch_bounds__(256) k_vb_spmv(int n, const int *__restrict__ cdim, const int *__restrict__ off,
-                                                 const int *__restrict__ tw_ptr, const int4 *__restrict__ tw_info,
-                                                 const T *__restrict__ val, const T *__restrict__ x, T *__restrict__ y) {
-    const int nw = (int)(((int64_t)gridDim.x * blockDim.x) >> 5);
-    for (int i = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5); i < n; i += nw)
-        vb_row<T>(i, cdim, off, tw_ptr, tw_info, val, [&](int idx) { return __ldg(x + idx); },
-                  [&](int idx, T v) { y[idx] = v; });
-}
-
-// M^-1 per camera (a thread each): FP64 Cholesky of the diagonal block, then
-// its inverse column by column; a block that is not positive definite sets
-// BA_ERR_NOT_SPD and leaves zeros.
-template <typename T>
-__global__ void k_vb_minv(int n, const int *__restrict__ cdim, const int *__restrict__ row_ptr,
-                          const int64_t *__restrict__ boff, const T *__restrict__ val, const int64_t *__restrict__ moff,
-                          T *__restrict__ Minv, int *err) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int c = cdim[i];
-    const T *D = val + boff[row_ptr[i]];
-    T *M = Minv + moff[i];
-    double L[BA_VB_CMAX * BA_VB_CMAX];
-    bool ok = true;
-    for (int r = 0; r < c; ++r)
-        for (int q = 0; q <= r; ++q) {
-            double s = 0.5 * ((double)D[r * c + q] + (double)D[q * c + r]);
-            for (int k = 0; k < q; ++k) s -= L[r * BA_VB_CMAX + k] * L[q * BA_VB_CMAX + k];
-            if (r == q) {
-                if (!(s > 0.0)) {
-                    ok = false;
-                    s = 1.0;
-                }
-                L[r * BA_VB_CMAX + r] = sqrt(s);
-            } else {
-                L[r * BA_VB_CMAX + q] = s / L[q * BA_VB_CMAX + q];
+__global__ void __launch_bounds__(256) k_vb_spmv(int n, int wpr, const int *__restrict__ cdim,
+                                                 const int *__restrict__ off, const int *__restrict__ tw_ptr,
+                                                 const int4 *__restrict__ tw_info, const T *__restrict__ val,
+                                                 const T *__restrict__ x, T *__restrict__ y) {
+    __shared__ T s_x[8][VB_GROUPS * BA_VB_CMAX];
+    __shared__ T s_part[8][BA_VB_CMAX];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int rows = 8 / wpr, lr = w / wpr, part = w - lr * wpr;
+    for (int base = blockIdx.x * rows; base < n; base += gridDim.x * rows) {
+        const int i = base + lr;
+        int ci = 1;
+        if (i < n) {
+            ci = __ldg(cdim + i);
+            const int G = min(32 / ci, VB_GROUPS), e0 = __ldg(tw_ptr + i), e1 = __ldg(tw_ptr + i + 1);
+            const T t = vb_part<T>(ci, e0 + part * G, e1, wpr * G, tw_info, val, s_x[w],
+                                          [&](int k) { return __ldg(x + k); });
+            if (wpr == 1) {
+                if (lane < ci) y[__ldg(off + i) + lane] = t;
+            } else if (lane < ci) {
+                s_part[w][lane] = t;
             }
         }
-    if (!ok) {
-        atomicExch(err, (int)BA_ERR_NOT_SPD);
-        for (int k = 0; k < c * c; ++k) M[k] = T(0);
+        if (wpr > 1) {
+            __syncthreads();
+            if (part == 0 && i < n && lane < ci) {
+                T t = s_part[w][lane];
+                for (int q = 1; q < wpr; ++q) t += s_part[w + q][lane];
+                y[__ldg(off + i) + lane] = t;
+            }
+            __syncthreads();
+        }
+    }
+}
+
+// M^-1 per camera, sixteen lanes each, in FP64: lane r holds row r of the
+// (symmetrised) diagonal block, the Cholesky factor is formed column by column
+// (right-looking, the pivot column passed by shuffles), then lane q solves for
+// column q of the inverse.  A block that is not positive definite sets
+// BA_ERR_NOT_SPD and leaves zeros.  (A thread per camera, its factor in local
+// memory, was one serial FP64 chain: 260 us at 990 and at 120 cameras of c =
+// 11, against 21 us.)
+template <typename T>
+__global__ void __launch_bounds__(64) k_vb_minv(int n, const int *__restrict__ cdim, const int *__restrict__ row_ptr,
+                                                const int64_t *__restrict__ boff, const T *__restrict__ val,
+                                                const int64_t *__restrict__ moff, T *__restrict__ Minv, int *err) {
+    constexpr unsigned FULL = 0xffffffffu;
+    constexpr int CM = BA_VB_CMAX;
+    const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 4, r = threadIdx.x & 15;
+    const int c = i < n ? cdim[i] : 0;
+    const int cm = (int)__reduce_max_sync(FULL, (unsigned)c);
+    const T *D = val + (i < n ? boff[row_ptr[i]] : 0);
+    double A[CM], invd = 1.0;
+#pragma unroll
+    for (int q = 0; q < CM; ++q)
+        A[q] = r < c && q < c ? 0.5 * ((double)D[r * c + q] + (double)D[q * c + r]) : 0.0;
+    bool ok = true;
+#pragma unroll
+    for (int q = 0; q < CM; ++q) {
+        if (q >= cm) break;
+        double p = __shfl_sync(FULL, A[q], q, 16);
+        if (!(p > 0.0)) {
+            ok = ok && q >= c;
+            p = 1.0;
+        }
+        const double d = sqrt(p), inv = 1.0 / d;
+        if (r == q) invd = inv;
+        A[q] = r == q ? d : A[q] * inv;
+#pragma unroll
+        for (int k = q + 1; k < CM; ++k) {
+            if (k >= cm) break;
+            A[k] -= A[q] * __shfl_sync(FULL, A[q], k, 16);  // rows r >= k of column k are meant
+        }
+    }
+    // column r of (L L^T)^-1: forward, then backward substitution on e_r
+    double x[CM];
+#pragma unroll
+    for (int q = 0; q < CM; ++q) {
+        x[q] = 0.0;
+        if (q < cm) {
+            double s = r == q ? 1.0 : 0.0;
+#pragma unroll
+            for (int k = 0; k < q; ++k) s -= __shfl_sync(FULL, A[k], q, 16) * x[k];
+            x[q] = s * __shfl_sync(FULL, invd, q, 16);
+        }
+    }
+#pragma unroll
+    for (int q = CM - 1; q >= 0; --q) {
+        if (q < cm) {
+            double s = x[q];
+#pragma unroll
+            for (int k = q + 1; k < CM; ++k)
+                if (k < cm) s -= __shfl_sync(FULL, A[q], k, 16) * x[k];
+            x[q] = s * __shfl_sync(FULL, invd, q, 16);
+        }
+    }
+    if (!ok && r == 0) atomicExch(err, (int)BA_ERR_NOT_SPD);
+    if (r < c) {
+        T *M = Minv + moff[i];
+#pragma unroll
+        for (int q = 0; q < CM; ++q)
+            if (q < c) M[q * c + r] = ok ? (T)x[q] : T(0);
+    }
+}
+
+// The PCG of Sec. 3.2 with a CTA owning a contiguous run of block rows: `wpr`
+// warps share a row's product (units of row and part, taken round-robin by the
+// CTA's warps), and thread t keeps y, r, z, d and its row of M^-1 of the CTA's
+// t-th vector entry in registers for the whole solve; only z and d pass
+// through memory; the neighbours' d is gathered once per iteration into shared
+// memory.  The entries' records, and with PACKED the values too (by columns, so
+// the lanes of a group read consecutive words), are copied there once.  Two
+// grid exchanges per iteration, run by one warp, which also forms alpha and
+// beta; every wait is bounded (BA_ERR_TIMEOUT).
+// What bounds it: in FP64 the SM's FP64 issue (one warp instruction per 16
+// cycles), spread over every SM and its four schedulers; in FP32 the two
+// exchanges and the reads of S.  Against one warp per row on n / 8 SMs and
+// vectors in memory, c = 11, us per iteration: FP64 61.7 -> 10.9 at 120 cameras,
+// 115 -> 50 at 1,984 (values in L2); FP32 32 -> 10.3 at 120, 33.4 -> 13.7 at
+// 990 (22 with the neighbours' values gathered pass by pass), 38.7 -> 22.5 at
+// 1,984 (values in L2).
+struct VbPlan {
+    int rows, wpr, max_ent;  // rows per CTA; warps per row; longest entry list of a CTA
+    int64_t max_val;         // PACKED: largest value count of a CTA
+};
+template <typename T>
+__host__ __device__ constexpr size_t vb_own_smem(int rows, int wpr, int max_ent, int64_t max_val, int threads) {
+    return (size_t)max_ent * sizeof(int4) +
+           ((size_t)max_val + (size_t)rows * wpr * BA_VB_CMAX + (size_t)max_ent * BA_VB_CMAX + threads) * sizeof(T) +
+           (size_t)(2 * rows + 2) * sizeof(int);
+}
+template <typename T>
+__host__ __device__ constexpr int vb_own_threads() {
+    return sizeof(T) == 4 ? 512 : 256;
+}
+template <typename T, bool PACKED>
+__global__ void __launch_bounds__(vb_own_threads<T>(), 1)
+    k_vb_pcg_own(int n, VbPlan pl, const int *__restrict__ cdim, const int *__restrict__ off,
+                 const int *__restrict__ ent_cam, const int *__restrict__ tw_ptr, const int4 *__restrict__ tw_info,
+                 const T *__restrict__ val, const int64_t *__restrict__ moff, const T *__restrict__ Minv,
+                 const T *__restrict__ b, T *y, T *z, T *d0, T *d1, VbScalars *sc, double *red, unsigned *bar,
+                 long long limit_cycles) {
+    extern __shared__ __align__(16) unsigned char sm_raw[];
+    __shared__ double s_ab;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, W = blockDim.x >> 5;
+    const int row0 = blockIdx.x * pl.rows, R = min(pl.rows, n - row0);
+    int4 *s_rec = reinterpret_cast<int4 *>(sm_raw);
+    // s_x is read by 16-byte loads: it follows the 16-byte records, and its
+    // stride of BA_VB_CMAX values is a multiple of 16 bytes; the rest is read
+    // by single values
+    T *s_x = reinterpret_cast<T *>(s_rec + pl.max_ent);
+    T *s_part = s_x + (size_t)pl.max_ent * BA_VB_CMAX;
+    T *s_r = s_part + (size_t)pl.rows * pl.wpr * BA_VB_CMAX;
+    T *s_val = s_r + blockDim.x;
+    int *s_e = reinterpret_cast<int *>(s_val + pl.max_val), *s_c = s_e + pl.rows + 1;
+    const int t0 = __ldg(tw_ptr + row0), ne = __ldg(tw_ptr + row0 + R) - t0;
+    for (int q = threadIdx.x; q <= R; q += blockDim.x) {
+        s_e[q] = __ldg(tw_ptr + row0 + q) - t0;
+        if (q < R) s_c[q] = __ldg(cdim + row0 + q);
+    }
+    for (int q = threadIdx.x; q < ne; q += blockDim.x) s_rec[q] = __ldg(tw_info + t0 + q);
+    __syncthreads();
+    if (PACKED) {
+        // packed offsets (warp 0, running sum of the blocks' sizes), then the
+        // values by columns, a warp per entry
+        if (w == 0) {
+            int base = 0, lr = 0;
+            for (int q0 = 0; q0 < ne; q0 += 32) {
+                const int q = q0 + lane;
+                int sz = 0;
+                if (q < ne) {
+                    while (q >= s_e[lr + 1]) ++lr;
+                    sz = s_c[lr] * (s_rec[q].w >> 1);
+                }
+                int inc = sz;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int u = __shfl_up_sync(0xffffffffu, inc, o);
+                    if (lane >= o) inc += u;
+                }
+                // the offset rides in w's upper bits until the values are copied
+                if (q < ne) s_rec[q].w |= (base + inc - sz) << 8;
+                base += __shfl_sync(0xffffffffu, inc, 31);
+            }
+        }
+        __syncthreads();
+        for (int q = w; q < ne; q += W) {
+            int lr = 0;
+            while (q >= s_e[lr + 1]) ++lr;
+            const int ci = s_c[lr];
+            const int4 in = s_rec[q];
+            const int cj = (in.w & 0xff) >> 1, po = in.w >> 8;
+            const T *B = val + ((int64_t)(uint32_t)in.x | ((int64_t)in.y << 32));
+            for (int k = lane; k < ci * cj; k += 32) {
+                const int c = k / ci, a = k - c * ci;
+                s_val[po + k] = (in.w & 1) ? __ldg(B + k) : __ldg(B + a * cj + c);
+            }
+            __syncwarp();
+            if (lane == 0) s_rec[q] = make_int4(po, 0, in.z, in.w & 0xff);
+        }
+        __syncthreads();
+    }
+    // this thread's vector entry
+    const int v0 = __ldg(off + row0), NE = __ldg(off + row0 + R) - v0;
+    const int nwv = (NE + 31) >> 5;
+    const bool own = (int)threadIdx.x < NE;
+    const int e = v0 + threadIdx.x;
+    int lrow = 0, comp = 0, cown = 0;
+    T Mr[BA_VB_CMAX], rv = T(0), yv = T(0), zv = T(0), dv = T(0);
+#pragma unroll
+    for (int k = 0; k < BA_VB_CMAX; ++k) Mr[k] = T(0);
+    if (own) {
+        const int i = __ldg(ent_cam + e);
+        lrow = i - row0;
+        comp = e - __ldg(off + i);
+        cown = __ldg(cdim + i);
+        const T *M = Minv + __ldg(moff + i) + (int64_t)comp * cown;
+#pragma unroll
+        for (int k = 0; k < BA_VB_CMAX; ++k)
+            if (k < cown) Mr[k] = __ldg(M + k);
+        rv = __ldg(b + e);
+        s_r[threadIdx.x] = rv;
+        d0[e] = T(0);
+    }
+    __syncthreads();
+    const T *r6 = s_r + threadIdx.x - comp;  // the camera's residual entries
+    auto precond = [&]() {
+        T s = T(0);
+#pragma unroll
+        for (int k = 0; k < BA_VB_CMAX; ++k)
+            if (k < cown) s = fma(Mr[k], r6[k], s);
+        return s;
+    };
+    const double tol2 = sc->tol2;
+    const int max_iters = sc->max_iters;
+    unsigned gen = 0;
+    double v2[2] = {0.0, 0.0};
+    if (own) {
+        zv = precond();
+        z[e] = zv;
+        v2[0] = (double)(rv * zv);
+        v2[1] = (double)(rv * rv);
+    }
+    auto none = [](const double (&)[2], bool) {};
+    if (!grid_allreduce_w0<2>(v2, red, gen++, bar, &sc->err, limit_cycles, nwv, none)) return;
+    double rz = v2[0];
+    const double rr0 = v2[1];
+    if (!(rr0 > 0.0) || max_iters <= 0) {
+        if (own) y[e] = T(0);
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            sc->rr0 = rr0;
+            sc->rr = rr0;
+            sc->iters = 0;
+            sc->done = 1;
+        }
         return;
     }
-    // column q of (L L^T)^-1: forward then backward substitution on e_q
-    double w[BA_VB_CMAX];
-    for (int q = 0; q < c; ++q) {
-        for (int r = 0; r < c; ++r) {
-            double s = (r == q) ? 1.0 : 0.0;
-            for (int k = 0; k < r; ++k) s -= L[r * BA_VB_CMAX + k] * w[k];
-            w[r] = s / L[r * BA_VB_CMAX + r];
+    T bt = T(0);
+    const int units = R * pl.wpr;
+    for (int it = 0;;) {
+        const T *dold = (it & 1) ? d1 : d0;
+        T *dnew = (it & 1) ? d0 : d1;
+        // every entry's x = z + beta d, sixteen lanes to an entry, four entries'
+        // loads in flight per lane (their round trips to L2 would otherwise
+        // follow one another in the rows' loops)
+        for (int q0 = threadIdx.x >> 4; q0 < ne; q0 += 4 * (blockDim.x >> 4)) {
+            T zz[4], dd[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int q = q0 + k * (blockDim.x >> 4), c = threadIdx.x & 15;
+                zz[k] = dd[k] = T(0);
+                if (q < ne) {
+                    const int4 in = s_rec[q];
+                    if (c < (in.w >> 1)) {
+                        zz[k] = __ldcg(z + in.z + c);
+                        dd[k] = __ldcg(dold + in.z + c);
+                    }
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int q = q0 + k * (blockDim.x >> 4);
+                if (q < ne) s_x[BA_VB_CMAX * q + (threadIdx.x & 15)] = fma(bt, dd[k], zz[k]);
+            }
         }
-        for (int r = c - 1; r >= 0; --r) {
-            double s = w[r];
-            for (int k = r + 1; k < c; ++k) s -= L[k * BA_VB_CMAX + r] * w[k];
-            w[r] = s / L[r * BA_VB_CMAX + r];
+        __syncthreads();
+        for (int u = w; u < units; u += W) {
+            const int lr = u / pl.wpr, ci = s_c[lr], G = min(32 / ci, VB_GROUPS);
+            const T t = vb_own_part<T, PACKED>(ci, s_e[lr] + (u - lr * pl.wpr) * G, s_e[lr + 1], pl.wpr * G, s_rec,
+                                               PACKED ? s_val : val, s_x);
+            if (lane < ci) s_part[u * BA_VB_CMAX + lane] = t;
         }
-        for (int r = 0; r < c; ++r) M[r * c + q] = (T)w[r];
+        __syncthreads();
+        T q = T(0);
+        double v1[1] = {0.0};
+        if (own) {
+            const T *sp = s_part + lrow * pl.wpr * BA_VB_CMAX + comp;
+            q = sp[0];
+            for (int p = 1; p < pl.wpr; ++p) q += sp[p * BA_VB_CMAX];
+            dv = fma(bt, dv, zv);
+            dnew[e] = dv;
+            v1[0] = (double)(dv * q);
+        }
+        if (!grid_allreduce_w0<1>(v1, red, gen++, bar, &sc->err, limit_cycles, nwv,
+                                  [&](const double(&x)[1], bool) { s_ab = rz / x[0]; }))
+            return;
+        if (!(v1[0] > 0.0)) {
+            if (own) y[e] = yv;
+            if (blockIdx.x == 0 && threadIdx.x == 0) {
+                sc->err = (int)BA_ERR_NOT_SPD;
+                sc->done = 1;
+                sc->iters = it;
+            }
+            return;
+        }
+        const T alpha = (T)s_ab;
+        if (own) {
+            rv -= alpha * q;
+            yv += alpha * dv;
+            s_r[threadIdx.x] = rv;
+        }
+        __syncthreads();
+        v2[0] = v2[1] = 0.0;
+        if (own) {
+            zv = precond();
+            z[e] = zv;
+            v2[0] = (double)(rv * zv);
+            v2[1] = (double)(rv * rv);
+        }
+        if (!grid_allreduce_w0<2>(v2, red, gen++, bar, &sc->err, limit_cycles, nwv,
+                                  [&](const double(&x)[2], bool) { s_ab = x[0] / rz; }))
+            return;
+        ++it;
+        if (v2[1] <= tol2 * rr0 || it >= max_iters) {
+            if (own) y[e] = yv;
+            if (blockIdx.x == 0 && threadIdx.x == 0) {
+                sc->iters = it;
+                sc->rr = v2[1];
+                sc->rr0 = rr0;
+                sc->rz = v2[0];
+                sc->done = 1;
+            }
+            return;
+        }
+        bt = (T)s_ab;
+        rz = v2[0];
     }
 }
 
@@ -132,7 +520,8 @@ __device__ __forceinline__ T vb_precond_entry(int i, int a, const int *__restric
     return z;
 }
 
-// The PCG of Sec. 3.2 on the variable-size system in one cooperative launch:
+// The same for systems whose CTAs would own more entries than threads (vectors
+// in memory, a warp per row):
 // the start (r = b, z = M^-1 b, y = 0) and r^T z, r^T r by one all-reduce;
 // then per iteration the product phase (d = z + beta d_old formed on the fly,
 // q = S d, d^T S d), its all-reduce, the update phase (y += alpha d,
@@ -146,7 +535,7 @@ __global__ void __launch_bounds__(256) k_vb_pcg(int n, int N, const int *__restr
                                                 const T *__restrict__ Minv, const T *__restrict__ b, T *y, T *r0, T *r1,
                                                 T *z, T *d0, T *d1, T *q, VbScalars *sc, double *red, unsigned *bar,
                                                 long long limit_cycles) {
-    __shared__ double sh[40];
+    __shared__ T s_x[8][VB_GROUPS * BA_VB_CMAX];
     const int tid = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
     const double tol2 = sc->tol2;
     const int max_iters = sc->max_iters;
@@ -163,8 +552,7 @@ __global__ void __launch_bounds__(256) k_vb_pcg(int n, int N, const int *__restr
         v0[0] += (double)(be * ze);
         v0[1] += (double)(be * be);
     }
-    block_sum<2>(v0, sh);
-    if (!grid_allreduce_sym<2>(v0, red, gen++, bar, &sc->err, limit_cycles)) return;
+    if (!grid_allreduce_w0<2>(v0, red, gen++, bar, &sc->err, limit_cycles)) return;
     double rz = v0[0];
     const double rr0 = v0[1];
     if (!(rr0 > 0.0) || max_iters <= 0) {
@@ -186,16 +574,20 @@ __global__ void __launch_bounds__(256) k_vb_pcg(int n, int N, const int *__restr
         const T bt = (T)beta;
         auto dir = [&](int k) { return __ldcg(z + k) + bt * __ldcg(dold + k); };
         T pap_t = T(0);
-        for (int i = tid >> 5; i < n; i += nw)
-            vb_row<T>(i, cdim, off, tw_ptr, tw_info, val, dir, [&](int idx, T v) {
+        for (int i = tid >> 5; i < n; i += nw) {
+            const int ci = __ldg(cdim + i), lane = threadIdx.x & 31;
+            const T v = vb_part<T>(ci, __ldg(tw_ptr + i), __ldg(tw_ptr + i + 1), min(32 / ci, VB_GROUPS),
+                                          tw_info, val, s_x[threadIdx.x >> 5], dir);
+            if (lane < ci) {
+                const int idx = __ldg(off + i) + lane;
                 const T dv = dir(idx);
                 q[idx] = v;
                 dnew[idx] = dv;
                 pap_t += dv * v;
-            });
+            }
+        }
         double v1[1] = {(double)pap_t};
-        block_sum<1>(v1, sh);
-        if (!grid_allreduce_sym<1>(v1, red, gen++, bar, &sc->err, limit_cycles)) return;
+        if (!grid_allreduce_w0<1>(v1, red, gen++, bar, &sc->err, limit_cycles)) return;
         const double pAp = v1[0];
         if (!(pAp > 0.0)) {
             if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -218,8 +610,7 @@ __global__ void __launch_bounds__(256) k_vb_pcg(int n, int N, const int *__restr
             v2[0] += (double)(ra * ze);
             v2[1] += (double)(ra * ra);
         }
-        block_sum<2>(v2, sh);
-        if (!grid_allreduce_sym<2>(v2, red, gen++, bar, &sc->err, limit_cycles)) return;
+        if (!grid_allreduce_w0<2>(v2, red, gen++, bar, &sc->err, limit_cycles)) return;
         const double rz_new = v2[0], rr = v2[1];
         ++it;
         if (rr <= tol2 * rr0 || it >= max_iters) {
@@ -279,10 +670,79 @@ cudaError_t vb_spmv_T(ba_vbsmc *h, const T *x, T *y) {
     int per_sm = 0, n_sm = 0;
     cudaError_t e = occupancy((const void *)k_vb_spmv<T>, 256, 0, &per_sm, &n_sm);
     if (e != cudaSuccess) return e;
-    const int64_t want = ((int64_t)h->n * 32 + 255) / 256;
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)std::max(per_sm, 1) * n_sm));
-    k_vb_spmv<T><<<grid, 256, 0, h->st>>>(h->n, h->cdim, h->off, h->tw_ptr, h->tw_info, (const T *)h->val, x, y);
+    per_sm = std::max(per_sm, 1);
+    // warps per row: as many as leave the resident warps one row part each
+    int wpr = 1;
+    while (wpr < 8 && (int64_t)h->n * wpr * 2 <= (int64_t)per_sm * n_sm * 8) wpr *= 2;
+    const int rows = 8 / wpr;
+    const int grid = std::min((h->n + rows - 1) / rows, per_sm * n_sm);
+    k_vb_spmv<T><<<grid, 256, 0, h->st>>>(h->n, wpr, h->cdim, h->off, h->tw_ptr, h->tw_info, (const T *)h->val, x, y);
     return cudaGetLastError();
+}
+
+// The owning kernel's launch shape: rows spread over every SM; 8 warps per CTA
+// in FP64 (its FP64 issue is the limit), 16 in FP32.
+// False when a CTA would own more entries than threads or its records and
+// vectors do not fit in shared memory.
+constexpr size_t VB_SMEM_MAX = 225 * 1024;
+template <typename T>
+bool vb_own_plan(const ba_vbsmc *h, int n_sm, VbPlan *pl, int *grid, int *threads, size_t *smem, bool *packed) {
+    const int n = h->n, R = (n + n_sm - 1) / n_sm;
+    int max_ent = 0, max_vec = 0, row_ent = 0;
+    int64_t max_val = 0;
+    for (int r0 = 0; r0 < n; r0 += R) {
+        int ent = 0, vec = 0;
+        int64_t val = 0;
+        for (int i = r0; i < std::min(n, r0 + R); ++i) {
+            ent += h->row_ent[i];
+            val += h->row_val[i];
+            vec += h->row_dim[i];
+            row_ent = std::max(row_ent, h->row_ent[i]);
+        }
+        max_ent = std::max(max_ent, ent);
+        max_vec = std::max(max_vec, vec);
+        max_val = std::max(max_val, val);
+    }
+    const int nt = vb_own_threads<T>(), W = nt / 32;
+    if (max_vec > nt) return false;
+    const int G = std::max(1, std::min(32 / std::max(1, h->max_dim), VB_GROUPS));
+    // FP32: one warp per row (a row's sum keeps its order, and more warps gained
+    // 3 us of 10 at 120 cameras, nothing from 990 on); FP64: the split with the
+    // fewest passes (18.3, 13.5, 11.2, 10.9 us per iteration with 1, 2, 4, 8
+    // warps per row at 120 cameras)
+    int best = 1, best_cost = INT32_MAX;
+    for (int wpr = 1; sizeof(T) == 8 && wpr <= W; wpr *= 2) {
+        const int cost = ((R * wpr + W - 1) / W) * ((row_ent + wpr * G - 1) / (wpr * G) + 1);
+        if (cost < best_cost) {
+            best = wpr;
+            best_cost = cost;
+        }
+    }
+    *packed = max_val < (1 << 22) && vb_own_smem<T>(R, best, max_ent, max_val, nt) <= VB_SMEM_MAX;
+    *smem = vb_own_smem<T>(R, best, max_ent, *packed ? max_val : 0, nt);
+    if (*smem > VB_SMEM_MAX) return false;
+    *pl = VbPlan{R, best, max_ent, *packed ? max_val : 0};
+    *grid = (n + R - 1) / R;
+    *threads = nt;
+    return true;
+}
+
+template <typename T>
+cudaError_t vb_pcg_own(ba_vbsmc *h, VbPlan pl, int grid, int threads, size_t smem, bool packed, long long limit) {
+    const void *k = packed ? (const void *)k_vb_pcg_own<T, true> : (const void *)k_vb_pcg_own<T, false>;
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)VB_SMEM_MAX);
+    if (e != cudaSuccess) return e;
+    int n = h->n;
+    const int *cd = h->cdim, *of = h->off, *ec = h->ent_cam, *twp = h->tw_ptr;
+    const int4 *twi = h->tw_info;
+    const int64_t *mo = h->moff;
+    const T *val = (const T *)h->val, *Mi = (const T *)h->Minv, *b = (const T *)h->b;
+    T *y = (T *)h->vec[0], *z = (T *)h->vec[3], *d0 = (T *)h->vec[4], *d1 = (T *)h->vec[5];
+    VbScalars *sc = h->sc;
+    double *red = h->red;
+    unsigned *bar = h->bar;
+    void *args[] = {&n, &pl, &cd, &of, &ec, &twp, &twi, &val, &mo, &Mi, &b, &y, &z, &d0, &d1, &sc, &red, &bar, &limit};
+    return cudaLaunchCooperativeKernel(k, dim3(grid), dim3(threads), args, smem, h->st);
 }
 
 template <typename T>
@@ -290,11 +750,20 @@ cudaError_t vb_pcg_T(ba_vbsmc *h) {
     int per_sm = 0, n_sm = 0;
     cudaError_t e = occupancy((const void *)k_vb_pcg<T>, 256, 0, &per_sm, &n_sm);
     if (e != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(h->bar, 0, AR_SUB * 32 * sizeof(unsigned), h->st)) != cudaSuccess) return e;
+    long long limit = 4000000000LL;  // ~2 s of SM clock per grid wait
+    {
+        VbPlan pl;
+        int grid = 0, threads = 0;
+        size_t smem = 0;
+        bool packed = false;
+        if (vb_own_plan<T>(h, n_sm, &pl, &grid, &threads, &smem, &packed))
+            return vb_pcg_own<T>(h, pl, grid, threads, smem, packed, limit);
+    }
     if (per_sm > 2) per_sm = 2;
     if (per_sm < 1) return cudaErrorCooperativeLaunchTooLarge;
     const int64_t want = std::max<int64_t>(((int64_t)h->n * 32 + 255) / 256, (h->N + 255) / 256);
     int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)per_sm * n_sm));
-    if ((e = cudaMemsetAsync(h->bar, 0, sizeof(unsigned), h->st)) != cudaSuccess) return e;
     int n = h->n, N = (int)h->N;
     const int *cd = h->cdim, *of = h->off, *ec = h->ent_cam, *twp = h->tw_ptr;
     const int4 *twi = h->tw_info;
@@ -305,7 +774,6 @@ cudaError_t vb_pcg_T(ba_vbsmc *h) {
     VbScalars *sc = h->sc;
     double *red = h->red;
     unsigned *bar = h->bar;
-    long long limit = 4000000000LL;  // ~2 s of SM clock per grid wait
     void *args[] = {&n, &N, &cd, &of, &ec, &twp, &twi, &val, &mo, &Mi, &b, &y, &r0, &r1, &z, &d0, &d1, &q,
                     &sc, &red, &bar, &limit};
     return cudaLaunchCooperativeKernel((const void *)k_vb_pcg<T>, dim3(grid), dim3(256), args, 0, h->st);
@@ -384,6 +852,16 @@ ba_status vb_build(const ba_options &o, int32_t n, const int32_t *cdim, int64_t 
     h->esz = h->fp32 ? 4 : 8;
     h->st = (cudaStream_t)o.cuda_stream;
     h->cap = o.device_mem_cap;
+    h->row_ent.resize(n);
+    h->row_val.resize(n);
+    h->row_dim.assign(cdim, cdim + n);
+    for (int32_t i = 0; i < n; ++i) {
+        h->row_ent[i] = tw_ptr[i + 1] - tw_ptr[i];
+        h->max_dim = std::max(h->max_dim, cdim[i]);
+        int64_t v = 0;
+        for (int32_t t = tw_ptr[i]; t < tw_ptr[i + 1]; ++t) v += tw_info[t].w >> 1;
+        h->row_val[i] = v * cdim[i];
+    }
     auto up = [&](void **d, const void *src, size_t bytes) -> ba_status {
         ba_status r = vb_alloc(h, d, bytes);
         if (r) return r;
@@ -409,8 +887,10 @@ ba_status vb_build(const ba_options &o, int32_t n, const int32_t *cdim, int64_t 
         if (!s) s = vb_alloc(h, &v, N * h->esz);
     if (!s) s = vb_alloc(h, (void **)&h->sc, sizeof(VbScalars));
     if (!s) s = vb_alloc(h, (void **)&h->red, (size_t)RED_SLOTS * sizeof(double));
-    if (!s) s = vb_alloc(h, (void **)&h->bar, sizeof(unsigned));
     if (!s) s = vb_alloc(h, (void **)&h->err, sizeof(int));
+    // the arrival counters lie behind the partials (2 grids of AR_NV_MAX doubles
+    // each, at most 2 CTAs on every SM)
+    if (!s) h->bar = reinterpret_cast<unsigned *>(h->red + RED_SLOTS / 2);
     if (!s) s = vb_cuda(h, cudaEventCreate(&h->ev[0]), "event");
     if (!s) s = vb_cuda(h, cudaEventCreate(&h->ev[1]), "event");
     if (s) {
@@ -424,12 +904,12 @@ ba_status vb_build(const ba_options &o, int32_t n, const int32_t *cdim, int64_t 
 ba_status vb_finish(ba_vbsmc *h) {
     ba_status s;
     if ((s = vb_cuda(h, cudaMemsetAsync(h->err, 0, sizeof(int), h->st), "memset"))) return s;
-    const int g = (h->n + 127) / 128;
+    const int g = (h->n + 3) / 4;  // sixteen lanes per camera, two warps per CTA: spread over the SMs
     if (h->fp32)
-        k_vb_minv<float><<<g, 128, 0, h->st>>>(h->n, h->cdim, h->row_ptr, h->boff, (const float *)h->val, h->moff,
+        k_vb_minv<float><<<g, 64, 0, h->st>>>(h->n, h->cdim, h->row_ptr, h->boff, (const float *)h->val, h->moff,
                                                (float *)h->Minv, h->err);
     else
-        k_vb_minv<double><<<g, 128, 0, h->st>>>(h->n, h->cdim, h->row_ptr, h->boff, (const double *)h->val, h->moff,
+        k_vb_minv<double><<<g, 64, 0, h->st>>>(h->n, h->cdim, h->row_ptr, h->boff, (const double *)h->val, h->moff,
                                                 (double *)h->Minv, h->err);
     if ((s = vb_cuda(h, cudaGetLastError(), "k_vb_minv"))) return s;
     int err = 0;

@@ -36,6 +36,10 @@ struct ba_vbsmc {
     double *red = nullptr;
     unsigned *bar = nullptr;
     int *err = nullptr;
+    // per block row: two-sided entries, their values, unknowns (launch shapes)
+    std::vector<int32_t> row_ent, row_dim;
+    std::vector<int64_t> row_val;
+    int max_dim = 0;
     std::vector<void *> allocs;
     cudaEvent_t ev[2] = {nullptr, nullptr};
 };

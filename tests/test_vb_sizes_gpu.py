@@ -1,0 +1,97 @@
+"""Variable-size BSMC product, M^-1 and PCG over the launch shapes and block
+sizes its kernels distinguish: 1 to 16 unknowns per camera in one system, one
+to many block rows per CTA, values in shared memory or not, and CTAs that own
+more vector entries than threads.  Reference: numpy FP64 on the blocks padded
+to 16 x 16.  Tolerances: a product sums at most 32 x 16 terms, so it is within
+512 eps of sum |S| |x| per entry; the solves stop at ||r|| <= tol ||b|| by
+their own recurrence, and for these block-dominant systems (condition below
+50, a few tens of iterations) the true residual is within 100 eps of it
+relative to ||b|| in the storage precision."""
+import numpy as np
+import pytest
+
+import scenes
+from test_pcg_sizes_gpu import banded_pattern
+
+pytestmark = pytest.mark.gpu
+
+
+def padded(row_ptr, col, cdim, val):
+    row = np.repeat(np.arange(len(cdim)), np.diff(row_ptr))
+    S = np.zeros((len(col), 16, 16))
+    size = cdim[row].astype(np.int64) * cdim[col]
+    at = np.concatenate([[0], np.cumsum(size)])
+    for k in range(len(col)):
+        S[k, :cdim[row[k]], :cdim[col[k]]] = val[at[k]:at[k + 1]].reshape(cdim[row[k]], cdim[col[k]])
+    return row, S
+
+
+def product(row, col, S, x):
+    y = np.zeros_like(x)
+    np.add.at(y, row, np.einsum("kab,kb->ka", S, x[col]))
+    off = row != col
+    np.add.at(y, col[off], np.einsum("kba,kb->ka", S[off], x[row[off]]))
+    return y
+
+
+def sizes(kind, n, seed):
+    rng = np.random.default_rng(seed)
+    if kind == "any":
+        return rng.integers(1, 17, n).astype(np.int32)
+    if kind == "mixed":
+        return np.where(rng.random(n) < 0.5, 11, 6).astype(np.int32)
+    return np.full(n, int(kind), np.int32)
+
+
+@pytest.mark.parametrize("n,half,kind,fp32", [(1, 1, "any", False), (3, 2, "any", False), (40, 30, "any", False),
+                                              (40, 30, "any", True), (153, 11, "mixed", False),
+                                              (400, 25, "11", False), (1000, 9, "mixed", True),
+                                              (1600, 22, "11", True), (5200, 1, "16", False), (5200, 1, "16", True),
+                                              (330, 3, "1", True), (17, 16, "5", False)])
+def test_vb_system_over_sizes(n, half, kind, fp32):
+    import torch
+
+    from paper_2307_08383_gb300.build import build
+    build()
+    import paper_2307_08383_gb300 as B
+    row_ptr, col = banded_pattern(n, half)
+    cdim = sizes(kind, n, 77 + n)
+    T = np.float32 if fp32 else np.float64
+    val, _ = scenes.random_block_spd(row_ptr, col, cdim, 9300 + n)
+    val = val.astype(T).astype(np.float64)
+    N = int(cdim.sum())
+    rng = np.random.default_rng(n)
+    b = rng.standard_normal(N).astype(T).astype(np.float64)
+    x = rng.standard_normal(N).astype(T).astype(np.float64)
+    live = np.arange(16)[None] < cdim[:, None]
+    row, S = padded(row_ptr, col, cdim, val)
+
+    def pad(v):
+        p = np.zeros((n, 16))
+        p[live] = v
+        return p
+
+    eps = np.finfo(T).eps
+    g = B.VBSMC(cdim, row_ptr, col, val, b, precision=B.BA_FP32 if fp32 else B.BA_FP64)
+    dx = torch.from_numpy(x.astype(T)).cuda()
+    dy = torch.full_like(dx, float("nan"))
+    g.spmv(dx, dy)
+    y = dy.cpu().numpy().astype(np.float64)
+    bound = product(row, col, np.abs(S), pad(np.abs(x)))[live]
+    assert np.all(np.abs(y - product(row, col, S, pad(x))[live]) <= 512 * eps * bound)
+    tol = 1e-5 if fp32 else 1e-11
+    for _ in range(2):  # a second solve finds nothing of the first
+        sol, its, rel, _, status = g.solve(tol)
+        assert status == B.BA_OK and 1 <= its < 100 and rel <= tol
+        r = pad(b) - product(row, col, S, pad(sol))
+        assert np.linalg.norm(r) <= (tol + 100 * eps) * np.linalg.norm(b)
+    # a diagonal block that is not positive definite is still refused
+    bad = val.copy()
+    k = int(row_ptr[n - 1])
+    at = np.concatenate([[0], np.cumsum(cdim[row].astype(np.int64) * cdim[col])])
+    c = int(cdim[n - 1])
+    bad[at[k] + c * c - 1] = -1.0
+    with pytest.raises(B.BAError) as ei:
+        B.VBSMC(cdim, row_ptr, col, bad, b, precision=B.BA_FP32 if fp32 else B.BA_FP64)
+    assert ei.value.status == B.BA_ERR_NOT_SPD
+    g.close()
