@@ -7,7 +7,7 @@
 // d = 1 + k1 r2 + k2 r2^2 the projection is u = f d xh + cx, v = f d yh + cy.
 // A camera has c_i = 6 (interiors fixed) or 11 unknowns.  Three kernels:
 //   k_vbi_linearize  e and J of every observation (Eq. 1), rows of
-//                    [J_c (2 x 11) | J_p (2 x 3) | e (2)] in the storage
+//                    [J_c (11 x 2) | J_p (2 x 3) | e (2)] in the storage
 //                    precision (X_cam in FP64, the rest in that precision);
 //   k_vbi_points     per point, in FP64, V_k (damped), its Cholesky factor
 //                    L, V_k^-1 and l_p (Eq. 3), and per observation the
@@ -28,7 +28,11 @@
 
 namespace ba {
 
-constexpr int VJW = 32;      // J row (T): J_c 2 x 11 at 0, 11 | J_p 2 x 3 at 22, 25 | e at 28, 29 | pad
+// J row (T): J_c by columns, the two rows of column c at 2 c, 2 c + 1 (c < 11) |
+// pad 22, 23 | J_p 2 x 3 at 24, 27 | e at 30, 31.  A column is one aligned pair
+// (the block kernels load the columns they need), J_p and e one aligned
+// 32-byte stretch in FP32.
+constexpr int VJW = 32, VJP = 24, VJE = 30;
 constexpr int VPW = 8;       // factor row (T): P = J_p L^-T (2 x 3) at 0, 3 | e^ = e + P L^-1 l_p at 6, 7
 constexpr int VB_CI = 11;    // unknowns of a self-calibrating camera
 constexpr int VB_NT = 4;     // block entries per lane: 4 x 32 >= 11 x 11
@@ -95,22 +99,22 @@ __global__ void __launch_bounds__(256) k_vbi_linearize(int64_t m, const int *__r
         T *o = J + a * VJW;
         const T ph[2] = {xh, yh};
         for (int r = 0; r < 2; ++r) {
-            T *jc = o + VB_CI * r, *jp = o + 22 + 3 * r;
+            T *jc = o + r, *jp = o + VJP + 3 * r;  // column c at jc[2 c]
             for (int c = 0; c < 3; ++c) {
-                jc[c] = A[r][0] * Mx[0][c] + A[r][1] * Mx[1][c] + A[r][2] * Mx[2][c];
-                jc[3 + c] = A[r][c];
+                jc[2 * c] = A[r][0] * Mx[0][c] + A[r][1] * Mx[1][c] + A[r][2] * Mx[2][c];
+                jc[2 * (3 + c)] = A[r][c];
                 jp[c] = A[r][0] * (T)R[c] + A[r][1] * (T)R[3 + c] + A[r][2] * (T)R[6 + c];
             }
-            jc[6] = d * ph[r];                 // f
-            jc[7] = r == 0 ? T(1) : T(0);      // cx
-            jc[8] = r == 0 ? T(0) : T(1);      // cy
-            jc[9] = f * ph[r] * r2;            // k1
-            jc[10] = f * ph[r] * r2 * r2;      // k2
+            jc[12] = d * ph[r];                // f
+            jc[14] = r == 0 ? T(1) : T(0);     // cx
+            jc[16] = r == 0 ? T(0) : T(1);     // cy
+            jc[18] = f * ph[r] * r2;           // k1
+            jc[20] = f * ph[r] * r2 * r2;      // k2
         }
-        o[28] = pr.e0;
-        o[29] = pr.e1;
-        o[30] = T(0);
-        o[31] = T(0);
+        o[VJE] = pr.e0;
+        o[VJE + 1] = pr.e1;
+        o[22] = T(0);
+        o[23] = T(0);
     }
 }
 
@@ -129,8 +133,8 @@ __global__ void __launch_bounds__(256) k_vbi_points(int64_t P, const int *__rest
         for (int a = trk_ptr[k]; a < trk_ptr[k + 1]; ++a) {
             const T *o = J + (int64_t)a * VJW;
             double jp[6];
-            for (int q = 0; q < 6; ++q) jp[q] = (double)o[22 + q];
-            const double e0 = (double)o[28], e1 = (double)o[29];
+            for (int q = 0; q < 6; ++q) jp[q] = (double)o[VJP + q];
+            const double e0 = (double)o[VJE], e1 = (double)o[VJE + 1];
             for (int m = 0; m < 3; ++m) {
                 for (int n = 0; n < 3; ++n) V[m][n] += jp[m] * jp[n] + jp[3 + m] * jp[3 + n];
                 l[m] -= jp[m] * e0 + jp[3 + m] * e1;
@@ -159,107 +163,302 @@ __global__ void __launch_bounds__(256) k_vbi_points(int64_t P, const int *__rest
             const T *o = J + (int64_t)a * VJW;
             T *pe = PE + (int64_t)a * VPW;
             for (int r = 0; r < 2; ++r) {
-                const double j0 = (double)o[22 + 3 * r], j1 = (double)o[23 + 3 * r], j2 = (double)o[24 + 3 * r];
+                const double j0 = (double)o[VJP + 3 * r], j1 = (double)o[VJP + 1 + 3 * r], j2 = (double)o[VJP + 2 + 3 * r];
                 // P = J_p L^-T: P_c = sum_k J_k (L^-1)_ck over k <= c
                 const double P0 = j0 * m00, P1 = j0 * m10 + j1 * m11, P2 = j0 * m20 + j1 * m21 + j2 * m22;
                 pe[3 * r] = (T)P0;
                 pe[3 * r + 1] = (T)P1;
                 pe[3 * r + 2] = (T)P2;
-                pe[6 + r] = (T)((double)o[28 + r] + P0 * q0 + P1 * q1 + P2 * q2);
+                pe[6 + r] = (T)((double)o[VJE + r] + P0 * q0 + P1 * q1 + P2 * q2);
             }
         }
     }
 }
 
-// A warp per stored block (beta, gamma) and its list of slot pairs (a, b).
-// A slot is an observation's J_c columns that belong to one block: for a
-// block of camera i (c_i = 6 or 11) the first c_i columns, for the block of a
-// physical camera whose images share interiors the five interior columns;
-// jc0[beta] is the first J_c column of block beta's slots (null: 0).  The
-// pairs of a block are its slots' pairs within each point (every ordered
-// pair, a in beta and b in gamma).  Per pair the 2 x 2 middle factor is
-// -P_a P_b^T, or I - P_a P_a^T when both slots belong to one observation
-// (that adds U = J_c^T J_c, the coupling of an image and its physical camera
-// included); lanes 16.. form its product with the c_gamma columns of J_c,b,
-// lanes 0.. stage J_c,a's c_beta columns, and every lane adds
-// J_c,a^T (M J_c,b) for its entries.  Summed over a point's slot pairs this is
-// U - W_beta V_k^-1 W_gamma^T with W_beta summed over the point's slots in
-// beta.  On a diagonal block a slot paired with itself also gives b_beta's
-// term -J_c,a^T e^_a and the U diagonal that damps the block at the end.
+// The block kernels: a warp per stored block (beta, gamma) and its list of
+// slot pairs (a, b).  A slot is an observation's J_c columns that belong to one
+// block: for a block of camera i (c_i = 6 or 11) the first c_i columns, for the
+// block of a physical camera whose images share interiors the five interior
+// columns; jc0[beta] is the first J_c column of block beta's slots (null: 0).
+// The pairs of a block are its slots' pairs within each point (every ordered
+// pair, a in beta and b in gamma).  Per pair the 2 x 2 middle factor M is
+// -P_a P_b^T, or I - P_a P_a^T when both slots belong to one observation (that
+// adds U = J_c^T J_c, the coupling of an image and its physical camera
+// included), and the block gains J_c,a^T (M J_c,b).  Summed over a point's slot
+// pairs this is U - W_beta V_k^-1 W_gamma^T with W_beta summed over the point's
+// slots in beta.  On a diagonal block a slot paired with itself also gives
+// b_beta's term -J_c,a^T e^_a and the U diagonal that damps the block at the
+// end.  The factors M of 32 pairs are formed at once, one pair to a lane, and
+// handed to the warp by shuffles.
+
+// a b + c d with one rounding fewer
 template <typename T>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 4) k_vbi_blocks(int64_t nnzb, const int *__restrict__ brow,
-                                                    const int *__restrict__ col, const int *__restrict__ cdim,
-                                                    const int *__restrict__ jc0, const int *__restrict__ off,
-                                                    const int64_t *__restrict__ boff,
-                                                    const int *__restrict__ pptr, const int2 *__restrict__ plist,
-                                                    const T *__restrict__ J, const T *__restrict__ PE,
-                                                    double lambda, T *__restrict__ val, T *__restrict__ b) {
-    __shared__ T sm[8][4 * 16];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    T *Jca = sm[w], *Tb = Jca + 32;  // J_c,a columns (2 x 16), M J_c,b (2 x 16)
+__device__ __forceinline__ T dot2(T a, T b, T c, T d) {
+    return fma(a, b, c * d);
+}
+
+// One pair's middle factor from the factor rows of its observations (and the
+// first row's e^).
+template <typename T>
+__device__ __forceinline__ void vbi_middle(const T *__restrict__ Pa, const T *__restrict__ Pb, bool same, T (&M)[4],
+                                           T (&eh)[2]) {
+    T a[8], b[8];
+    if constexpr (sizeof(T) == 4) {
+        const float4 *p = reinterpret_cast<const float4 *>(Pa), *q = reinterpret_cast<const float4 *>(Pb);
+        const float4 a0 = __ldg(p), a1 = __ldg(p + 1), b0 = __ldg(q), b1 = __ldg(q + 1);
+        a[0] = a0.x; a[1] = a0.y; a[2] = a0.z; a[3] = a0.w; a[4] = a1.x; a[5] = a1.y; a[6] = a1.z; a[7] = a1.w;
+        b[0] = b0.x; b[1] = b0.y; b[2] = b0.z; b[3] = b0.w; b[4] = b1.x; b[5] = b1.y;
+    } else {
+        const double2 *p = reinterpret_cast<const double2 *>(Pa), *q = reinterpret_cast<const double2 *>(Pb);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const double2 u = __ldg(p + k), v = __ldg(q + k);
+            a[2 * k] = u.x; a[2 * k + 1] = u.y;
+            b[2 * k] = v.x; b[2 * k + 1] = v.y;
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int v = 0; v < 2; ++v)
+            M[2 * u + v] = (same && u == v ? T(1) : T(0)) -
+                           fma(a[3 * u + 2], b[3 * v + 2], dot2(a[3 * u], b[3 * v], a[3 * u + 1], b[3 * v + 1]));
+    eh[0] = a[6];
+    eh[1] = a[7];
+}
+
+// FP32: the block as a 4 x 8 grid of lanes, each with up to 3 x 2 entries in
+// registers and the columns it needs loaded straight from the J rows (a row
+// column is an 8-byte pair; the lanes of a group share the words), so a pair
+// costs five loads, six shuffles and about thirty multiply-adds per lane with no
+// shared memory and no barrier, and several pairs' loads are in flight.  A
+// block's pairs are added in list order, each as acc + (j0 t0 + j1 t1).
+// (Before, both J rows passed through shared memory with two warp barriers per
+// pair, and every lane formed M: 1031 -> 386 us at 990 cameras of c = 11, 485,000
+// observations, the same bits.)
+__global__ void __launch_bounds__(256) k_vbi_blocks32(int64_t nnzb, const int *__restrict__ brow,
+                                                      const int *__restrict__ col, const int *__restrict__ cdim,
+                                                      const int *__restrict__ jc0, const int *__restrict__ off,
+                                                      const int64_t *__restrict__ boff, const int *__restrict__ pptr,
+                                                      const int2 *__restrict__ plist, const float *__restrict__ J,
+                                                      const float *__restrict__ PE, double lambda,
+                                                      float *__restrict__ val, float *__restrict__ b) {
+    constexpr unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, rg = lane >> 3, cg = lane & 7;
+    const float2 *J2 = reinterpret_cast<const float2 *>(J);
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t k = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; k < nnzb; k += nw) {
-        const int i = brow[k], j = col[k], ci = cdim[i], cj = cdim[j], nel = ci * cj;
-        const int ai = jc0 ? jc0[i] : 0, aj = jc0 ? jc0[j] : 0;
+        const int i = brow[k], j = col[k], ci = cdim[i], cj = cdim[j];
+        const int rpl = (ci + 3) >> 2, cpl = (cj + 7) >> 3;  // rows and columns per lane
+        const int r0 = rpl * rg, c0 = cpl * cg;
+        const int ja0 = (jc0 ? jc0[i] : 0) + r0, jb0 = (jc0 ? jc0[j] : 0) + c0;
         const bool diag = i == j;
-        T acc[VB_NT], dU[VB_NT], bacc = T(0);
-        // this lane's entries (row, column) of the block, fixed for its pairs
-        int er[VB_NT], ec[VB_NT];
+        bool ron[3], con[2];
 #pragma unroll
-        for (int t = 0; t < VB_NT; ++t) {
-            acc[t] = dU[t] = T(0);
-            const int E = lane + 32 * t;
-            er[t] = E < nel ? E / cj : 0;
-            ec[t] = E < nel ? E - er[t] * cj : 0;
-        }
-        for (int p = pptr[k]; p < pptr[k + 1]; ++p) {  // warp-uniform
-            const int2 pr = plist[p];
-            const bool same = pr.x == pr.y;
-            const T *Ja = J + (int64_t)pr.x * VJW, *Jb = J + (int64_t)pr.y * VJW;
-            const T *Pa = PE + (int64_t)pr.x * VPW, *Pb = PE + (int64_t)pr.y * VPW;
-            if (lane < 16) {
-                const int r = lane;
-                if (r < ci) {
-                    const T j0 = Ja[ai + r], j1 = Ja[VB_CI + ai + r];
-                    Jca[r] = j0;
-                    Jca[16 + r] = j1;
-                    if (diag && same) bacc -= j0 * Pa[6] + j1 * Pa[7];
+        for (int u = 0; u < 3; ++u) ron[u] = u < rpl && r0 + u < ci;
+#pragma unroll
+        for (int v = 0; v < 2; ++v) con[v] = v < cpl && c0 + v < cj;
+        float acc[3][2], dU[3], bacc[3];
+#pragma unroll
+        for (int u = 0; u < 3; ++u) acc[u][0] = acc[u][1] = dU[u] = bacc[u] = 0.f;
+        const int p1 = pptr[k + 1];
+        for (int p0 = pptr[k]; p0 < p1; p0 += 32) {
+            const int cnt = min(32, p1 - p0);
+            int2 pr = make_int2(0, 0);
+            float M[4] = {0.f, 0.f, 0.f, 0.f}, eh[2] = {0.f, 0.f};
+            if (lane < cnt) {
+                pr = __ldg(plist + p0 + lane);
+                vbi_middle<float>(PE + (int64_t)pr.x * VPW, PE + (int64_t)pr.y * VPW, pr.x == pr.y, M, eh);
+            }
+#pragma unroll 4
+            for (int q = 0; q < cnt; ++q) {
+                const int x = __shfl_sync(FULL, pr.x, q), y = __shfl_sync(FULL, pr.y, q);
+                const float m00 = __shfl_sync(FULL, M[0], q), m01 = __shfl_sync(FULL, M[1], q),
+                            m10 = __shfl_sync(FULL, M[2], q), m11 = __shfl_sync(FULL, M[3], q);
+                const float2 *ra = J2 + (int64_t)x * (VJW / 2) + ja0, *rb = J2 + (int64_t)y * (VJW / 2) + jb0;
+                float2 a[3], t[2];
+#pragma unroll
+                for (int u = 0; u < 3; ++u) a[u] = ron[u] ? __ldg(ra + u) : make_float2(0.f, 0.f);
+#pragma unroll
+                for (int v = 0; v < 2; ++v) {
+                    const float2 w = con[v] ? __ldg(rb + v) : make_float2(0.f, 0.f);
+                    t[v] = make_float2(dot2(m00, w.x, m01, w.y), dot2(m10, w.x, m11, w.y));
                 }
-            } else {
-                const int c = lane - 16;
-                if (c < cj) {
-                    // M = (same ? I : 0) - P_a P_b^T
-                    T M[2][2];
-                    for (int u = 0; u < 2; ++u)
-                        for (int v = 0; v < 2; ++v)
-                            M[u][v] = (same && u == v ? T(1) : T(0)) -
-                                      (Pa[3 * u] * Pb[3 * v] + Pa[3 * u + 1] * Pb[3 * v + 1] + Pa[3 * u + 2] * Pb[3 * v + 2]);
-                    const T j0 = Jb[aj + c], j1 = Jb[VB_CI + aj + c];
-                    Tb[c] = M[0][0] * j0 + M[0][1] * j1;
-                    Tb[16 + c] = M[1][0] * j0 + M[1][1] * j1;
+#pragma unroll
+                for (int u = 0; u < 3; ++u)
+#pragma unroll
+                    for (int v = 0; v < 2; ++v) acc[u][v] += dot2(a[u].x, t[v].x, a[u].y, t[v].y);
+                if (diag && x == y) {
+                    const float e0 = __shfl_sync(FULL, eh[0], q), e1 = __shfl_sync(FULL, eh[1], q);
+#pragma unroll
+                    for (int u = 0; u < 3; ++u) {
+                        bacc[u] -= dot2(a[u].x, e0, a[u].y, e1);
+                        dU[u] += dot2(a[u].x, a[u].x, a[u].y, a[u].y);
+                    }
+                }
+            }
+        }
+        float *out = val + boff[k];
+#pragma unroll
+        for (int u = 0; u < 3; ++u) {
+            if (!ron[u]) continue;
+            const int r = r0 + u;
+#pragma unroll
+            for (int v = 0; v < 2; ++v) {
+                const int c = c0 + v;
+                if (!con[v]) continue;
+                out[r * cj + c] = diag && r == c ? fmaf((float)lambda, clampT(dU[u]), acc[u][v]) : acc[u][v];
+            }
+            if (diag && cg == 0) b[off[i] + r] = bacc[u];
+        }
+    }
+}
+
+// FP64: an SM issues one FP64 warp instruction per 16 cycles, so the pairs are
+// staged four at a time (J_c,a and M J_c,b in the warp's shared memory, 6 FP64
+// instructions per four pairs) and every lane adds its four entries of the
+// block with 8 per pair (32 before, M and the products formed pair by pair).
+// A block of more than VB64_SPLIT pairs (a diagonal block, mostly) is shared by
+// the CTA's eight warps, which take batches of 32 pairs in turn and join their
+// sums in shared memory.  1778 -> 297 us at 120 cameras (half of them c = 11),
+// 58,000 observations.
+constexpr int VB64_SPLIT = 96;
+struct Vbi64Sums {
+    double acc[VB_NT], du, bacc;  // entries lane + 32 t; row `lane`'s U diagonal and b
+};
+// pairs p0 + 32 (first + k step), ... of a block into s
+__device__ __forceinline__ void vbi64_pairs(int p0, int p1, int first, int step, int ci, int cj, int ai, int aj,
+                                            bool diag, const int2 *__restrict__ plist, const double2 *__restrict__ J2,
+                                            const double *__restrict__ PE, double *sm, Vbi64Sums &s) {
+    constexpr unsigned FULL = 0xffffffffu;
+    constexpr int SP = 4;  // pairs staged at a time
+    const int lane = threadIdx.x & 31, nel = ci * cj;
+    double *sA = sm, *sT = sm + SP * 2 * VB_CI;  // [pair][row][column]
+    int er[VB_NT], ec[VB_NT];
+#pragma unroll
+    for (int t = 0; t < VB_NT; ++t) {
+        const int E = lane + 32 * t;
+        er[t] = E < nel ? E / cj : 0;
+        ec[t] = E < nel ? E - er[t] * cj : 0;
+    }
+    for (int pb = p0 + 32 * first; pb < p1; pb += 32 * step) {
+        const int cnt = min(32, p1 - pb);
+        int2 pr = make_int2(0, 0);
+        double M[4] = {0.0, 0.0, 0.0, 0.0}, eh[2] = {0.0, 0.0};
+        if (lane < cnt) {
+            pr = __ldg(plist + pb + lane);
+            vbi_middle<double>(PE + (int64_t)pr.x * VPW, PE + (int64_t)pr.y * VPW, pr.x == pr.y, M, eh);
+        }
+        for (int q0 = 0; q0 < cnt; q0 += SP) {
+            // stage: item (pair, row, column) over the lanes
+            double av[3], tv[3];
+#pragma unroll
+            for (int h = 0; h < 3; ++h) {
+                const int it = lane + 32 * h, qq = it / (2 * VB_CI), rem = it - qq * 2 * VB_CI;
+                const int u = rem >= VB_CI ? 1 : 0, c = rem - u * VB_CI, q = min(q0 + qq, 31);
+                const int x = __shfl_sync(FULL, pr.x, q), y = __shfl_sync(FULL, pr.y, q);
+                const double m0 = __shfl_sync(FULL, M[0], q), m1 = __shfl_sync(FULL, M[1], q),
+                             m2 = __shfl_sync(FULL, M[2], q), m3 = __shfl_sync(FULL, M[3], q);
+                const bool on = qq < SP && q0 + qq < cnt;
+                double2 a = make_double2(0.0, 0.0), w = a;
+                if (on && c < ci) a = __ldg(J2 + (int64_t)x * (VJW / 2) + ai + c);
+                if (on && c < cj) w = __ldg(J2 + (int64_t)y * (VJW / 2) + aj + c);
+                av[h] = u ? a.y : a.x;
+                tv[h] = (u ? m2 : m0) * w.x + (u ? m3 : m1) * w.y;
+            }
+            __syncwarp();
+#pragma unroll
+            for (int h = 0; h < 3; ++h) {
+                const int it = lane + 32 * h;
+                if (it < SP * 2 * VB_CI) {
+                    sA[it] = av[h];
+                    sT[it] = tv[h];
                 }
             }
             __syncwarp();
 #pragma unroll
-            for (int t = 0; t < VB_NT; ++t) {
-                if (lane + 32 * t < nel) {
-                    const int r = er[t], c = ec[t];
-                    acc[t] += Jca[r] * Tb[c] + Jca[16 + r] * Tb[16 + c];
-                    if (diag && same && r == c) dU[t] += Jca[r] * Jca[r] + Jca[16 + r] * Jca[16 + r];
+            for (int qq = 0; qq < SP; ++qq) {
+                const double *A = sA + qq * 2 * VB_CI, *Tq = sT + qq * 2 * VB_CI;
+#pragma unroll
+                for (int t = 0; t < VB_NT; ++t) {
+                    if (32 * t >= nel) break;
+                    s.acc[t] = fma(A[er[t]], Tq[ec[t]], s.acc[t]);
+                    s.acc[t] = fma(A[VB_CI + er[t]], Tq[VB_CI + ec[t]], s.acc[t]);
+                }
+                if (diag) {
+                    const int q = min(q0 + qq, 31);
+                    const bool same = q0 + qq < cnt && __shfl_sync(FULL, pr.x, q) == __shfl_sync(FULL, pr.y, q);
+                    const double e0 = __shfl_sync(FULL, eh[0], q), e1 = __shfl_sync(FULL, eh[1], q);
+                    if (same && lane < ci) {
+                        const double j0 = A[lane], j1 = A[VB_CI + lane];
+                        s.du = fma(j0, j0, s.du);
+                        s.du = fma(j1, j1, s.du);
+                        s.bacc = fma(-j0, e0, s.bacc);
+                        s.bacc = fma(-j1, e1, s.bacc);
+                    }
                 }
             }
-            __syncwarp();
         }
+    }
+}
+__global__ void __launch_bounds__(256) k_vbi_blocks64(int64_t nnzb, const int *__restrict__ brow,
+                                                      const int *__restrict__ col, const int *__restrict__ cdim,
+                                                      const int *__restrict__ jc0, const int *__restrict__ off,
+                                                      const int64_t *__restrict__ boff, const int *__restrict__ pptr,
+                                                      const int2 *__restrict__ plist, const double *__restrict__ J,
+                                                      const double *__restrict__ PE, double lambda,
+                                                      double *__restrict__ val, double *__restrict__ b) {
+    __shared__ double sm[8][2 * 4 * 2 * VB_CI];     // staging per warp
+    __shared__ double join[8][(VB_NT + 2) * 32];    // a shared block's sums per warp
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const double2 *J2 = reinterpret_cast<const double2 *>(J);
+    auto finish = [&](int64_t k, int i, int cj, int nel, int ci, bool diag, const Vbi64Sums &s) {
+#pragma unroll
         for (int t = 0; t < VB_NT; ++t) {
-            const int E = lane + 32 * t;
-            if (E < nel) {
-                const int r = E / cj, c = E - r * cj;
-                T v = acc[t];
-                if (diag && r == c) v += (T)lambda * clampT(dU[t]);
-                val[boff[k] + E] = v;
+            const int E = lane + 32 * t, r = E / cj, c = E - r * cj;
+            const double d = __shfl_sync(0xffffffffu, s.du, min(r, 31));
+            if (E < nel) val[boff[k] + E] = diag && r == c ? fma(lambda, clampT(d), s.acc[t]) : s.acc[t];
+        }
+        if (diag && lane < ci) b[off[i] + lane] = s.bacc;
+    };
+    for (int64_t k0 = blockIdx.x * (int64_t)8; k0 < nnzb; k0 += (int64_t)gridDim.x * 8) {
+        const int nb = (int)min((int64_t)8, nnzb - k0);
+        // blocks of few pairs: one to a warp
+        if (w < nb) {
+            const int64_t k = k0 + w;
+            const int p0 = pptr[k], p1 = pptr[k + 1];
+            if (p1 - p0 <= VB64_SPLIT) {
+                const int i = brow[k], j = col[k], ci = cdim[i], cj = cdim[j];
+                Vbi64Sums s = {};
+                vbi64_pairs(p0, p1, 0, 1, ci, cj, jc0 ? jc0[i] : 0, jc0 ? jc0[j] : 0, i == j, plist, J2, PE, sm[w], s);
+                finish(k, i, cj, ci * cj, ci, i == j, s);
             }
         }
-        if (diag && lane < ci) b[off[i] + lane] = (T)bacc;
+        // the others: the CTA's warps together
+        for (int q = 0; q < nb; ++q) {
+            const int64_t k = k0 + q;
+            const int p0 = pptr[k], p1 = pptr[k + 1];
+            if (p1 - p0 <= VB64_SPLIT) continue;  // CTA-uniform
+            const int i = brow[k], j = col[k], ci = cdim[i], cj = cdim[j];
+            Vbi64Sums s = {};
+            vbi64_pairs(p0, p1, w, 8, ci, cj, jc0 ? jc0[i] : 0, jc0 ? jc0[j] : 0, i == j, plist, J2, PE, sm[w], s);
+            __syncthreads();  // the previous block's sums have been read
+#pragma unroll
+            for (int t = 0; t < VB_NT; ++t) join[w][32 * t + lane] = s.acc[t];
+            join[w][32 * VB_NT + lane] = s.du;
+            join[w][32 * (VB_NT + 1) + lane] = s.bacc;
+            __syncthreads();
+            if (w == (q & 7)) {
+                s = {};
+                for (int h = 0; h < 8; ++h) {
+#pragma unroll
+                    for (int t = 0; t < VB_NT; ++t) s.acc[t] += join[h][32 * t + lane];
+                    s.du += join[h][32 * VB_NT + lane];
+                    s.bacc += join[h][32 * (VB_NT + 1) + lane];
+                }
+                finish(k, i, cj, ci * cj, ci, i == j, s);
+            }
+        }
     }
 }
 
@@ -279,7 +478,7 @@ __global__ void __launch_bounds__(256) k_vbi_cost(int64_t m, const T *__restrict
                                                   unsigned *ctr) {
     double v[1] = {0.0};
     for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < m; a += (int64_t)gridDim.x * blockDim.x) {
-        const double e0 = (double)J[a * VJW + 28], e1 = (double)J[a * VJW + 29];
+        const double e0 = (double)J[a * VJW + VJE], e1 = (double)J[a * VJW + VJE + 1];
         v[0] += e0 * e0 + e1 * e1;
     }
     grid_sum<1>(v, red, ctr, [&](double *t) { sc->cost = 0.5 * t[0]; });
@@ -303,10 +502,10 @@ __global__ void __launch_bounds__(256) k_vbi_backsub(int64_t P, const int *__res
             const T *dc = dxc + off[i];
             double t0 = 0.0, t1 = 0.0;
             for (int c = 0; c < ci; ++c) {
-                t0 += (double)o[c] * (double)dc[c];
-                t1 += (double)o[VB_CI + c] * (double)dc[c];
+                t0 += (double)o[2 * c] * (double)dc[c];
+                t1 += (double)o[2 * c + 1] * (double)dc[c];
             }
-            for (int m = 0; m < 3; ++m) s[m] -= (double)o[22 + m] * t0 + (double)o[25 + m] * t1;
+            for (int m = 0; m < 3; ++m) s[m] -= (double)o[VJP + m] * t0 + (double)o[VJP + 3 + m] * t1;
         }
         const double *vi = Vinv + 9 * k;
         for (int m = 0; m < 3; ++m) {
@@ -367,14 +566,14 @@ __global__ void __launch_bounds__(256) k_vbi_trial(int64_t m, const int *__restr
         const T *dc = dxc + off[i];
         T t0 = T(0), t1 = T(0);
         for (int c = 0; c < ci; ++c) {
-            t0 += o[c] * dc[c];
-            t1 += o[VB_CI + c] * dc[c];
+            t0 += o[2 * c] * dc[c];
+            t1 += o[2 * c + 1] * dc[c];
         }
         for (int c = 0; c < 3; ++c) {
-            t0 += o[22 + c] * (T)dxp[3 * (int64_t)k + c];
-            t1 += o[25 + c] * (T)dxp[3 * (int64_t)k + c];
+            t0 += o[VJP + c] * (T)dxp[3 * (int64_t)k + c];
+            t1 += o[VJP + 3 + c] * (T)dxp[3 * (int64_t)k + c];
         }
-        v[1] -= (double)(t0 * (T(2) * o[28] + t0) + t1 * (T(2) * o[29] + t1));
+        v[1] -= (double)(t0 * (T(2) * o[VJE] + t0) + t1 * (T(2) * o[VJE + 1] + t1));
     }
     grid_sum<3>(v, red, ctr, [&](double *t) {
         sc->cost_trial = 0.5 * t[0];
@@ -506,13 +705,13 @@ cudaError_t vbi_form(ba_vbsmc *h, const VbiDev &d, int64_t P, double lambda) {
     if (h->fp32) {
         k_vbi_points<float><<<g2, 256, 0, h->st>>>(P, d.trk, (const float *)d.J, lambda, d.Vinv, d.lp, (float *)d.PE,
                                                    d.err);
-        k_vbi_blocks<float><<<g3, 256, 0, h->st>>>(h->nnzb, h->brow, h->col, h->cdim, d.jc0, h->off, h->boff, d.pptr,
+        k_vbi_blocks32<<<g3, 256, 0, h->st>>>(h->nnzb, h->brow, h->col, h->cdim, d.jc0, h->off, h->boff, d.pptr,
                                                    d.plist, (const float *)d.J, (const float *)d.PE, lambda,
                                                    (float *)h->val, (float *)h->b);
     } else {
         k_vbi_points<double><<<g2, 256, 0, h->st>>>(P, d.trk, (const double *)d.J, lambda, d.Vinv, d.lp,
                                                     (double *)d.PE, d.err);
-        k_vbi_blocks<double><<<g3, 256, 0, h->st>>>(h->nnzb, h->brow, h->col, h->cdim, d.jc0, h->off, h->boff,
+        k_vbi_blocks64<<<g3, 256, 0, h->st>>>(h->nnzb, h->brow, h->col, h->cdim, d.jc0, h->off, h->boff,
                                                     d.pptr, d.plist, (const double *)d.J, (const double *)d.PE,
                                                     lambda, (double *)h->val, (double *)h->b);
     }
