@@ -5,14 +5,16 @@
 // exterior and five interior unknowns per camera.  The interiors are
 // [f, cx, cy, k1, k2]: with xh = x/z, yh = y/z, r2 = xh^2 + yh^2 and
 // d = 1 + k1 r2 + k2 r2^2 the projection is u = f d xh + cx, v = f d yh + cy.
-// A camera has c_i = 6 (interiors fixed) or 11 unknowns.  Three kernels:
+// A camera has c_i = 6 (interiors fixed) or 11 unknowns.  Four kernels:
 //   k_vbi_linearize  e and J of every observation (Eq. 1), rows of
 //                    [J_c (11 x 2) | J_p (2 x 3) | e (2)] in the storage
 //                    precision (X_cam in FP64, the rest in that precision);
-//   k_vbi_points     per point, in FP64, V_k (damped), its Cholesky factor
-//                    L, V_k^-1 and l_p (Eq. 3), and per observation the
-//                    factor row P = J_p L^-T and e^ = e + P L^-1 l_p;
-//   k_vbi_blocks     a warp per stored block (i, j): the sum over its point
+//   k_vbi_factor     per point, in FP64, V_k (damped) and l_p (Eq. 3), the
+//                    inverse M = L^-1 of V_k's Cholesky factor and q = M l_p;
+//   k_vbi_rows       per observation, in FP64, the factor row P = J_p M^T and
+//                    e^ = e + P q;
+//   k_vbi_blocks32 / k_vbi_blocks64
+//                    a warp per stored block (i, j): the sum over its point
 //                    pairs of -J_c,a^T (P_a P_b^T) J_c,b = -W_a V_k^-1 W_b^T
 //                    (Eq. 4), plus U_i (damped) and b_i = -sum J_c^T e^ on
 //                    the diagonal, in the storage precision.  The pairs of a
@@ -38,14 +40,16 @@ constexpr int VB_CI = 11;    // unknowns of a self-calibrating camera
 constexpr int VB_NT = 4;     // block entries per lane: 4 x 32 >= 11 x 11
 
 // Per camera [R (9), t (3)] in FP64, R = Exp(omega).
+__device__ __forceinline__ void vbi_camera(const double *cam, double *out) {
+    double q[4], R[9];
+    quat_exp(cam, q);
+    quat_to_R(q, R);
+    for (int k = 0; k < 9; ++k) out[k] = R[k];
+    for (int k = 0; k < 3; ++k) out[9 + k] = cam[3 + k];
+}
 __global__ void k_vbi_camcache(int n, const double *__restrict__ cams, double *__restrict__ camc) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    double q[4], R[9];
-    quat_exp(cams + 6 * i, q);
-    quat_to_R(q, R);
-    for (int k = 0; k < 9; ++k) camc[12 * i + k] = R[k];
-    for (int k = 0; k < 3; ++k) camc[12 * i + 9 + k] = cams[6 * i + 3 + k];
+    if (i < n) vbi_camera(cams + 6 * i, camc + 12 * i);
 }
 
 // X_cam = R X + t in FP64 (no cancellation of the large world coordinates),
@@ -71,106 +75,196 @@ __device__ __forceinline__ VbiProj<T> vbi_project(const double *__restrict__ cam
     return o;
 }
 
-template <typename T>
-__global__ void __launch_bounds__(256) k_vbi_linearize(int64_t m, const int *__restrict__ ocam,
-                                                       const int *__restrict__ opt, const double *__restrict__ uv,
-                                                       const double *__restrict__ camc,
-                                                       const double *__restrict__ intr,
-                                                       const double *__restrict__ pts, T *__restrict__ J) {
-    for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < m; a += (int64_t)gridDim.x * blockDim.x) {
-        const int i = ocam[a], k = opt[a];
-        const VbiProj<T> pr = vbi_project<T>(camc, intr, pts, i, k, uv + 2 * a);
-        const double *R = camc + 12 * i, *kk = intr + 5 * i;
-        const T f = (T)kk[0], k1 = (T)kk[3], k2 = (T)kk[4];
-        const T z = pr.Xc[2], xh = pr.xh, yh = pr.yh, r2 = pr.r2, d = pr.d;
-        const T g = T(2) * (k1 + T(2) * k2 * r2);
-        // image-plane Jacobian D of (f d xh, f d yh) w.r.t. (xh, yh), then A = D d(xh, yh)/dX_cam
-        const T D00 = f * (d + g * xh * xh), D01 = f * g * xh * yh, D11 = f * (d + g * yh * yh);
-        T A[2][3];
-        A[0][0] = D00 / z;
-        A[0][1] = D01 / z;
-        A[0][2] = -(D00 * xh + D01 * yh) / z;
-        A[1][0] = D01 / z;
-        A[1][1] = D11 / z;
-        A[1][2] = -(D01 * xh + D11 * yh) / z;
-        // dX_cam/d(d_omega) = -[X_cam]x (camera-frame update), dX_cam/d(dt) = I, dX_cam/dX = R
-        const T *Xc = pr.Xc;
-        const T Mx[3][3] = {{T(0), Xc[2], -Xc[1]}, {-Xc[2], T(0), Xc[0]}, {Xc[1], -Xc[0], T(0)}};
-        T *o = J + a * VJW;
-        const T ph[2] = {xh, yh};
-        for (int r = 0; r < 2; ++r) {
-            T *jc = o + r, *jp = o + VJP + 3 * r;  // column c at jc[2 c]
-            for (int c = 0; c < 3; ++c) {
-                jc[2 * c] = A[r][0] * Mx[0][c] + A[r][1] * Mx[1][c] + A[r][2] * Mx[2][c];
-                jc[2 * (3 + c)] = A[r][c];
-                jp[c] = A[r][0] * (T)R[c] + A[r][1] * (T)R[3 + c] + A[r][2] * (T)R[6 + c];
-            }
-            jc[12] = d * ph[r];                // f
-            jc[14] = r == 0 ? T(1) : T(0);     // cx
-            jc[16] = r == 0 ? T(0) : T(1);     // cy
-            jc[18] = f * ph[r] * r2;           // k1
-            jc[20] = f * ph[r] * r2 * r2;      // k2
+// FP32 to FP64 without the FP64 pipe's conversion (16 cycles per warp, as much as
+// a multiply-add there; this is about six on the integer pipe): the exponent
+// rebiased, the mantissa shifted.  Exact; denormals, infinities and NaN take
+// the conversion.
+__device__ __forceinline__ double widen(float f) {
+    const unsigned u = __float_as_uint(f), m = u << 1;
+    if (m != 0u && m - 0x01000000u >= 0xfe000000u) return (double)f;
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (m ? 0x38000000u : 0u))),
+                            (int)(u << 29));
+}
+__device__ __forceinline__ double widen(double d) { return d; }
+
+// N values from a 16-byte aligned address with 16-byte loads.
+template <int N, typename T>
+__device__ __forceinline__ void load_vec(const T *__restrict__ p, T (&v)[N]) {
+    static_assert(N * sizeof(T) % 16 == 0, "whole 16-byte words");
+    if constexpr (sizeof(T) == 4) {
+        const float4 *q = reinterpret_cast<const float4 *>(p);
+#pragma unroll
+        for (int k = 0; k < N / 4; ++k) {
+            const float4 t = __ldg(q + k);
+            v[4 * k] = t.x; v[4 * k + 1] = t.y; v[4 * k + 2] = t.z; v[4 * k + 3] = t.w;
         }
-        o[VJE] = pr.e0;
-        o[VJE + 1] = pr.e1;
-        o[22] = T(0);
-        o[23] = T(0);
+    } else {
+        const double2 *q = reinterpret_cast<const double2 *>(p);
+#pragma unroll
+        for (int k = 0; k < N / 2; ++k) {
+            const double2 t = __ldg(q + k);
+            v[2 * k] = t.x; v[2 * k + 1] = t.y;
+        }
     }
 }
 
-// Per point, in FP64: V_k = sum J_p^T J_p + lambda clamp(diag), its
-// Cholesky factor V_k = L L^T (the three pivots must be positive), V_k^-1
-// and l_p = -sum J_p^T e for Eq. 5; then per observation of the point the
-// factor row P_a = J_p,a L^-T and e^_a = e_a + P_a (L^-1 l_p), in T, so that
-// -W_a V^-1 W_b^T = -J_c,a^T (P_a P_b^T) J_c,b and
-// -J_c,a^T e_a - W_a V^-1 l_p = -J_c,a^T e^_a (the block kernel's products).
+struct VbiScalars {
+    double cost, cost_trial, model;
+    unsigned long long n_cheir_trial;
+};
+
+// A thread per observation; a warp's 32 rows leave through shared memory, so
+// that each is written as whole lines.  With sc, also F = 1/2 sum ||e||^2 of the
+// stored e (FP64 sum).  (Rows written value by value from the threads, with the
+// cost in a pass of its own, took 101 us for 485,000 observations in FP32; this
+// takes 47.)
+constexpr int VLT = 128;  // threads per CTA
 template <typename T>
-__global__ void __launch_bounds__(256) k_vbi_points(int64_t P, const int *__restrict__ trk_ptr,
-                                                    const T *__restrict__ J, double lambda, double *__restrict__ Vinv,
-                                                    double *__restrict__ lp, T *__restrict__ PE, int *err) {
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < P; k += (int64_t)gridDim.x * blockDim.x) {
-        double V[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}}, l[3] = {0, 0, 0};
-        for (int a = trk_ptr[k]; a < trk_ptr[k + 1]; ++a) {
-            const T *o = J + (int64_t)a * VJW;
-            double jp[6];
-            for (int q = 0; q < 6; ++q) jp[q] = (double)o[VJP + q];
-            const double e0 = (double)o[VJE], e1 = (double)o[VJE + 1];
-            for (int m = 0; m < 3; ++m) {
-                for (int n = 0; n < 3; ++n) V[m][n] += jp[m] * jp[n] + jp[3 + m] * jp[3 + n];
-                l[m] -= jp[m] * e0 + jp[3 + m] * e1;
+__global__ void __launch_bounds__(VLT) k_vbi_linearize(int64_t m, const int *__restrict__ ocam,
+                                                       const int *__restrict__ opt, const double *__restrict__ uv,
+                                                       const double *__restrict__ camc,
+                                                       const double *__restrict__ intr,
+                                                       const double *__restrict__ pts, T *__restrict__ J,
+                                                       VbiScalars *sc, double *red, unsigned *ctr) {
+    __shared__ T rows[VLT / 32][32][VJW + 1];
+    const int lane = threadIdx.x & 31;
+    T(*row)[VJW + 1] = rows[threadIdx.x >> 5];
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    double F[1] = {0.0};
+    for (int64_t base = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); base < m; base += stride) {
+        const int64_t a = base + lane;
+        if (a < m) {
+            const int i = ocam[a], k = opt[a];
+            const VbiProj<T> pr = vbi_project<T>(camc, intr, pts, i, k, uv + 2 * a);
+            const double *R = camc + 12 * i, *kk = intr + 5 * i;
+            const T f = (T)kk[0], k1 = (T)kk[3], k2 = (T)kk[4];
+            const T z = pr.Xc[2], xh = pr.xh, yh = pr.yh, r2 = pr.r2, d = pr.d;
+            const T g = T(2) * (k1 + T(2) * k2 * r2);
+            // image-plane Jacobian D of (f d xh, f d yh) w.r.t. (xh, yh), then A = D d(xh, yh)/dX_cam
+            const T D00 = f * (d + g * xh * xh), D01 = f * g * xh * yh, D11 = f * (d + g * yh * yh);
+            T A[2][3];
+            A[0][0] = D00 / z;
+            A[0][1] = D01 / z;
+            A[0][2] = -(D00 * xh + D01 * yh) / z;
+            A[1][0] = D01 / z;
+            A[1][1] = D11 / z;
+            A[1][2] = -(D01 * xh + D11 * yh) / z;
+            // dX_cam/d(d_omega) = -[X_cam]x (camera-frame update), dX_cam/d(dt) = I, dX_cam/dX = R
+            const T *Xc = pr.Xc;
+            const T Mx[3][3] = {{T(0), Xc[2], -Xc[1]}, {-Xc[2], T(0), Xc[0]}, {Xc[1], -Xc[0], T(0)}};
+            T *o = row[lane];
+            const T ph[2] = {xh, yh};
+            for (int r = 0; r < 2; ++r) {
+                T *jc = o + r, *jp = o + VJP + 3 * r;  // column c at jc[2 c]
+                for (int c = 0; c < 3; ++c) {
+                    jc[2 * c] = A[r][0] * Mx[0][c] + A[r][1] * Mx[1][c] + A[r][2] * Mx[2][c];
+                    jc[2 * (3 + c)] = A[r][c];
+                    jp[c] = A[r][0] * (T)R[c] + A[r][1] * (T)R[3 + c] + A[r][2] * (T)R[6 + c];
+                }
+                jc[12] = d * ph[r];                // f
+                jc[14] = r == 0 ? T(1) : T(0);     // cx
+                jc[16] = r == 0 ? T(0) : T(1);     // cy
+                jc[18] = f * ph[r] * r2;           // k1
+                jc[20] = f * ph[r] * r2 * r2;      // k2
+            }
+            o[VJE] = pr.e0;
+            o[VJE + 1] = pr.e1;
+            o[22] = T(0);
+            o[23] = T(0);
+            if (sc) {
+                const double e0 = widen(pr.e0), e1 = widen(pr.e1);
+                F[0] += e0 * e0 + e1 * e1;
             }
         }
-        for (int m = 0; m < 3; ++m) V[m][m] += lambda * clampT(V[m][m]);
-        // V = L L^T, M = L^-1 (lower)
-        const double d0 = sqrt(V[0][0]), c10 = V[0][1] / d0, c20 = V[0][2] / d0;
-        const double s11 = V[1][1] - c10 * c10, d1 = sqrt(s11), c21 = (V[1][2] - c20 * c10) / d1;
-        const double s22 = V[2][2] - c20 * c20 - c21 * c21, d2 = sqrt(s22);
-        const bool ok = V[0][0] > 0.0 && s11 > 0.0 && s22 > 0.0;
+        __syncwarp();
+        const int nr = (int)min((int64_t)32, m - base);
+        T *out = J + base * VJW + lane;
+#pragma unroll 8
+        for (int r = 0; r < nr; ++r) out[r * VJW] = row[r][lane];
+        __syncwarp();
+    }
+    if (sc) grid_sum<1>(F, red, ctr, [&](double *t) { sc->cost = 0.5 * t[0]; });
+}
+
+// Per point, in FP64: V_k = sum J_p^T J_p + lambda clamp(diag), its Cholesky
+// factor V_k = L L^T (the three pivots must be positive), l_p = -sum J_p^T e;
+// stored per point: M = L^-1 (m00 m10 m11 m20 m21 m22) and q = M l_p, from
+// which Eq. 5 and the factor rows follow.  A thread per point, in the order
+// `ord` of track lengths, so that the threads of a warp loop alike (bound by
+// FP64 issue; in the points' own order a warp runs its longest track, 2.6
+// times the mean).  With k_vbi_rows 96 us at 99,000 points, 485,000
+// observations, against 275 us for one kernel in the points' own order that
+// also formed the factor rows.
+template <typename T>
+__global__ void __launch_bounds__(128) k_vbi_factor(int64_t P, const int *__restrict__ ord,
+                                                    const int *__restrict__ trk_ptr, const T *__restrict__ J,
+                                                    double lambda, double *__restrict__ Mq, int *err) {
+    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < P; x += (int64_t)gridDim.x * blockDim.x) {
+        const int k = __ldg(ord + x);
+        double v00 = 0, v01 = 0, v02 = 0, v11 = 0, v12 = 0, v22 = 0, l0 = 0, l1 = 0, l2 = 0;
+        const int a1 = __ldg(trk_ptr + k + 1);
+        for (int a = __ldg(trk_ptr + k); a < a1; ++a) {
+            T s[8];
+            load_vec<8>(J + (int64_t)a * VJW + VJP, s);
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                const double p0 = widen(s[3 * r]), p1 = widen(s[3 * r + 1]), p2 = widen(s[3 * r + 2]);
+                const double e = widen(s[6 + r]);
+                v00 = fma(p0, p0, v00); v01 = fma(p0, p1, v01); v02 = fma(p0, p2, v02);
+                v11 = fma(p1, p1, v11); v12 = fma(p1, p2, v12); v22 = fma(p2, p2, v22);
+                l0 = fma(-p0, e, l0); l1 = fma(-p1, e, l1); l2 = fma(-p2, e, l2);
+            }
+        }
+        v00 += lambda * clampT(v00);
+        v11 += lambda * clampT(v11);
+        v22 += lambda * clampT(v22);
+        const double d0 = sqrt(v00), c10 = v01 / d0, c20 = v02 / d0;
+        const double s11 = v11 - c10 * c10, d1 = sqrt(s11), c21 = (v12 - c20 * c10) / d1;
+        const double s22 = v22 - c20 * c20 - c21 * c21, d2 = sqrt(s22);
+        const bool ok = v00 > 0.0 && s11 > 0.0 && s22 > 0.0;
         double m00 = 1.0 / d0, m11 = 1.0 / d1, m22 = 1.0 / d2;
         double m10 = -c10 * m00 * m11, m21 = -c21 * m11 * m22, m20 = -(c20 * m00 + c21 * m10) * m22;
         if (!ok) {
             atomicExch(err, (int)BA_ERR_NOT_SPD);
             m00 = m11 = m22 = m10 = m21 = m20 = 0.0;
         }
-        // V^-1 = M^T M
-        const double Mm[3][3] = {{m00, 0.0, 0.0}, {m10, m11, 0.0}, {m20, m21, m22}};
-        double *vi = Vinv + 9 * k;
-        for (int r = 0; r < 3; ++r)
-            for (int c = 0; c < 3; ++c) vi[3 * r + c] = Mm[0][r] * Mm[0][c] + Mm[1][r] * Mm[1][c] + Mm[2][r] * Mm[2][c];
-        for (int m = 0; m < 3; ++m) lp[3 * k + m] = l[m];
-        const double q0 = m00 * l[0], q1 = m10 * l[0] + m11 * l[1], q2 = m20 * l[0] + m21 * l[1] + m22 * l[2];
-        for (int a = trk_ptr[k]; a < trk_ptr[k + 1]; ++a) {
-            const T *o = J + (int64_t)a * VJW;
-            T *pe = PE + (int64_t)a * VPW;
-            for (int r = 0; r < 2; ++r) {
-                const double j0 = (double)o[VJP + 3 * r], j1 = (double)o[VJP + 1 + 3 * r], j2 = (double)o[VJP + 2 + 3 * r];
-                // P = J_p L^-T: P_c = sum_k J_k (L^-1)_ck over k <= c
-                const double P0 = j0 * m00, P1 = j0 * m10 + j1 * m11, P2 = j0 * m20 + j1 * m21 + j2 * m22;
-                pe[3 * r] = (T)P0;
-                pe[3 * r + 1] = (T)P1;
-                pe[3 * r + 2] = (T)P2;
-                pe[6 + r] = (T)((double)o[VJE + r] + P0 * q0 + P1 * q1 + P2 * q2);
-            }
+        double *o = Mq + 9 * (int64_t)k;
+        o[0] = m00; o[1] = m10; o[2] = m11; o[3] = m20; o[4] = m21; o[5] = m22;
+        o[6] = m00 * l0;
+        o[7] = m10 * l0 + m11 * l1;
+        o[8] = m20 * l0 + m21 * l1 + m22 * l2;
+    }
+}
+
+// Per observation, in FP64, the factor row P = J_p M^T and e^ = e + P q of its
+// point, stored in T, so that -W_a V^-1 W_b^T = -J_c,a^T (P_a P_b^T) J_c,b and
+// -J_c,a^T e_a - W_a V^-1 l_p = -J_c,a^T e^_a (the block kernels' products).
+template <typename T>
+__global__ void __launch_bounds__(256) k_vbi_rows(int64_t m, const int *__restrict__ opt, const T *__restrict__ J,
+                                                  const double *__restrict__ Mq, T *__restrict__ PE) {
+    for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < m; a += (int64_t)gridDim.x * blockDim.x) {
+        T s[8], o[8];
+        load_vec<8>(J + a * VJW + VJP, s);
+        const double *w = Mq + 9 * (int64_t)__ldg(opt + a);
+        const double m00 = __ldg(w), m10 = __ldg(w + 1), m11 = __ldg(w + 2), m20 = __ldg(w + 3), m21 = __ldg(w + 4),
+                     m22 = __ldg(w + 5), q0 = __ldg(w + 6), q1 = __ldg(w + 7), q2 = __ldg(w + 8);
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+            const double j0 = widen(s[3 * r]), j1 = widen(s[3 * r + 1]), j2 = widen(s[3 * r + 2]);
+            // P = J_p L^-T: P_c = sum_k J_k (L^-1)_ck over k <= c
+            const double P0 = j0 * m00, P1 = j0 * m10 + j1 * m11, P2 = j0 * m20 + j1 * m21 + j2 * m22;
+            o[3 * r] = (T)P0;
+            o[3 * r + 1] = (T)P1;
+            o[3 * r + 2] = (T)P2;
+            o[6 + r] = (T)(widen(s[6 + r]) + P0 * q0 + P1 * q1 + P2 * q2);
+        }
+        T *pe = PE + a * VPW;
+        if constexpr (sizeof(T) == 4) {
+            reinterpret_cast<float4 *>(pe)[0] = make_float4(o[0], o[1], o[2], o[3]);
+            reinterpret_cast<float4 *>(pe)[1] = make_float4(o[4], o[5], o[6], o[7]);
+        } else {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) reinterpret_cast<double2 *>(pe)[q] = make_double2(o[2 * q], o[2 * q + 1]);
         }
     }
 }
@@ -236,7 +330,8 @@ __device__ __forceinline__ void vbi_middle(const T *__restrict__ Pa, const T *__
 // (Before, both J rows passed through shared memory with two warp barriers per
 // pair, and every lane formed M: 1031 -> 386 us at 990 cameras of c = 11, 485,000
 // observations, the same bits.)
-__global__ void __launch_bounds__(256) k_vbi_blocks32(int64_t nnzb, const int *__restrict__ brow,
+constexpr int VB32_WARPS = 2;  // per CTA: few, so that a block of many pairs holds back few others
+__global__ void __launch_bounds__(32 * VB32_WARPS) k_vbi_blocks32(int64_t nnzb, const int *__restrict__ brow,
                                                       const int *__restrict__ col, const int *__restrict__ cdim,
                                                       const int *__restrict__ jc0, const int *__restrict__ off,
                                                       const int64_t *__restrict__ boff, const int *__restrict__ pptr,
@@ -246,8 +341,8 @@ __global__ void __launch_bounds__(256) k_vbi_blocks32(int64_t nnzb, const int *_
     constexpr unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31, rg = lane >> 3, cg = lane & 7;
     const float2 *J2 = reinterpret_cast<const float2 *>(J);
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t k = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; k < nnzb; k += nw) {
+    const int64_t k = blockIdx.x * (int64_t)VB32_WARPS + (threadIdx.x >> 5);
+    if (k < nnzb) {
         const int i = brow[k], j = col[k], ci = cdim[i], cj = cdim[j];
         const int rpl = (ci + 3) >> 2, cpl = (cj + 7) >> 3;  // rows and columns per lane
         const int r0 = rpl * rg, c0 = cpl * cg;
@@ -319,10 +414,11 @@ __global__ void __launch_bounds__(256) k_vbi_blocks32(int64_t nnzb, const int *_
 // instructions per four pairs) and every lane adds its four entries of the
 // block with 8 per pair (32 before, M and the products formed pair by pair).
 // A block of more than VB64_SPLIT pairs (a diagonal block, mostly) is shared by
-// the CTA's eight warps, which take batches of 32 pairs in turn and join their
+// the CTA's VB64_WARPS warps, which take batches of 32 pairs in turn and join their
 // sums in shared memory.  1778 -> 297 us at 120 cameras (half of them c = 11),
 // 58,000 observations.
 constexpr int VB64_SPLIT = 96;
+constexpr int VB64_WARPS = 8;
 struct Vbi64Sums {
     double acc[VB_NT], du, bacc;  // entries lane + 32 t; row `lane`'s U diagonal and b
 };
@@ -401,15 +497,15 @@ __device__ __forceinline__ void vbi64_pairs(int p0, int p1, int first, int step,
         }
     }
 }
-__global__ void __launch_bounds__(256) k_vbi_blocks64(int64_t nnzb, const int *__restrict__ brow,
+__global__ void __launch_bounds__(32 * VB64_WARPS) k_vbi_blocks64(int64_t nnzb, const int *__restrict__ brow,
                                                       const int *__restrict__ col, const int *__restrict__ cdim,
                                                       const int *__restrict__ jc0, const int *__restrict__ off,
                                                       const int64_t *__restrict__ boff, const int *__restrict__ pptr,
                                                       const int2 *__restrict__ plist, const double *__restrict__ J,
                                                       const double *__restrict__ PE, double lambda,
                                                       double *__restrict__ val, double *__restrict__ b) {
-    __shared__ double sm[8][2 * 4 * 2 * VB_CI];     // staging per warp
-    __shared__ double join[8][(VB_NT + 2) * 32];    // a shared block's sums per warp
+    __shared__ double sm[VB64_WARPS][2 * 4 * 2 * VB_CI];     // staging per warp
+    __shared__ double join[VB64_WARPS][(VB_NT + 2) * 32];    // a shared block's sums per warp
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const double2 *J2 = reinterpret_cast<const double2 *>(J);
     auto finish = [&](int64_t k, int i, int cj, int nel, int ci, bool diag, const Vbi64Sums &s) {
@@ -421,8 +517,9 @@ __global__ void __launch_bounds__(256) k_vbi_blocks64(int64_t nnzb, const int *_
         }
         if (diag && lane < ci) b[off[i] + lane] = s.bacc;
     };
-    for (int64_t k0 = blockIdx.x * (int64_t)8; k0 < nnzb; k0 += (int64_t)gridDim.x * 8) {
-        const int nb = (int)min((int64_t)8, nnzb - k0);
+    {
+        const int64_t k0 = blockIdx.x * (int64_t)VB64_WARPS;
+        const int nb = (int)min((int64_t)VB64_WARPS, nnzb - k0);
         // blocks of few pairs: one to a warp
         if (w < nb) {
             const int64_t k = k0 + w;
@@ -441,16 +538,16 @@ __global__ void __launch_bounds__(256) k_vbi_blocks64(int64_t nnzb, const int *_
             if (p1 - p0 <= VB64_SPLIT) continue;  // CTA-uniform
             const int i = brow[k], j = col[k], ci = cdim[i], cj = cdim[j];
             Vbi64Sums s = {};
-            vbi64_pairs(p0, p1, w, 8, ci, cj, jc0 ? jc0[i] : 0, jc0 ? jc0[j] : 0, i == j, plist, J2, PE, sm[w], s);
+            vbi64_pairs(p0, p1, w, VB64_WARPS, ci, cj, jc0 ? jc0[i] : 0, jc0 ? jc0[j] : 0, i == j, plist, J2, PE, sm[w], s);
             __syncthreads();  // the previous block's sums have been read
 #pragma unroll
             for (int t = 0; t < VB_NT; ++t) join[w][32 * t + lane] = s.acc[t];
             join[w][32 * VB_NT + lane] = s.du;
             join[w][32 * (VB_NT + 1) + lane] = s.bacc;
             __syncthreads();
-            if (w == (q & 7)) {
+            if (w == q % VB64_WARPS) {
                 s = {};
-                for (int h = 0; h < 8; ++h) {
+                for (int h = 0; h < VB64_WARPS; ++h) {
 #pragma unroll
                     for (int t = 0; t < VB_NT; ++t) s.acc[t] += join[h][32 * t + lane];
                     s.du += join[h][32 * VB_NT + lane];
@@ -463,66 +560,84 @@ __global__ void __launch_bounds__(256) k_vbi_blocks64(int64_t nnzb, const int *_
 }
 
 // ---------------------------------------------------------------------------
-// LM iteration with interiors: cost, Eq. 5, the trial state and its cost, and
-// the model decrease of the gain ratio (all FP64)
+// LM iteration with interiors: Eq. 5, the trial state and its cost, and the
+// model decrease of the gain ratio (all FP64)
 // ---------------------------------------------------------------------------
 
-struct VbiScalars {
-    double cost, cost_trial, model;
-    unsigned long long n_cheir_trial;
-};
-
-// F = 1/2 sum ||e||^2 from the stored rows (after k_vbi_linearize), FP64 sum
+// Eq. 5, first half: per observation J_p,a^T (J_c,a dx_c) in FP64 (the sum over
+// the camera's c_i columns; dxc is the solve's vector, c_i entries per camera at
+// off[i]) into `g`, three doubles at the start of the observation's factor row
+// (rewritten by the next formation).  A thread per observation, so that no
+// thread waits for a longer track.
 template <typename T>
-__global__ void __launch_bounds__(256) k_vbi_cost(int64_t m, const T *__restrict__ J, VbiScalars *sc, double *red,
-                                                  unsigned *ctr) {
-    double v[1] = {0.0};
+__global__ void __launch_bounds__(256) k_vbi_jdx(int64_t m, const int *__restrict__ ocam, const T *__restrict__ J,
+                                                 const int *__restrict__ cdim, const int *__restrict__ off,
+                                                 const T *__restrict__ dxc, T *__restrict__ g) {
     for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < m; a += (int64_t)gridDim.x * blockDim.x) {
-        const double e0 = (double)J[a * VJW + VJE], e1 = (double)J[a * VJW + VJE + 1];
-        v[0] += e0 * e0 + e1 * e1;
+        const int i = __ldg(ocam + a), ci = __ldg(cdim + i);
+        const T *dc = dxc + __ldg(off + i);
+        T o[VJW];
+        load_vec<VJW>(J + a * VJW, o);
+        double t0 = 0.0, t1 = 0.0;
+#pragma unroll
+        for (int c = 0; c < VB_CI; ++c) {
+            if (c >= ci) break;
+            const double d = widen(__ldg(dc + c));
+            t0 = fma(widen(o[2 * c]), d, t0);
+            t1 = fma(widen(o[2 * c + 1]), d, t1);
+        }
+        double *w = reinterpret_cast<double *>(g + a * VPW);
+        double c3[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) c3[q] = fma(widen(o[VJP + q]), t0, widen(o[VJP + 3 + q]) * t1);
+        *reinterpret_cast<double2 *>(w) = make_double2(c3[0], c3[1]);
+        w[2] = c3[2];
     }
-    grid_sum<1>(v, red, ctr, [&](double *t) { sc->cost = 0.5 * t[0]; });
 }
 
-// Eq. 5 per point: dx_p = V^-1 (l_p - sum_a W_a^T dx_c,cam(a)) with
-// W_a^T dx = J_p,a^T (J_c,a dx) over the camera's c_i columns; the trial
-// point X + dx_p.  dxc is the solve's vector (c_i entries per camera at off[i]).
+// Eq. 5, second half, per point (in the order of track lengths): with V^-1 =
+// M^T M and q = M l_p, dx_p = M^T (q - M sum_a J_p,a^T J_c,a dx_c), and the
+// trial point X + dx_p.  One pass over tracks and FP64 conversions of every J_c
+// value by a thread per point took 261 us at 485,000 observations; the two
+// kernels take 56.
 template <typename T>
-__global__ void __launch_bounds__(256) k_vbi_backsub(int64_t P, const int *__restrict__ trk_ptr,
-                                                     const int *__restrict__ ocam, const T *__restrict__ J,
-                                                     const double *__restrict__ Vinv, const double *__restrict__ lp,
-                                                     const int *__restrict__ cdim, const int *__restrict__ off,
-                                                     const T *__restrict__ dxc, const double *__restrict__ pts,
-                                                     double *__restrict__ dxp, double *__restrict__ pts_t) {
-    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < P; k += (int64_t)gridDim.x * blockDim.x) {
-        double s[3] = {lp[3 * k], lp[3 * k + 1], lp[3 * k + 2]};
-        for (int a = trk_ptr[k]; a < trk_ptr[k + 1]; ++a) {
-            const T *o = J + (int64_t)a * VJW;
-            const int i = ocam[a], ci = cdim[i];
-            const T *dc = dxc + off[i];
-            double t0 = 0.0, t1 = 0.0;
-            for (int c = 0; c < ci; ++c) {
-                t0 += (double)o[2 * c] * (double)dc[c];
-                t1 += (double)o[2 * c + 1] * (double)dc[c];
-            }
-            for (int m = 0; m < 3; ++m) s[m] -= (double)o[VJP + m] * t0 + (double)o[VJP + 3 + m] * t1;
+__global__ void __launch_bounds__(128) k_vbi_dxp(int64_t P, const int *__restrict__ ord,
+                                                 const int *__restrict__ trk_ptr, const T *__restrict__ g,
+                                                 const double *__restrict__ Mq, const double *__restrict__ pts,
+                                                 double *__restrict__ dxp, double *__restrict__ pts_t) {
+    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < P; x += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t k = __ldg(ord + x);
+        double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+        const int a1 = __ldg(trk_ptr + k + 1);
+        for (int a = __ldg(trk_ptr + k); a < a1; ++a) {
+            const double *w = reinterpret_cast<const double *>(g + (int64_t)a * VPW);
+            const double2 u = *reinterpret_cast<const double2 *>(w);
+            s0 += u.x;
+            s1 += u.y;
+            s2 += w[2];
         }
-        const double *vi = Vinv + 9 * k;
-        for (int m = 0; m < 3; ++m) {
-            const double d = vi[3 * m] * s[0] + vi[3 * m + 1] * s[1] + vi[3 * m + 2] * s[2];
-            dxp[3 * k + m] = d;
-            pts_t[3 * k + m] = pts[3 * k + m] + d;
+        const double *w = Mq + 9 * k;
+        const double m00 = w[0], m10 = w[1], m11 = w[2], m20 = w[3], m21 = w[4], m22 = w[5];
+        const double u0 = w[6] - m00 * s0, u1 = w[7] - (m10 * s0 + m11 * s1),
+                     u2 = w[8] - (m20 * s0 + m21 * s1 + m22 * s2);
+        const double d[3] = {m00 * u0 + m10 * u1 + m20 * u2, m11 * u1 + m21 * u2, m22 * u2};
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            dxp[3 * k + q] = d[q];
+            pts_t[3 * k + q] = pts[3 * k + q] + d[q];
         }
     }
 }
 
 // The trial cameras: the pose perturbed in the camera frame,
 // R <- Exp(d_omega) R, t <- Exp(d_omega) t + dt (unit quaternions), and the
-// interiors of a self-calibrating camera (c_i = 11) moved additively.
+// interiors of a self-calibrating camera (c_i = 11) moved additively; also the
+// trial cameras' [R, t].
 template <typename T>
 __global__ void k_vbi_update_cams(int n, const double *__restrict__ cams, const double *__restrict__ intr,
                                   const int *__restrict__ cdim, const int *__restrict__ off, const T *__restrict__ dxc,
-                                  double *__restrict__ cams_t, double *__restrict__ intr_t) {
+                                  double *__restrict__ cams_t, double *__restrict__ intr_t,
+                                  double *__restrict__ camc_t) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const T *dc = dxc + off[i];
@@ -540,6 +655,7 @@ __global__ void k_vbi_update_cams(int n, const double *__restrict__ cams, const 
         cams_t[6 * i + r] = w[r];
         cams_t[6 * i + 3 + r] = Rd[3 * r] * t[0] + Rd[3 * r + 1] * t[1] + Rd[3 * r + 2] * t[2] + (double)dc[3 + r];
     }
+    vbi_camera(cams_t + 6 * i, camc_t + 12 * i);
     const bool self_cal = cdim[i] == VB_CI;
     for (int r = 0; r < 5; ++r) intr_t[5 * i + r] = intr[5 * i + r] + (self_cal ? (double)dc[6 + r] : 0.0);
 }
@@ -560,20 +676,25 @@ __global__ void __launch_bounds__(256) k_vbi_trial(int64_t m, const int *__restr
     for (int64_t a = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; a < m; a += (int64_t)gridDim.x * blockDim.x) {
         const int i = ocam[a], k = opt[a], ci = cdim[i];
         const VbiProj<T> pr = vbi_project<T>(camc_t, intr_t, pts_t, i, k, uv + 2 * a);
-        v[0] += (double)pr.e0 * (double)pr.e0 + (double)pr.e1 * (double)pr.e1;
+        const double e0 = widen(pr.e0), e1 = widen(pr.e1);
+        v[0] += e0 * e0 + e1 * e1;
         v[2] += pr.Xc[2] <= T(1e-6) ? 1.0 : 0.0;
-        const T *o = J + a * VJW;
+        T o[VJW];
+        load_vec<VJW>(J + a * VJW, o);
         const T *dc = dxc + off[i];
         T t0 = T(0), t1 = T(0);
-        for (int c = 0; c < ci; ++c) {
-            t0 += o[2 * c] * dc[c];
-            t1 += o[2 * c + 1] * dc[c];
+#pragma unroll
+        for (int c = 0; c < VB_CI; ++c) {
+            if (c >= ci) break;
+            const T d = __ldg(dc + c);
+            t0 = fma(o[2 * c], d, t0);
+            t1 = fma(o[2 * c + 1], d, t1);
         }
         for (int c = 0; c < 3; ++c) {
             t0 += o[VJP + c] * (T)dxp[3 * (int64_t)k + c];
             t1 += o[VJP + 3 + c] * (T)dxp[3 * (int64_t)k + c];
         }
-        v[1] -= (double)(t0 * (T(2) * o[VJE] + t0) + t1 * (T(2) * o[VJE + 1] + t1));
+        v[1] -= widen(t0 * (T(2) * o[VJE] + t0) + t1 * (T(2) * o[VJE + 1] + t1));
     }
     grid_sum<3>(v, red, ctr, [&](double *t) {
         sc->cost_trial = 0.5 * t[0];
@@ -674,57 +795,93 @@ ba_status vbi_layout(int32_t nblk, int64_t P, const std::vector<int32_t> &trk_pt
     return BA_OK;
 }
 
+// The points in the order of their track lengths (stable).
+std::vector<int32_t> order_by_length(const std::vector<int32_t> &trk_ptr, int64_t P) {
+    int32_t most = 0;
+    for (int64_t k = 0; k < P; ++k) most = std::max(most, trk_ptr[k + 1] - trk_ptr[k]);
+    std::vector<int64_t> at((size_t)most + 2, 0);
+    for (int64_t k = 0; k < P; ++k) at[trk_ptr[k + 1] - trk_ptr[k] + 1]++;
+    for (int32_t l = 0; l <= most; ++l) at[l + 1] += at[l];
+    std::vector<int32_t> ord(P);
+    for (int64_t k = 0; k < P; ++k) ord[at[trk_ptr[k + 1] - trk_ptr[k]]++] = (int32_t)k;
+    return ord;
+}
+
 // Device inputs of the formation, owned by the caller of vbi_form.
 struct VbiDev {
     int *ocam = nullptr, *opt = nullptr, *trk = nullptr, *pptr = nullptr, *jc0 = nullptr, *err = nullptr;
+    int *ord = nullptr;  // points by track length
     int2 *plist = nullptr;
-    double *uv = nullptr, *Vinv = nullptr, *lp = nullptr, *camc = nullptr;
+    double *uv = nullptr, *Mq = nullptr, *camc = nullptr;  // Mq: 9 values per point (k_vbi_factor)
     void *J = nullptr, *PE = nullptr;  // rows in the storage precision: VJW and VPW values per observation
 };
 
-// e and J at (cams, intr, pts): the cameras' [R, t] into d.camc, then the rows.
-cudaError_t vbi_linearize(ba_vbsmc *h, const VbiDev &d, int64_t m, int n, const double *cams, const double *intr,
-                          const double *pts) {
-    k_vbi_camcache<<<(n + 127) / 128, 128, 0, h->st>>>(n, cams, d.camc);
-    const int g1 = (int)std::min<int64_t>((m + 255) / 256, 152 * 16);
-    if (h->fp32)
-        k_vbi_linearize<float><<<g1, 256, 0, h->st>>>(m, d.ocam, d.opt, d.uv, d.camc, intr, pts, (float *)d.J);
-    else
-        k_vbi_linearize<double><<<g1, 256, 0, h->st>>>(m, d.ocam, d.opt, d.uv, d.camc, intr, pts, (double *)d.J);
+// e and J at (cams, intr, pts): the cameras' [R, t] into d.camc, then the rows
+// and, with sc, their cost.
+template <typename T>
+cudaError_t vbi_linearize_T(ba_vbsmc *h, const VbiDev &d, int64_t m, int n, const double *cams, const double *intr,
+                            const double *pts, VbiScalars *sc, double *red, unsigned *ctr) {
+    k_vbi_camcache<<<(n + 31) / 32, 32, 0, h->st>>>(n, cams, d.camc);
+    const int g = (int)std::min<int64_t>((m + VLT - 1) / VLT, 152 * 16);
+    k_vbi_linearize<T><<<g, VLT, 0, h->st>>>(m, d.ocam, d.opt, d.uv, d.camc, intr, pts, (T *)d.J, sc, red, ctr);
     return cudaGetLastError();
 }
+cudaError_t vbi_linearize(ba_vbsmc *h, const VbiDev &d, int64_t m, int n, const double *cams, const double *intr,
+                          const double *pts, VbiScalars *sc = nullptr, double *red = nullptr,
+                          unsigned *ctr = nullptr) {
+    return h->fp32 ? vbi_linearize_T<float>(h, d, m, n, cams, intr, pts, sc, red, ctr)
+                   : vbi_linearize_T<double>(h, d, m, n, cams, intr, pts, sc, red, ctr);
+}
 
-// From the stored rows: V_k^-1, l_p and the factor rows per point, then the
-// damped RCS into h's values and b (queued on h's stream; M^-1 is left to
-// vb_finish).
-cudaError_t vbi_form(ba_vbsmc *h, const VbiDev &d, int64_t P, double lambda) {
+// From the stored rows: M and q per point, the factor rows, then the damped
+// RCS into h's values and b (queued on h's stream; M^-1 is left to vb_finish).
+template <typename T>
+void vbi_factor_T(ba_vbsmc *h, const VbiDev &d, int64_t P, int64_t m, double lambda) {
+    const int gp = (int)std::min<int64_t>((P + 127) / 128, 152 * 16), gm = (int)std::min<int64_t>((m + 255) / 256, 152 * 16);
+    k_vbi_factor<T><<<gp, 128, 0, h->st>>>(P, d.ord, d.trk, (const T *)d.J, lambda, d.Mq, d.err);
+    k_vbi_rows<T><<<gm, 256, 0, h->st>>>(m, d.opt, (const T *)d.J, d.Mq, (T *)d.PE);
+}
+cudaError_t vbi_form(ba_vbsmc *h, const VbiDev &d, int64_t P, int64_t m, double lambda) {
     cudaError_t e = cudaMemsetAsync(d.err, 0, sizeof(int), h->st);
     if (e != cudaSuccess) return e;
-    const int g2 = (int)std::min<int64_t>((P + 255) / 256, 152 * 16);
-    const int g3 = (int)std::min<int64_t>((h->nnzb * 32 + 255) / 256, 152 * 16);
     if (h->fp32) {
-        k_vbi_points<float><<<g2, 256, 0, h->st>>>(P, d.trk, (const float *)d.J, lambda, d.Vinv, d.lp, (float *)d.PE,
-                                                   d.err);
-        k_vbi_blocks32<<<g3, 256, 0, h->st>>>(h->nnzb, h->brow, h->col, h->cdim, d.jc0, h->off, h->boff, d.pptr,
-                                                   d.plist, (const float *)d.J, (const float *)d.PE, lambda,
-                                                   (float *)h->val, (float *)h->b);
+        vbi_factor_T<float>(h, d, P, m, lambda);
+        const int64_t g = (h->nnzb + VB32_WARPS - 1) / VB32_WARPS;
+        k_vbi_blocks32<<<(unsigned)g, 32 * VB32_WARPS, 0, h->st>>>(
+            h->nnzb, h->brow, h->col, h->cdim, d.jc0, h->off, h->boff, d.pptr, d.plist, (const float *)d.J,
+            (const float *)d.PE, lambda, (float *)h->val, (float *)h->b);
     } else {
-        k_vbi_points<double><<<g2, 256, 0, h->st>>>(P, d.trk, (const double *)d.J, lambda, d.Vinv, d.lp,
-                                                    (double *)d.PE, d.err);
-        k_vbi_blocks64<<<g3, 256, 0, h->st>>>(h->nnzb, h->brow, h->col, h->cdim, d.jc0, h->off, h->boff,
-                                                    d.pptr, d.plist, (const double *)d.J, (const double *)d.PE,
-                                                    lambda, (double *)h->val, (double *)h->b);
+        vbi_factor_T<double>(h, d, P, m, lambda);
+        const int64_t g = (h->nnzb + VB64_WARPS - 1) / VB64_WARPS;
+        k_vbi_blocks64<<<(unsigned)g, 32 * VB64_WARPS, 0, h->st>>>(
+            h->nnzb, h->brow, h->col, h->cdim, d.jc0, h->off, h->boff, d.pptr, d.plist, (const double *)d.J,
+            (const double *)d.PE, lambda, (double *)h->val, (double *)h->b);
     }
     return cudaGetLastError();
 }
 
-// F of the stored rows into sc->cost (FP64 sum)
-cudaError_t vbi_cost(ba_vbsmc *h, const VbiDev &d, int64_t m, VbiScalars *sc, double *red, unsigned *ctr) {
-    const int g = (int)std::min<int64_t>((m + 255) / 256, 152 * 4);
-    if (h->fp32)
-        k_vbi_cost<float><<<g, 256, 0, h->st>>>(m, (const float *)d.J, sc, red, ctr);
-    else
-        k_vbi_cost<double><<<g, 256, 0, h->st>>>(m, (const double *)d.J, sc, red, ctr);
+// Eq. 5 and the trial state of an LM step from the solution dxc: the points
+// and the cameras (with their [R, t]); then, after ev, the trial cost.
+struct VbiTrial {
+    const double *cams, *intr, *pts;
+    double *cams_t, *intr_t, *pts_t, *camc_t, *dxp;
+    VbiScalars *sc;
+    double *red;
+    unsigned *ctr;
+};
+template <typename T>
+cudaError_t vbi_trial_T(ba_vbsmc *h, const VbiDev &d, int64_t P, int64_t m, int n, const VbiTrial &t, cudaEvent_t ev) {
+    const T *dxc = (const T *)h->vec[0];
+    const int gp = (int)std::min<int64_t>((P + 127) / 128, 152 * 16), gm = (int)std::min<int64_t>((m + 255) / 256, 152 * 16);
+    const int go = (int)std::min<int64_t>((m + 255) / 256, 152 * 4);
+    k_vbi_jdx<T><<<gm, 256, 0, h->st>>>(m, d.ocam, (const T *)d.J, h->cdim, h->off, dxc, (T *)d.PE);
+    k_vbi_dxp<T><<<gp, 128, 0, h->st>>>(P, d.ord, d.trk, (const T *)d.PE, d.Mq, t.pts, t.dxp, t.pts_t);
+    k_vbi_update_cams<T><<<(n + 31) / 32, 32, 0, h->st>>>(n, t.cams, t.intr, h->cdim, h->off, dxc, t.cams_t, t.intr_t,
+                                                          t.camc_t);
+    const cudaError_t e = cudaEventRecord(ev, h->st);
+    if (e != cudaSuccess) return e;
+    k_vbi_trial<T><<<go, 256, 0, h->st>>>(m, d.ocam, d.opt, d.uv, (const T *)d.J, h->cdim, h->off, dxc, t.dxp, t.camc_t,
+                                          t.intr_t, t.pts_t, t.sc, t.red, t.ctr);
     return cudaGetLastError();
 }
 
@@ -746,6 +903,7 @@ ba_status vbi_create(const ba_options &o, int32_t nblk, const std::vector<int32_
     step(sc.put((void **)&d.ocam, hs.obs_cam.data(), n_obs * sizeof(int32_t)));
     step(sc.put((void **)&d.opt, hs.obs_pt.data(), n_obs * sizeof(int32_t)));
     step(sc.put((void **)&d.trk, hs.trk_ptr.data(), (n_pts + 1) * sizeof(int32_t)));
+    step(sc.put((void **)&d.ord, order_by_length(hs.trk_ptr, n_pts).data(), n_pts * sizeof(int32_t)));
     step(sc.put((void **)&d.pptr, L.pptr.data(), L.pptr.size() * sizeof(int32_t)));
     step(sc.put((void **)&d.plist, L.plist.data(), L.plist.size() * sizeof(int2)));
     if (jc0) step(sc.put((void **)&d.jc0, jc0->data(), jc0->size() * sizeof(int32_t)));
@@ -756,8 +914,7 @@ ba_status vbi_create(const ba_options &o, int32_t nblk, const std::vector<int32_
     step(sc.alloc((void **)&d.J, (size_t)n_obs * VJW * h->esz));
     step(sc.alloc((void **)&d.PE, (size_t)n_obs * VPW * h->esz));
     step(sc.alloc((void **)&d.camc, (size_t)n_cams * 12 * sizeof(double)));
-    step(sc.alloc((void **)&d.Vinv, (size_t)n_pts * 9 * sizeof(double)));
-    step(sc.alloc((void **)&d.lp, (size_t)n_pts * 3 * sizeof(double)));
+    step(sc.alloc((void **)&d.Mq, (size_t)n_pts * 9 * sizeof(double)));
     step(sc.alloc((void **)&d.err, sizeof(int)));
     if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();
@@ -765,7 +922,7 @@ ba_status vbi_create(const ba_options &o, int32_t nblk, const std::vector<int32_
         return set_error(BA_ERR_OOM, "cudaMalloc failed");
     }
     if (e == cudaSuccess) e = vbi_linearize(h, d, n_obs, n_cams, d_cams, d_intr, d_pts);
-    if (e == cudaSuccess) e = vbi_form(h, d, n_pts, lambda);
+    if (e == cudaSuccess) e = vbi_form(h, d, n_pts, n_obs, lambda);
     int flag = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&flag, d.err, sizeof(int), cudaMemcpyDeviceToHost, h->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);
@@ -988,6 +1145,7 @@ ba_status ba_vbi_problem_create(const ba_options *opt, int32_t n_cams, const dou
     if (!s) s = vbi_put(p, (void **)&p->d.ocam, hs.obs_cam.data(), n_obs * sizeof(int32_t));
     if (!s) s = vbi_put(p, (void **)&p->d.opt, hs.obs_pt.data(), n_obs * sizeof(int32_t));
     if (!s) s = vbi_put(p, (void **)&p->d.trk, hs.trk_ptr.data(), (n_pts + 1) * sizeof(int32_t));
+    if (!s) s = vbi_put(p, (void **)&p->d.ord, order_by_length(hs.trk_ptr, n_pts).data(), n_pts * sizeof(int32_t));
     if (!s) s = vbi_put(p, (void **)&p->d.pptr, L.pptr.data(), L.pptr.size() * sizeof(int32_t));
     if (!s) s = vbi_put(p, (void **)&p->d.plist, L.plist.data(), L.plist.size() * sizeof(int2));
     if (!s) s = vbi_put(p, (void **)&p->d.uv, uv.data(), uv.size() * sizeof(double));
@@ -995,8 +1153,7 @@ ba_status ba_vbi_problem_create(const ba_options *opt, int32_t n_cams, const dou
     if (!s) s = vbi_alloc(p, (void **)&p->d.PE, (size_t)n_obs * VPW * p->h->esz);
     if (!s) s = vbi_alloc(p, (void **)&p->d.camc, (size_t)n_cams * 12 * sizeof(double));
     if (!s) s = vbi_alloc(p, (void **)&p->camc_t, (size_t)n_cams * 12 * sizeof(double));
-    if (!s) s = vbi_alloc(p, (void **)&p->d.Vinv, (size_t)n_pts * 9 * sizeof(double));
-    if (!s) s = vbi_alloc(p, (void **)&p->d.lp, P3);
+    if (!s) s = vbi_alloc(p, (void **)&p->d.Mq, (size_t)n_pts * 9 * sizeof(double));
     if (!s) s = vbi_alloc(p, (void **)&p->d.err, sizeof(int));
     if (!s) s = vbi_put(p, (void **)&p->cams, cams, C6);
     if (!s) s = vbi_put(p, (void **)&p->intr, intr, C5);
@@ -1031,13 +1188,13 @@ ba_status ba_vbi_lm_step(ba_vbi_problem *p, ba_step_info *info) {
     const bool relin = !p->linearized;
     if ((s = vbi_fail(p, cudaEventRecord(p->ev[0], st), "event"))) return s;
     if (relin) {
-        if ((s = vbi_fail(p, vbi_linearize(h, p->d, p->m, p->n, p->cams, p->intr, p->pts), "k_vbi_linearize")))
+        if ((s = vbi_fail(p, vbi_linearize(h, p->d, p->m, p->n, p->cams, p->intr, p->pts, p->sc, p->red, p->ctr),
+                          "k_vbi_linearize")))
             return s;
-        if ((s = vbi_fail(p, vbi_cost(h, p->d, p->m, p->sc, p->red, p->ctr), "k_vbi_cost"))) return s;
     }
     if ((s = vbi_fail(p, cudaEventRecord(p->ev[1], st), "event"))) return s;
     // Eq. 3-4 with c_i unknowns per camera, then the block-Jacobi M^-1
-    if ((s = vbi_fail(p, vbi_form(h, p->d, p->P, p->lambda), "forming the RCS"))) return s;
+    if ((s = vbi_fail(p, vbi_form(h, p->d, p->P, p->m, p->lambda), "forming the RCS"))) return s;
     int flag = 0;
     if ((s = vbi_fail(p, cudaMemcpyAsync(&flag, p->d.err, sizeof(int), cudaMemcpyDeviceToHost, st), "copy")))
         return s;
@@ -1063,33 +1220,11 @@ ba_status ba_vbi_lm_step(ba_vbi_problem *p, ba_step_info *info) {
     }
     if ((s = vbi_fail(p, cudaEventRecord(p->ev[3], st), "event"))) return s;
     // Eq. 5, the trial state, its cost and the model decrease
-    const int gp = (int)std::min<int64_t>((p->P + 255) / 256, 152 * 16);
-    const int go = (int)std::min<int64_t>((p->m + 255) / 256, 152 * 4);
-    const int gc = (p->n + 127) / 128;
-    if (h->fp32) {
-        const float *dxc = (const float *)h->vec[0];
-        k_vbi_backsub<float><<<gp, 256, 0, st>>>(p->P, p->d.trk, p->d.ocam, (const float *)p->d.J, p->d.Vinv,
-                                                 p->d.lp, h->cdim, h->off, dxc, p->pts, p->dxp, p->pts_t);
-        k_vbi_update_cams<float><<<gc, 128, 0, st>>>(p->n, p->cams, p->intr, h->cdim, h->off, dxc, p->cams_t,
-                                                     p->intr_t);
-        k_vbi_camcache<<<gc, 128, 0, st>>>(p->n, p->cams_t, p->camc_t);
-        if ((s = vbi_fail(p, cudaEventRecord(p->ev[4], st), "event"))) return s;
-        k_vbi_trial<float><<<go, 256, 0, st>>>(p->m, p->d.ocam, p->d.opt, p->d.uv, (const float *)p->d.J, h->cdim,
-                                               h->off, dxc, p->dxp, p->camc_t, p->intr_t, p->pts_t, p->sc, p->red,
-                                               p->ctr + 1);
-    } else {
-        const double *dxc = (const double *)h->vec[0];
-        k_vbi_backsub<double><<<gp, 256, 0, st>>>(p->P, p->d.trk, p->d.ocam, (const double *)p->d.J, p->d.Vinv,
-                                                  p->d.lp, h->cdim, h->off, dxc, p->pts, p->dxp, p->pts_t);
-        k_vbi_update_cams<double><<<gc, 128, 0, st>>>(p->n, p->cams, p->intr, h->cdim, h->off, dxc, p->cams_t,
-                                                      p->intr_t);
-        k_vbi_camcache<<<gc, 128, 0, st>>>(p->n, p->cams_t, p->camc_t);
-        if ((s = vbi_fail(p, cudaEventRecord(p->ev[4], st), "event"))) return s;
-        k_vbi_trial<double><<<go, 256, 0, st>>>(p->m, p->d.ocam, p->d.opt, p->d.uv, (const double *)p->d.J, h->cdim,
-                                                h->off, dxc, p->dxp, p->camc_t, p->intr_t, p->pts_t, p->sc, p->red,
-                                                p->ctr + 1);
-    }
-    if ((s = vbi_fail(p, cudaGetLastError(), "trial kernels"))) return s;
+    const VbiTrial t{p->cams, p->intr, p->pts, p->cams_t, p->intr_t, p->pts_t, p->camc_t, p->dxp, p->sc, p->red,
+                     p->ctr + 1};
+    const cudaError_t te = h->fp32 ? vbi_trial_T<float>(h, p->d, p->P, p->m, p->n, t, p->ev[4])
+                                   : vbi_trial_T<double>(h, p->d, p->P, p->m, p->n, t, p->ev[4]);
+    if ((s = vbi_fail(p, te, "trial kernels"))) return s;
     if ((s = vbi_fail(p, cudaEventRecord(p->ev[5], st), "event"))) return s;
     if ((s = vbi_fail(p, cudaMemcpyAsync(p->sc_host, p->sc, sizeof(VbiScalars), cudaMemcpyDeviceToHost, st), "copy")))
         return s;
@@ -1187,9 +1322,9 @@ ba_status ba_vbi_get_lm_state(const ba_vbi_problem *p, double *lambda, double *n
         if (!p->linearized) {  // the cost of the current state
             ba_vbi_problem *q = const_cast<ba_vbi_problem *>(p);
             ba_status s;
-            if ((s = vbi_fail(q, vbi_linearize(p->h, p->d, p->m, p->n, p->cams, p->intr, p->pts), "k_vbi_linearize")))
+            if ((s = vbi_fail(q, vbi_linearize(p->h, p->d, p->m, p->n, p->cams, p->intr, p->pts, p->sc, p->red,
+                                               p->ctr), "k_vbi_linearize")))
                 return s;
-            if ((s = vbi_fail(q, vbi_cost(p->h, p->d, p->m, p->sc, p->red, p->ctr), "k_vbi_cost"))) return s;
             if ((s = vbi_fail(q, cudaMemcpyAsync(p->sc_host, p->sc, sizeof(VbiScalars), cudaMemcpyDeviceToHost,
                                                  p->h->st), "copy")))
                 return s;
