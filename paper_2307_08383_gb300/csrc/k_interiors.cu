@@ -26,6 +26,7 @@
 #include <vector>
 
 #include "device_util.cuh"
+#include "tma_util.cuh"
 #include "vbsmc_internal.h"
 
 namespace ba {
@@ -322,90 +323,152 @@ __device__ __forceinline__ void vbi_middle(const T *__restrict__ Pa, const T *__
 }
 
 // FP32: the block as a 4 x 8 grid of lanes, each with up to 3 x 2 entries in
-// registers and the columns it needs loaded straight from the J rows (a row
-// column is an 8-byte pair; the lanes of a group share the words), so a pair
-// costs five loads, six shuffles and about thirty multiply-adds per lane with no
-// shared memory and no barrier, and several pairs' loads are in flight.  A
-// block's pairs are added in list order, each as acc + (j0 t0 + j1 t1).
-// (Before, both J rows passed through shared memory with two warp barriers per
-// pair, and every lane formed M: 1031 -> 386 us at 990 cameras of c = 11, 485,000
-// observations, the same bits.)
-constexpr int VB32_WARPS = 2;  // per CTA: few, so that a block of many pairs holds back few others
-__global__ void __launch_bounds__(32 * VB32_WARPS) k_vbi_blocks32(int64_t nnzb, const int *__restrict__ brow,
+// registers.  The heads of the pairs' J rows (96 bytes: the columns) come eight
+// pairs at a time by asynchronous copies into one half of the warp's stage
+// while the other half is used, so a pair costs five shared loads, four shuffles
+// and about thirty multiply-adds per lane, with no wait of its own.  A block's
+// pairs are added in list order, each as acc + (j0 t0 + j1 t1).  Bound by
+// instruction issue (57 per pair and warp).  990 cameras of c = 11, 485,000
+// observations, 2.1 M pairs: 173 us; 386 with the columns loaded by the lanes
+// straight from the rows (waits for L1 and L2), 1031 with both rows passed
+// through shared memory pair by pair; the same bits.
+constexpr int VB32_FETCH = 8;  // pairs copied at a time: 16 row heads, two halves per warp
+static_assert(VB32_FETCH * 12 % 32 == 0, "whole turns of a warp");
+// RPL x CPL entries per lane (the lanes beyond the block's edge repeat its last
+// row or column, so that the loop has no predicates).
+template <int RPL, int CPL, bool DIAG>
+__device__ __forceinline__ void vbi32_block(int p0, int p1, int ci, int cj, int ai, int aj,
+                                            const int2 *__restrict__ plist, const float *__restrict__ J,
+                                            const float *__restrict__ PE, float lambda, float *__restrict__ out,
+                                            float *__restrict__ b, float *stage) {
+    constexpr unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, rg = lane >> 3, cg = lane & 7;
+    // byte offsets of this lane's columns within a J row
+    int ra[RPL], rb[CPL];
+#pragma unroll
+    for (int u = 0; u < RPL; ++u) ra[u] = 8 * (ai + min(RPL * rg + u, ci - 1));
+#pragma unroll
+    for (int v = 0; v < CPL; ++v) rb[v] = 8 * (aj + min(CPL * cg + v, cj - 1));
+    float acc[RPL][CPL], dU[RPL], bacc[RPL];
+#pragma unroll
+    for (int u = 0; u < RPL; ++u) {
+        dU[u] = bacc[u] = 0.f;
+#pragma unroll
+        for (int v = 0; v < CPL; ++v) acc[u][v] = 0.f;
+    }
+    for (; p0 < p1; p0 += 32) {
+        const int cnt = min(32, p1 - p0);
+        int2 pr = make_int2(0, 0);
+        float M[4] = {0.f, 0.f, 0.f, 0.f}, eh[2] = {0.f, 0.f};
+        if (lane < cnt) pr = __ldg(plist + p0 + lane);
+        // copies of pairs q0 .. q0 + 7 into half `h` of the stage, 16 bytes to a
+        // lane and turn: row c / 6 of the sixteen, part c % 6 of its columns
+        auto fetch = [&](int q0, int h) {
+#pragma unroll
+            for (int t = 0; t < VB32_FETCH * 12 / 32; ++t) {
+                const int c = lane + 32 * t, row = c / 6, part = c - 6 * row, q = q0 + (row >> 1);
+                const int x = __shfl_sync(FULL, pr.x, q & 31), y = __shfl_sync(FULL, pr.y, q & 31);
+                if (q < cnt)
+                    cp_async16(stage + h * (VB32_FETCH * 48) + row * 24 + 4 * part,
+                               J + (int64_t)((row & 1) ? y : x) * VJW + 4 * part);
+            }
+            cp_async_commit();
+        };
+        fetch(0, 0);
+        if (lane < cnt) vbi_middle<float>(PE + (int64_t)pr.x * VPW, PE + (int64_t)pr.y * VPW, pr.x == pr.y, M, eh);
+        for (int q0 = 0, h = 0; q0 < cnt; q0 += VB32_FETCH, h ^= 1) {
+            if (q0 + VB32_FETCH < cnt) {
+                fetch(q0 + VB32_FETCH, h ^ 1);
+                cp_async_wait<1>();
+            } else {
+                cp_async_wait<0>();
+            }
+            __syncwarp();
+            const char *st = reinterpret_cast<const char *>(stage + h * (VB32_FETCH * 48));
+            const int nq = min(VB32_FETCH, cnt - q0);
+#pragma unroll 4
+            for (int qq = 0; qq < nq; ++qq) {
+                const int q = q0 + qq;
+                const float m00 = __shfl_sync(FULL, M[0], q), m01 = __shfl_sync(FULL, M[1], q),
+                            m10 = __shfl_sync(FULL, M[2], q), m11 = __shfl_sync(FULL, M[3], q);
+                const char *ja = st + 192 * qq, *jb = ja + 96;
+                float2 a[RPL], t[CPL];
+#pragma unroll
+                for (int u = 0; u < RPL; ++u) a[u] = *reinterpret_cast<const float2 *>(ja + ra[u]);
+#pragma unroll
+                for (int v = 0; v < CPL; ++v) {
+                    const float2 w = *reinterpret_cast<const float2 *>(jb + rb[v]);
+                    t[v] = make_float2(dot2(m00, w.x, m01, w.y), dot2(m10, w.x, m11, w.y));
+                }
+#pragma unroll
+                for (int u = 0; u < RPL; ++u)
+#pragma unroll
+                    for (int v = 0; v < CPL; ++v) acc[u][v] += dot2(a[u].x, t[v].x, a[u].y, t[v].y);
+                if (DIAG && __shfl_sync(FULL, pr.x, q) == __shfl_sync(FULL, pr.y, q)) {
+                    const float e0 = __shfl_sync(FULL, eh[0], q), e1 = __shfl_sync(FULL, eh[1], q);
+#pragma unroll
+                    for (int u = 0; u < RPL; ++u) {
+                        bacc[u] -= dot2(a[u].x, e0, a[u].y, e1);
+                        dU[u] += dot2(a[u].x, a[u].x, a[u].y, a[u].y);
+                    }
+                }
+            }
+            __syncwarp();  // this half may be refilled
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < RPL; ++u) {
+        const int r = RPL * rg + u;
+        if (r >= ci) continue;
+#pragma unroll
+        for (int v = 0; v < CPL; ++v) {
+            const int c = CPL * cg + v;
+            if (c < cj) out[r * cj + c] = DIAG && r == c ? fmaf(lambda, clampT(dU[u]), acc[u][v]) : acc[u][v];
+        }
+        if (DIAG && cg == 0) b[r] = bacc[u];
+    }
+}
+
+constexpr int VB32_WARPS = 1;  // per CTA: a block of many pairs holds back no others (1: 173 us, 2: 184, 4: 178)
+__global__ void __launch_bounds__(32 * VB32_WARPS) k_vbi_blocks32(int n, const int *__restrict__ row_ptr,
+                                                      int64_t nnzb, const int *__restrict__ brow,
                                                       const int *__restrict__ col, const int *__restrict__ cdim,
                                                       const int *__restrict__ jc0, const int *__restrict__ off,
                                                       const int64_t *__restrict__ boff, const int *__restrict__ pptr,
                                                       const int2 *__restrict__ plist, const float *__restrict__ J,
                                                       const float *__restrict__ PE, double lambda,
                                                       float *__restrict__ val, float *__restrict__ b) {
-    constexpr unsigned FULL = 0xffffffffu;
-    const int lane = threadIdx.x & 31, rg = lane >> 3, cg = lane & 7;
-    const float2 *J2 = reinterpret_cast<const float2 *>(J);
-    const int64_t k = blockIdx.x * (int64_t)VB32_WARPS + (threadIdx.x >> 5);
-    if (k < nnzb) {
-        const int i = brow[k], j = col[k], ci = cdim[i], cj = cdim[j];
-        const int rpl = (ci + 3) >> 2, cpl = (cj + 7) >> 3;  // rows and columns per lane
-        const int r0 = rpl * rg, c0 = cpl * cg;
-        const int ja0 = (jc0 ? jc0[i] : 0) + r0, jb0 = (jc0 ? jc0[j] : 0) + c0;
-        const bool diag = i == j;
-        bool ron[3], con[2];
-#pragma unroll
-        for (int u = 0; u < 3; ++u) ron[u] = u < rpl && r0 + u < ci;
-#pragma unroll
-        for (int v = 0; v < 2; ++v) con[v] = v < cpl && c0 + v < cj;
-        float acc[3][2], dU[3], bacc[3];
-#pragma unroll
-        for (int u = 0; u < 3; ++u) acc[u][0] = acc[u][1] = dU[u] = bacc[u] = 0.f;
-        const int p1 = pptr[k + 1];
-        for (int p0 = pptr[k]; p0 < p1; p0 += 32) {
-            const int cnt = min(32, p1 - p0);
-            int2 pr = make_int2(0, 0);
-            float M[4] = {0.f, 0.f, 0.f, 0.f}, eh[2] = {0.f, 0.f};
-            if (lane < cnt) {
-                pr = __ldg(plist + p0 + lane);
-                vbi_middle<float>(PE + (int64_t)pr.x * VPW, PE + (int64_t)pr.y * VPW, pr.x == pr.y, M, eh);
-            }
-#pragma unroll 4
-            for (int q = 0; q < cnt; ++q) {
-                const int x = __shfl_sync(FULL, pr.x, q), y = __shfl_sync(FULL, pr.y, q);
-                const float m00 = __shfl_sync(FULL, M[0], q), m01 = __shfl_sync(FULL, M[1], q),
-                            m10 = __shfl_sync(FULL, M[2], q), m11 = __shfl_sync(FULL, M[3], q);
-                const float2 *ra = J2 + (int64_t)x * (VJW / 2) + ja0, *rb = J2 + (int64_t)y * (VJW / 2) + jb0;
-                float2 a[3], t[2];
-#pragma unroll
-                for (int u = 0; u < 3; ++u) a[u] = ron[u] ? __ldg(ra + u) : make_float2(0.f, 0.f);
-#pragma unroll
-                for (int v = 0; v < 2; ++v) {
-                    const float2 w = con[v] ? __ldg(rb + v) : make_float2(0.f, 0.f);
-                    t[v] = make_float2(dot2(m00, w.x, m01, w.y), dot2(m10, w.x, m11, w.y));
-                }
-#pragma unroll
-                for (int u = 0; u < 3; ++u)
-#pragma unroll
-                    for (int v = 0; v < 2; ++v) acc[u][v] += dot2(a[u].x, t[v].x, a[u].y, t[v].y);
-                if (diag && x == y) {
-                    const float e0 = __shfl_sync(FULL, eh[0], q), e1 = __shfl_sync(FULL, eh[1], q);
-#pragma unroll
-                    for (int u = 0; u < 3; ++u) {
-                        bacc[u] -= dot2(a[u].x, e0, a[u].y, e1);
-                        dU[u] += dot2(a[u].x, a[u].x, a[u].y, a[u].y);
-                    }
-                }
-            }
-        }
-        float *out = val + boff[k];
-#pragma unroll
-        for (int u = 0; u < 3; ++u) {
-            if (!ron[u]) continue;
-            const int r = r0 + u;
-#pragma unroll
-            for (int v = 0; v < 2; ++v) {
-                const int c = c0 + v;
-                if (!con[v]) continue;
-                out[r * cj + c] = diag && r == c ? fmaf((float)lambda, clampT(dU[u]), acc[u][v]) : acc[u][v];
-            }
-            if (diag && cg == 0) b[off[i] + r] = bacc[u];
-        }
+    __shared__ __align__(16) float stage[VB32_WARPS][2 * VB32_FETCH * 48];
+    // the diagonal blocks (every observation of a camera) first: they have the
+    // most pairs, and one started last would run alone
+    int64_t k = blockIdx.x * (int64_t)VB32_WARPS + (threadIdx.x >> 5);
+    const bool first = k < n;
+    if (first)
+        k = row_ptr[k];
+    else
+        k -= n;
+    if (k >= nnzb) return;
+    const int i = brow[k], j = col[k], ci = cdim[i], cj = cdim[j], p0 = pptr[k], p1 = pptr[k + 1];
+    if (!first && i == j) return;
+    const int ai = jc0 ? jc0[i] : 0, aj = jc0 ? jc0[j] : 0;
+    float *out = val + boff[k], *bi = b + off[i];
+    const float lam = (float)lambda;
+    // up to 4 x 2 = 8 rows and 8 x 1 columns, or 12 rows and 16 columns (c <= 11)
+    if (i == j) {
+        if (ci <= 8)
+            vbi32_block<2, 1, true>(p0, p1, ci, cj, ai, aj, plist, J, PE, lam, out, bi, stage[threadIdx.x >> 5]);
+        else
+            vbi32_block<3, 2, true>(p0, p1, ci, cj, ai, aj, plist, J, PE, lam, out, bi, stage[threadIdx.x >> 5]);
+    } else if (ci <= 8) {
+        if (cj <= 8)
+            vbi32_block<2, 1, false>(p0, p1, ci, cj, ai, aj, plist, J, PE, lam, out, bi, stage[threadIdx.x >> 5]);
+        else
+            vbi32_block<2, 2, false>(p0, p1, ci, cj, ai, aj, plist, J, PE, lam, out, bi, stage[threadIdx.x >> 5]);
+    } else {
+        if (cj <= 8)
+            vbi32_block<3, 1, false>(p0, p1, ci, cj, ai, aj, plist, J, PE, lam, out, bi, stage[threadIdx.x >> 5]);
+        else
+            vbi32_block<3, 2, false>(p0, p1, ci, cj, ai, aj, plist, J, PE, lam, out, bi, stage[threadIdx.x >> 5]);
     }
 }
 
@@ -846,9 +909,9 @@ cudaError_t vbi_form(ba_vbsmc *h, const VbiDev &d, int64_t P, int64_t m, double 
     if (e != cudaSuccess) return e;
     if (h->fp32) {
         vbi_factor_T<float>(h, d, P, m, lambda);
-        const int64_t g = (h->nnzb + VB32_WARPS - 1) / VB32_WARPS;
+        const int64_t g = (h->n + h->nnzb + VB32_WARPS - 1) / VB32_WARPS;
         k_vbi_blocks32<<<(unsigned)g, 32 * VB32_WARPS, 0, h->st>>>(
-            h->nnzb, h->brow, h->col, h->cdim, d.jc0, h->off, h->boff, d.pptr, d.plist, (const float *)d.J,
+            h->n, h->row_ptr, h->nnzb, h->brow, h->col, h->cdim, d.jc0, h->off, h->boff, d.pptr, d.plist, (const float *)d.J,
             (const float *)d.PE, lambda, (float *)h->val, (float *)h->b);
     } else {
         vbi_factor_T<double>(h, d, P, m, lambda);
