@@ -96,6 +96,18 @@ template <> struct RunSum<double> {
     __device__ __forceinline__ double get() const { return s; }
 };
 
+// FP32 to FP64 without the FP64 pipe's conversion (16 cycles per warp, as much as
+// a multiply-add there; this is about six on the integer pipe): the exponent
+// rebiased, the mantissa shifted.  Exact; denormals, infinities and NaN take
+// the conversion.
+__device__ __forceinline__ double widen(float f) {
+    const unsigned u = __float_as_uint(f), m = u << 1;
+    if (m != 0u && m - 0x01000000u >= 0xfe000000u) return (double)f;
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (m ? 0x38000000u : 0u))),
+                            (int)(u << 29));
+}
+__device__ __forceinline__ double widen(double d) { return d; }
+
 // In-place Cholesky of a symmetric 6x6 (row-major, lower triangle used) and
 // the inverse A^-1 = L^-T L^-1 written full.  Returns false if not SPD.
 template <typename T>
@@ -568,6 +580,48 @@ __device__ __forceinline__ void block_apply(const TV (&Sv)[36], const TV (&x)[6]
     }
 }
 
+// Sums of six values over the warp by recursive halving (eight adds per lane
+// instead of thirty: the adds of an FP64 row sum took as long as a quarter of
+// its products).  Lane l ends with the total of component fold6_comp(l); the
+// additions pair the lanes as the xor butterfly 16, 8, 4, 2, 1 does, so the
+// totals are its bits.
+__device__ __forceinline__ int fold6_comp(int lane) {
+    return ((lane & 16) ? 3 : 0) + ((lane & 8) ? 2 : ((lane & 4) ? 1 : 0));
+}
+__device__ __forceinline__ bool fold6_owner(int lane) { return (lane & 3) == 0 && (lane & 12) != 12; }
+template <typename TV>
+__device__ __forceinline__ TV warp_fold6(const TV (&a)[6], int lane) {
+    const unsigned M = 0xffffffffu;
+    const bool b16 = lane & 16, b8 = lane & 8, b4 = lane & 4;
+    TV k[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) k[c] = (b16 ? a[3 + c] : a[c]) + __shfl_xor_sync(M, b16 ? a[c] : a[3 + c], 16);
+    const TV r0 = __shfl_xor_sync(M, b8 ? k[0] : k[2], 8), r1 = __shfl_xor_sync(M, k[1], 8);
+    const TV u = (b8 ? k[2] : k[0]) + r0, v = k[1] + r1;
+    TV t = (b8 || !b4) ? u : v;
+    t += __shfl_xor_sync(M, (b8 || b4) ? u : v, 4);
+    t += __shfl_xor_sync(M, t, 2);
+    t += __shfl_xor_sync(M, t, 1);
+    return t;
+}
+
+// Six FP32 reductions into a camera vector (24 B, 8-byte aligned).
+__device__ __forceinline__ void red_add2_f(float *a, float u, float v) {
+    asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(a), "f"(u), "f"(v) : "memory");
+}
+__device__ __forceinline__ void red_add4_f(float *a, float u0, float u1, float u2, float u3) {
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(a), "f"(u0), "f"(u1), "f"(u2), "f"(u3)
+                 : "memory");
+}
+__device__ __forceinline__ void red_add6_f(float *qj, const float (&t)[6]) {
+    if ((reinterpret_cast<uintptr_t>(qj) & 15u) == 0) {
+        red_add4_f(qj, t[0], t[1], t[2], t[3]);
+        red_add2_f(qj + 4, t[4], t[5]);
+    } else {
+        red_add2_f(qj, t[0], t[1]);
+        red_add4_f(qj + 2, t[2], t[3], t[4], t[5]);
+    }
+}
 // One stored linearization row (JW values, 16-byte aligned, read-only) into
 // registers with vector loads.
 __device__ __forceinline__ void load_jrow(const float *__restrict__ s, float (&v)[JW]) {

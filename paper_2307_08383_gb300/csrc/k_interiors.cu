@@ -76,18 +76,6 @@ __device__ __forceinline__ VbiProj<T> vbi_project(const double *__restrict__ cam
     return o;
 }
 
-// FP32 to FP64 without the FP64 pipe's conversion (16 cycles per warp, as much as
-// a multiply-add there; this is about six on the integer pipe): the exponent
-// rebiased, the mantissa shifted.  Exact; denormals, infinities and NaN take
-// the conversion.
-__device__ __forceinline__ double widen(float f) {
-    const unsigned u = __float_as_uint(f), m = u << 1;
-    if (m != 0u && m - 0x01000000u >= 0xfe000000u) return (double)f;
-    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (m ? 0x38000000u : 0u))),
-                            (int)(u << 29));
-}
-__device__ __forceinline__ double widen(double d) { return d; }
-
 // N values from a 16-byte aligned address with 16-byte loads.
 template <int N, typename T>
 __device__ __forceinline__ void load_vec(const T *__restrict__ p, T (&v)[N]) {

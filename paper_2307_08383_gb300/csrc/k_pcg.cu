@@ -40,31 +40,6 @@ __device__ __forceinline__ void gather_x(const TV *__restrict__ xz, const TV *__
     }
 }
 
-// Sums of six values over the warp by recursive halving (eight adds per lane
-// instead of thirty: the adds of an FP64 row sum took as long as a quarter of
-// its products).  Lane l ends with the total of component fold6_comp(l); the
-// additions pair the lanes as the xor butterfly 16, 8, 4, 2, 1 does, so the
-// totals are its bits.
-__device__ __forceinline__ int fold6_comp(int lane) {
-    return ((lane & 16) ? 3 : 0) + ((lane & 8) ? 2 : ((lane & 4) ? 1 : 0));
-}
-__device__ __forceinline__ bool fold6_owner(int lane) { return (lane & 3) == 0 && (lane & 12) != 12; }
-template <typename TV>
-__device__ __forceinline__ TV warp_fold6(const TV (&a)[6], int lane) {
-    const unsigned M = 0xffffffffu;
-    const bool b16 = lane & 16, b8 = lane & 8, b4 = lane & 4;
-    TV k[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) k[c] = (b16 ? a[3 + c] : a[c]) + __shfl_xor_sync(M, b16 ? a[c] : a[3 + c], 16);
-    const TV r0 = __shfl_xor_sync(M, b8 ? k[0] : k[2], 8), r1 = __shfl_xor_sync(M, k[1], 8);
-    const TV u = (b8 ? k[2] : k[0]) + r0, v = k[1] + r1;
-    TV t = (b8 || !b4) ? u : v;
-    t += __shfl_xor_sync(M, (b8 || b4) ? u : v, 4);
-    t += __shfl_xor_sync(M, t, 2);
-    t += __shfl_xor_sync(M, t, 1);
-    return t;
-}
-
 // q = S x over BSMC without atomics: a warp per block row i walks the row's
 // two-sided entry list - the stored blocks (i, j >= i), applied as S_ij x_j,
 // then the blocks (j < i, i) of column i, applied as S_ji^T x_j - so q_i is
@@ -133,22 +108,6 @@ __device__ __forceinline__ double spmv_rows(int n, const int *__restrict__ tw_pt
 // entry.  d^T S d is summed per block as (2 for j > i, 1 for j = i)
 // d_i^T S_ij d_j, so it needs no complete q.  The order of q's terms is not
 // fixed (floating-point reductions).
-__device__ __forceinline__ void red_add2_f(float *a, float u, float v) {
-    asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(a), "f"(u), "f"(v) : "memory");
-}
-__device__ __forceinline__ void red_add4_f(float *a, float u0, float u1, float u2, float u3) {
-    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(a), "f"(u0), "f"(u1), "f"(u2), "f"(u3)
-                 : "memory");
-}
-__device__ __forceinline__ void red_add6_f(float *qj, const float (&t)[6]) {
-    if ((reinterpret_cast<uintptr_t>(qj) & 15u) == 0) {
-        red_add4_f(qj, t[0], t[1], t[2], t[3]);
-        red_add2_f(qj + 4, t[4], t[5]);
-    } else {
-        red_add2_f(qj, t[0], t[1]);
-        red_add4_f(qj + 2, t[2], t[3], t[4], t[5]);
-    }
-}
 __device__ __forceinline__ double spmv_rows_once(int n, const int *__restrict__ row_ptr,
                                                  const int *__restrict__ col, const float *__restrict__ S,
                                                  const float *__restrict__ z, const float *__restrict__ dold,

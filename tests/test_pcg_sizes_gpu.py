@@ -79,3 +79,31 @@ def test_fp64_pcg_over_launch_shapes(n, half):
         assert np.linalg.norm(b - product(row_ptr, col, val, x)) <= 1.01 * tol * np.linalg.norm(b)
         assert np.linalg.norm(x - ref) <= 1e-8 * np.linalg.norm(ref)
     g.close()
+
+
+@pytest.mark.parametrize("n,half,shift", [(1, 1, 0), (7, 6, 1), (153, 20, 0), (200, 199, 0), (200, 199, 1),
+                                          (1300, 33, 0), (8192, 3, 1)])
+def test_static_pcg_over_launch_shapes(n, half, shift):
+    """The allocation-free solve: one to 54 rows per CTA, rows of more than a
+    warp's blocks, CTAs whose blocks exceed their shared memory share, and
+    arrays at a 4-byte offset (shift).  FP32 recurrence to 1e-5: the true
+    residual is within 100 eps of it."""
+    import torch
+
+    from paper_2307_08383_gb300.build import build
+    build()
+    import paper_2307_08383_gb300 as B
+    row_ptr, col, val, b = system(n, half, 9200 + n)
+    val, b = val.astype(np.float32), b.astype(np.float32)
+    dev = [torch.from_numpy(row_ptr).cuda(), torch.from_numpy(col).cuda()]
+    flat = [torch.zeros(a.size + 1, device="cuda") for a in (val, b, b)]
+    for t, a in zip(flat[:2], (val, b)):
+        t[shift:shift + a.size] = torch.from_numpy(a.reshape(-1)).cuda()
+    ptr = [t.data_ptr() + 4 * shift for t in flat]
+    for _ in range(2):
+        status, its, rel = B.ba_pcg_solve_static(n, len(col), dev[0].data_ptr(), dev[1].data_ptr(), ptr[0], ptr[1],
+                                                 ptr[2], 1e-5, 0, torch.cuda.current_stream().cuda_stream)
+        assert status == B.BA_OK and 1 <= its < 40 and rel <= 1e-5
+        x = flat[2][shift:shift + b.size].cpu().numpy().astype(np.float64).reshape(n, 6)
+        r = b - product(row_ptr, col, val.astype(np.float64), x)
+        assert np.linalg.norm(r) <= (1e-5 + 100 * np.finfo(np.float32).eps) * np.linalg.norm(b)
