@@ -215,6 +215,7 @@ struct ba_problem {
     uint32_t *tw_meta = nullptr;   // per entry: local row | halo index << 16 (per-CTA aligned)
     int32_t *meta_off = nullptr, *halo_ptr = nullptr, *halo_col = nullptr, *own_base = nullptr;
     int split_grid = 0;            // 0: not partitioned yet, < 0: unavailable
+    bool split_cluster = false;    // the grid runs as one thread-block cluster
     int split_slot_floats = 0;
     size_t split_smem = 0;
     double ph_sum[4] = {};  // split CG phase totals over solves (profile >= 2)

@@ -691,10 +691,22 @@ __device__ __forceinline__ df32 warp_sum_df(df32 v) {
     return v;
 }
 
-// Block sum of NV double-floats; the totals are valid in every lane of warp 0.
-template <int NV>
+// Sum over the warp's first N lanes (a power of two), valid in lane 0.
+template <int N>
+__device__ __forceinline__ df32 warp_sum_df_n(df32 v) {
+#pragma unroll
+    for (int o = N / 2; o > 0; o >>= 1) {
+        const df32 u = {__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)};
+        v = df_add(v, u);
+    }
+    return v;
+}
+
+// Block sum of NV double-floats over NW warps (a power of two, the whole CTA);
+// the totals are valid in lane 0 of warp 0.
+template <int NV, int NW>
 __device__ __forceinline__ void block_sum_df(df32 (&v)[NV], float2 *sh) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
     for (int i = 0; i < NV; ++i) v[i] = warp_sum_df(v[i]);
     if (lane == 0)
@@ -704,8 +716,8 @@ __device__ __forceinline__ void block_sum_df(df32 (&v)[NV], float2 *sh) {
     if (w == 0) {
 #pragma unroll
         for (int i = 0; i < NV; ++i) {
-            const float2 t = lane < nw ? sh[lane * NV + i] : make_float2(0.f, 0.f);
-            v[i] = warp_sum_df(df32{t.x, t.y});
+            const float2 t = lane < NW ? sh[lane * NV + i] : make_float2(0.f, 0.f);
+            v[i] = warp_sum_df_n<NW>(df32{t.x, t.y});
         }
     }
     __syncthreads();
@@ -723,12 +735,12 @@ __device__ __forceinline__ void block_sum_df(df32 (&v)[NV], float2 *sh) {
 // for a given launch shape, so every CTA gets the same bits.  `bar` holds
 // AR_SUB * 32 words, zero at launch; `sh` holds NV * warps float2, `s_ok` is
 // shared.  Every thread of the CTA calls this (it holds __syncthreads); the
-// CTA's own partial is v as left by block_sum_df (valid in warp 0).  Once
+// CTA's own partial is v as left by block_sum_df (valid in thread 0).  Once
 // every CTA has arrived, every thread runs after_wait() (what the grid wrote
 // before arriving is visible to it) right after issuing its partial reads;
 // meant for asynchronous copies that overlap the rest.  On return the
 // totals are valid in thread 0 only (as double-floats); false on timeout.
-template <int NV, class F>
+template <int NV, int NW, class F>
 __device__ __forceinline__ bool grid_allreduce_df(df32 (&v)[NV], double *part, unsigned gen, unsigned *bar,
                                                   int *err, long long limit_cycles, df32 (&tot)[NV], float2 *sh,
                                                   int *s_ok, F &&after_wait) {
@@ -785,7 +797,7 @@ __device__ __forceinline__ bool grid_allreduce_df(df32 (&v)[NV], double *part, u
                 acc[k] = df_add(acc[k], df32{u.x, u.y});
             }
     }
-    block_sum_df<NV>(acc, sh);
+    block_sum_df<NV, NW>(acc, sh);
     if (threadIdx.x == 0)
 #pragma unroll
         for (int k = 0; k < NV; ++k) tot[k] = acc[k];

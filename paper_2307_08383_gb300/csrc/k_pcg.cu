@@ -1009,6 +1009,66 @@ __device__ __forceinline__ void split_halo_apply(int H, int ob, int R, bool firs
     }
 }
 
+// The all-reduce of the split CG when its CTAs are one thread-block cluster:
+// warp 0 of each CTA stores the CTA's NV double-float partials into every CTA's
+// shared memory and arrives at its barrier (release), waits (bounded) for the
+// arrivals at its own, and adds the partials in a fixed order: the same bits
+// everywhere, without a round trip to L2.  Two barriers alternate by call, so
+// that a CTA one call ahead never completes a phase another still waits for:
+// its arrival at call g + 2 needs every CTA's at g + 1.  What the CTAs wrote to
+// global memory before the call is visible after it.  Every thread of the CTA
+// calls this; after_wait() runs in every thread once all have arrived; totals
+// in warp 0; false on timeout.
+constexpr int CL_MAX = 16;  // CTAs per cluster at most
+template <int NV>
+struct ClusterSlots {
+    float2 part[2][CL_MAX][NV];
+    uint64_t bar[2];
+};
+template <int NV, class F>
+__device__ __forceinline__ bool cluster_allreduce_df(df32 (&v)[NV], ClusterSlots<NV> &cl, unsigned gen, int *err,
+                                                     long long limit_cycles, df32 (&tot)[NV], int *s_ok,
+                                                     F &&after_wait) {
+    const unsigned h = gen & 1u;
+    const int lane = threadIdx.x & 31;
+    if (threadIdx.x < 32) {
+#pragma unroll
+        for (int k = 0; k < NV; ++k)
+            v[k] = df32{__shfl_sync(0xffffffffu, v[k].hi, 0), __shfl_sync(0xffffffffu, v[k].lo, 0)};
+        if (lane < (int)gridDim.x) {
+#pragma unroll
+            for (int k = 0; k < NV; ++k)
+                cluster_store2(cluster_peer_addr(&cl.part[h][blockIdx.x][k], lane), v[k].hi, v[k].lo);
+            cluster_arrive(cluster_peer_addr(&cl.bar[h], lane));
+        }
+        bool ok = true;
+        const long long t0 = clock64();
+        while (!cluster_try_wait(&cl.bar[h], (gen >> 1) & 1u))
+            if (clock64() - t0 > limit_cycles) {
+                ok = false;
+                break;
+            }
+        ok = __all_sync(0xffffffffu, ok) != 0;
+        if (lane == 0) {
+            *s_ok = ok ? 1 : 0;
+            if (!ok) atomicExch(err, (int)BA_ERR_TIMEOUT);
+        }
+    }
+    __syncthreads();
+    const bool ok = *s_ok != 0;
+    if (ok) {
+        after_wait();
+        if (threadIdx.x < 32) {
+#pragma unroll
+            for (int k = 0; k < NV; ++k) {
+                const float2 u = lane < (int)gridDim.x ? cl.part[h][lane & (CL_MAX - 1)][k] : make_float2(0.f, 0.f);
+                tot[k] = warp_sum_df_n<CL_MAX>(df32{u.x, u.y});
+            }
+        }
+    }
+    return ok;
+}
+
 // CG on S^ x^ = r^_0 (Chronopoulos-Gear), with per iteration k
 //   p = r + beta p,  s = w + beta s,  x^ += alpha p,  r -= alpha s,  w = S^ r,
 //   gamma = r.r, delta = w.r, beta' = gamma'/gamma,
@@ -1018,7 +1078,9 @@ __device__ __forceinline__ void split_halo_apply(int H, int ob, int R, bool firs
 // own p, s, x^, r, w (a thread's first element keeps p, x^ and its row of H
 // in registers across iterations).  The stop test uses the original
 // residual norm ||H r^|| (block-Jacobi: ||L r^||).  One grid all-reduce of
-// (gamma, delta, ||H r||^2) ends each phase.
+// (gamma, delta, ||H r||^2) ends each phase; with CLUSTER the grid is one
+// thread-block cluster and the all-reduce stays in its shared memory.
+template <bool CLUSTER>
 __global__ void __launch_bounds__(SPLIT_WARPS * 32, SPLIT_CTAS_PER_SM) k_pcg_split(const int *__restrict__ cta_rows, const int *__restrict__ tw_ptr,
                                                       const uint32_t *__restrict__ tw_meta,
                                                       const int *__restrict__ meta_off,
@@ -1028,10 +1090,18 @@ __global__ void __launch_bounds__(SPLIT_WARPS * 32, SPLIT_CTAS_PER_SM) k_pcg_spl
                                                       const float *__restrict__ Sh, const float *__restrict__ H,
                                                       const float *__restrict__ Shd, int diag_ident,
                                                       float *x, float *p, float *rec0, float *rec1, DevScalars *sc,
-                                                      double *red, unsigned *bar, long long limit_cycles) {
+                                                      double *red, unsigned *bar, long long limit_cycles,
+                                                      int short_by) {
     extern __shared__ __align__(16) float sdyn[];
     __shared__ uint64_t mbar[SPLIT_NBUF * SPLIT_WARPS];
+    __shared__ ClusterSlots<3> cl;
     if (sc->done) return;
+    if (CLUSTER) {
+        // (short_by 1: the armed test of the timeout path, one arrival too few)
+        if (threadIdx.x < 2) mbar_init(&cl.bar[threadIdx.x], gridDim.x + short_by);
+        cluster_fence_init();
+        cluster_sync_all();  // every CTA runs and its barriers are set before a peer arrives
+    }
     const int rb = __ldg(cta_rows + blockIdx.x), re = __ldg(cta_rows + blockIdx.x + 1);
     const int eb = __ldg(tw_ptr + rb), ee = __ldg(tw_ptr + re);
     const int hb = __ldg(halo_ptr + blockIdx.x), NH = __ldg(halo_ptr + blockIdx.x + 1) - hb;
@@ -1114,6 +1184,13 @@ __global__ void __launch_bounds__(SPLIT_WARPS * 32, SPLIT_CTAS_PER_SM) k_pcg_spl
         if (has0) x[6 * (int64_t)(rb + lr0) + c0] = x0;
         cp_async_wait_all();
         split_drain(pp, limit_cycles);
+        if (CLUSTER) cluster_sync_all();  // no CTA ends while a peer may still write to it
+    };
+    auto allreduce = [&](df32(&v)[3], df32(&t)[3], unsigned g, auto &&hook) {
+        if constexpr (CLUSTER)
+            return cluster_allreduce_df<3>(v, cl, g, &sc->err, limit_cycles, t, &s_arok, hook);
+        else
+            return grid_allreduce_df<3, SPLIT_WARPS>(v, red, g, bar, &sc->err, limit_cycles, t, sh_df, &s_arok, hook);
     };
     // phase timing (thread 0 of each CTA, profile >= 2): passes, combine, all-reduce
     const bool prof = sc->prof_on != 0 && threadIdx.x == 0;
@@ -1144,10 +1221,9 @@ __global__ void __launch_bounds__(SPLIT_WARPS * 32, SPLIT_CTAS_PER_SM) k_pcg_spl
             rp.add(hr * hr);
         }
         df32 v[3] = {{gp.s, gp.c}, {dp.s, dp.c}, {rp.s, rp.c}};
-        block_sum_df<3>(v, sh_df);
+        block_sum_df<3, SPLIT_WARPS>(v, sh_df);
         df32 t[3];
-        const bool ok2 = grid_allreduce_df<3>(v, red, gen++, bar, &sc->err, limit_cycles, t, sh_df, &s_arok,
-                                              [&]() { split_halo_fetch(halo_col, hb, NH, hj0, rec0, hx); });
+        const bool ok2 = allreduce(v, t, gen++, [&]() { split_halo_fetch(halo_col, hb, NH, hj0, rec0, hx); });
         if (threadIdx.x == 0) decide(ok2, t, true);
         __syncthreads();
     }
@@ -1218,11 +1294,10 @@ __global__ void __launch_bounds__(SPLIT_WARPS * 32, SPLIT_CTAS_PER_SM) k_pcg_spl
             rp.add(hr * hr);
         }
         df32 v[3] = {{gp.s, gp.c}, {dp.s, dp.c}, {rp.s, rp.c}};
-        block_sum_df<3>(v, sh_df);
+        block_sum_df<3, SPLIT_WARPS>(v, sh_df);
         if (prof) t2 = global_ns();
         df32 t[3];
-        const bool ok2 = grid_allreduce_df<3>(v, red, gen++, bar, &sc->err, limit_cycles, t, sh_df, &s_arok,
-                                              [&]() { split_halo_fetch(halo_col, hb, NH, hj0, rn, hx); });
+        const bool ok2 = allreduce(v, t, gen++, [&]() { split_halo_fetch(halo_col, hb, NH, hj0, rn, hx); });
         if (threadIdx.x == 0) {
             if (prof) {
                 const unsigned long long t3 = global_ns();
@@ -1527,6 +1602,26 @@ cudaError_t launch_split_prepare(ba_problem *p, bool from_minv) {
     return cudaGetLastError();
 }
 
+// Systems of at most this many entries run the split CG in one cluster of up
+// to CL_MAX CTAs, whose all-reduce takes 1.3 us instead of 2.5; with more, the
+// passes on sixteen SMs outweigh that.  Per iteration, cluster against grid: 24
+// cameras 3.9 / 4.7 us, 128 (7,700 entries) 4.0 / 5.15, 200 (12,000) 4.8 / 5.1,
+// 288 (17,500) 5.05 / 5.07, 392 6.0 / 5.1, 1,250 11.6 / 5.6
+constexpr int64_t SPLIT_CLUSTER_ENTRIES = 14 * 1024;
+static cudaLaunchConfig_t split_cluster_config(int grid, size_t smem, cudaStream_t st, cudaLaunchAttribute *at) {
+    at->id = cudaLaunchAttributeClusterDimension;
+    at->val.clusterDim.x = (unsigned)grid;
+    at->val.clusterDim.y = at->val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(SPLIT_WARPS * 32);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
 // Work partition of the split CG, made once per problem on the host: the
 // grid size; each CTA's row range (contiguous rows, about equal entries + a
 // fixed cost per row); its halo (the sorted distinct columns of its entries;
@@ -1562,12 +1657,19 @@ static cudaError_t split_partition(ba_problem *p) {
     int dev = 0, n_sm = 0, bps = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    constexpr int SMEM_MAX = 226 * 1024, ROW_COST = 8;  // 227 KB per CTA less the static part
-    if ((e = cudaFuncSetAttribute(k_pcg_split, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX)) != cudaSuccess)
+    constexpr int ROW_COST = 8;
+    constexpr int SMEM_MAX = 226 * 1024, SMEM_CLUSTER = 224 * 1024;  // 227 KB per CTA less the static part
+    for (const void *k : {(const void *)k_pcg_split<false>, (const void *)k_pcg_split<true>}) {
+        if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      k == (const void *)k_pcg_split<true> ? SMEM_CLUSTER : SMEM_MAX)) != cudaSuccess)
+            return e;
+        if ((e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                      (int)cudaSharedmemCarveoutMaxShared)) != cudaSuccess)
+            return e;
+    }
+    if ((e = cudaFuncSetAttribute(k_pcg_split<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess)
         return e;
-    if ((e = cudaFuncSetAttribute(k_pcg_split, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                  (int)cudaSharedmemCarveoutMaxShared)) != cudaSuccess)
-        return e;
+    bool cluster = E <= SPLIT_CLUSTER_ENTRIES;
     auto unavailable = [&]() {
         p->split_grid = -1;
         return cudaSuccess;
@@ -1576,10 +1678,15 @@ static cudaError_t split_partition(ba_problem *p) {
     size_t smem = SPLIT_STAGE_BYTES;
     int slot_floats = 0, G = 0;
     for (int attempt = 0; attempt < 4; ++attempt) {
-        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_pcg_split, SPLIT_WARPS * 32, smem)) != cudaSuccess) return e;
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_pcg_split<false>, SPLIT_WARPS * 32, smem)) != cudaSuccess) return e;
         bps = std::min(bps, SPLIT_CTAS_PER_SM);
         if (bps < 1) return unavailable();
-        const int g = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)bps * n_sm, (E + 255) / 256));
+        int g = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)bps * n_sm, (E + 255) / 256));
+        if (cluster) {  // the power of two below, at most CL_MAX, no more CTAs than rows
+            int c = 1;
+            while (2 * c <= std::min(std::min(g, CL_MAX), n)) c *= 2;
+            g = c;
+        }
         if (g == G) break;
         G = g;
         rows.assign(G + 1, n);
@@ -1648,10 +1755,26 @@ static cudaError_t split_partition(ba_problem *p) {
         }
         smem = SPLIT_STAGE_BYTES +
                ((size_t)slot_floats + (size_t)HX * Hmax + 20 * (size_t)Rmax) * sizeof(float);
+        if (cluster && smem > (size_t)SMEM_CLUSTER) {  // start over as a grid over all SMs
+            cluster = false;
+            smem = SPLIT_STAGE_BYTES;
+            G = 0;
+            attempt = -1;
+            continue;
+        }
         if (smem > (size_t)SMEM_MAX || Hmax > 0xFFFF || Rmax > 0xFFFE) return unavailable();
     }
+    if (cluster) {
+        cudaLaunchAttribute at;
+        const cudaLaunchConfig_t cfg = split_cluster_config(G, smem, p->st, &at);
+        int clusters = 0;
+        if (cudaOccupancyMaxActiveClusters(&clusters, k_pcg_split<true>, &cfg) != cudaSuccess || clusters < 1) {
+            cudaGetLastError();
+            cluster = false;  // no room for such a cluster: the same partition as a grid
+        }
+    }
     // the occupancy at the final shared-memory size must keep the grid resident
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_pcg_split, SPLIT_WARPS * 32, smem)) != cudaSuccess) return e;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_pcg_split<false>, SPLIT_WARPS * 32, smem)) != cudaSuccess) return e;
     if (G < 1 || (int64_t)bps * n_sm < G) return unavailable();
     // packed entry metadata, per CTA from a 16-byte aligned offset (+ padding
     // for the rounded-up copy of a CTA's last pass)
@@ -1692,6 +1815,7 @@ static cudaError_t split_partition(ba_problem *p) {
     p->split_slot_floats = slot_floats;
     p->split_smem = smem;
     p->split_grid = G;
+    p->split_cluster = cluster;
     return cudaSuccess;
 }
 
@@ -1740,10 +1864,17 @@ cudaError_t launch_pcg_split(ba_problem *p) {
         double *red = p->red;
         unsigned *bar = p->ar_bar;
         long long limit = test_limit > 0 ? test_limit : 4000000000LL;  // ~2 s of SM clock per wait
+        int short_by = test_limit > 0 ? 1 : 0;
         void *args[] = {&cr, &twp, &meta, &mo, &hp, &hc, &ob, &sf, &Sh, &H, &Shd, &ident, &x, &pp, &rec0, &rec1, &sc,
-                        &red, &bar, &limit};
-        e = cudaLaunchCooperativeKernel((const void *)k_pcg_split, dim3(p->split_grid), dim3(SPLIT_WARPS * 32), args,
-                                        p->split_smem, p->st);
+                        &red, &bar, &limit, &short_by};
+        if (p->split_cluster) {
+            cudaLaunchAttribute at;
+            const cudaLaunchConfig_t cfg = split_cluster_config(p->split_grid, p->split_smem, p->st, &at);
+            e = cudaLaunchKernelExC(&cfg, (const void *)k_pcg_split<true>, args);
+        } else {
+            e = cudaLaunchCooperativeKernel((const void *)k_pcg_split<false>, dim3(p->split_grid),
+                                            dim3(SPLIT_WARPS * 32), args, p->split_smem, p->st);
+        }
     }
     ktimer_end(p, K_PCG_LOOP, ev);
     p->launches += 1;
