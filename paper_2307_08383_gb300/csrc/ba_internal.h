@@ -216,7 +216,7 @@ struct ba_problem {
     int32_t *meta_off = nullptr, *halo_ptr = nullptr, *halo_col = nullptr, *own_base = nullptr;
     int split_grid = 0;            // 0: not partitioned yet, < 0: unavailable
     bool split_cluster = false;    // the grid runs as one thread-block cluster
-    int split_slot_floats = 0;
+    int split_slot_floats = 0, split_stage_floats = 0;
     size_t split_smem = 0;
     double ph_sum[4] = {};  // split CG phase totals over solves (profile >= 2)
     double ph_imbalance = 0.0;  // last split solve: busiest CTA's work / mean CTA's

@@ -828,7 +828,12 @@ __device__ __forceinline__ float next_r(float r, float w, float s, float a, floa
 // entries' packed (local row, halo index) arrive by 1-D bulk copies into one
 // of the warp's SPLIT_NBUF buffers; since S^ does not change during the
 // solve, each refill fetches the warp's pass SPLIT_NBUF positions ahead,
-// wrapping into the next iteration.  The pass loop thus reads shared memory only.  A segmented
+// wrapping into the next iteration.  Where the CTA's passes all fit in shared
+// memory (about 42), each has a buffer of its own, filled once: a warp's third
+// pass otherwise waits about 1 us in every iteration for a refill issued in
+// it (with the rows' starts in shared memory too: 2,556 cameras, 33 passes,
+// 6.40 -> 6.07 us per iteration; 512 cameras 5.02 -> 4.74).  The pass loop reads shared
+// memory only.  A segmented
 // shuffle scan over the pass (entries are sorted by row) leaves each row
 // segment's sum in its last lane, which stores it in a slot: (q, 0) if the
 // segment opens pass q, (q, 1) if it closes it, else the row's own slot.  The
@@ -848,6 +853,7 @@ struct SplitPipe {
     const uint32_t *meta;  // this CTA's packed entry metadata (16-byte aligned base)
     int eb, ee, m;   // entry range; passes of this warp
     uint32_t seq;    // passes this warp has consumed so far
+    bool res;        // every pass of the CTA has its own buffer
 };
 
 __device__ __forceinline__ float *pass_buf(const SplitPipe &pp, uint32_t s) {
@@ -866,11 +872,38 @@ __device__ __forceinline__ void split_issue(const SplitPipe &pp, uint32_t s) {
     bulk_g2s(buf, pp.Sh + (int64_t)(pp.eb + 32 * q) * BW, sbytes, bar);
     bulk_g2s(buf + PASS_S_BYTES / 4, pp.meta + 32 * q, mbytes, bar);
 }
+// lane 0: the warp's first copies - the passes its buffers hold, or (res) all of
+// its passes, into the buffers of their own on the warp's first barrier
+__device__ __forceinline__ void split_start(const SplitPipe &pp) {
+    if ((threadIdx.x & 31) != 0 || pp.m == 0) return;
+    if (!pp.res) {
+        for (uint32_t q = 0; q < (uint32_t)SPLIT_NBUF; ++q) split_issue(pp, q);
+        return;
+    }
+    const int wid = threadIdx.x >> 5;
+    uint64_t *bar = pp.mbar + SPLIT_NBUF * wid;
+    uint32_t total = 0;
+    for (int k = 0; k < pp.m; ++k) {
+        const int cnt = min(32, pp.ee - pp.eb - 32 * (wid + SPLIT_WARPS * k));
+        total += (uint32_t)cnt * BW * 4 + (uint32_t)((cnt + 3) & ~3) * 4;
+    }
+    mbar_expect_tx(bar, total);
+    for (int k = 0; k < pp.m; ++k) {
+        const int q = wid + SPLIT_WARPS * k, cnt = min(32, pp.ee - pp.eb - 32 * q);
+        float *buf = pp.stage + (size_t)q * (PASS_BYTES / 4);
+        bulk_g2s(buf, pp.Sh + (int64_t)(pp.eb + 32 * q) * BW, (uint32_t)cnt * BW * 4, bar);
+        bulk_g2s(buf + PASS_S_BYTES / 4, pp.meta + 32 * q, (uint32_t)((cnt + 3) & ~3) * 4, bar);
+    }
+}
 
 // lane 0: wait (bounded) for the copies still in flight before the CTA leaves
 __device__ __forceinline__ void split_drain(const SplitPipe &pp, long long limit) {
     if ((threadIdx.x & 31) != 0 || pp.m == 0) return;
     const int wid = threadIdx.x >> 5;
+    if (pp.res) {
+        mbar_wait(pp.mbar + SPLIT_NBUF * wid, 0u, limit);
+        return;
+    }
     for (uint32_t s = pp.seq; s < pp.seq + SPLIT_NBUF; ++s)
         mbar_wait(pp.mbar + SPLIT_NBUF * wid + s % SPLIT_NBUF, (s / SPLIT_NBUF) & 1u, limit);
 }
@@ -878,7 +911,7 @@ __device__ __forceinline__ void split_drain(const SplitPipe &pp, long long limit
 // One sweep of the warp's passes over the halo vectors hx.  False on an
 // mbarrier timeout (then the warp stops; callers agree CTA-wide with
 // __syncthreads_and and leave).
-__device__ __forceinline__ bool split_passes(SplitPipe &pp, int rb, const int *__restrict__ tw_ptr, const float *hx,
+__device__ __forceinline__ bool split_passes(SplitPipe &pp, const int *row_ent, const float *hx,
                                              float *slot, float *rowacc, int *err, long long limit) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int eb = pp.eb, ee = pp.ee;
@@ -886,13 +919,15 @@ __device__ __forceinline__ bool split_passes(SplitPipe &pp, int rb, const int *_
         const int q = wid + SPLIT_WARPS * k;
         const int t = eb + 32 * q + lane;
         const bool valid = t < ee;
-        const uint32_t b = pp.seq % SPLIT_NBUF;
+        const uint32_t b = pp.res ? 0u : pp.seq % SPLIT_NBUF;
         // every lane observes the copy's completion; the outcome is warp-uniform
-        if (!__all_sync(0xffffffffu, mbar_wait(pp.mbar + SPLIT_NBUF * wid + b, (pp.seq / SPLIT_NBUF) & 1u, limit))) {
+        // (res: the one phase that the first wait saw complete)
+        if (!__all_sync(0xffffffffu, mbar_wait(pp.mbar + SPLIT_NBUF * wid + b,
+                                               pp.res ? 0u : (pp.seq / SPLIT_NBUF) & 1u, limit))) {
             if (lane == 0) atomicExch(err, (int)BA_ERR_TIMEOUT);
             return false;
         }
-        const float *buf = pass_buf(pp, pp.seq);
+        const float *buf = pp.res ? pp.stage + (size_t)q * (PASS_BYTES / 4) : pass_buf(pp, pp.seq);
         int lr = 0xFFFF;
         float y[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
         if (valid) {
@@ -915,7 +950,7 @@ __device__ __forceinline__ bool split_passes(SplitPipe &pp, int rb, const int *_
             }
         }
         __syncwarp();
-        if (lane == 0) split_issue(pp, pp.seq + SPLIT_NBUF);  // this buffer is free again
+        if (!pp.res && lane == 0) split_issue(pp, pp.seq + SPLIT_NBUF);  // this buffer is free again
         ++pp.seq;
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
@@ -929,8 +964,7 @@ __device__ __forceinline__ bool split_passes(SplitPipe &pp, int rb, const int *_
         }
         const int ld = __shfl_down_sync(0xffffffffu, lr, 1);
         if (valid && (lane == 31 || ld != lr)) {
-            const int i = rb + lr;
-            const int rs = __ldg(tw_ptr + i), rend = __ldg(tw_ptr + i + 1);
+            const int rs = row_ent[lr], rend = row_ent[lr + 1];
             const int ps = eb + 32 * q, pe = min(ps + 32, ee);
             float *dst = rs <= ps ? slot + 12 * q : (rend >= pe ? slot + 12 * q + 6 : rowacc + 6 * lr);
 #pragma unroll
@@ -1087,6 +1121,7 @@ __global__ void __launch_bounds__(SPLIT_WARPS * 32, SPLIT_CTAS_PER_SM) k_pcg_spl
                                                       const int *__restrict__ halo_ptr,
                                                       const int *__restrict__ halo_col,
                                                       const int *__restrict__ own_base, int slot_floats,
+                                                      int stage_floats,
                                                       const float *__restrict__ Sh, const float *__restrict__ H,
                                                       const float *__restrict__ Shd, int diag_ident,
                                                       float *x, float *p, float *rec0, float *rec1, DevScalars *sc,
@@ -1107,29 +1142,26 @@ __global__ void __launch_bounds__(SPLIT_WARPS * 32, SPLIT_CTAS_PER_SM) k_pcg_spl
     const int hb = __ldg(halo_ptr + blockIdx.x), NH = __ldg(halo_ptr + blockIdx.x + 1) - hb;
     const int ob = __ldg(own_base + blockIdx.x);
     const int R = re - rb, P = (ee - eb + 31) >> 5, wid = threadIdx.x >> 5;
-    // dynamic shared memory: copy buffers | slots + row sums | halo | own records
-    float *slot = sdyn + SPLIT_STAGE_BYTES / 4, *rowacc = slot + 12 * P;
+    // dynamic shared memory: copy buffers | slots + row sums | halo | own records | row starts
+    float *slot = sdyn + stage_floats, *rowacc = slot + 12 * P;
     float *hx = slot + slot_floats, *own = hx + HX * NH;
+    int *s_row = reinterpret_cast<int *>(own + 20 * R);  // first entry of each of the CTA's rows, and the end
+    for (int q = threadIdx.x; q <= R; q += blockDim.x) s_row[q] = __ldg(tw_ptr + rb + q);
     const int hj0 = (int)threadIdx.x < NH ? __ldg(halo_col + hb + threadIdx.x) : 0;
     SplitPipe pp{sdyn, mbar, Sh, tw_meta + __ldg(meta_off + blockIdx.x), eb, ee,
-                 wid < P ? (P - 1 - wid) / SPLIT_WARPS + 1 : 0, 0u};
+                 wid < P ? (P - 1 - wid) / SPLIT_WARPS + 1 : 0, 0u, stage_floats * 4 != SPLIT_STAGE_BYTES};
     if (threadIdx.x < SPLIT_NBUF * SPLIT_WARPS) mbar_init(&mbar[threadIdx.x], 1);
     fence_proxy_async();
     __syncthreads();
-    if ((threadIdx.x & 31) == 0 && pp.m > 0)
-        for (uint32_t q = 0; q < (uint32_t)SPLIT_NBUF; ++q) split_issue(pp, q);
-    // this thread's first (row, component): p, x^, its row of H and the row's
-    // entry range stay in registers
+    split_start(pp);
+    // this thread's first (row, component): p, x^ and its row of H stay in registers
     const int u0 = threadIdx.x;
     const bool has0 = u0 < 6 * R;
     const int lr0 = u0 / 6, c0 = u0 - 6 * lr0;
     float p0 = 0.f, x0 = 0.f, h0[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    int rs0 = 0, re0 = 0;
     if (has0) {
 #pragma unroll
         for (int k = 0; k < 6; ++k) h0[k] = __ldg(H + 36 * (int64_t)(rb + lr0) + 6 * c0 + k);
-        rs0 = __ldg(tw_ptr + rb + lr0);
-        re0 = __ldg(tw_ptr + rb + lr0 + 1);
     }
     unsigned gen = 0;
     // The recurrence's scalars live in thread 0, which decides alpha, beta and
@@ -1199,7 +1231,7 @@ __global__ void __launch_bounds__(SPLIT_WARPS * 32, SPLIT_CTAS_PER_SM) k_pcg_spl
         split_halo_fetch(halo_col, hb, NH, hj0, rec0, hx);
         split_halo_apply(NH, ob, R, true, 0.f, 0.f, hx, own);
         __syncthreads();
-        const bool ok = __syncthreads_and(split_passes(pp, rb, tw_ptr, hx, slot, rowacc, &sc->err, limit_cycles));
+        const bool ok = __syncthreads_and(split_passes(pp, s_row, hx, slot, rowacc, &sc->err, limit_cycles));
         if (!ok) {
             leave();
             return;
@@ -1207,7 +1239,7 @@ __global__ void __launch_bounds__(SPLIT_WARPS * 32, SPLIT_CTAS_PER_SM) k_pcg_spl
         RunSum<float> gp, dp, rp;
         for (int u = threadIdx.x; u < 6 * R; u += blockDim.x) {
             const int lr = u / 6, c = u - 6 * lr, i = rb + lr;
-            const int rs = u == u0 ? rs0 : __ldg(tw_ptr + i), rend = u == u0 ? re0 : __ldg(tw_ptr + i + 1);
+            const int rs = s_row[lr], rend = s_row[lr + 1];
             const float *r6 = hx + HX * (ob + lr);
             const float wc = split_combine(lr, c, rs, rend, eb, ee, slot, rowacc) + split_diag(i, c, r6, Shd, diag_ident);
             rec0[(int64_t)SREC * i + 6 + c] = wc;
@@ -1256,7 +1288,7 @@ __global__ void __launch_bounds__(SPLIT_WARPS * 32, SPLIT_CTAS_PER_SM) k_pcg_spl
         if (prof) t0 = global_ns();
         split_halo_apply(NH, ob, R, false, a, b, hx, own);
         __syncthreads();
-        const bool ok = __syncthreads_and(split_passes(pp, rb, tw_ptr, hx, slot, rowacc, &sc->err, limit_cycles));
+        const bool ok = __syncthreads_and(split_passes(pp, s_row, hx, slot, rowacc, &sc->err, limit_cycles));
         if (!ok) {
             leave();
             return;
@@ -1266,7 +1298,7 @@ __global__ void __launch_bounds__(SPLIT_WARPS * 32, SPLIT_CTAS_PER_SM) k_pcg_spl
         for (int u = threadIdx.x; u < 6 * R; u += blockDim.x) {
             const int lr = u / 6, c = u - 6 * lr, i = rb + lr, e = 6 * i + c;
             const bool first = u == u0;
-            const int rs = first ? rs0 : __ldg(tw_ptr + i), rend = first ? re0 : __ldg(tw_ptr + i + 1);
+            const int rs = s_row[lr], rend = s_row[lr + 1];
             const float *rnew = hx + HX * (ob + lr);  // this row's new residual (all six components)
             const float w_e = split_combine(lr, c, rs, rend, eb, ee, slot, rowacc) + split_diag(i, c, rnew, Shd, diag_ident);
             const float *o6 = own + 20 * lr;
@@ -1605,8 +1637,8 @@ cudaError_t launch_split_prepare(ba_problem *p, bool from_minv) {
 // Systems of at most this many entries run the split CG in one cluster of up
 // to CL_MAX CTAs, whose all-reduce takes 1.3 us instead of 2.5; with more, the
 // passes on sixteen SMs outweigh that.  Per iteration, cluster against grid: 24
-// cameras 3.9 / 4.7 us, 128 (7,700 entries) 4.0 / 5.15, 200 (12,000) 4.8 / 5.1,
-// 288 (17,500) 5.05 / 5.07, 392 6.0 / 5.1, 1,250 11.6 / 5.6
+// cameras 3.4 / 4.4 us, 128 (7,700 entries) 3.6 / 4.8, 200 (12,000) 4.3 / 4.7,
+// 288 (17,500) 4.7 / 4.7, 392 5.5 / 4.7
 constexpr int64_t SPLIT_CLUSTER_ENTRIES = 14 * 1024;
 static cudaLaunchConfig_t split_cluster_config(int grid, size_t smem, cudaStream_t st, cudaLaunchAttribute *at) {
     at->id = cudaLaunchAttributeClusterDimension;
@@ -1676,7 +1708,7 @@ static cudaError_t split_partition(ba_problem *p) {
     };
     std::vector<int32_t> rows, hptr, hcol, obase;
     size_t smem = SPLIT_STAGE_BYTES;
-    int slot_floats = 0, G = 0;
+    int slot_floats = 0, stage_bytes = SPLIT_STAGE_BYTES, G = 0;
     for (int attempt = 0; attempt < 4; ++attempt) {
         if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_pcg_split<false>, SPLIT_WARPS * 32, smem)) != cudaSuccess) return e;
         bps = std::min(bps, SPLIT_CTAS_PER_SM);
@@ -1735,7 +1767,7 @@ static cudaError_t split_partition(ba_problem *p) {
         hptr.assign(G + 1, 0);
         hcol.clear();
         obase.assign(G, 0);
-        int Hmax = 0, Rmax = 0;
+        int Hmax = 0, Rmax = 0, Pmax = 1;
         slot_floats = 0;
         std::vector<int32_t> cols;
         for (int k = 0; k < G; ++k) {
@@ -1751,10 +1783,15 @@ static cudaError_t split_partition(ba_problem *p) {
             const int64_t P = ((int64_t)twp[rows[k + 1]] - twp[rows[k]] + 31) / 32;
             Hmax = std::max(Hmax, (int)cols.size());
             Rmax = std::max(Rmax, R);
+            Pmax = std::max(Pmax, (int)P);
             slot_floats = std::max(slot_floats, (int)(12 * P + 6 * R + 3) & ~3);
         }
-        smem = SPLIT_STAGE_BYTES +
-               ((size_t)slot_floats + (size_t)HX * Hmax + 20 * (size_t)Rmax) * sizeof(float);
+        const size_t rest = ((size_t)slot_floats + (size_t)HX * Hmax + 21 * (size_t)Rmax + 1) * sizeof(float);
+        // a buffer for every pass where they fit (one more where their number
+        // is that of the streaming buffers: the kernel tells the modes by it)
+        const size_t own = (size_t)PASS_BYTES * (Pmax == SPLIT_WARPS * SPLIT_NBUF ? Pmax + 1 : Pmax);
+        stage_bytes = own + rest <= (size_t)(cluster ? SMEM_CLUSTER : SMEM_MAX) ? (int)own : SPLIT_STAGE_BYTES;
+        smem = stage_bytes + rest;
         if (cluster && smem > (size_t)SMEM_CLUSTER) {  // start over as a grid over all SMs
             cluster = false;
             smem = SPLIT_STAGE_BYTES;
@@ -1813,6 +1850,7 @@ static cudaError_t split_partition(ba_problem *p) {
         *u.first = d;
     }
     p->split_slot_floats = slot_floats;
+    p->split_stage_floats = stage_bytes / 4;
     p->split_smem = smem;
     p->split_grid = G;
     p->split_cluster = cluster;
@@ -1854,7 +1892,7 @@ cudaError_t launch_pcg_split(ba_problem *p) {
         const int *cr = p->cta_rows, *twp = p->tws_ptr, *mo = p->meta_off, *hp = p->halo_ptr, *hc = p->halo_col,
                   *ob = p->own_base;
         const uint32_t *meta = p->tw_meta;
-        int sf = p->split_slot_floats;
+        int sf = p->split_slot_floats, stf = p->split_stage_floats;
         const float *Sh = p->Sh, *H = p->Hs, *Shd = p->Shd;
         int ident = p->minv_learned ? 0 : 1;
         float **v = (float **)p->sv.pv;
@@ -1865,7 +1903,7 @@ cudaError_t launch_pcg_split(ba_problem *p) {
         unsigned *bar = p->ar_bar;
         long long limit = test_limit > 0 ? test_limit : 4000000000LL;  // ~2 s of SM clock per wait
         int short_by = test_limit > 0 ? 1 : 0;
-        void *args[] = {&cr, &twp, &meta, &mo, &hp, &hc, &ob, &sf, &Sh, &H, &Shd, &ident, &x, &pp, &rec0, &rec1, &sc,
+        void *args[] = {&cr, &twp, &meta, &mo, &hp, &hc, &ob, &sf, &stf, &Sh, &H, &Shd, &ident, &x, &pp, &rec0, &rec1, &sc,
                         &red, &bar, &limit, &short_by};
         if (p->split_cluster) {
             cudaLaunchAttribute at;
