@@ -698,18 +698,19 @@ static ba_status solve_once_view(ba_problem *p, ba_step_info *info) {
         // One host synchronisation per sweep: the first sweep always runs (r = b;
         // a zero b stops its PCG at once), and a sweep's PCG, accumulation and
         // residual are queued together and read back once.
-        CK(p, launch_resid64(p, false));  // r64 = b, x64 implicit 0
+        // the split CG's first sweep reads b itself (its init also forms ||b||)
+        if (!split) CK(p, launch_resid64(p, false));  // r64 = b, x64 implicit 0
         bool first = true;
         for (int o = 0; o < p->opt.refine_max; ++o) {
             if (!first) {
                 if (p->sc_host->rr64 <= tol * tol * p->sc_host->bb64) { converged = true; break; }
                 if (p->sc_host->bb64 == 0.0) { converged = true; break; }
             }
-            CK(p, launch_refine_rhs(p, p->sv.pv[1]));  // r buffer doubles as the rhs (copied by init)
+            if (!split) CK(p, launch_refine_rhs(p, p->sv.pv[1]));  // r buffer doubles as the rhs (copied by init)
             const double rho = first ? 1.0 : std::sqrt(p->sc_host->rr64 / p->sc_host->bb64);
             const double inner = std::min(0.9, std::max(p->opt.inner_rel_tol, tol / rho));
             if (split) {
-                CK(p, launch_split_init(p, (const float *)p->sv.pv[1], inner, max_iters));
+                CK(p, launch_split_init(p, first, inner, max_iters));
                 CK(p, launch_pcg_split(p));
             } else {
                 CK(p, launch_pcg_init(p, p->sv.pv[1], inner, max_iters));
@@ -717,7 +718,7 @@ static ba_status solve_once_view(ba_problem *p, ba_step_info *info) {
             }
             CK(p, split ? launch_accumulate_split(p, first) : launch_accumulate_solution(p, first));
             first = false;
-            CK(p, launch_resid64(p, true));
+            CK(p, launch_resid64(p, true, split));
             if ((s = sync_scalars(p))) return s;
             if (split && p->opt.profile >= 2) {
                 for (int k = 0; k < 4; ++k) p->ph_sum[k] += p->sc_host->ph[k];

@@ -257,7 +257,7 @@ cudaError_t launch_form_rcs(ba_problem *p, double lambda);
 cudaError_t launch_pcg_init(ba_problem *p, const void *rhs_T, double tol, int max_iters);
 cudaError_t launch_pcg_loop(ba_problem *p);
 cudaError_t launch_pcg_implicit(ba_problem *p);  // the loop on the implicit operator (k_formats.cu)
-cudaError_t launch_resid64(ba_problem *p, bool from_x64);
+cudaError_t launch_resid64(ba_problem *p, bool from_x64, bool split = false);
 cudaError_t launch_solution_to_step(ba_problem *p);
 cudaError_t launch_refine_rhs(ba_problem *p, void *rhs_T);
 cudaError_t launch_back_substitute(ba_problem *p);
@@ -272,7 +272,7 @@ cudaError_t launch_demote(ba_problem *p);                     // S32, Minv32 fro
 // and x64 (+)= G x^
 cudaError_t launch_split_prepare(ba_problem *p, bool from_minv);
 bool split_available(ba_problem *p);  // partitions on first use
-cudaError_t launch_split_init(ba_problem *p, const float *rhs, double tol, int max_iters);
+cudaError_t launch_split_init(ba_problem *p, bool first, double tol, int max_iters);
 cudaError_t launch_pcg_split(ba_problem *p);
 cudaError_t launch_accumulate_split(ba_problem *p, bool first);
 // y = S x for one FP32 vector (learned-preconditioner probes)

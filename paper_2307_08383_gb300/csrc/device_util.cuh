@@ -108,51 +108,62 @@ __device__ __forceinline__ double widen(float f) {
 }
 __device__ __forceinline__ double widen(double d) { return d; }
 
-// In-place Cholesky of a symmetric 6x6 (row-major, lower triangle used) and
-// the inverse A^-1 = L^-T L^-1 written full.  Returns false if not SPD.
+// Cholesky of symmetric 6x6 matrices, eight lanes each (lane r < 6 of a group
+// holds row r in a; lanes 6 and 7 hold zeros): on return a holds row r of L
+// (columns k <= r), x column r of L^-1 (rows k >= r, zeros above), and the
+// result is false in the whole group if a pivot is not positive.  One thread
+// per matrix ran some 450 FP64 instructions of 64 cycles each; a group runs
+// about 170, its pivots' one division per column.
 template <typename T>
-__device__ bool spd_inverse6(const T *A, T *Ainv) {
-    T L[21];  // packed lower: L[i*(i+1)/2 + j]
+__device__ __forceinline__ bool chol6_lanes(T (&a)[6], T (&x)[6]) {
+    constexpr unsigned FULL = 0xffffffffu;
+    const int r = threadIdx.x & 7;
+    bool ok = true;
+    T invd = T(1);
 #pragma unroll
-    for (int i = 0; i < 6; ++i) {
-#pragma unroll
-        for (int j = 0; j <= i; ++j) {
-            T s = A[i * 6 + j];
-#pragma unroll
-            for (int k = 0; k < j; ++k) s -= L[i * (i + 1) / 2 + k] * L[j * (j + 1) / 2 + k];
-            if (i == j) {
-                if (!(s > T(0))) return false;
-                L[i * (i + 1) / 2 + i] = sqrt(s);
-            } else {
-                L[i * (i + 1) / 2 + j] = s / L[j * (j + 1) / 2 + j];
-            }
+    for (int q = 0; q < 6; ++q) {
+        T p = __shfl_sync(FULL, a[q], q, 8);
+        if (!(p > T(0))) {
+            ok = false;
+            p = T(1);
         }
+        const T s = sqrt(p), inv = T(1) / s;
+        if (r == q) invd = inv;
+        a[q] = r == q ? s : a[q] * inv;
+#pragma unroll
+        for (int k = q + 1; k < 6; ++k) a[k] -= a[q] * __shfl_sync(FULL, a[q], k, 8);  // rows r >= k are meant
     }
-    // Li = L^-1 (lower)
-    T Li[21];
 #pragma unroll
-    for (int i = 0; i < 6; ++i) {
-        Li[i * (i + 1) / 2 + i] = T(1) / L[i * (i + 1) / 2 + i];
+    for (int q = 0; q < 6; ++q) {
+        const T dq = __shfl_sync(FULL, invd, q, 8);
+        T s = T(0);
 #pragma unroll
-        for (int j = 0; j < i; ++j) {
-            T s = T(0);
-#pragma unroll
-            for (int k = j; k < i; ++k) s += L[i * (i + 1) / 2 + k] * Li[k * (k + 1) / 2 + j];
-            Li[i * (i + 1) / 2 + j] = -s * Li[i * (i + 1) / 2 + i];
-        }
+        for (int k = 0; k < q; ++k) s += __shfl_sync(FULL, a[k], q, 8) * x[k];
+        x[q] = q < r ? T(0) : (q == r ? dq : -s * dq);
     }
-    // A^-1 = Li^T Li
+    return ok;
+}
+// Row r of the inverse, from chol6_lanes' x: (L^-1)^T L^-1.
+template <typename T>
+__device__ __forceinline__ void inv6_row(const T (&x)[6], T (&out)[6]) {
 #pragma unroll
-    for (int i = 0; i < 6; ++i)
+    for (int c = 0; c < 6; ++c) {
+        T s = T(0);
 #pragma unroll
-        for (int j = i; j < 6; ++j) {
-            T s = T(0);
+        for (int k = c; k < 6; ++k) s += x[k] * __shfl_sync(0xffffffffu, x[k], c, 8);
+        out[c] = s;
+    }
+}
+// A lane's row of six values to an 8-byte aligned address.
+__device__ __forceinline__ void store6(float *p, const float (&v)[6]) {
+    float2 *q = reinterpret_cast<float2 *>(p);
 #pragma unroll
-            for (int k = j; k < 6; ++k) s += Li[k * (k + 1) / 2 + i] * Li[k * (k + 1) / 2 + j];
-            Ainv[i * 6 + j] = s;
-            Ainv[j * 6 + i] = s;
-        }
-    return true;
+    for (int k = 0; k < 3; ++k) q[k] = make_float2(v[2 * k], v[2 * k + 1]);
+}
+__device__ __forceinline__ void store6(double *p, const double (&v)[6]) {
+    double2 *q = reinterpret_cast<double2 *>(p);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) q[k] = make_double2(v[2 * k], v[2 * k + 1]);
 }
 
 // Quaternion (w, x, y, z) of the rotation vector v.
@@ -689,6 +700,23 @@ __device__ __forceinline__ df32 warp_sum_df(df32 v) {
         v = df_add(v, u);
     }
     return v;
+}
+
+// warp_fold6 for double-floats: component fold6_comp(lane) of the six sums.
+__device__ __forceinline__ df32 shfl_xor_df(df32 v, int o) {
+    return {__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)};
+}
+__device__ __forceinline__ df32 warp_fold6_df(const df32 (&a)[6], int lane) {
+    const bool b16 = lane & 16, b8 = lane & 8, b4 = lane & 4;
+    df32 k[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) k[c] = df_add(b16 ? a[3 + c] : a[c], shfl_xor_df(b16 ? a[c] : a[3 + c], 16));
+    const df32 r0 = shfl_xor_df(b8 ? k[0] : k[2], 8), r1 = shfl_xor_df(k[1], 8);
+    const df32 u = df_add(b8 ? k[2] : k[0], r0), v = df_add(k[1], r1);
+    df32 t = (b8 || !b4) ? u : v;
+    t = df_add(t, shfl_xor_df((b8 || b4) ? u : v, 4));
+    t = df_add(t, shfl_xor_df(t, 2));
+    return df_add(t, shfl_xor_df(t, 1));
 }
 
 // Sum over the warp's first N lanes (a power of two), valid in lane 0.

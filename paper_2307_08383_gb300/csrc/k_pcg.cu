@@ -175,8 +175,8 @@ __global__ void __launch_bounds__(256) k_spmv64(int n, const int *__restrict__ t
     spmv_rows<TS, double, false>(n, tw_ptr, tw_ent, S, x, nullptr, nullptr, q, 0.0);
 }
 
-// q = S x to about 2^-44 relative on the FP32 pipe, for the refinement
-// residual of FP32 problems (FP64 arithmetic runs at a small fraction of the
+// r64 = b - S x with S x to about 2^-44 relative on the FP32 pipe, ||r64||^2 and
+// ||b||^2, for the refinement of FP32 problems (FP64 arithmetic runs at a small fraction of the
 // FP32 rate on GB300).  x arrives split in FP32 pairs (xh + xl, k_split_x);
 // S is FP32.  Each product is the exact s xh (FMA TwoProd) plus s xl, added
 // with TwoSum (double-float).  A warp per block row over its two-sided
@@ -192,11 +192,14 @@ __global__ void k_split_x(int64_t cnt, const double *__restrict__ x, float2 *__r
         xs[i] = make_float2(h, l);
     }
 }
-__global__ void __launch_bounds__(256) k_spmv_df(int n, const int *__restrict__ tw_ptr, const int2 *__restrict__ tw_ent,
-                                                 const float *__restrict__ S, const float2 *__restrict__ xs, double *q) {
-    const int lane = threadIdx.x & 31;
+__global__ void __launch_bounds__(256) k_resid_df(int n, const int *__restrict__ tw_ptr, const int2 *__restrict__ tw_ent,
+                                                  const float *__restrict__ S, const float2 *__restrict__ xs,
+                                                  const float *__restrict__ b, double *r64, DevScalars *sc,
+                                                  double *red, unsigned *ctr) {
+    const int lane = threadIdx.x & 31, comp = fold6_comp(lane);
     const int warp = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
     const int nw = (int)(((int64_t)gridDim.x * blockDim.x) >> 5);
+    double v[2] = {0.0, 0.0};
     for (int i = warp; i < n; i += nw) {
         df32 acc[6];
 #pragma unroll
@@ -208,15 +211,15 @@ __global__ void __launch_bounds__(256) k_spmv_df(int n, const int *__restrict__ 
             float sb[36];  // the block, 16-byte loads
 #pragma unroll
             for (int q = 0; q < 9; ++q) {
-                const float4 v = __ldg(s4 + q);
-                sb[4 * q] = v.x; sb[4 * q + 1] = v.y; sb[4 * q + 2] = v.z; sb[4 * q + 3] = v.w;
+                const float4 u = __ldg(s4 + q);
+                sb[4 * q] = u.x; sb[4 * q + 1] = u.y; sb[4 * q + 2] = u.z; sb[4 * q + 3] = u.w;
             }
             float xh[6], xl[6];
 #pragma unroll
             for (int c = 0; c < 6; ++c) {
-                const float2 v = __ldcg(xs + 6 * (int64_t)e.y + c);
-                xh[c] = v.x;
-                xl[c] = v.y;
+                const float2 u = __ldcg(xs + 6 * (int64_t)e.y + c);
+                xh[c] = u.x;
+                xl[c] = u.y;
             }
 #pragma unroll
             for (int r = 0; r < 6; ++r)
@@ -228,12 +231,19 @@ __global__ void __launch_bounds__(256) k_spmv_df(int n, const int *__restrict__ 
                     acc[r] = df_add(acc[r], df32{ph, pl});
                 }
         }
-#pragma unroll
-        for (int r = 0; r < 6; ++r) acc[r] = warp_sum_df(acc[r]);
-#pragma unroll
-        for (int r = 0; r < 6; ++r)
-            if (lane == r) q[6 * (int64_t)i + r] = (double)acc[r].hi + (double)acc[r].lo;
+        const df32 q = warp_fold6_df(acc, lane);
+        if (fold6_owner(lane)) {
+            const int e = 6 * i + comp;
+            const double bi = widen(__ldg(b + e)), ri = bi - ((double)q.hi + (double)q.lo);
+            r64[e] = ri;
+            v[0] += ri * ri;
+            v[1] += bi * bi;
+        }
     }
+    grid_sum<2>(v, red, ctr, [&](double *t) {
+        sc->rr64 = t[0];
+        sc->bb64 = t[1];
+    });
 }
 
 template <typename T>
@@ -594,38 +604,6 @@ __global__ void __launch_bounds__(256) k_back_sub(int64_t P, const int *__restri
 // Split-preconditioned CG for FP32 solves
 // --------------------------------------------------------------------------
 
-// Cholesky A = L L^T of a symmetric 6x6 (row-major, lower triangle read) and
-// L^-1, both packed lower (index k(k+1)/2 + l).  False if A is not SPD.
-__device__ bool chol6_with_inverse(const double *A, double *L, double *Li) {
-#pragma unroll
-    for (int i = 0; i < 6; ++i) {
-#pragma unroll
-        for (int j = 0; j <= i; ++j) {
-            double s = A[i * 6 + j];
-#pragma unroll
-            for (int k = 0; k < j; ++k) s -= L[i * (i + 1) / 2 + k] * L[j * (j + 1) / 2 + k];
-            if (i == j) {
-                if (!(s > 0.0)) return false;
-                L[i * (i + 1) / 2 + i] = sqrt(s);
-            } else {
-                L[i * (i + 1) / 2 + j] = s / L[j * (j + 1) / 2 + j];
-            }
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < 6; ++i) {
-        Li[i * (i + 1) / 2 + i] = 1.0 / L[i * (i + 1) / 2 + i];
-#pragma unroll
-        for (int j = 0; j < i; ++j) {
-            double s = 0.0;
-#pragma unroll
-            for (int k = j; k < i; ++k) s += L[i * (i + 1) / 2 + k] * Li[k * (k + 1) / 2 + j];
-            Li[i * (i + 1) / 2 + j] = -s * Li[i * (i + 1) / 2 + i];
-        }
-    }
-    return true;
-}
-
 // Per camera, in FP64, a factor G_i with M_i^-1 = G_i G_i^T and H_i = G_i^-T
 // (H r^ gives back the residual of the original system):
 //   block-Jacobi (from_minv = 0): S_ii = L L^T, G = L^-T, H = L;
@@ -633,56 +611,61 @@ __device__ bool chol6_with_inverse(const double *A, double *L, double *Li) {
 // Stored row-major FP32, n x 36 each.  The diagonal block of S^ = G^T S G is
 // the identity for block-Jacobi (L^-1 L L^T L^-T); for a given M^-1 it is
 // G_i^T S_ii G_i, written to Shd (n x 36).
+// Eight lanes per camera (chol6_lanes): 16 -> 8.7 us at 200 cameras against a
+// thread each.
 template <typename T>
-__global__ void __launch_bounds__(128) k_split_factor(int n, const int *__restrict__ row_ptr, const T *__restrict__ S,
-                                                      const T *__restrict__ Minv, int from_minv, float *__restrict__ G,
-                                                      float *__restrict__ H, float *__restrict__ Shd, DevScalars *sc) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const T *src = from_minv ? Minv + 36 * (int64_t)i : S + (int64_t)__ldg(row_ptr + i) * BW;
-    double A[36], L[21], Li[21];
+__global__ void __launch_bounds__(32) k_split_factor(int n, const int *__restrict__ row_ptr, const T *__restrict__ S,
+                                                     const T *__restrict__ Minv, int from_minv, float *__restrict__ G,
+                                                     float *__restrict__ H, float *__restrict__ Shd, DevScalars *sc) {
+    constexpr unsigned FULL = 0xffffffffu;
+    const int i = (blockIdx.x * 32 + threadIdx.x) >> 3, r = threadIdx.x & 7;
+    const bool on = i < n && r < 6;
+    const T *sd = S + (i < n ? (int64_t)__ldg(row_ptr + i) * BW : 0), *src = from_minv && i < n ? Minv + 36 * (int64_t)i : sd;
+    double a[6], x[6];
 #pragma unroll
-    for (int k = 0; k < 36; ++k) A[k] = (double)src[k];
-    float *g = G + 36 * (int64_t)i, *h = H + 36 * (int64_t)i;
-    if (!chol6_with_inverse(A, L, Li)) {
-        atomicExch(&sc->err, (int)BA_ERR_NOT_SPD);
+    for (int k = 0; k < 6; ++k) a[k] = on ? (double)src[6 * r + k] : (i < n ? 0.0 : 1.0);
+    const bool ok = chol6_lanes<double>(a, x);
+    float *g = G + 36 * (int64_t)i + 6 * r, *h = H + 36 * (int64_t)i + 6 * r;
+    float fl[6], fx[6];  // row r of L, row r of L^-T
 #pragma unroll
-        for (int k = 0; k < 36; ++k) g[k] = h[k] = (k % 7 == 0) ? 1.f : 0.f;
-        return;
+    for (int c = 0; c < 6; ++c) {
+        fl[c] = !ok ? (c == r ? 1.f : 0.f) : (c <= r ? (float)a[c] : 0.f);
+        fx[c] = !ok ? (c == r ? 1.f : 0.f) : (float)x[c];
     }
+    if (on) {
+        if (!ok && r == 0) atomicExch(&sc->err, (int)BA_ERR_NOT_SPD);
+        store6(g, from_minv ? fl : fx);
+        store6(h, from_minv ? fx : fl);
+    }
+    if (!from_minv) return;
+    // row r of S_ii G, then of G^T (S_ii G), with G = L (lower) in FP64
+    double s[6], sg[6];
 #pragma unroll
-    for (int a = 0; a < 6; ++a)
+    for (int k = 0; k < 6; ++k) s[k] = on ? (double)sd[6 * r + k] : 0.0;
 #pragma unroll
-        for (int c = 0; c < 6; ++c) {
-            const double low = a >= c ? L[a * (a + 1) / 2 + c] : 0.0;    // L[a][c]
-            const double lit = c >= a ? Li[c * (c + 1) / 2 + a] : 0.0;   // (L^-1)^T[a][c]
-            g[6 * a + c] = (float)(from_minv ? low : lit);
-            h[6 * a + c] = (float)(from_minv ? lit : low);
+    for (int c = 0; c < 6; ++c) {
+        sg[c] = 0.0;
+#pragma unroll
+        for (int k = c; k < 6; ++k) sg[c] += s[k] * __shfl_sync(FULL, a[c], k, 8);
+    }
+    float dr[6];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+        double v = 0.0;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            // L[k][r] from lane k, for k >= r
+            double lkr = 0.0;
+#pragma unroll
+            for (int m = 0; m <= k; ++m) {
+                const double t = __shfl_sync(FULL, a[m], k, 8);
+                if (m == r) lkr = t;
+            }
+            v += lkr * __shfl_sync(FULL, sg[c], k, 8);
         }
-    if (from_minv) {
-        // S_ii G, then G^T (S_ii G), with G = L (lower) in FP64
-        const T *sd = S + (int64_t)__ldg(row_ptr + i) * BW;
-        double SG[36];
-#pragma unroll
-        for (int a = 0; a < 6; ++a)
-#pragma unroll
-            for (int c = 0; c < 6; ++c) {
-                double v = 0.0;
-#pragma unroll
-                for (int k = c; k < 6; ++k) v += (double)sd[6 * a + k] * L[k * (k + 1) / 2 + c];
-                SG[6 * a + c] = v;
-            }
-        float *d = Shd + 36 * (int64_t)i;
-#pragma unroll
-        for (int a = 0; a < 6; ++a)
-#pragma unroll
-            for (int c = 0; c < 6; ++c) {
-                double v = 0.0;
-#pragma unroll
-                for (int k = a; k < 6; ++k) v += L[k * (k + 1) / 2 + a] * SG[6 * k + c];
-                d[6 * a + c] = (float)v;
-            }
+        dr[c] = (float)v;
     }
+    if (on && ok) store6(Shd + 36 * (int64_t)i + 6 * r, dr);
 }
 
 // S^ in two-sided entry order without the diagonal blocks (the split CG's
@@ -764,15 +747,27 @@ __device__ __forceinline__ void load_rec(const float *rec, int j, float (&v)[20]
     }
 }
 
-// r^_0 = G^T rhs per camera into record 0, s = 0 in both records, x^ = p = 0,
-// and the scalars of the solve.
-__global__ void __launch_bounds__(256) k_split_init(int n, const float *__restrict__ rhs, const float *__restrict__ G,
-                                                    float *rec0, float *rec1, float *x, float *p, DevScalars *sc,
-                                                    double tol2, int max_iters, int prof) {
+// r^_0 = G^T rhs per camera (rhs rounded to FP32) into record 0, s = 0 in both
+// records, x^ = p = 0, the scalars of the solve, and its all-reduce's arrival
+// counters (bar0: 0, or -1 for the armed test of the timeout path).  first:
+// also ||rhs||^2 = ||b||^2 for the refinement.
+template <typename T>
+__global__ void __launch_bounds__(64) k_split_init(int n, const T *__restrict__ rhs, const float *__restrict__ G,
+                                                   float *rec0, float *rec1, float *x, float *p, DevScalars *sc,
+                                                   double tol2, int max_iters, int prof, unsigned *bar, unsigned bar0,
+                                                   int first, double *red, unsigned *ctr) {
+    double v[1] = {0.0};
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         float b6[6];
 #pragma unroll
-        for (int c = 0; c < 6; ++c) b6[c] = rhs[6 * i + c];
+        for (int c = 0; c < 6; ++c) {
+            const T b = rhs[6 * i + c];
+            b6[c] = (float)b;
+            if (first) {
+                const double d = widen(b);
+                v[0] += d * d;
+            }
+        }
         const float *g = G + 36 * (int64_t)i;
         float *q0 = rec0 + (int64_t)SREC * i, *q1 = rec1 + (int64_t)SREC * i;
 #pragma unroll
@@ -787,17 +782,21 @@ __global__ void __launch_bounds__(256) k_split_init(int n, const float *__restri
             p[6 * i + a] = 0.f;
         }
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        sc->tol2 = tol2;
-        sc->max_iters = max_iters;
-        sc->iters = 0;
-        sc->alpha = 0.0;
-        sc->beta = 0.0;
-        sc->done = max_iters <= 0 ? 1 : 0;
-        sc->prof_on = prof;
-        for (int k = 0; k < 4; ++k) sc->ph[k] = 0.0;
-        sc->ph_work_max = 0ull;
+    if (blockIdx.x == 0) {
+        for (int k = threadIdx.x; k < AR_SUB * 32; k += blockDim.x) bar[k] = bar0;
+        if (threadIdx.x == 0) {
+            sc->tol2 = tol2;
+            sc->max_iters = max_iters;
+            sc->iters = 0;
+            sc->alpha = 0.0;
+            sc->beta = 0.0;
+            sc->done = max_iters <= 0 ? 1 : 0;
+            sc->prof_on = prof;
+            for (int k = 0; k < 4; ++k) sc->ph[k] = 0.0;
+            sc->ph_work_max = 0ull;
+        }
     }
+    if (first) grid_sum<1>(v, red, ctr, [&](double *t) { sc->rr64 = sc->bb64 = t[0]; });
 }
 
 __device__ __forceinline__ unsigned long long global_ns() {
@@ -1344,9 +1343,10 @@ __global__ void __launch_bounds__(SPLIT_WARPS * 32, SPLIT_CTAS_PER_SM) k_pcg_spl
     }
 }
 
-// x64 (+)= G x^ per camera (the solution of the original system)
+// x64 (+)= G x^ per camera (the solution of the original system); with xs, also
+// its FP32 pairs for k_resid_df
 __global__ void k_acc64_split(int n, const float *__restrict__ G, const float *__restrict__ xh, double *x64,
-                              int first) {
+                              int first, float2 *xs) {
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= 6 * n) return;
     const int i = e / 6, a = e - 6 * i;
@@ -1354,7 +1354,13 @@ __global__ void k_acc64_split(int n, const float *__restrict__ G, const float *_
     float t = 0.f;
 #pragma unroll
     for (int c = 0; c < 6; ++c) t = __fmaf_rn(__ldg(g + c), __ldcg(xh + 6 * i + c), t);
-    x64[e] = (first ? 0.0 : x64[e]) + (double)t;
+    const double v = (first ? 0.0 : x64[e]) + (double)t;
+    x64[e] = v;
+    if (xs) {
+        float h, l;
+        split_f64(v, h, l);
+        xs[e] = make_float2(h, l);
+    }
 }
 
 // --------------------------------------------------------------------------
@@ -1370,14 +1376,14 @@ static constexpr int VEC_CAP = 152 * 4;
 cudaError_t launch_pcg_init(ba_problem *p, const void *rhs, double tol, int max_iters) {
     cudaEvent_t ev;
     ktimer_begin(p, K_PCG_INIT, &ev);
-    const int g = grid_for(p->n, 256, VEC_CAP);
+    const int g = grid_for(p->n, 64, VEC_CAP);
     if (p->sv.f32)
-        k_pcg_init<float><<<g, 256, 0, p->st>>>(p->n, (const float *)rhs, (const float *)p->sv.Minv, (float *)p->sv.pv[0],
+        k_pcg_init<float><<<g, 64, 0, p->st>>>(p->n, (const float *)rhs, (const float *)p->sv.Minv, (float *)p->sv.pv[0],
                                                 (float *)p->sv.pv[1], (float *)p->sv.pv[2], (float *)p->sv.pv[3],
                                                 (float *)p->sv.pv[5], (float *)p->sv.pv[7], p->sc, tol * tol, max_iters, p->red,
                                                 p->counters + 2);
     else
-        k_pcg_init<double><<<g, 256, 0, p->st>>>(p->n, (const double *)rhs, (const double *)p->sv.Minv,
+        k_pcg_init<double><<<g, 64, 0, p->st>>>(p->n, (const double *)rhs, (const double *)p->sv.Minv,
                                                  (double *)p->sv.pv[0], (double *)p->sv.pv[1], (double *)p->sv.pv[2],
                                                  (double *)p->sv.pv[3], (double *)p->sv.pv[5], (double *)p->sv.pv[7], p->sc,
                                                  tol * tol, max_iters, p->red, p->counters + 2);
@@ -1489,25 +1495,29 @@ static cudaError_t ensure_xs(ba_problem *p) {
     return cudaSuccess;
 }
 
-// from_x64: r64 = b - S x64; else r64 = b (x64 = 0).
-cudaError_t launch_resid64(ba_problem *p, bool from_x64) {
+// from_x64: r64 = b - S x64; else r64 = b (x64 = 0).  split: the FP32 pairs of
+// x64 were written by launch_accumulate_split.
+cudaError_t launch_resid64(ba_problem *p, bool from_x64, bool split) {
     cudaEvent_t ev;
-    ktimer_begin(p, K_RESID64, &ev);
-    if (from_x64) {
-        const int gs = grid_for((int64_t)p->n * 32, 256, 152 * 8);
+    cudaError_t e;
+    // a warp per row: two rows to a CTA until every SM has several, else eight
+    const int th = p->n <= 152 * 8 ? 64 : 256, gs = grid_for((int64_t)p->n * 32, th, 152 * 8);
+    if (from_x64 && p->fp32) {
         // FP32 problems: double-float products on the FP32 pipe; FP64
         // problems keep FP64 arithmetic (their S is FP64)
-        if (p->fp32) {
-            cudaError_t e = ensure_xs(p);
-            if (e != cudaSuccess) return e;
-            const int64_t cnt = (int64_t)p->n * 6;
-            k_split_x<<<grid_for(cnt, 256, VEC_CAP), 256, 0, p->st>>>(cnt, p->x64, p->xs);
-            k_spmv_df<<<gs, 256, 0, p->st>>>(p->n, p->tw_ptr, p->tw_ent, (const float *)p->S, p->xs, p->q64);
-            p->launches += 1;
-        } else {
-            k_spmv64<double><<<gs, 256, 0, p->st>>>(p->n, p->tw_ptr, p->tw_ent, (const double *)p->S, p->x64, p->q64);
-        }
+        if ((e = ensure_xs(p)) != cudaSuccess) return e;
+        ktimer_begin(p, K_RESID64, &ev);
+        const int64_t cnt = (int64_t)p->n * 6;
+        if (!split) k_split_x<<<grid_for(cnt, 256, VEC_CAP), 256, 0, p->st>>>(cnt, p->x64, p->xs);
+        k_resid_df<<<gs, th, 0, p->st>>>(p->n, p->tw_ptr, p->tw_ent, (const float *)p->S, p->xs, (const float *)p->b,
+                                          p->r64, p->sc, p->red, p->counters + 6);
+        ktimer_end(p, K_RESID64, ev);
+        p->launches += split ? 1 : 2;
+        return cudaGetLastError();
     }
+    ktimer_begin(p, K_RESID64, &ev);
+    if (from_x64)
+        k_spmv64<double><<<gs, th, 0, p->st>>>(p->n, p->tw_ptr, p->tw_ent, (const double *)p->S, p->x64, p->q64);
     const int g = grid_for((int64_t)p->n * 6, 256, VEC_CAP);
     if (p->fp32)
         k_resid_fin<float><<<g, 256, 0, p->st>>>(p->n, (const float *)p->b, p->q64, p->r64, p->sc, p->red,
@@ -1616,9 +1626,9 @@ cudaError_t launch_split_prepare(ba_problem *p, bool from_minv) {
     if (e != cudaSuccess) return e;
     cudaEvent_t ev;
     ktimer_begin(p, K_SPLIT_PREP, &ev);
-    // the factors: a thread per camera in FP64, 32 to a CTA so that the
+    // the factors: eight lanes per camera in FP64, one warp to a CTA so that the
     // cameras spread over every SM's FP64 units; S^: a warp per block row
-    const int nb = (p->n + 31) / 32, ns = (int)(((int64_t)p->n * 32 + 127) / 128);
+    const int nb = (p->n + 3) / 4, ns = (int)(((int64_t)p->n * 32 + 127) / 128);
     if (p->fp32) {
         k_split_factor<float><<<nb, 32, 0, p->st>>>(p->n, p->row_ptr, (const float *)p->S, (const float *)p->Minv,
                                                      from_minv ? 1 : 0, p->Gs, p->Hs, p->Shd, p->sc);
@@ -1865,14 +1875,25 @@ bool split_available(ba_problem *p) {
     return p->split_grid > 0;
 }
 
-// vectors: pv[0] x^, pv[2] p of the active FP32 view; records in p->srec
-cudaError_t launch_split_init(ba_problem *p, const float *rhs, double tol, int max_iters) {
+// vectors: pv[0] x^, pv[2] p of the active FP32 view; records in p->srec.
+// first: the sweep's right-hand side is b, else the residual r64
+cudaError_t launch_split_init(ba_problem *p, bool first, double tol, int max_iters) {
+    const cudaError_t e = ensure_ar_bar(p);
+    if (e != cudaSuccess) return e;
     cudaEvent_t ev;
     ktimer_begin(p, K_PCG_INIT, &ev);
     float **v = (float **)p->sv.pv;
     float *rec0 = p->srec, *rec1 = p->srec + (size_t)SREC * p->n;
-    k_split_init<<<grid_for(p->n, 256, VEC_CAP), 256, 0, p->st>>>(p->n, rhs, p->Gs, rec0, rec1, v[0], v[2], p->sc,
-                                                                  tol * tol, max_iters, p->opt.profile >= 2);
+    const int g = grid_for(p->n, 64, VEC_CAP), prof = p->opt.profile >= 2 ? 1 : 0;
+    const unsigned bar0 = p->test_wait_limit > 0 ? ~0u : 0u;
+    if (first && p->fp32)
+        k_split_init<float><<<g, 64, 0, p->st>>>(p->n, (const float *)p->b, p->Gs, rec0, rec1, v[0], v[2], p->sc,
+                                                 tol * tol, max_iters, prof, p->ar_bar, bar0, 1, p->red,
+                                                 p->counters + 6);
+    else
+        k_split_init<double><<<g, 64, 0, p->st>>>(p->n, first ? (const double *)p->b : p->r64, p->Gs, rec0, rec1, v[0],
+                                                  v[2], p->sc, tol * tol, max_iters, prof, p->ar_bar, bar0,
+                                                  first ? 1 : 0, p->red, p->counters + 6);
     ktimer_end(p, K_PCG_INIT, ev);
     p->launches += 1;
     return cudaGetLastError();
@@ -1881,14 +1902,13 @@ cudaError_t launch_split_init(ba_problem *p, const float *rhs, double tol, int m
 cudaError_t launch_pcg_split(ba_problem *p) {
     cudaEvent_t ev;
     cudaError_t e = cudaSuccess;
-    if ((e = ensure_ar_bar(p)) != cudaSuccess) return e;
     ktimer_begin(p, K_PCG_LOOP, &ev);
-    // armed test of the timeout path: every counter starts at -1, so each one
-    // ends a call one arrival short of its target and the wait runs out
+    // armed test of the timeout path: every counter started at -1
+    // (launch_split_init), so each one ends a call one arrival short of its
+    // target and the wait runs out
     const long long test_limit = p->test_wait_limit;
     p->test_wait_limit = 0;
-    e = cudaMemsetAsync(p->ar_bar, test_limit > 0 ? 0xFF : 0, AR_SUB * 32 * sizeof(unsigned), p->st);
-    if (e == cudaSuccess) {
+    {
         const int *cr = p->cta_rows, *twp = p->tws_ptr, *mo = p->meta_off, *hp = p->halo_ptr, *hc = p->halo_col,
                   *ob = p->own_base;
         const uint32_t *meta = p->tw_meta;
@@ -1921,9 +1941,11 @@ cudaError_t launch_pcg_split(ba_problem *p) {
 }
 
 cudaError_t launch_accumulate_split(ba_problem *p, bool first) {
+    cudaError_t e;
+    if (p->fp32 && (e = ensure_xs(p)) != cudaSuccess) return e;
     const int cnt = p->n * 6;
-    k_acc64_split<<<(cnt + 255) / 256, 256, 0, p->st>>>(p->n, p->Gs, (const float *)p->sv.pv[0], p->x64,
-                                                        first ? 1 : 0);
+    k_acc64_split<<<(cnt + 127) / 128, 128, 0, p->st>>>(p->n, p->Gs, (const float *)p->sv.pv[0], p->x64,
+                                                        first ? 1 : 0, p->fp32 ? p->xs : nullptr);
     p->launches += 1;
     return cudaGetLastError();
 }

@@ -57,30 +57,29 @@ unsigned char *g_ptr[kMaxDevices] = {};
 // triangles, which the two-sided product would count twice - sets
 // BA_ERR_INVALID_ARG; a diagonal block that is not SPD sets BA_ERR_NOT_SPD.
 // Either error stops the solve before its first iteration.
-__global__ void k_static_minv(int n, int64_t nnzb, const int *__restrict__ row_ptr, const int *__restrict__ col,
-                              const float *__restrict__ val, float *__restrict__ Minv, StaticScalars *sc) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    double A[36], Ai[36];
-    const int rs = row_ptr[i], re = row_ptr[i + 1];
-    bool ok = rs >= 0 && re > rs && (int64_t)re <= nnzb && (i + 1 < n || (int64_t)re == nnzb) && col[rs] == i;
-    for (int k = rs + 1; ok && k < re; ++k) ok = col[k] > col[k - 1] && col[k] < n;
-    if (!ok) {
-        atomicExch(&sc->err, (int)BA_ERR_INVALID_ARG);
+// Eight lanes per camera (chol6_lanes, FP64).
+__global__ void __launch_bounds__(32) k_static_minv(int n, int64_t nnzb, const int *__restrict__ row_ptr,
+                                                    const int *__restrict__ col, const float *__restrict__ val,
+                                                    float *__restrict__ Minv, StaticScalars *sc) {
+    const int i = (blockIdx.x * 32 + threadIdx.x) >> 3, r = threadIdx.x & 7;
+    const int rs = i < n ? row_ptr[i] : 0, re = i < n ? row_ptr[i + 1] : 0;
+    bool ok = i < n && rs >= 0 && re > rs && (int64_t)re <= nnzb && (i + 1 < n || (int64_t)re == nnzb);
+    ok = ok && col[rs] == i;
+    for (int k = rs + 1 + r; ok && k < re; k += 8) ok = col[k] > col[k - 1] && col[k] < n;
+    ok = (__ballot_sync(0xffffffffu, ok) >> (threadIdx.x & 24) & 0xffu) == 0xffu;  // all eight lanes
+    double a[6], x[6], out[6];
+    const float *d = val + (int64_t)(ok ? rs : 0) * BW;
 #pragma unroll
-        for (int q = 0; q < 36; ++q) Minv[36 * (int64_t)i + q] = 0.f;
-        return;
+    for (int c = 0; c < 6; ++c) a[c] = ok && r < 6 ? (double)d[6 * r + c] : 0.0;
+    const bool spd = chol6_lanes<double>(a, x);
+    inv6_row<double>(x, out);
+    if (i >= n || r >= 6) return;
+    if (r == 0) {
+        if (!ok) atomicExch(&sc->err, (int)BA_ERR_INVALID_ARG);
+        else if (!spd) atomicCAS(&sc->err, 0, (int)BA_ERR_NOT_SPD);
     }
-    const float *d = val + (int64_t)rs * BW;
 #pragma unroll
-    for (int q = 0; q < 36; ++q) A[q] = d[q];
-    if (!spd_inverse6<double>(A, Ai)) {
-        atomicCAS(&sc->err, 0, (int)BA_ERR_NOT_SPD);
-#pragma unroll
-        for (int q = 0; q < 36; ++q) Ai[q] = 0.0;
-    }
-#pragma unroll
-    for (int q = 0; q < 36; ++q) Minv[36 * (int64_t)i + q] = (float)Ai[q];
+    for (int q = 0; q < 6; ++q) Minv[36 * (int64_t)i + 6 * r + q] = ok && spd ? (float)out[q] : 0.f;
 }
 
 // The whole solve in one cooperative launch.  CTA c owns block rows c R ..
@@ -314,7 +313,7 @@ extern "C" ba_status ba_pcg_solve_static(int32_t n, int64_t nnzb, const int32_t 
         return set_error(BA_ERR_CUDA, cudaGetErrorString(e));
     if ((e = cudaMemsetAsync(sc, 0, sizeof(StaticScalars), st)) != cudaSuccess)
         return set_error(BA_ERR_CUDA, cudaGetErrorString(e));
-    k_static_minv<<<(n + 31) / 32, 32, 0, st>>>(n, nnzb, row_ptr, col, val, Minv, sc);
+    k_static_minv<<<(n + 3) / 4, 32, 0, st>>>(n, nnzb, row_ptr, col, val, Minv, sc);
     if ((e = cudaGetLastError()) != cudaSuccess) return set_error(BA_ERR_CUDA, cudaGetErrorString(e));
     // shared memory for the blocks: what a CTA's share of them needs, with
     // half as much again for uneven rows, at most what a CTA can have

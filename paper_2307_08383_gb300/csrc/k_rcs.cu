@@ -401,56 +401,60 @@ __global__ void __launch_bounds__(256) k_rcs_reduce(int64_t nblk, const int *__r
     }
 }
 
-// K4: unpack the diagonal blocks, damp them, extract b, invert for M^-1.
+// K4: unpack the diagonal blocks, damp them, extract b, invert for M^-1: eight
+// lanes per camera (chol6_lanes), lane r row r.
 template <typename T>
-__global__ void k_rcs_diag(int n, const int *__restrict__ row_ptr, T *__restrict__ S, T *__restrict__ b,
-                           T *__restrict__ Minv, double lambda, DevScalars *sc) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    T *Sd = S + (int64_t)row_ptr[i] * BW;
-    T pk[36], A[36], Ai[36];
+__global__ void __launch_bounds__(32) k_rcs_diag(int n, const int *__restrict__ row_ptr, T *__restrict__ S,
+                                                 T *__restrict__ b, T *__restrict__ Minv, double lambda,
+                                                 DevScalars *sc) {
+    const int i = (blockIdx.x * 32 + threadIdx.x) >> 3, r = threadIdx.x & 7;
+    const bool on = i < n && r < 6;
+    T *Sd = S + (i < n ? (int64_t)row_ptr[i] * BW : 0);
+    T a[6], x[6], out[6];
 #pragma unroll
-    for (int q = 0; q < 36; ++q) pk[q] = Sd[q];
-#pragma unroll
-    for (int r = 0; r < 6; ++r)
-#pragma unroll
-        for (int c = r; c < 6; ++c) {
-            A[6 * r + c] = pk[up_idx(r, c)];
-            A[6 * c + r] = pk[up_idx(r, c)];
-        }
-    const T lam = (T)lambda;
-#pragma unroll
-    for (int r = 0; r < 6; ++r) A[7 * r] += lam * clampT(pk[21 + r]);
-#pragma unroll
-    for (int q = 0; q < 36; ++q) Sd[q] = A[q];
-#pragma unroll
-    for (int r = 0; r < 6; ++r) b[6 * i + r] = pk[27 + r];
-    if (!spd_inverse6<T>(A, Ai)) {
-        atomicExch(&sc->err, (int)BA_ERR_NOT_SPD);
-#pragma unroll
-        for (int q = 0; q < 36; ++q) Ai[q] = T(0);
+    for (int c = 0; c < 6; ++c) {
+        const int lo = min(r, c), hi = max(r, c);
+        a[c] = on ? Sd[6 * lo - lo * (lo - 1) / 2 + (hi - lo)] : (i < n ? T(0) : T(1));
     }
+    if (on) {
+        const T dmp = (T)lambda * clampT(Sd[21 + r]);
 #pragma unroll
-    for (int q = 0; q < 36; ++q) Minv[36 * (int64_t)i + q] = Ai[q];
+        for (int c = 0; c < 6; ++c)
+            if (c == r) a[c] += dmp;
+        b[6 * i + r] = Sd[27 + r];
+    }
+    __syncwarp();  // the packed block has been read
+    if (on) store6(Sd + 6 * r, a);
+    const bool ok = chol6_lanes<T>(a, x);
+    inv6_row<T>(x, out);
+    if (!on) return;
+    if (!ok) {
+        if (r == 0) atomicExch(&sc->err, (int)BA_ERR_NOT_SPD);
+#pragma unroll
+        for (int c = 0; c < 6; ++c) out[c] = T(0);
+    }
+    store6(Minv + 36 * (int64_t)i + 6 * r, out);
 }
 
 // Block-Jacobi only: M_i^-1 = S_ii^-1 (diagonal blocks stored full, first in each row).
 template <typename T>
-__global__ void k_block_jacobi(int n, const int *__restrict__ row_ptr, const T *__restrict__ S, T *__restrict__ Minv,
-                               DevScalars *sc) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    T A[36], Ai[36];
-    const T *d = S + (int64_t)row_ptr[i] * BW;
+__global__ void __launch_bounds__(32) k_block_jacobi(int n, const int *__restrict__ row_ptr, const T *__restrict__ S,
+                                                     T *__restrict__ Minv, DevScalars *sc) {
+    const int i = (blockIdx.x * 32 + threadIdx.x) >> 3, r = threadIdx.x & 7;
+    const bool on = i < n && r < 6;
+    const T *d = S + (i < n ? (int64_t)row_ptr[i] * BW : 0);
+    T a[6], x[6], out[6];
 #pragma unroll
-    for (int q = 0; q < 36; ++q) A[q] = d[q];
-    if (!spd_inverse6<T>(A, Ai)) {
-        atomicExch(&sc->err, (int)BA_ERR_NOT_SPD);
+    for (int c = 0; c < 6; ++c) a[c] = on ? d[6 * r + c] : (i < n ? T(0) : T(1));
+    const bool ok = chol6_lanes<T>(a, x);
+    inv6_row<T>(x, out);
+    if (!on) return;
+    if (!ok) {
+        if (r == 0) atomicExch(&sc->err, (int)BA_ERR_NOT_SPD);
 #pragma unroll
-        for (int q = 0; q < 36; ++q) Ai[q] = T(0);
+        for (int c = 0; c < 6; ++c) out[c] = T(0);
     }
-#pragma unroll
-    for (int q = 0; q < 36; ++q) Minv[36 * (int64_t)i + q] = Ai[q];
+    store6(Minv + 36 * (int64_t)i + 6 * r, out);
 }
 
 static inline int grid_for(int64_t work, int threads, int cap) {
@@ -478,11 +482,11 @@ static cudaError_t form_rcs_T(ba_problem *p, double lambda, size_t smem, long lo
 }
 
 cudaError_t launch_block_jacobi(ba_problem *p) {
-    const int nb = (p->n + 127) / 128;
+    const int nb = (p->n + 3) / 4;
     if (p->fp32)
-        k_block_jacobi<float><<<nb, 128, 0, p->st>>>(p->n, p->row_ptr, (const float *)p->S, (float *)p->Minv, p->sc);
+        k_block_jacobi<float><<<nb, 32, 0, p->st>>>(p->n, p->row_ptr, (const float *)p->S, (float *)p->Minv, p->sc);
     else
-        k_block_jacobi<double><<<nb, 128, 0, p->st>>>(p->n, p->row_ptr, (const double *)p->S, (double *)p->Minv, p->sc);
+        k_block_jacobi<double><<<nb, 32, 0, p->st>>>(p->n, p->row_ptr, (const double *)p->S, (double *)p->Minv, p->sc);
     p->launches += 1;
     return cudaGetLastError();
 }
@@ -514,12 +518,12 @@ cudaError_t launch_form_rcs(ba_problem *p, double lambda) {
     p->launches += 1;
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
     ktimer_begin(p, K_RCS_DIAG, &ev);
-    const int nb = (p->n + 127) / 128;
+    const int nb = (p->n + 3) / 4;
     if (p->fp32)
-        k_rcs_diag<float><<<nb, 128, 0, p->st>>>(p->n, p->row_ptr, (float *)p->S, (float *)p->b, (float *)p->Minv,
+        k_rcs_diag<float><<<nb, 32, 0, p->st>>>(p->n, p->row_ptr, (float *)p->S, (float *)p->b, (float *)p->Minv,
                                                  lambda, p->sc);
     else
-        k_rcs_diag<double><<<nb, 128, 0, p->st>>>(p->n, p->row_ptr, (double *)p->S, (double *)p->b,
+        k_rcs_diag<double><<<nb, 32, 0, p->st>>>(p->n, p->row_ptr, (double *)p->S, (double *)p->b,
                                                   (double *)p->Minv, lambda, p->sc);
     ktimer_end(p, K_RCS_DIAG, ev);
     p->launches += 1;
