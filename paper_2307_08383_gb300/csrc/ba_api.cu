@@ -282,32 +282,50 @@ ba_status ba_problem_create(const ba_options *opt, int32_t n_cams, const double 
     p->lambda = o.lambda0;
     p->nu = 2.0;
     std::string err;
-    ba_status s = symbolic_setup(n_cams, n_pts, n_obs, obs_cam, obs_pt, pts, p->obs_max, false, p->hs, err);
-    if (s != BA_OK) {
-        delete p;
-        return fail(s, err);
-    }
-    HostSetup &hs = p->hs;
-    p->nnzb = (int64_t)hs.col.size();
-    p->ngroups = (int64_t)hs.groups.size();
-    p->npart = (int64_t)hs.lb_gblk.size();
-    p->nitems = (int64_t)hs.items.size();
     const int64_t n = n_cams, P = n_pts, m = n_obs;
     const size_t E = p->esz;
-
-    // planned device bytes (checked against the cap before any allocation)
+    HostSetup &hs = p->hs;
+    // Point groups of equal size for whole rounds of the formation's CTAs (two
+    // to an SM in FP32, one in FP64), at most the default size.  50 cameras,
+    // FP64: 22 groups of 512 keep 22 SMs busy, formation 110 us and the step's
+    // point pass 26; 49 and 18 with 141 groups.  200 cameras, FP64: 374 -> 321
+    // us.  FP32 beyond one round keeps the default (200 cameras 22.6 / 21 us
+    // alone, no difference in the step; 1,770 cameras 114 both ways).  The few
+    // observations on top allow for whole tracks.
+    int target = p->obs_max;
+    const int64_t slots = p->fp32 ? 304 : 152, rounds = (m + slots * p->obs_max - 1) / (slots * p->obs_max);
+    if (o.group_max_obs <= 0 && (!p->fp32 || rounds == 1))
+        target = (int)std::min<int64_t>(p->obs_max, std::max<int64_t>(40, (m + slots * rounds - 1) / (slots * rounds) + 8));
     const size_t camc_w = p->fp32 ? CAMC32_W * 4 : 12 * 8;
-    size_t plan = 2 * (n * 6 * 8 + P * 3 * 8 + n * camc_w + (p->fp32 ? P * 6 * 4 + m * 2 * 4 : 0)) +
-                  m * 4 * 2 + (P + 1) * 4 + m * 16 + (p->fp32 ? m * 16 : 0) + m * JW * E + (n + 1) * 4 +
-                  p->nnzb * 4 + 2 * (n + 1) * 4 + 2 * p->nnzb * 4 + (2 * p->nnzb - n) * 8 + p->nnzb * BW * E + n * 6 * E + n * 36 * E + p->ngroups * sizeof(GroupDesc) +
-                  p->nitems * 8 + hs.contrib.size() * 4 + (p->nnzb + 1) * 4 + p->npart * 4 + p->npart * BW * E +
-                  P * 9 * E + 8 * n * 6 * E + 3 * n * 6 * 8 + n * 6 * E + P * 3 * E + sizeof(DevScalars) +
-                  RED_SLOTS * 8 + N_COUNTERS * 4;
+    size_t plan = 0;
+    for (;;) {
+        ba_status s = symbolic_setup(n_cams, n_pts, n_obs, obs_cam, obs_pt, pts, p->obs_max, false, hs, err, target);
+        if (s != BA_OK) {
+            delete p;
+            return fail(s, err);
+        }
+        p->nnzb = (int64_t)hs.col.size();
+        p->ngroups = (int64_t)hs.groups.size();
+        p->npart = (int64_t)hs.lb_gblk.size();
+        p->nitems = (int64_t)hs.items.size();
+
+        // planned device bytes (checked against the cap before any allocation)
+        plan = 2 * (n * 6 * 8 + P * 3 * 8 + n * camc_w + (p->fp32 ? P * 6 * 4 + m * 2 * 4 : 0)) +
+                      m * 4 * 2 + (P + 1) * 4 + m * 16 + (p->fp32 ? m * 16 : 0) + m * JW * E + (n + 1) * 4 +
+                      p->nnzb * 4 + 2 * (n + 1) * 4 + 2 * p->nnzb * 4 + (2 * p->nnzb - n) * 8 + p->nnzb * BW * E + n * 6 * E + n * 36 * E + p->ngroups * sizeof(GroupDesc) +
+                      p->nitems * 8 + hs.contrib.size() * 4 + (p->nnzb + 1) * 4 + p->npart * 4 + p->npart * BW * E +
+                      P * 9 * E + 8 * n * 6 * E + 3 * n * 6 * 8 + n * 6 * E + P * 3 * E + sizeof(DevScalars) +
+                      RED_SLOTS * 8 + N_COUNTERS * 4;
+        // smaller groups write more partials: a cap that only they exceed gets the default size
+        if (!o.device_mem_cap || plan <= o.device_mem_cap || target == p->obs_max) break;
+        target = p->obs_max;
+    }
     if (o.device_mem_cap && plan > o.device_mem_cap) {
         delete p;
         return fail(BA_ERR_OOM, "problem needs " + std::to_string(plan) + " device bytes, cap is " +
                                     std::to_string(o.device_mem_cap));
     }
+    p->obs_max = (hs.max_nobs + 7) & ~7;  // what the kernels' buffers hold
 #define AL(ptr, cnt)                                                                                  \
     do {                                                                                              \
         cudaError_t e_ = dalloc(p, &(ptr), (cnt));                                                    \

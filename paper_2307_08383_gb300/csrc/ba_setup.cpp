@@ -166,7 +166,8 @@ void order_items_for_banks(uint32_t *cl, const WorkItem *its, int32_t nit, const
 
 ba_status symbolic_setup(int32_t n, int64_t P, int64_t m, const int32_t *obs_cam,
                          const int64_t *obs_pt, const double *pts, int obs_max, bool pattern_only,
-                         HostSetup &hs, std::string &err) {
+                         HostSetup &hs, std::string &err, int obs_target) {
+    if (obs_target <= 0 || obs_target > obs_max) obs_target = obs_max;
     if (n <= 0 || P <= 0 || m <= 0) { err = "n_cams, n_pts and n_obs must be positive"; return BA_ERR_INVALID_ARG; }
     if (m >= (int64_t)INT32_MAX || P >= (int64_t)INT32_MAX) { err = "n_obs and n_pts must be < 2^31"; return BA_ERR_INVALID_ARG; }
     if (!obs_cam || !obs_pt) { err = "null observation index array"; return BA_ERR_INVALID_ARG; }
@@ -350,7 +351,7 @@ ba_status symbolic_setup(int32_t n, int64_t P, int64_t m, const int32_t *obs_cam
                   " observations; the limit is " + std::to_string(std::min(obs_max, 90));
             return BA_ERR_INVALID_ARG;
         }
-        if (g.npts > 0 && (g.nobs + L > obs_max || g.nc + npair > C_MAX || (int32_t)g_gblk.size() + fresh > LB_MAX))
+        if (g.npts > 0 && (g.nobs + L > obs_target || g.nc + npair > C_MAX || (int32_t)g_gblk.size() + fresh > LB_MAX))
             close_group();
         if (g.npts == 0) { g.obs_begin = tb; g.pt_begin = (int32_t)k; }
         int32_t q = 0;

@@ -362,8 +362,11 @@ __global__ void __launch_bounds__(FORM_THREADS) k_form_rcs(const GroupDesc *__re
 
 // K3: S[block] = sum of the block's partials in list order (fixed), a thread
 // per 16-byte chunk of the block (9 for FP32, 18 for FP64): the chunks of a
-// partial are read by consecutive threads, and each thread keeps four
-// partials' loads in flight before adding them in order.  (Writing each
+// partial are read by consecutive threads, and each thread keeps DEPTH
+// partials' loads in flight before adding them in order; with 8 also the next
+// ones' indices.  DEPTH 8 for small systems (few warps, long lists: a chain of
+// round trips; 50 cameras FP64 43 -> 29 us, 200 cameras FP32 19 -> 12), 4 for
+// large ones (bandwidth: 1,770 cameras FP32 27 us, 31 with 8).  (Writing each
 // partial straight to a block-ordered slot in RCS formation made this
 // reduction contiguous but cost the formation more than it saved here.)
 __device__ __forceinline__ void add16(float4 &s, const float4 v) {
@@ -372,7 +375,7 @@ __device__ __forceinline__ void add16(float4 &s, const float4 v) {
 __device__ __forceinline__ void add16(double2 &s, const double2 v) {
     s.x += v.x; s.y += v.y;
 }
-template <typename T>
+template <typename T, int DEPTH>
 __global__ void __launch_bounds__(256) k_rcs_reduce(int64_t nblk, const int *__restrict__ pptr, const int *__restrict__ plist,
                                                     const T *__restrict__ part, T *__restrict__ S) {
     using V = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
@@ -386,17 +389,38 @@ __global__ void __launch_bounds__(256) k_rcs_reduce(int64_t nblk, const int *__r
         int q = __ldg(pptr + blk);
         V s;
         std::memset(&s, 0, sizeof(V));
-        for (; q + 4 <= q1; q += 4) {
-            const int i0 = __ldg(plist + q), i1 = __ldg(plist + q + 1), i2 = __ldg(plist + q + 2),
-                      i3 = __ldg(plist + q + 3);
-            const V v0 = pv[(int64_t)i0 * NCH + c], v1 = pv[(int64_t)i1 * NCH + c], v2 = pv[(int64_t)i2 * NCH + c],
-                    v3 = pv[(int64_t)i3 * NCH + c];
-            add16(s, v0);
-            add16(s, v1);
-            add16(s, v2);
-            add16(s, v3);
+        if constexpr (DEPTH == 4) {
+            for (; q + 4 <= q1; q += 4) {
+                const int i0 = __ldg(plist + q), i1 = __ldg(plist + q + 1), i2 = __ldg(plist + q + 2),
+                          i3 = __ldg(plist + q + 3);
+                const V v0 = pv[(int64_t)i0 * NCH + c], v1 = pv[(int64_t)i1 * NCH + c], v2 = pv[(int64_t)i2 * NCH + c],
+                        v3 = pv[(int64_t)i3 * NCH + c];
+                add16(s, v0);
+                add16(s, v1);
+                add16(s, v2);
+                add16(s, v3);
+            }
+            for (; q < q1; ++q) add16(s, pv[(int64_t)__ldg(plist + q) * NCH + c]);
+        } else {
+            int id[DEPTH];
+            if (q < q1) {
+#pragma unroll
+                for (int k = 0; k < DEPTH; ++k) id[k] = __ldg(plist + min(q + k, q1 - 1));
+            }
+            for (; q < q1; q += DEPTH) {
+                V v[DEPTH];
+#pragma unroll
+                for (int k = 0; k < DEPTH; ++k)
+                    if (q + k < q1) v[k] = pv[(int64_t)id[k] * NCH + c];
+                if (q + DEPTH < q1) {
+#pragma unroll
+                    for (int k = 0; k < DEPTH; ++k) id[k] = __ldg(plist + min(q + DEPTH + k, q1 - 1));
+                }
+#pragma unroll
+                for (int k = 0; k < DEPTH; ++k)
+                    if (q + k < q1) add16(s, v[k]);
+            }
         }
-        for (; q < q1; ++q) add16(s, pv[(int64_t)__ldg(plist + q) * NCH + c]);
         sv[x] = s;
     }
 }
@@ -508,12 +532,18 @@ cudaError_t launch_form_rcs(ba_problem *p, double lambda) {
     p->launches += 1;
     if ((err = cudaGetLastError()) != cudaSuccess) return err;
     ktimer_begin(p, K_RCS_REDUCE, &ev);
-    const int g = grid_for(p->nnzb * (int64_t)(BW * p->esz / 16), 256, 152 * 16);
+    // CTAs of two warps until every SM has several (the adds of an FP64 CTA of
+    // eight are its SM's FP64 issue)
+    const int64_t chunks = p->nnzb * (int64_t)(BW * p->esz / 16);
+    const bool small = chunks <= 152 * 1024;
+    const int th = small ? 64 : 256, g = grid_for(chunks, th, 152 * 16);
+    auto reduce = [&](auto kernel, auto *part, auto *S) {
+        kernel<<<g, th, 0, p->st>>>(p->nnzb, p->pptr, p->plist, part, S);
+    };
     if (p->fp32)
-        k_rcs_reduce<float><<<g, 256, 0, p->st>>>(p->nnzb, p->pptr, p->plist, (const float *)p->part, (float *)p->S);
+        reduce(small ? k_rcs_reduce<float, 8> : k_rcs_reduce<float, 4>, (const float *)p->part, (float *)p->S);
     else
-        k_rcs_reduce<double><<<g, 256, 0, p->st>>>(p->nnzb, p->pptr, p->plist, (const double *)p->part,
-                                                   (double *)p->S);
+        reduce(small ? k_rcs_reduce<double, 8> : k_rcs_reduce<double, 4>, (const double *)p->part, (double *)p->S);
     ktimer_end(p, K_RCS_REDUCE, ev);
     p->launches += 1;
     if ((err = cudaGetLastError()) != cudaSuccess) return err;

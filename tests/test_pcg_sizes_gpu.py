@@ -107,3 +107,49 @@ def test_static_pcg_over_launch_shapes(n, half, shift):
         x = flat[2][shift:shift + b.size].cpu().numpy().astype(np.float64).reshape(n, 6)
         r = b - product(row_ptr, col, val.astype(np.float64), x)
         assert np.linalg.norm(r) <= (1e-5 + 100 * np.finfo(np.float32).eps) * np.linalg.norm(b)
+
+
+@pytest.mark.parametrize("n,half", [(1, 1), (2, 1), (24, 23), (128, 60), (160, 63), (160, 75), (1500, 20),
+                                    (2600, 40), (2600, 62)])
+def test_fp32_split_cg_over_launch_shapes(n, half):
+    """FP32: one cluster (up to 14,336 off-diagonal entries) and a CTA per SM;
+    passes held in shared memory and passes copied again each iteration.  The
+    refinement stops at a true residual of 1e-6 ||b||; the step is returned
+    in FP32, which adds at most 2^-24 ||S|| ||x|| <= 2^-24 cond(S) ||b||,
+    cond(S) < 150 (see above)."""
+    from paper_2307_08383_gb300.build import build
+    build()
+    import paper_2307_08383_gb300 as B
+    row_ptr, col, val, b = system(n, half, 9300 + n)
+    val, b = val.astype(np.float32).astype(np.float64), b.astype(np.float32).astype(np.float64)
+    g = B.Problem.from_rcs(row_ptr, col, val, b, precision=B.BA_FP32, pcg_rel_tol=1e-6)
+    for _ in range(2):
+        info, conv = g.solve_rcs()
+        assert conv and 1 <= info["pcg_iters"] < 200
+        x = g.step()[0].reshape(n, 6)
+        assert np.linalg.norm(b - product(row_ptr, col, val, x)) <= (1e-6 + 150 * 2.0 ** -24) * np.linalg.norm(b)
+    g.close()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+@pytest.mark.parametrize("cams,pts", [(8, 60), (16, 2500), (40, 6000)])
+def test_group_sizes_from_the_problem(prec, cams, pts):
+    """Point groups sized by the problem against the largest ones: the same
+    system, its sums in another order (64 cameras' worth of terms a block at
+    most 2^13 eps of the block's norm)."""
+    from paper_2307_08383_gb300.build import build
+    build()
+    import paper_2307_08383_gb300 as B
+    s = scenes.ring_scene(n_cams=cams, n_pts=pts, seed=9400 + cams)
+    out = []
+    for kw in ({}, {"group_max_obs": 512}):
+        g = B.Problem(s.cams0, s.pts0, s.obs_cam, s.obs_pt, s.obs_uv,
+                      precision=B.BA_FP64 if prec == "fp64" else B.BA_FP32, **kw)
+        g.linearize()
+        g.form_rcs(1e-4)
+        out.append((g.stats()["n_groups"], *g.rcs()))
+        g.close()
+    assert out[0][0] >= out[1][0]
+    eps = np.finfo(np.float64 if prec == "fp64" else np.float32).eps
+    for a, c in zip(out[0][3:], out[1][3:]):
+        assert np.abs(np.asarray(a) - np.asarray(c)).max() <= 2 ** 13 * eps * np.abs(np.asarray(c)).max()
