@@ -454,6 +454,7 @@ ba_status ba_problem_create(const ba_options *opt, int32_t n_cams, const double 
     std::vector<int32_t>().swap(hs.tw_ptr);
     std::vector<int2>().swap(hs.tw_ent);
     default_view(p);
+    if (e == cudaSuccess) prepare_pcg(p);
     if (e == cudaSuccess) e = launch_prepare_state(p, p->cur);
     if (e == cudaSuccess) e = cudaStreamSynchronize(p->st);
     if (e != cudaSuccess) {
@@ -541,6 +542,7 @@ ba_status ba_problem_create_rcs(const ba_options *opt, int32_t n, int64_t nnzb, 
     up_ok(cudaMemsetAsync(p->counters, 0, N_COUNTERS * 4, p->st));
     std::vector<int2>().swap(p->hs.tw_ent);
     std::vector<int32_t>().swap(p->hs.tw_ptr);
+    if (e == cudaSuccess) prepare_pcg(p);
     if (e == cudaSuccess) e = launch_block_jacobi(p);
     if (e == cudaSuccess) e = cudaStreamSynchronize(p->st);
     if (e != cudaSuccess) {

@@ -224,6 +224,8 @@ struct ba_problem {
     double ph_imbalance = 0.0;  // last split solve: busiest CTA's work / mean CTA's
     bool minv_learned = false;  // Minv holds the learned M^-1 (else block-Jacobi)
     float2 *xs = nullptr;  // x64 split in FP32 pairs (refinement residual of FP32 problems)
+    unsigned char *mail = nullptr;  // mailboxes of the register-resident FP64 PCG
+    unsigned mail_epoch = 0;        // its launches
     unsigned *ar_bar = nullptr;  // arrival counters of the split CG's all-reduce (one per line)
     // > 0: the next PCG launch (split or standard recurrence) starts its
     // all-reduce counters one arrival short and waits at most this many SM
@@ -258,6 +260,7 @@ cudaError_t launch_cost(ba_problem *p, StateBuf &s, bool trial);
 cudaError_t launch_form_rcs(ba_problem *p, double lambda);
 cudaError_t launch_pcg_init(ba_problem *p, const void *rhs_T, double tol, int max_iters);
 cudaError_t launch_pcg_loop(ba_problem *p);
+void prepare_pcg(ba_problem *p);
 cudaError_t launch_pcg_implicit(ba_problem *p);  // the loop on the implicit operator (k_formats.cu)
 cudaError_t launch_resid64(ba_problem *p, bool from_x64, bool split = false);
 cudaError_t launch_solution_to_step(ba_problem *p);

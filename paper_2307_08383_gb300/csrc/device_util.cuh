@@ -477,6 +477,114 @@ __device__ __forceinline__ bool grid_exchange(double (&v)[NV], double *part, uns
     return ok;
 }
 
+// A 16-byte slot of payload and tag, moved by one 128-bit access: a reader
+// that sees the tag has the payload, with no flag to wait for and no second
+// round trip.  (Relaxed: acquiring polls would not overlap one another.)
+__device__ __forceinline__ void st_slot(void *p, unsigned long long a, unsigned long long b) {
+    asm volatile("{\n\t.reg .b128 t;\n\tmov.b128 t, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], t;\n\t}" ::"l"(p), "l"(a),
+                 "l"(b)
+                 : "memory");
+}
+__device__ __forceinline__ void ld_slot(const void *p, unsigned long long &a, unsigned long long &b) {
+    asm volatile("{\n\t.reg .b128 t;\n\tld.relaxed.gpu.global.b128 t, [%2];\n\tmov.b128 {%0, %1}, t;\n\t}"
+                 : "=l"(a), "=l"(b)
+                 : "l"(p)
+                 : "memory");
+}
+// Whether a bounded poll gives up: its cycles are used up, or (looked at every
+// 64th time) another wait of the launch has timed out.
+__device__ __forceinline__ bool poll_over(long long t0, long long limit_cycles, unsigned n, int *err) {
+    return clock64() - t0 > limit_cycles || ((n & 63u) == 63u && *(volatile int *)err == (int)BA_ERR_TIMEOUT);
+}
+
+// The exchange of a grid all-reduce by mailboxes, run by one warp per CTA of a
+// cooperative launch; the totals alone cross, nothing else is ordered.  Post:
+// every lane stores the CTA's partials (v, the same in all lanes) with the
+// call's tag into the mailboxes of CTAs lane, lane + 32, ...  Wait: every lane
+// polls the CTA's own mailbox for the partials of the same CTAs (bounded) and
+// the warp adds them.  Totals in every lane, the same bits in every CTA; false
+// on timeout (the error word is set).  `mail` holds mail_bytes(gridDim.x)
+// bytes; `epoch` numbers the launches that use it from 1 on, `gen` the launch's
+// calls (two sets in turn: a set is written again only two calls later, by a
+// CTA that has every CTA's partials of call gen + 1, sent after reading call
+// gen).  miss: 0 (set, the tag waited for is one that nobody posts).
+// Against grid_exchange: a store and a poll instead of a store, its
+// acknowledged release, an atomic, a poll and a read.  One slot per CTA that
+// all the others poll was slower than either at 100 CTAs and more (its few
+// lines are read by every SM while they are written).
+__host__ __device__ constexpr size_t mail_bytes(int grid) { return (size_t)2 * 2 * 16 * grid * grid; }
+struct Mail {
+    unsigned char *box;
+    unsigned epoch, miss;
+};
+template <int NV>
+__device__ __forceinline__ void mail_post(const double (&v)[NV], const Mail &m, unsigned gen) {
+    const unsigned G = gridDim.x;
+    const unsigned long long tag = ((unsigned long long)m.epoch << 32) | gen;
+    unsigned char *o = m.box + ((size_t)(gen & 1u) * G * 2 * G + blockIdx.x) * 16;
+    for (unsigned b = threadIdx.x & 31; b < G; b += 32) {
+#pragma unroll
+        for (int k = 0; k < NV; ++k)
+            st_slot(o + ((size_t)b * 2 + k) * G * 16, (unsigned long long)__double_as_longlong(v[k]), tag);
+    }
+}
+template <int NV>
+__device__ __forceinline__ bool mail_wait(double (&v)[NV], const Mail &m, unsigned gen, int *err,
+                                          long long limit_cycles) {
+    const unsigned G = gridDim.x, lane = threadIdx.x & 31;
+    const unsigned long long tag = ((unsigned long long)(m.epoch + m.miss) << 32) | gen;
+    const unsigned char *in = m.box + ((size_t)(gen & 1u) * G + blockIdx.x) * 2 * G * 16;
+    double acc[NV];
+#pragma unroll
+    for (int k = 0; k < NV; ++k) acc[k] = 0.0;
+    bool ok = true;
+    const long long t0 = clock64();
+    for (unsigned b0 = 0; b0 < G && ok; b0 += 160) {
+        unsigned long long u[NV][5], t[NV][5];
+#pragma unroll
+        for (int k = 0; k < NV; ++k)
+#pragma unroll
+            for (int q = 0; q < 5; ++q) {
+                u[k][q] = 0ull;
+                t[k][q] = tag;
+            }
+        for (unsigned n = 0;; ++n) {
+#pragma unroll
+            for (int k = 0; k < NV; ++k)
+#pragma unroll
+                for (int q = 0; q < 5; ++q) {
+                    const unsigned b = b0 + lane + 32 * q;
+                    if (b < G) ld_slot(in + ((size_t)k * G + b) * 16, u[k][q], t[k][q]);
+                }
+            bool all = true;
+#pragma unroll
+            for (int q = 0; q < 5; ++q) all = all && t[0][q] == tag && t[NV - 1][q] == tag;
+            if (all) break;
+            if (poll_over(t0, limit_cycles, n, err)) {
+                ok = false;
+                break;
+            }
+        }
+        __syncwarp();
+        ok = __all_sync(0xffffffffu, ok) != 0;
+        // (64 cycles an add: none for the stretches that the grid does not reach)
+#pragma unroll
+        for (int q = 0; q < 5; ++q)
+            if (b0 + 32 * q < G) {
+#pragma unroll
+                for (int k = 0; k < NV; ++k) {
+                    const double x = __longlong_as_double((long long)u[k][q]);
+                    acc[k] = b0 + q == 0 ? x : acc[k] + x;
+                }
+            }
+    }
+    if (!ok && lane == 0) atomicExch(err, (int)BA_ERR_TIMEOUT);
+    const double tot = warp_fold<NV>(acc);
+    v[0] = __shfl_sync(0xffffffffu, tot, 0);
+    if (NV == 2) v[NV - 1] = __shfl_sync(0xffffffffu, tot, 16);
+    return ok;
+}
+
 // grid_allreduce_sym for kernels of few warps per CTA: v holds the own
 // partials of every thread of the first nwv warps (at most 16 warps per CTA),
 // and warp 0 alone runs the exchange, so that a call costs one warp-wide fold

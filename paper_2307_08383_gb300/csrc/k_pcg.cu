@@ -389,26 +389,31 @@ __global__ void __launch_bounds__(256) k_pcg_persist(int n, const int *__restric
 // CTA c owns rows c R .. c R + R - 1 (R <= RES64_ROWS), `wpr` warps to a row, one
 // two-sided entry to a lane (already transposed where the entry asks for it,
 // so that no warp runs both forms of the product); lane 6 lr + a of warp 0
-// keeps y, r, d and a row of M^-1 of entry (lr, a) for the whole solve.  Only
-// z and d pass through memory (the neighbours' gather), and warp 0 alone runs
-// the two exchanges of an iteration; the gathers are issued as soon as the
-// second has seen every CTA arrive.
+// keeps y, r, d and a row of M^-1 of entry (lr, a) for the whole solve, every
+// lane the direction of its own column.  Only z passes through memory, in
+// slots of value and tag (the iteration), which the neighbours' gather polls
+// without waiting for the grid; warp 0 alone runs the two exchanges of an
+// iteration, which carry their totals and order nothing else (no release).
+// A z slot is written again only after the next iteration's first exchange,
+// which every CTA enters with its gather done.
 // What bounds it: FP64 warp instructions of 64 cycles each for one warp (16
 // with all four of an SM's schedulers busy) - 50 per row half, about 60 in the
-// scalar chain - and two grid exchanges of about 1.2 us.  Against
-// k_pcg_persist (which re-reads S and passes r and q through L2 each
-// iteration): 14 -> 9.2 us per iteration at 200 cameras, 12 -> 7.1 at 50.
+// scalar chain - and the exchanges' round trips.  Against k_pcg_persist (which
+// re-reads S and passes r and q through L2 each iteration): 14 -> 8.5 us per
+// iteration at 200 cameras, 12 -> 5.9 at 50 (9.2 and 7.1 with exchanges by
+// arrival counters that also publish z and d).
 constexpr int RES64_ROWS = 5;   // 6 R owner lanes in one warp
 constexpr int RES64_WARPS = 8;  // warps per CTA at most
 __global__ void __launch_bounds__(32 * RES64_WARPS, 1)
     k_pcg64_res(int n, int rows, int wpr, const int *__restrict__ tw_ptr, const int2 *__restrict__ tw_ent,
                 const double *__restrict__ S, const double *__restrict__ Minv, double *__restrict__ y,
-                const double *__restrict__ r0, double *z, double *d0, double *d1, DevScalars *sc, double *red,
-                unsigned *bar, long long limit_cycles) {
+                const double *__restrict__ r0, const double *__restrict__ z0, double *za, double *zb, DevScalars *sc,
+                Mail mail, long long limit_cycles) {
     __shared__ double s_part[RES64_WARPS][6];
     __shared__ double s_beta;
-    __shared__ int s_ctl;  // 0 go on, 1 leave
+    __shared__ int s_go, s_ctl, s_bad;  // nonzero: leave after the first exchange, after the second, after the gather
     if (sc->done) return;
+    if (threadIdx.x == 0) s_bad = 0;  // ordered by the first barrier
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int comp = fold6_comp(lane);
     const bool writes = fold6_owner(lane);
@@ -437,7 +442,7 @@ __global__ void __launch_bounds__(32 * RES64_WARPS, 1)
     double rv = 0.0, yv = 0.0, zv = 0.0, dv = 0.0, Mr[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
     if (own) {
         rv = r0[6 * oi + oc];
-        zv = __ldcg(z + 6 * oi + oc);
+        zv = z0[6 * oi + oc];
 #pragma unroll
         for (int c = 0; c < 6; ++c) Mr[c] = __ldg(Minv + 36 * (int64_t)oi + 6 * oc + c);
     }
@@ -445,98 +450,120 @@ __global__ void __launch_bounds__(32 * RES64_WARPS, 1)
     const double thr = sc->tol2 * sc->rr0;
     const int max_iters = sc->max_iters;
     unsigned gen = 0;
-    double zj[6], dj[6];
-    load6(z + 6 * j, zj);
-    load6(d0 + 6 * j, dj);
-    for (int it = 0;;) {
-        double *dnew = (it & 1) ? d0 : d1;
-        double x[6], acc[6];
+    // z's slots: entries 0..2 of a camera in za, 3..5 in zb (tags zero at launch)
+    unsigned char *const sa = reinterpret_cast<unsigned char *>(za), *const sb = reinterpret_cast<unsigned char *>(zb);
+    double zj[6], xj[6];  // of this lane's column: z, and the direction d
+    load6(z0 + 6 * j, zj);
 #pragma unroll
-        for (int c = 0; c < 6; ++c) x[c] = zj[c] + beta * dj[c];
+    for (int c = 0; c < 6; ++c) xj[c] = 0.0;
+    unsigned long long zu[6], zt[6];
+    auto fetch = [&]() {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            ld_slot(sa + 16 * (3 * j + c), zu[c], zt[c]);
+            ld_slot(sb + 16 * (3 * j + c), zu[3 + c], zt[3 + c]);
+        }
+    };
+    // the slots' values once all six carry the tag (bounded)
+    auto gather = [&](unsigned long long tag) {
+        const long long t0 = clock64();
+        for (unsigned t = 0;; ++t) {
+            bool all = true;
+#pragma unroll
+            for (int c = 0; c < 6; ++c) all = all && zt[c] == tag;
+            if (all) break;
+            if (poll_over(t0, limit_cycles, t, &sc->err)) {
+                s_bad = 1;
+                atomicExch(&sc->err, (int)BA_ERR_TIMEOUT);
+                break;
+            }
+            fetch();
+        }
+#pragma unroll
+        for (int c = 0; c < 6; ++c) zj[c] = __longlong_as_double((long long)zu[c]);
+    };
+    for (int it = 0;;) {
+        double acc[6];
+#pragma unroll
+        for (int c = 0; c < 6; ++c) xj[c] = zj[c] + beta * xj[c];
 #pragma unroll
         for (int r = 0; r < 6; ++r) {
-            acc[r] = Sv[6 * r] * x[0];
+            acc[r] = Sv[6 * r] * xj[0];
 #pragma unroll
-            for (int c = 1; c < 6; ++c) acc[r] += Sv[6 * r + c] * x[c];
+            for (int c = 1; c < 6; ++c) acc[r] += Sv[6 * r + c] * xj[c];
         }
         const double pr = warp_fold6(acc, lane);
         if (writes) s_part[w][comp] = pr;
         __syncthreads();
         if (w == 0) {
-            double q = 0.0, v1[1] = {0.0};
+            double q = 0.0, v1[1] = {0.0}, v2[2] = {0.0, 0.0};
             if (own) {
                 q = s_part[ol * wpr][oc];
                 for (int p = 1; p < wpr; ++p) q += s_part[ol * wpr + p][oc];
                 dv = zv + beta * dv;
-                dnew[6 * oi + oc] = dv;
                 v1[0] = dv * q;
             }
             v1[0] = warp_fold<1>(v1);
-            bool ok = grid_exchange<1>(v1, red, gen++, bar, &sc->err, limit_cycles, []() {});
+            mail_post<1>(v1, mail, gen);
+            const double inv_rz = 1.0 / rz;  // for beta, while the partials travel
+            const bool ok = mail_wait<1>(v1, mail, gen, &sc->err, limit_cycles);
+            ++gen;
             const double pAp = v1[0];
-            int ctl = 0;
-            if (!ok || !(pAp > 0.0)) {
-                ctl = 1;
-                if (ok && blockIdx.x == 0 && lane == 0) {
-                    sc->err = (int)BA_ERR_NOT_SPD;
-                    sc->done = 1;
-                    sc->iters = it;
-                }
-            }
-            if (ctl == 0) {
+            const bool go = ok && pAp > 0.0;
+            if (go) {
                 const double alpha = rz / pAp;
                 rv -= alpha * q;
-                yv += alpha * dv;
                 double zn = 0.0;
                 const int l6 = lane < 30 ? 6 * ol : 0;
 #pragma unroll
                 for (int c = 0; c < 6; ++c) zn += Mr[c] * __shfl_sync(0xffffffffu, rv, l6 + c);
                 zv = zn;
-                if (own) z[6 * oi + oc] = zv;
-                double v2[2] = {rv * zv, rv * rv};
+                if (own)
+                    st_slot((oc < 3 ? sa : sb - 48) + 16 * (3 * oi + oc), __double_as_longlong(zv),
+                            (unsigned long long)(it + 1));
+                v2[0] = rv * zv;
+                v2[1] = rv * rv;
                 const double f = warp_fold<2>(v2);
-                v2[0] = f;
+                v2[0] = __shfl_sync(0xffffffffu, f, 0);
                 v2[1] = __shfl_sync(0xffffffffu, f, 16);
-                if (lane == 0) s_ctl = 0;
-                ok = grid_exchange<2>(v2, red, gen++, bar, &sc->err, limit_cycles, [&]() {
-                    __syncthreads();  // the other warps' gathers start here
-                    load6(z + 6 * j, zj);
-                    load6(dnew + 6 * j, dj);
-                });
-                ++it;
-                if (!ok) {
-                    ctl = 2;  // the others still wait at the first barrier
-                } else if (v2[1] <= thr || it >= max_iters) {
-                    ctl = 1;
-                    if (blockIdx.x == 0 && lane == 0) {
-                        sc->iters = it;
-                        sc->rr = v2[1];
-                        sc->rz = v2[0];
-                        sc->done = 1;
-                    }
-                } else {
-                    beta = v2[0] / rz;
-                    rz = v2[0];
-                }
-                if (lane == 0) {
-                    s_ctl = ctl;
-                    s_beta = beta;
-                }
-                if (ctl == 2) __syncthreads();
-                __syncthreads();
-                if (ctl) break;
-                continue;
+                mail_post<2>(v2, mail, gen);
+                yv += alpha * dv;
+            } else if (ok && blockIdx.x == 0 && lane == 0) {
+                sc->err = (int)BA_ERR_NOT_SPD;
+                sc->done = 1;
+                sc->iters = it;
             }
-            if (lane == 0) s_ctl = 1;
+            if (lane == 0) s_go = go ? 0 : 1;
+            __syncthreads();  // the other warps' gathers start here
+            if (!go) break;
+            fetch();
+            const bool ok2 = mail_wait<2>(v2, mail, gen, &sc->err, limit_cycles);
+            ++gen;
+            int ctl = ok2 ? 0 : 1;
+            if (ok2 && (v2[1] <= thr || it + 1 >= max_iters)) {
+                ctl = 1;
+                if (blockIdx.x == 0 && lane == 0) {
+                    sc->iters = it + 1;
+                    sc->rr = v2[1];
+                    sc->rz = v2[0];
+                    sc->done = 1;
+                }
+            }
+            beta = v2[0] * inv_rz;
+            rz = v2[0];
+            if (lane == 0) {
+                s_ctl = ctl;
+                s_beta = beta;
+            }
+            gather((unsigned long long)(it + 1));
+        } else {
             __syncthreads();
-            __syncthreads();
-            break;
+            if (s_go) break;
+            fetch();
+            gather((unsigned long long)(it + 1));
         }
         __syncthreads();
-        load6(z + 6 * j, zj);
-        load6(dnew + 6 * j, dj);
-        __syncthreads();
-        if (s_ctl) break;
+        if (s_ctl | s_bad) break;
         beta = s_beta;
         ++it;
     }
@@ -1417,18 +1444,39 @@ static bool res64_fits(const ba_problem *p, int n_sm) {
     const int rows = (p->n + n_sm - 1) / n_sm;
     return p->hs.max_row_ent > 0 && rows <= RES64_ROWS && rows * res64_wpr(p) <= RES64_WARPS;
 }
-static cudaError_t launch_res64(ba_problem *p, int n_sm, long long limit) {
+static int res64_grid(const ba_problem *p, int n_sm) {
+    const int rows = (p->n + n_sm - 1) / n_sm;
+    return (p->n + rows - 1) / rows;
+}
+// Its mailboxes (1.5 MB for a CTA on every SM), made with the problem where
+// they fit under the cap; without them the loop is not used.
+void prepare_pcg(ba_problem *p) {
+    int dev = 0, n_sm = 0;
+    if (p->fp32 || cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || !res64_fits(p, n_sm))
+        return;
+    const size_t bytes = mail_bytes(res64_grid(p, n_sm));
+    if (p->opt.device_mem_cap && p->dev_bytes + bytes > p->opt.device_mem_cap) return;
+    void *v = nullptr;
+    if (cudaMalloc(&v, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
+    p->allocs.push_back(v);
+    p->dev_bytes += bytes;
+    if (cudaMemsetAsync(v, 0, bytes, p->st) == cudaSuccess) p->mail = (unsigned char *)v;
+}
+static cudaError_t launch_res64(ba_problem *p, int n_sm, unsigned miss, long long limit) {
     int n = p->n, rows = (n + n_sm - 1) / n_sm, wpr = res64_wpr(p);
-    const int grid = (n + rows - 1) / rows;
+    const int grid = res64_grid(p, n_sm);
     const int *twp = p->tw_ptr;
     const int2 *twe = p->tw_ent;
     const double *S = (const double *)p->sv.S, *Mi = (const double *)p->sv.Minv, *r = (const double *)p->sv.pv[1];
-    double *y = (double *)p->sv.pv[0], *z = (double *)p->sv.pv[2], *d0 = (double *)p->sv.pv[3],
-           *d1 = (double *)p->sv.pv[4];
+    const double *z = (const double *)p->sv.pv[2];
+    double *y = (double *)p->sv.pv[0], *za = (double *)p->sv.pv[5], *zb = (double *)p->sv.pv[7];
     DevScalars *sc = p->sc;
-    double *red = p->red;
-    unsigned *bar = p->ar_bar;
-    void *args[] = {&n, &rows, &wpr, &twp, &twe, &S, &Mi, &y, &r, &z, &d0, &d1, &sc, &red, &bar, &limit};
+    Mail mail{p->mail, ++p->mail_epoch, miss};
+    void *args[] = {&n, &rows, &wpr, &twp, &twe, &S, &Mi, &y, &r, &z, &za, &zb, &sc, &mail, &limit};
     return cudaLaunchCooperativeKernel((const void *)k_pcg64_res, dim3(grid), dim3(32 * rows * wpr), args, 0, p->st);
 }
 
@@ -1451,12 +1499,12 @@ static cudaError_t pcg_loop_T(ba_problem *p) {
     // armed test of the timeout path: every counter starts at -1, one arrival short
     const long long test_limit = p->test_wait_limit;
     p->test_wait_limit = 0;
+    const long long limit_cycles = test_limit > 0 ? test_limit : 4000000000LL;  // ~2 s of SM clock per wait
+    if (sizeof(T) == 8 && p->mail && res64_fits(p, n_sm)) return launch_res64(p, n_sm, test_limit > 0 ? 1u : 0u, limit_cycles);
     if ((e = ensure_ar_bar(p)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(p->ar_bar, test_limit > 0 ? 0xFF : 0, AR_SUB * 32 * sizeof(unsigned), p->st)) !=
         cudaSuccess)
         return e;
-    const long long limit_cycles = test_limit > 0 ? test_limit : 4000000000LL;  // ~2 s of SM clock per wait
-    if (sizeof(T) == 8 && res64_fits(p, n_sm)) return launch_res64(p, n_sm, limit_cycles);
     int n = p->n;
     const int *twp = p->tw_ptr, *rp = p->row_ptr, *cl = p->col;
     const int2 *twe = p->tw_ent;

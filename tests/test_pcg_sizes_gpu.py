@@ -109,6 +109,22 @@ def test_static_pcg_over_launch_shapes(n, half, shift):
         assert np.linalg.norm(r) <= (1e-5 + 100 * np.finfo(np.float32).eps) * np.linalg.norm(b)
 
 
+@pytest.mark.parametrize("n,half", [(3, 2), (152, 9), (200, 199)])
+def test_fp64_pcg_without_mailboxes(n, half):
+    """A cap on device memory that the mailboxes would exceed: the loop that
+    exchanges by counters solves the same systems."""
+    from paper_2307_08383_gb300.build import build
+    build()
+    import paper_2307_08383_gb300 as B
+    row_ptr, col, val, b = system(n, half, 9100 + n)
+    ref, its = pcg(row_ptr, col, val, b, 1e-10)
+    g = B.Problem.from_rcs(row_ptr, col, val, b, precision=B.BA_FP64, pcg_rel_tol=1e-10, device_mem_cap=1)
+    info, conv = g.solve_rcs()
+    assert conv and abs(info["pcg_iters"] - its) <= 1
+    assert np.linalg.norm(g.step()[0].reshape(n, 6) - ref) <= 1e-8 * np.linalg.norm(ref)
+    g.close()
+
+
 @pytest.mark.parametrize("n,half", [(1, 1), (2, 1), (24, 23), (128, 60), (160, 63), (160, 75), (1500, 20),
                                     (2600, 40), (2600, 62)])
 def test_fp32_split_cg_over_launch_shapes(n, half):
