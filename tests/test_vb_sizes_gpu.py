@@ -95,3 +95,39 @@ def test_vb_system_over_sizes(n, half, kind, fp32):
         B.VBSMC(cdim, row_ptr, col, bad, b, precision=B.BA_FP32 if fp32 else B.BA_FP64)
     assert ei.value.status == B.BA_ERR_NOT_SPD
     g.close()
+
+
+@pytest.mark.parametrize("capped", [False, True])
+def test_interiors_state_round_trip(capped):
+    """The state set and read back bit for bit, unchanged by a refused one, and
+    the LM step from it the same, with the points' order kept on the device or
+    (under a cap that leaves no room for it) sent with each call."""
+    from paper_2307_08383_gb300.build import build
+    build()
+    import paper_2307_08383_gb300 as B
+    s = scenes.shuffled(scenes.aerial_small(n_along=5, n_across=4, pts_per_cam=30, seed=9500), 3)
+    intr = scenes.interiors0(s.n_cams, seed=9501)
+    args = (s.cams0, intr, np.full(s.n_cams, 11, np.int32), s.pts0, s.obs_cam, s.obs_pt, s.obs_uv)
+    ref = B.VBIProblem(*args, precision=B.BA_FP64)
+    g = B.VBIProblem(*args, precision=B.BA_FP64, device_mem_cap=ref.info()["device_bytes"] - 1 if capped else 0)
+    want = ref.lm_step()
+    rng = np.random.default_rng(9502)
+    cams, ins, pts = (a + 1e-3 * rng.standard_normal(a.shape) for a in (s.cams0, intr, s.pts0))
+    g.set_state(cams, ins, pts, 1e-3, 2.0)
+    for a, b in zip(g.state(), (cams, ins, pts)):
+        assert np.array_equal(a.reshape(b.shape), b)
+    for k, v in ((0, np.nan), (pts.size - 1, np.inf)):
+        bad = pts.copy()
+        bad.flat[k] = v
+        with pytest.raises(B.BAError):
+            g.set_state(s.cams0, intr, bad, 1e-3, 2.0)
+        for a, b in zip(g.state(), (cams, ins, pts)):
+            assert np.array_equal(a.reshape(b.shape), b)
+    g.set_state(s.cams0, intr, s.pts0, 1e-4, 2.0)
+    info = g.lm_step()
+    assert (info["cost_before"], info["accepted"]) == (want["cost_before"], want["accepted"])
+    assert abs(info["cost_after"] - want["cost_after"]) <= 1e-12 * want["cost_after"]
+    for a, b in zip(g.step(), ref.step()):
+        assert np.linalg.norm(a - b) <= 1e-9 * np.linalg.norm(b)
+    ref.close()
+    g.close()
