@@ -285,17 +285,18 @@ ba_status ba_problem_create(const ba_options *opt, int32_t n_cams, const double 
     const int64_t n = n_cams, P = n_pts, m = n_obs;
     const size_t E = p->esz;
     HostSetup &hs = p->hs;
-    // Point groups of equal size for whole rounds of the formation's CTAs (two
-    // to an SM in FP32, one in FP64), at most the default size.  50 cameras,
-    // FP64: 22 groups of 512 keep 22 SMs busy, formation 110 us and the step's
-    // point pass 26; 49 and 18 with 141 groups.  200 cameras, FP64: 374 -> 321
-    // us.  FP32 beyond one round keeps the default (200 cameras 22.6 / 21 us
-    // alone, no difference in the step; 1,770 cameras 114 both ways).  The few
-    // observations on top allow for whole tracks.
+    // FP64: point groups of equal size for whole rounds of the formation's CTAs
+    // (one to an SM), at most the default size.  50 cameras: 22 groups of 512
+    // keep 22 SMs busy, formation 110 us and the step's point pass 26; 49 and 18
+    // with 141 groups.  200 cameras: 374 -> 321 us.  The few observations on top
+    // allow for whole tracks.  FP32 keeps the default: smaller groups leave more
+    // of each block's sum to the chain over partials (8 to 60 cameras: the median
+    // error of an LM step's cost grew by 1.7).
     int target = p->obs_max;
-    const int64_t slots = p->fp32 ? 304 : 152, rounds = (m + slots * p->obs_max - 1) / (slots * p->obs_max);
-    if (o.group_max_obs <= 0 && (!p->fp32 || rounds == 1))
+    if (o.group_max_obs <= 0 && !p->fp32) {
+        const int64_t slots = 152, rounds = (m + slots * p->obs_max - 1) / (slots * p->obs_max);
         target = (int)std::min<int64_t>(p->obs_max, std::max<int64_t>(40, (m + slots * rounds - 1) / (slots * rounds) + 8));
+    }
     const size_t camc_w = p->fp32 ? CAMC32_W * 4 : 12 * 8;
     size_t plan = 0;
     for (;;) {

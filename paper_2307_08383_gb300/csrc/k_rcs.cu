@@ -384,7 +384,8 @@ __global__ void __launch_bounds__(FORM_THREADS) k_form_rcs(const GroupDesc *__re
 // per 16-byte chunk of the block (9 for FP32, 18 for FP64): the chunks of a
 // partial are read by consecutive threads, and each thread keeps DEPTH
 // partials' loads in flight before adding them in order; with 8 also the next
-// ones' indices.  DEPTH 8 for small systems (few warps, long lists: a chain of
+// ones' indices, and the eight are added in pairs first (a chain an eighth as
+// long).  DEPTH 8 for small systems (few warps, long lists: a chain of
 // round trips; 50 cameras FP64 43 -> 29 us, 200 cameras FP32 19 -> 12), 4 for
 // large ones (bandwidth: 1,770 cameras FP32 27 us, 31 with 8).  (Writing each
 // partial straight to a block-ordered slot in RCS formation made this
@@ -430,15 +431,19 @@ __global__ void __launch_bounds__(256) k_rcs_reduce(int64_t nblk, const int *__r
             for (; q < q1; q += DEPTH) {
                 V v[DEPTH];
 #pragma unroll
-                for (int k = 0; k < DEPTH; ++k)
+                for (int k = 0; k < DEPTH; ++k) {
+                    std::memset(&v[k], 0, sizeof(V));
                     if (q + k < q1) v[k] = pv[(int64_t)id[k] * NCH + c];
+                }
                 if (q + DEPTH < q1) {
 #pragma unroll
                     for (int k = 0; k < DEPTH; ++k) id[k] = __ldg(plist + min(q + DEPTH + k, q1 - 1));
                 }
 #pragma unroll
-                for (int k = 0; k < DEPTH; ++k)
-                    if (q + k < q1) add16(s, v[k]);
+                for (int h = DEPTH / 2; h > 0; h /= 2)
+#pragma unroll
+                    for (int k = 0; k < h; ++k) add16(v[k], v[k + h]);
+                add16(s, v[0]);
             }
         }
         sv[x] = s;
