@@ -252,14 +252,11 @@ ba_status ktimer_flush(ba_problem *p);
 // launchers (kernels in the .cu files); each returns cudaGetLastError()
 cudaError_t launch_prepare_state(ba_problem *p, StateBuf &s);
 // caller-order point I/O through a device staging buffer (d_perm, stage_pts)
-// points between the caller's order and the internal one, and the check of a
-// caller's values, on any stream (bad: set to 1 by a value that is not finite)
-cudaError_t run_count_nonfinite(cudaStream_t st, const double *a, int64_t cnt, unsigned *bad);
-cudaError_t run_gather_pts(cudaStream_t st, int64_t P, const int32_t *perm, const double *user, double *internal);
-cudaError_t run_scatter_pts(cudaStream_t st, int64_t P, const int32_t *perm, const double *internal, double *user);
 cudaError_t launch_count_nonfinite(ba_problem *p, const double *a, int64_t cnt, unsigned *bad);
 cudaError_t launch_gather_pts(ba_problem *p, const double *user, double *internal);
 cudaError_t launch_scatter_pts(ba_problem *p, const void *internal, bool internal_fp32, double *user);
+// the check alone, on any stream: sets bad if a value is not finite
+cudaError_t run_count_nonfinite(cudaStream_t st, const double *a, int64_t cnt, unsigned *bad);
 cudaError_t launch_linearize(ba_problem *p);
 cudaError_t launch_cost(ba_problem *p, StateBuf &s, bool trial);
 cudaError_t launch_form_rcs(ba_problem *p, double lambda);

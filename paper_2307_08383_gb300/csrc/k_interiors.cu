@@ -1029,7 +1029,6 @@ struct ba_vbi_problem {
     double *cams = nullptr, *intr = nullptr, *pts = nullptr, *cams_t = nullptr, *intr_t = nullptr, *pts_t = nullptr;
     double *dxp = nullptr, *red = nullptr, *camc_t = nullptr;
     unsigned *ctr = nullptr;
-    int32_t *perm = nullptr;  // internal -> the caller's point
     VbiScalars *sc = nullptr, *sc_host = nullptr;
     std::vector<void *> allocs;
     cudaEvent_t ev[6] = {};
@@ -1065,28 +1064,6 @@ ba_status vbi_put(ba_vbi_problem *p, void **dptr, const void *src, size_t bytes)
     ba_status s = vbi_alloc(p, dptr, bytes);
     if (s) return s;
     return vbi_fail(p, cudaMemcpy(*dptr, src, bytes, cudaMemcpyHostToDevice), "upload");
-}
-
-// The point permutation on the device; without a place of its own it is copied
-// to the P, e^ rows, which every formation writes before it reads them.
-cudaError_t vbi_perm(ba_vbi_problem *p, const int32_t **perm) {
-    *perm = p->perm ? p->perm : (const int32_t *)p->d.PE;
-    if (p->perm) return cudaSuccess;
-    const std::vector<int32_t> t(p->hs.pt_perm.begin(), p->hs.pt_perm.end());
-    return cudaMemcpyAsync(p->d.PE, t.data(), t.size() * sizeof(int32_t), cudaMemcpyHostToDevice, p->h->st);
-}
-
-// Device points (internal order) to the caller's array, in their order by way
-// of the trial points' array (no step is in flight between calls).
-ba_status vbi_get_points(ba_vbi_problem *p, const double *src, double *dst) {
-    cudaStream_t st = p->h->st;
-    const int32_t *perm = nullptr;
-    ba_status s;
-    if ((s = vbi_fail(p, vbi_perm(p, &perm), "copy"))) return s;
-    if ((s = vbi_fail(p, run_scatter_pts(st, p->P, perm, src, p->pts_t), "k_scatter_pts"))) return s;
-    if ((s = vbi_fail(p, cudaMemcpyAsync(dst, p->pts_t, (size_t)p->P * 24, cudaMemcpyDeviceToHost, st), "copy")))
-        return s;
-    return vbi_fail(p, cudaStreamSynchronize(st), "sync");
 }
 
 void vbi_free(ba_vbi_problem *p) {
@@ -1239,10 +1216,6 @@ ba_status ba_vbi_problem_create(const ba_options *opt, int32_t n_cams, const dou
     if (!s) s = vbi_alloc(p, (void **)&p->red, (size_t)RED_SLOTS * sizeof(double));
     if (!s) s = vbi_alloc(p, (void **)&p->ctr, 64);
     if (!s) s = vbi_alloc(p, (void **)&p->sc, sizeof(VbiScalars));
-    // (not under a cap that it would exceed: vbi_perm)
-    const size_t PB = (size_t)n_pts * sizeof(int32_t);
-    if (!s && (!o.device_mem_cap || (size_t)p->dev_bytes + p->h->dev_bytes + std::max<size_t>(PB, 16) <= o.device_mem_cap))
-        s = vbi_put(p, (void **)&p->perm, std::vector<int32_t>(hs.pt_perm.begin(), hs.pt_perm.end()).data(), PB);
     if (!s) s = vbi_fail(p, cudaMemset(p->ctr, 0, 64), "memset");
     if (!s) s = vbi_fail(p, cudaMallocHost((void **)&p->sc_host, sizeof(VbiScalars)), "cudaMallocHost");
     for (auto &e : p->ev)
@@ -1358,7 +1331,9 @@ ba_status ba_vbi_get_state(const ba_vbi_problem *p, double *cams, double *intr, 
         return s;
     if (intr && (s = vbi_fail(q, cudaMemcpy(intr, p->intr, (size_t)p->n * 40, cudaMemcpyDeviceToHost), "copy")))
         return s;
-    if (pts && (s = vbi_get_points(q, p->pts, pts))) return s;
+    // (the points keep the caller's order: pattern-only setup)
+    if (pts && (s = vbi_fail(q, cudaMemcpy(pts, p->pts, (size_t)p->P * 24, cudaMemcpyDeviceToHost), "copy")))
+        return s;
     return BA_OK;
 }
 
@@ -1371,22 +1346,20 @@ ba_status ba_vbi_set_state(ba_vbi_problem *p, const double *cams, const double *
         return set_error(BA_ERR_INVALID_ARG, "lambda and nu must be finite and > 0");
     if (!finite_n(cams, (int64_t)p->n * 6) || !finite_n(intr, (int64_t)p->n * 5))
         return set_error(BA_ERR_NONFINITE, "non-finite state value");
-    // the points go to the trial points' array in the caller's order and are
-    // checked and permuted on the device (on the host this call and
-    // ba_vbi_get_state were 0.6 ms longer at 99,000 points); the state changes
-    // only when every value is finite
+    // the points go to the trial points' array and are checked there; the
+    // arrays change places only when every value is finite (checked and copied
+    // by way of a host vector, this call and ba_vbi_get_state took 0.6 ms more
+    // at 99,000 points)
     cudaStream_t st = p->h->st;
     ba_status s;
     unsigned bad = 0, *flag = p->ctr + 15;
-    const int32_t *perm = nullptr;
     if ((s = vbi_fail(p, cudaMemcpyAsync(p->pts_t, pts, (size_t)p->P * 24, cudaMemcpyHostToDevice, st), "copy"))) return s;
     if ((s = vbi_fail(p, cudaMemsetAsync(flag, 0, sizeof(unsigned), st), "memset"))) return s;
     if ((s = vbi_fail(p, run_count_nonfinite(st, p->pts_t, p->P * 3, flag), "k_count_nonfinite"))) return s;
     if ((s = vbi_fail(p, cudaMemcpyAsync(&bad, flag, sizeof(unsigned), cudaMemcpyDeviceToHost, st), "copy"))) return s;
     if ((s = vbi_fail(p, cudaStreamSynchronize(st), "sync"))) return s;
     if (bad) return set_error(BA_ERR_NONFINITE, "non-finite state value");
-    if ((s = vbi_fail(p, vbi_perm(p, &perm), "copy"))) return s;
-    if ((s = vbi_fail(p, run_gather_pts(st, p->P, perm, p->pts_t, p->pts), "k_gather_pts"))) return s;
+    std::swap(p->pts, p->pts_t);
     if ((s = vbi_fail(p, cudaMemcpyAsync(p->cams, cams, (size_t)p->n * 48, cudaMemcpyHostToDevice, st), "copy"))) return s;
     if ((s = vbi_fail(p, cudaMemcpyAsync(p->intr, intr, (size_t)p->n * 40, cudaMemcpyHostToDevice, st), "copy"))) return s;
     if ((s = vbi_fail(p, cudaStreamSynchronize(st), "sync"))) return s;
@@ -1436,7 +1409,7 @@ ba_status ba_vbi_get_step(const ba_vbi_problem *p, double *dxc, double *dxp) {
             dxc[k] = p->h->fp32 ? (double)reinterpret_cast<const float *>(raw.data())[k]
                                 : reinterpret_cast<const double *>(raw.data())[k];
     }
-    if (dxp && (s = vbi_get_points(q, p->dxp, dxp))) return s;
+    if (dxp && (s = vbi_fail(q, cudaMemcpy(dxp, p->dxp, (size_t)p->P * 24, cudaMemcpyDeviceToHost), "copy"))) return s;
     return BA_OK;
 }
 

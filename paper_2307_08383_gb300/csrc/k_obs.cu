@@ -888,27 +888,23 @@ cudaError_t run_count_nonfinite(cudaStream_t st, const double *a, int64_t cnt, u
     k_count_nonfinite<<<grid_for(cnt, 256, GRID_CAP), 256, 0, st>>>(cnt, a, bad);
     return cudaGetLastError();
 }
-cudaError_t run_gather_pts(cudaStream_t st, int64_t P, const int32_t *perm, const double *user, double *internal) {
-    k_gather_pts<<<grid_for(P, 256, GRID_CAP), 256, 0, st>>>(P, perm, user, internal);
-    return cudaGetLastError();
-}
-cudaError_t run_scatter_pts(cudaStream_t st, int64_t P, const int32_t *perm, const double *internal, double *user) {
-    k_scatter_pts<double><<<grid_for(P, 256, GRID_CAP), 256, 0, st>>>(P, perm, internal, user);
-    return cudaGetLastError();
-}
 cudaError_t launch_count_nonfinite(ba_problem *p, const double *a, int64_t cnt, unsigned *bad) {
     p->launches += 1;
     return run_count_nonfinite(p->st, a, cnt, bad);
 }
 cudaError_t launch_gather_pts(ba_problem *p, const double *user, double *internal) {
+    k_gather_pts<<<grid_for(p->P, 256, GRID_CAP), 256, 0, p->st>>>(p->P, p->d_perm, user, internal);
     p->launches += 1;
-    return run_gather_pts(p->st, p->P, p->d_perm, user, internal);
+    return cudaGetLastError();
 }
 cudaError_t launch_scatter_pts(ba_problem *p, const void *internal, bool internal_fp32, double *user) {
+    if (internal_fp32)
+        k_scatter_pts<float><<<grid_for(p->P, 256, GRID_CAP), 256, 0, p->st>>>(p->P, p->d_perm,
+                                                                              (const float *)internal, user);
+    else
+        k_scatter_pts<double><<<grid_for(p->P, 256, GRID_CAP), 256, 0, p->st>>>(p->P, p->d_perm,
+                                                                               (const double *)internal, user);
     p->launches += 1;
-    if (!internal_fp32) return run_scatter_pts(p->st, p->P, p->d_perm, (const double *)internal, user);
-    k_scatter_pts<float><<<grid_for(p->P, 256, GRID_CAP), 256, 0, p->st>>>(p->P, p->d_perm, (const float *)internal,
-                                                                          user);
     return cudaGetLastError();
 }
 
