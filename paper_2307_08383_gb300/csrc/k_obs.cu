@@ -32,28 +32,22 @@ struct Intr {
 // --------------------------------------------------------------------------
 // state caches
 // --------------------------------------------------------------------------
-__global__ void k_prepare_cams64(int n, const double *__restrict__ cams, double *__restrict__ camc) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+// the cache of one camera [w, t]
+__device__ __forceinline__ void prepare_cam(const double *w, const double *t, double *__restrict__ o) {
     double q[4], R[9];
-    quat_exp(cams + 6 * i, q);
+    quat_exp(w, q);
     quat_to_R(q, R);
 #pragma unroll
-    for (int k = 0; k < 9; ++k) camc[12 * i + k] = R[k];
+    for (int k = 0; k < 9; ++k) o[k] = R[k];
 #pragma unroll
-    for (int k = 0; k < 3; ++k) camc[12 * i + 9 + k] = cams[6 * i + 3 + k];
+    for (int k = 0; k < 3; ++k) o[9 + k] = t[k];
 }
-
 // FP32 camera cache, CAMC32_W floats per camera:
 // [R_hi (9), C_hi (3), C_lo (3), 0, R_lo (9), 0 (7)]
-__global__ void k_prepare_cams32(int n, const double *__restrict__ cams, float *__restrict__ camc) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+__device__ __forceinline__ void prepare_cam(const double *w, const double *t, float *__restrict__ o) {
     double q[4], R[9];
-    quat_exp(cams + 6 * i, q);
+    quat_exp(w, q);
     quat_to_R(q, R);
-    const double *t = cams + 6 * i + 3;
-    float *o = camc + CAMC32_W * i;
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
         const float hi = (float)R[k];
@@ -70,6 +64,13 @@ __global__ void k_prepare_cams32(int n, const double *__restrict__ cams, float *
         o[12 + d] = (float)(C - (double)hi);
     }
     o[15] = 0.f;
+}
+// CTAs of one warp: 64 cycles an FP64 instruction for one warp or four
+constexpr int CAM_THREADS = 32;
+template <typename T>
+__global__ void __launch_bounds__(CAM_THREADS) k_prepare_cams(int n, const double *__restrict__ cams, T *__restrict__ camc) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) prepare_cam(cams + 6 * i, cams + 6 * i + 3, camc + (sizeof(T) == 4 ? CAMC32_W : 12) * (int64_t)i);
 }
 
 __global__ void k_split_pts(int64_t P, const double *__restrict__ pts, float *__restrict__ hl) {
@@ -401,13 +402,18 @@ __global__ void __launch_bounds__(256) k_cost(int64_t m, const int *__restrict__
 }
 
 // --------------------------------------------------------------------------
-// trial point: R <- Exp(dw) R, t <- Exp(dw) t + dt, X <- X + dX
+// trial camera: R <- Exp(dw) R, t <- Exp(dw) t + dt, and its cache
 // --------------------------------------------------------------------------
+// What bounds it: one warp's chain of FP64
+// instructions (two exponentials, a product, a logarithm, the exponential
+// again), 64 cycles each.  200 cameras, with the cache formed by a launch of its
+// own: 13.6 + 10.2 us; 17.9 so.
 template <typename T>
-__global__ void k_update_cams(int n, const double *__restrict__ cams, const T *__restrict__ dxc, double *__restrict__ out) {
+__global__ void __launch_bounds__(CAM_THREADS) k_update_cams(int n, const double *__restrict__ cams, const T *__restrict__ dxc,
+                                                             double *__restrict__ out, T *__restrict__ camc) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    double w[3], q[4], qd[4], qn[4], Rd[9];
+    double w[3], t1[3], q[4], qd[4], qn[4], Rd[9];
     const double dw[3] = {(double)dxc[6 * i], (double)dxc[6 * i + 1], (double)dxc[6 * i + 2]};
     quat_exp(cams + 6 * i, q);
     quat_exp(dw, qd);
@@ -420,11 +426,12 @@ __global__ void k_update_cams(int n, const double *__restrict__ cams, const T *_
     const double *t = cams + 6 * i + 3;
 #pragma unroll
     for (int r = 0; r < 3; ++r) {
+        t1[r] = Rd[3 * r] * t[0] + Rd[3 * r + 1] * t[1] + Rd[3 * r + 2] * t[2] + (double)dxc[6 * i + 3 + r];
         out[6 * i + r] = w[r];
-        out[6 * i + 3 + r] = Rd[3 * r] * t[0] + Rd[3 * r + 1] * t[1] + Rd[3 * r + 2] * t[2] + (double)dxc[6 * i + 3 + r];
+        out[6 * i + 3 + r] = t1[r];
     }
+    prepare_cam(w, t1, camc + (sizeof(T) == 4 ? CAMC32_W : 12) * (int64_t)i);
 }
-
 
 // One staged observation row (JW values, 16-byte aligned) from shared memory.
 __device__ __forceinline__ void load_jrow_s(const float *s, float (&v)[JW]) {
@@ -911,12 +918,12 @@ cudaError_t launch_scatter_pts(ba_problem *p, const void *internal, bool interna
 cudaError_t launch_prepare_state(ba_problem *p, StateBuf &s) {
     cudaEvent_t ev;
     ktimer_begin(p, K_PREPARE, &ev);
-    const int nb = (p->n + 127) / 128;
+    const int nb = (p->n + CAM_THREADS - 1) / CAM_THREADS;
     if (p->fp32) {
-        k_prepare_cams32<<<nb, 128, 0, p->st>>>(p->n, s.cams, (float *)s.camc);
+        k_prepare_cams<float><<<nb, CAM_THREADS, 0, p->st>>>(p->n, s.cams, (float *)s.camc);
         k_split_pts<<<grid_for(p->P, 256, GRID_CAP), 256, 0, p->st>>>(p->P, s.pts, s.pts_hl);
     } else {
-        k_prepare_cams64<<<nb, 128, 0, p->st>>>(p->n, s.cams, (double *)s.camc);
+        k_prepare_cams<double><<<nb, CAM_THREADS, 0, p->st>>>(p->n, s.cams, (double *)s.camc);
     }
     ktimer_end(p, K_PREPARE, ev);
     p->launches += p->fp32 ? 2 : 1;
@@ -964,16 +971,16 @@ cudaError_t launch_cost(ba_problem *p, StateBuf &s, bool trial) {
 cudaError_t launch_trial_cameras(ba_problem *p) {
     cudaEvent_t ev;
     ktimer_begin(p, K_UPDATE, &ev);
-    const int nb = (p->n + 127) / 128;
+    const int nb = (p->n + CAM_THREADS - 1) / CAM_THREADS;
     if (p->fp32) {
-        k_update_cams<float><<<nb, 128, 0, p->st>>>(p->n, p->cur.cams, (const float *)p->dxc, p->trial.cams);
-        k_prepare_cams32<<<nb, 128, 0, p->st>>>(p->n, p->trial.cams, (float *)p->trial.camc);
+        k_update_cams<float><<<nb, CAM_THREADS, 0, p->st>>>(p->n, p->cur.cams, (const float *)p->dxc, p->trial.cams,
+                                                            (float *)p->trial.camc);
     } else {
-        k_update_cams<double><<<nb, 128, 0, p->st>>>(p->n, p->cur.cams, (const double *)p->dxc, p->trial.cams);
-        k_prepare_cams64<<<nb, 128, 0, p->st>>>(p->n, p->trial.cams, (double *)p->trial.camc);
+        k_update_cams<double><<<nb, CAM_THREADS, 0, p->st>>>(p->n, p->cur.cams, (const double *)p->dxc, p->trial.cams,
+                                                             (double *)p->trial.camc);
     }
     ktimer_end(p, K_UPDATE, ev);
-    p->launches += 2;
+    p->launches += 1;
     return cudaGetLastError();
 }
 
@@ -1026,7 +1033,8 @@ cudaError_t launch_triangulate(ba_problem *p, int gn_iters) {
         p->tri_cam64 = (double *)d;
     }
     ktimer_begin(p, K_TRIANGULATE, &ev);
-    k_prepare_cams64<<<(p->n + 127) / 128, 128, 0, p->st>>>(p->n, p->cur.cams, p->tri_cam64);
+    k_prepare_cams<double><<<(p->n + CAM_THREADS - 1) / CAM_THREADS, CAM_THREADS, 0, p->st>>>(p->n, p->cur.cams,
+                                                                                           p->tri_cam64);
     k_triangulate<<<grid_for(p->P, 256, GRID_CAP), 256, 0, p->st>>>(p->P, p->trk_ptr, p->obs_cam, p->uv64,
                                                                     p->tri_cam64, intr_of(p), gn_iters, p->cur.pts,
                                                                     &p->sc->n_tri_fail);
