@@ -215,113 +215,10 @@ __device__ __forceinline__ void quat_to_R(const double *q, double *R) {
     R[6] = 2 * (x * z - w * y);     R[7] = 2 * (y * z + w * x);     R[8] = 1 - 2 * (x * x + y * y);
 }
 
-template <typename T> __device__ __forceinline__ void red_add(T *p, T v) { atomicAdd(p, v); }
-
-// Grid-wide barrier for a cooperative launch (all CTAs co-resident).
-// bar[0] counts arrivals, bar[1] is the generation.  The wait is bounded by
-// about `limit_cycles` SM clocks; on timeout it sets *err = BA_ERR_TIMEOUT and
-// returns false, and the caller must leave the kernel.
-__device__ __forceinline__ bool grid_barrier(unsigned *bar, int *err, long long limit_cycles) {
-    __shared__ int s_ok;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        volatile unsigned *vgen = bar + 1;
-        const unsigned g0 = *vgen;
-        __threadfence();
-        const unsigned arrived = atomicAdd(bar, 1u);
-        int ok = 1;
-        if (arrived == gridDim.x - 1) {
-            atomicExch(bar, 0u);
-            __threadfence();
-            atomicAdd(bar + 1, 1u);
-        } else {
-            const long long t0 = clock64();
-            while (*vgen == g0) {
-                if (clock64() - t0 > limit_cycles || *(volatile int *)err == (int)BA_ERR_TIMEOUT) {
-                    atomicExch(err, (int)BA_ERR_TIMEOUT);
-                    ok = 0;
-                    break;
-                }
-                __nanosleep(64);
-            }
-        }
-        __threadfence();
-        s_ok = ok;
-    }
-    __syncthreads();
-    return s_ok != 0;
-}
-
-// Grid-wide all-reduce fused with a barrier (cooperative launch).  On entry
-// v holds this CTA's partial in thread 0; every CTA stores it, the last CTA
-// to arrive adds the partials in CTA order, publishes the totals in bcast and
-// releases the others; on return every thread holds the totals.  Waits are
-// bounded as in grid_barrier; returns false on timeout.
-__device__ __forceinline__ unsigned atom_add_release(unsigned *p, unsigned v) {
-    unsigned old;
-    asm volatile("atom.add.release.gpu.global.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
-    return old;
-}
 __device__ __forceinline__ unsigned ld_acquire(const unsigned *p) {
     unsigned v;
     asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
-}
-
-template <int NV>
-__device__ __forceinline__ bool grid_allreduce(double (&v)[NV], double *part, double *bcast, unsigned *bar, int *err,
-                                               long long limit_cycles) {
-    __shared__ int s_last, s_ok;
-    __shared__ double s_tot[NV];
-    __shared__ double s_red[32 * NV];
-    unsigned g0 = 0;
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int k = 0; k < NV; ++k) part[blockIdx.x * NV + k] = v[k];
-        g0 = ld_acquire(bar + 1);
-        // release: the partial above is visible to whoever sees this arrival
-        const unsigned arrived = atom_add_release(bar, 1u);
-        s_last = (arrived == gridDim.x - 1);
-        s_ok = 1;
-    }
-    __syncthreads();
-    if (s_last) {
-        if (threadIdx.x == 0) ld_acquire(bar);  // acquire: every CTA's partial is visible
-        __syncthreads();
-        double acc[NV];
-#pragma unroll
-        for (int k = 0; k < NV; ++k) acc[k] = 0.0;
-        for (unsigned b = threadIdx.x; b < gridDim.x; b += blockDim.x)
-#pragma unroll
-            for (int k = 0; k < NV; ++k) acc[k] += __ldcg(part + b * NV + k);
-        block_sum<NV>(acc, s_red);
-        if (threadIdx.x == 0) {
-#pragma unroll
-            for (int k = 0; k < NV; ++k) {
-                __stcg(bcast + k, acc[k]);
-                s_tot[k] = acc[k];
-            }
-            atomicExch(bar, 0u);
-            atom_add_release(bar + 1, 1u);  // release: totals and the reset counter
-        }
-    } else if (threadIdx.x == 0) {
-        const long long t0 = clock64();
-        while (ld_acquire(bar + 1) == g0) {
-            if (clock64() - t0 > limit_cycles || *(volatile int *)err == (int)BA_ERR_TIMEOUT) {
-                atomicExch(err, (int)BA_ERR_TIMEOUT);
-                s_ok = 0;
-                break;
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < NV; ++k) s_tot[k] = __ldcg(bcast + k);
-    }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < NV; ++k) v[k] = s_tot[k];
-    const bool ok = s_ok != 0;
-    __syncthreads();
-    return ok;
 }
 
 __device__ __forceinline__ void red_add_release(unsigned *p, unsigned v) {

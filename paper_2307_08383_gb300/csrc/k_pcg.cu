@@ -8,11 +8,12 @@
 //   d = M^-1 r+ + beta d.
 // The whole recurrence runs in one persistent cooperative kernel: per
 // iteration a BSMC SpMV phase forms d = z + beta d_old on the fly (double-
-// buffered d), q = S d and d^T S d; a grid barrier; an update phase does the
-// axpys, z = M^-1 r and the two dot products; a second barrier.  Every CTA
+// buffered d), q = S d and d^T S d; a grid exchange; an update phase does the
+// axpys, z = M^-1 r and the two dot products; a second exchange.  Every CTA
 // sums the per-CTA partials in the same order, so all CTAs take the same
-// alpha, beta and stop decision without a third barrier.  Barrier waits are
-// bounded; a timeout sets an error flag and every CTA leaves.
+// alpha, beta and stop decision without a third.  The waits are bounded; a
+// timeout sets an error flag and every CTA leaves.  Small FP64 systems keep S
+// and the vectors in registers (k_pcg64_res).
 //
 // FP32 solves instead run CG on the split-preconditioned system
 // S^ = G^T S G (M^-1 = G G^T per camera, G from a Cholesky factor), which is
@@ -843,24 +844,22 @@ __device__ __forceinline__ float next_r(float r, float w, float s, float a, floa
 // [eb, ee), cut into passes of 32 consecutive entries; warp w of the
 // SPLIT_WARPS takes passes w, w + SPLIT_WARPS, ...  The cameras the CTA's
 // entries reference (its halo, a few hundred at the benchmark size, with one
-// CTA per SM) are gathered once per iteration from the
-// previous iteration's records, each transformed once into the vector the
-// SpMV applies, x_j = r_j - alpha (w_j + beta s_j), and kept in shared
+// CTA per SM) are gathered once per iteration from the previous iteration's
+// records, each transformed once into the vector the SpMV applies, x_j = r_j - alpha (w_j + beta s_j), and kept in shared
 // memory.  The gather of iteration k + 1 is issued (16-byte asynchronous
 // copies of the 80-byte records into the halo area, transformed there in
 // place) as soon as the all-reduce that ends iteration k has seen every CTA
 // arrive, so its L2 round trip overlaps the partial reads, the block sum and
-// the scalar update.  A pass's 32 S^ blocks (4.6 KB, contiguous in entry order) and the
-// entries' packed (local row, halo index) arrive by 1-D bulk copies into one
-// of the warp's SPLIT_NBUF buffers; since S^ does not change during the
+// the scalar update.  A pass's 32 S^ blocks (4.6 KB, contiguous in entry
+// order) and the entries' packed (local row, halo index) arrive by 1-D bulk
+// copies into one of the warp's SPLIT_NBUF buffers; since S^ does not change during the
 // solve, each refill fetches the warp's pass SPLIT_NBUF positions ahead,
 // wrapping into the next iteration.  Where the CTA's passes all fit in shared
 // memory (about 42), each has a buffer of its own, filled once: a warp's third
 // pass otherwise waits about 1 us in every iteration for a refill issued in
 // it (with the rows' starts in shared memory too: 2,556 cameras, 33 passes,
-// 6.40 -> 6.07 us per iteration; 512 cameras 5.02 -> 4.74).  The pass loop reads shared
-// memory only.  A segmented
-// shuffle scan over the pass (entries are sorted by row) leaves each row
+// 6.40 -> 6.07 us per iteration; 512 cameras 5.02 -> 4.74).  The pass loop
+// reads shared memory only.  A segmented shuffle scan over the pass (entries are sorted by row) leaves each row
 // segment's sum in its last lane, which stores it in a slot: (q, 0) if the
 // segment opens pass q, (q, 1) if it closes it, else the row's own slot.  The
 // sums depend only on the entry order: deterministic.
