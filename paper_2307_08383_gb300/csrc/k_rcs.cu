@@ -384,8 +384,8 @@ __global__ void __launch_bounds__(FORM_THREADS) k_form_rcs(const GroupDesc *__re
 // per 16-byte chunk of the block (9 for FP32, 18 for FP64): the chunks of a
 // partial are read by consecutive threads, and each thread keeps DEPTH
 // partials' loads in flight before adding them in order; with 8 also the next
-// ones' indices, and the eight are added in pairs first (a chain an eighth as
-// long).  DEPTH 8 for small systems (few warps, long lists: a chain of
+// ones' indices, and in FP64, whose smaller groups make more partials, the eight
+// are added in pairs first (a chain an eighth as long).  DEPTH 8 for small systems (few warps, long lists: a chain of
 // round trips; 50 cameras FP64 43 -> 29 us, 200 cameras FP32 19 -> 12), 4 for
 // large ones (bandwidth: 1,770 cameras FP32 27 us, 31 with 8).  (Writing each
 // partial straight to a block-ordered slot in RCS formation made this
@@ -439,11 +439,17 @@ __global__ void __launch_bounds__(256) k_rcs_reduce(int64_t nblk, const int *__r
 #pragma unroll
                     for (int k = 0; k < DEPTH; ++k) id[k] = __ldg(plist + min(q + DEPTH + k, q1 - 1));
                 }
+                if constexpr (sizeof(T) == 8) {
 #pragma unroll
-                for (int h = DEPTH / 2; h > 0; h /= 2)
+                    for (int h = DEPTH / 2; h > 0; h /= 2)
 #pragma unroll
-                    for (int k = 0; k < h; ++k) add16(v[k], v[k + h]);
-                add16(s, v[0]);
+                        for (int k = 0; k < h; ++k) add16(v[k], v[k + h]);
+                    add16(s, v[0]);
+                } else {
+#pragma unroll
+                    for (int k = 0; k < DEPTH; ++k)
+                        if (q + k < q1) add16(s, v[k]);
+                }
             }
         }
         sv[x] = s;
