@@ -300,7 +300,8 @@ ba_status ba_problem_create(const ba_options *opt, int32_t n_cams, const double 
     const size_t camc_w = p->fp32 ? CAMC32_W * 4 : 12 * 8;
     size_t plan = 0;
     for (;;) {
-        ba_status s = symbolic_setup(n_cams, n_pts, n_obs, obs_cam, obs_pt, pts, p->obs_max, false, hs, err, target);
+        ba_status s = symbolic_setup(n_cams, n_pts, n_obs, obs_cam, obs_pt, pts, p->obs_max, false, hs, err, target,
+                                     !p->fp32);
         if (s != BA_OK) {
             delete p;
             return fail(s, err);

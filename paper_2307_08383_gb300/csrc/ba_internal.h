@@ -99,10 +99,11 @@ void build_twosided(HostSetup &hs, int32_t n);
 // Validates the observation set and builds everything above.  Returns BA_OK or
 // BA_ERR_INVALID_ARG with a message.  Tracks of more than obs_max observations
 // are refused; point groups are closed at obs_target observations (0: obs_max;
-// a longer track is a group of its own).
+// a longer track is a group of its own).  even_items: blocks ordered so that a
+// warp's work items are of one size.
 ba_status symbolic_setup(int32_t n, int64_t P, int64_t m, const int32_t *obs_cam,
                          const int64_t *obs_pt, const double *pts, int obs_max, bool pattern_only,
-                         HostSetup &hs, std::string &err, int obs_target = 0);
+                         HostSetup &hs, std::string &err, int obs_target = 0, bool even_items = false);
 
 // A parameter state with its derived per-camera / per-point caches.
 struct StateBuf {
