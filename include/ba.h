@@ -409,10 +409,9 @@ ba_status ba_tc_gemm(int32_t M, int32_t N, int32_t K, const float *A, int64_t a_
  * current; make that first call before any stream capture.  All calls share
  * the one array: calls that overlap on the GPU race on it.  Each call clears
  * the parts that must start at zero.  The call allocates nothing (no
- * cudaMalloc / cudaFree), runs the iterations in one cooperative launch and
- * synchronises the stream once, to read its outcome.  Errors:
- * BA_ERR_INVALID_ARG, BA_ERR_NOT_SPD, BA_ERR_NO_CONVERGENCE (x holds the last
- * iterate), BA_ERR_TIMEOUT (a grid wait gave up), BA_ERR_CUDA. */
+ * cudaMalloc / cudaFree) and synchronises the stream every eight iterations
+ * to read the stop flag.  Errors: BA_ERR_INVALID_ARG, BA_ERR_NOT_SPD,
+ * BA_ERR_NO_CONVERGENCE (x holds the last iterate), BA_ERR_CUDA. */
 ba_status ba_pcg_solve_static(int32_t n, int64_t nnzb, const int32_t *row_ptr, const int32_t *col,
                               const float *val, const float *b, float *x, double rel_tol,
                               int32_t max_iters, void *cuda_stream, int32_t *iters_out,
