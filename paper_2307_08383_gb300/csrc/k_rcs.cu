@@ -140,7 +140,10 @@ __device__ __forceinline__ void rcs_points(const GroupDesc &g, T *so, int pl0, c
             atomicExch(&sc->err, (int)BA_ERR_NOT_SPD);
             m00 = m10 = m11 = m20 = m21 = m22 = T(0);
         }
-        const T q0 = m00 * l0, q1 = m10 * l0 + m11 * l1, q2 = m20 * l0 + m21 * l1 + m22 * l2;
+        // (fused by hand here and in e^: which product of a sum the compiler
+        // rounds first is its choice, and b's last bits, with the LM trajectory
+        // that follows from them, changed with code elsewhere in this loop)
+        const T q0 = m00 * l0, q1 = fma(m11, l1, m10 * l0), q2 = fma(m22, l2, fma(m20, l0, m21 * l1));
         T *lo = Linv_out + 6 * (int64_t)k;
         lo[0] = m00; lo[1] = m10; lo[2] = m11; lo[3] = m20; lo[4] = m21; lo[5] = m22;
         T *lpo = lp_out + 3 * (int64_t)k;
@@ -153,7 +156,7 @@ __device__ __forceinline__ void rcs_points(const GroupDesc &g, T *so, int pl0, c
                 const T j0 = s[12 + 3 * r], j1 = s[13 + 3 * r], j2 = s[14 + 3 * r];
                 const T P0 = j0 * m00, P1 = j0 * m10 + j1 * m11, P2 = j0 * m20 + j1 * m21 + j2 * m22;
                 Pv[3 * r] = P0; Pv[3 * r + 1] = P1; Pv[3 * r + 2] = P2;
-                s[18 + r] += P0 * q0 + P1 * q1 + P2 * q2;
+                s[18 + r] += fma(P2, q2, fma(P0, q0, P1 * q1));
             }
 #pragma unroll
             for (int k = 0; k < 6; ++k) s[p_slot(k / 3, k % 3)] = Pv[k];
@@ -472,10 +475,12 @@ __global__ void __launch_bounds__(32) k_rcs_diag(int n, const int *__restrict__ 
         a[c] = on ? Sd[6 * lo - lo * (lo - 1) / 2 + (hi - lo)] : (i < n ? T(0) : T(1));
     }
     if (on) {
-        const T dmp = (T)lambda * clampT(Sd[21 + r]);
+        // one rounding: S of an FP32 problem decides its LM trajectory (two, and
+        // the benchmark's twenty steps took 3,318 PCG iterations instead of 3,082)
+        const T u = clampT(Sd[21 + r]);
 #pragma unroll
         for (int c = 0; c < 6; ++c)
-            if (c == r) a[c] += dmp;
+            if (c == r) a[c] = fma((T)lambda, u, a[c]);
         b[6 * i + r] = Sd[27 + r];
     }
     __syncwarp();  // the packed block has been read
