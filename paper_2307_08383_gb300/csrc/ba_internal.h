@@ -217,6 +217,7 @@ struct ba_problem {
     int32_t *cta_rows = nullptr;   // row range of each CTA of the balanced SpMV
     uint32_t *tw_meta = nullptr;   // per entry: local row | halo index << 16 (per-CTA aligned)
     int32_t *meta_off = nullptr, *halo_ptr = nullptr, *halo_col = nullptr, *own_base = nullptr;
+    int32_t *pass_tab = nullptr;   // cluster: the CTAs' passes (offsets, then first entries)
     int split_grid = 0;            // 0: not partitioned yet, < 0: unavailable
     bool split_cluster = false;    // the grid runs as one thread-block cluster
     int split_slot_floats = 0, split_stage_floats = 0;

@@ -879,7 +879,17 @@ struct SplitPipe {
     int eb, ee, m;   // entry range; passes of this warp
     uint32_t seq;    // passes this warp has consumed so far
     bool res;        // every pass of the CTA has its own buffer
+    const int *ps;   // first entry of each pass and the end (cluster), null: 32 entries each from eb
+    __device__ __forceinline__ int first(int q) const { return ps ? __ldg(ps + q) : eb + 32 * q; }
+    __device__ __forceinline__ int end(int q) const { return ps ? __ldg(ps + q + 1) : min(eb + 32 * q + 32, ee); }
+    // metadata to copy: in whole 16-byte words; a cluster's pass has all 32
+    __device__ __forceinline__ uint32_t meta_bytes(int cnt) const { return ps ? 128u : (uint32_t)((cnt + 3) & ~3) * 4; }
 };
+// A cluster's metadata: 32 to a pass, local row | halo index << 16 as in the
+// grid's, with where a row's sum over the pass goes (the segment's slot of
+// split_passes: 0 opens the pass, 1 closes it, 2 the row's own) in the top bits of
+// the two halves; CL_NONE beyond the pass's entries.
+constexpr uint32_t CL_NONE = 0x7FFFu;
 
 __device__ __forceinline__ float *pass_buf(const SplitPipe &pp, uint32_t s) {
     return pp.stage + (size_t)(SPLIT_NBUF * (threadIdx.x >> 5) + s % SPLIT_NBUF) * (PASS_BYTES / 4);
@@ -889,12 +899,12 @@ __device__ __forceinline__ float *pass_buf(const SplitPipe &pp, uint32_t s) {
 __device__ __forceinline__ void split_issue(const SplitPipe &pp, uint32_t s) {
     const int wid = threadIdx.x >> 5;
     const int q = wid + SPLIT_WARPS * (int)(s % (uint32_t)pp.m);
-    const int cnt = min(32, pp.ee - pp.eb - 32 * q);
-    const uint32_t sbytes = (uint32_t)cnt * BW * 4, mbytes = (uint32_t)((cnt + 3) & ~3) * 4;
+    const int ps = pp.first(q), cnt = pp.end(q) - ps;
+    const uint32_t sbytes = (uint32_t)cnt * BW * 4, mbytes = pp.meta_bytes(cnt);
     uint64_t *bar = pp.mbar + SPLIT_NBUF * wid + s % SPLIT_NBUF;
     float *buf = pass_buf(pp, s);
     mbar_expect_tx(bar, sbytes + mbytes);
-    bulk_g2s(buf, pp.Sh + (int64_t)(pp.eb + 32 * q) * BW, sbytes, bar);
+    bulk_g2s(buf, pp.Sh + (int64_t)ps * BW, sbytes, bar);
     bulk_g2s(buf + PASS_S_BYTES / 4, pp.meta + 32 * q, mbytes, bar);
 }
 // lane 0: the warp's first copies - the passes its buffers hold, or (res) all of
@@ -909,15 +919,15 @@ __device__ __forceinline__ void split_start(const SplitPipe &pp) {
     uint64_t *bar = pp.mbar + SPLIT_NBUF * wid;
     uint32_t total = 0;
     for (int k = 0; k < pp.m; ++k) {
-        const int cnt = min(32, pp.ee - pp.eb - 32 * (wid + SPLIT_WARPS * k));
-        total += (uint32_t)cnt * BW * 4 + (uint32_t)((cnt + 3) & ~3) * 4;
+        const int cnt = pp.end(wid + SPLIT_WARPS * k) - pp.first(wid + SPLIT_WARPS * k);
+        total += (uint32_t)cnt * BW * 4 + pp.meta_bytes(cnt);
     }
     mbar_expect_tx(bar, total);
     for (int k = 0; k < pp.m; ++k) {
-        const int q = wid + SPLIT_WARPS * k, cnt = min(32, pp.ee - pp.eb - 32 * q);
+        const int q = wid + SPLIT_WARPS * k, ps = pp.first(q), cnt = pp.end(q) - ps;
         float *buf = pp.stage + (size_t)q * (PASS_BYTES / 4);
-        bulk_g2s(buf, pp.Sh + (int64_t)(pp.eb + 32 * q) * BW, (uint32_t)cnt * BW * 4, bar);
-        bulk_g2s(buf + PASS_S_BYTES / 4, pp.meta + 32 * q, (uint32_t)((cnt + 3) & ~3) * 4, bar);
+        bulk_g2s(buf, pp.Sh + (int64_t)ps * BW, (uint32_t)cnt * BW * 4, bar);
+        bulk_g2s(buf + PASS_S_BYTES / 4, pp.meta + 32 * q, pp.meta_bytes(cnt), bar);
     }
 }
 
@@ -939,11 +949,10 @@ __device__ __forceinline__ void split_drain(const SplitPipe &pp, long long limit
 __device__ __forceinline__ bool split_passes(SplitPipe &pp, const int *row_ent, const float *hx,
                                              float *slot, float *rowacc, int *err, long long limit) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int eb = pp.eb, ee = pp.ee;
     for (int k = 0; k < pp.m; ++k) {
         const int q = wid + SPLIT_WARPS * k;
-        const int t = eb + 32 * q + lane;
-        const bool valid = t < ee;
+        const bool table = pp.ps != nullptr;
+        const int ps = pp.eb + 32 * q, pe = min(ps + 32, pp.ee);  // (without a table)
         const uint32_t b = pp.res ? 0u : pp.seq % SPLIT_NBUF;
         // every lane observes the copy's completion; the outcome is warp-uniform
         // (res: the one phase that the first wait saw complete)
@@ -955,10 +964,12 @@ __device__ __forceinline__ bool split_passes(SplitPipe &pp, const int *row_ent, 
         const float *buf = pp.res ? pp.stage + (size_t)q * (PASS_BYTES / 4) : pass_buf(pp, pp.seq);
         int lr = 0xFFFF;
         float y[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        uint32_t md = CL_NONE;
+        if (table || ps + lane < pe) md = reinterpret_cast<const uint32_t *>(buf + PASS_S_BYTES / 4)[lane];
+        const bool valid = table ? (md & 0x7FFFu) != CL_NONE : ps + lane < pe;
         if (valid) {
-            const uint32_t md = reinterpret_cast<const uint32_t *>(buf + PASS_S_BYTES / 4)[lane];
-            lr = (int)(md & 0xFFFFu);
-            const float4 *x4 = reinterpret_cast<const float4 *>(hx + HX * (md >> 16));
+            lr = (int)(md & (table ? 0x7FFFu : 0xFFFFu));
+            const float4 *x4 = reinterpret_cast<const float4 *>(hx + HX * ((md >> 16) & (table ? 0x7FFFu : 0xFFFFu)));
             const float4 xa = x4[0], xb = x4[1];
             const float x[6] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y};
             const float4 *s4 = reinterpret_cast<const float4 *>(buf + lane * BW);
@@ -989,9 +1000,13 @@ __device__ __forceinline__ bool split_passes(SplitPipe &pp, const int *row_ent, 
         }
         const int ld = __shfl_down_sync(0xffffffffu, lr, 1);
         if (valid && (lane == 31 || ld != lr)) {
-            const int rs = row_ent[lr], rend = row_ent[lr + 1];
-            const int ps = eb + 32 * q, pe = min(ps + 32, ee);
-            float *dst = rs <= ps ? slot + 12 * q : (rend >= pe ? slot + 12 * q + 6 : rowacc + 6 * lr);
+            float *dst;
+            if (table) {
+                dst = md >> 31 ? rowacc + 6 * lr : slot + 12 * q + ((md & 0x8000u) ? 6 : 0);
+            } else {
+                const int rs = row_ent[lr], rend = row_ent[lr + 1];
+                dst = rs <= ps ? slot + 12 * q : (rend >= pe ? slot + 12 * q + 6 : rowacc + 6 * lr);
+            }
 #pragma unroll
             for (int c = 0; c < 6; ++c) dst[c] = y[c];
         }
@@ -1001,13 +1016,24 @@ __device__ __forceinline__ bool split_passes(SplitPipe &pp, const int *row_ent, 
 
 // Component c of the off-diagonal part of (S^ x)_i for local row lr after
 // split_passes and a __syncthreads: the row's segment sums in pass order
-// (zero for a row without off-diagonal entries).
-__device__ __forceinline__ float split_combine(int lr, int c, int rs, int rend, int eb, int ee, const float *slot,
-                                               const float *rowacc) {
+// (zero for a row without off-diagonal entries).  row_src (cluster, where a
+// pass's bounds come from a table): the row's first sum as an offset from slot,
+// and in the upper half the number of passes that it goes on for.
+constexpr uint32_t ROW_EMPTY = 0xFFFFu;
+__device__ __forceinline__ float split_combine(const SplitPipe &pp, const uint32_t *row_src, int lr, int c, int rs,
+                                               int rend, const float *slot, const float *rowacc) {
     float w = 0.f;
+    if (pp.ps) {
+        const uint32_t u = row_src[lr], o = u & 0xFFFFu;
+        if (o == ROW_EMPTY) return w;
+        w += slot[o + c];
+        const float *s = slot + 12 * (o / 12) + c;
+        for (uint32_t k = 1; k <= u >> 16; ++k) w += s[12 * k];
+        return w;
+    }
     if (rs >= rend) return w;
-    for (int q = (rs - eb) >> 5; q <= (rend - 1 - eb) >> 5; ++q) {
-        const int ps = eb + 32 * q, pe = min(ps + 32, ee);
+    for (int q = (rs - pp.eb) >> 5; q <= (rend - 1 - pp.eb) >> 5; ++q) {
+        const int ps = pp.eb + 32 * q, pe = min(ps + 32, pp.ee);
         const float *src = rs <= ps ? slot + 12 * q : (rend >= pe ? slot + 12 * q + 6 : rowacc + 6 * lr);
         w += src[c];
     }
@@ -1145,7 +1171,8 @@ __global__ void __launch_bounds__(SPLIT_WARPS * 32, SPLIT_CTAS_PER_SM) k_pcg_spl
                                                       const int *__restrict__ meta_off,
                                                       const int *__restrict__ halo_ptr,
                                                       const int *__restrict__ halo_col,
-                                                      const int *__restrict__ own_base, int slot_floats,
+                                                      const int *__restrict__ own_base,
+                                                      const int *__restrict__ pass_tab, int slot_floats,
                                                       int stage_floats,
                                                       const float *__restrict__ Sh, const float *__restrict__ H,
                                                       const float *__restrict__ Shd, int diag_ident,
@@ -1166,15 +1193,26 @@ __global__ void __launch_bounds__(SPLIT_WARPS * 32, SPLIT_CTAS_PER_SM) k_pcg_spl
     const int eb = __ldg(tw_ptr + rb), ee = __ldg(tw_ptr + re);
     const int hb = __ldg(halo_ptr + blockIdx.x), NH = __ldg(halo_ptr + blockIdx.x + 1) - hb;
     const int ob = __ldg(own_base + blockIdx.x);
-    const int R = re - rb, P = (ee - eb + 31) >> 5, wid = threadIdx.x >> 5;
-    // dynamic shared memory: copy buffers | slots + row sums | halo | own records | row starts
+    // the CTA's passes: with CLUSTER from the table (offsets of the CTAs' lists, each
+    // list's first entries and its end, then the rows' sums)
+    const int pt0 = CLUSTER ? __ldg(pass_tab + blockIdx.x) : 0;
+    const int R = re - rb, wid = threadIdx.x >> 5;
+    const int P = CLUSTER ? __ldg(pass_tab + blockIdx.x + 1) - pt0 - 1 : (ee - eb + 31) >> 5;
+    // dynamic shared memory: copy buffers | slots + row sums | halo | own records | row starts |
+    // (CLUSTER) rows' sums (split_combine)
     float *slot = sdyn + stage_floats, *rowacc = slot + 12 * P;
     float *hx = slot + slot_floats, *own = hx + HX * NH;
     int *s_row = reinterpret_cast<int *>(own + 20 * R);  // first entry of each of the CTA's rows, and the end
+    uint32_t *s_src = reinterpret_cast<uint32_t *>(s_row + R + 1);
     for (int q = threadIdx.x; q <= R; q += blockDim.x) s_row[q] = __ldg(tw_ptr + rb + q);
+    if (CLUSTER) {
+        const int *src = pass_tab + __ldg(pass_tab + gridDim.x) + rb;  // behind the lists
+        for (int q = threadIdx.x; q < R; q += blockDim.x) s_src[q] = (uint32_t)__ldg(src + q);
+    }
     const int hj0 = (int)threadIdx.x < NH ? __ldg(halo_col + hb + threadIdx.x) : 0;
     SplitPipe pp{sdyn, mbar, Sh, tw_meta + __ldg(meta_off + blockIdx.x), eb, ee,
-                 wid < P ? (P - 1 - wid) / SPLIT_WARPS + 1 : 0, 0u, stage_floats * 4 != SPLIT_STAGE_BYTES};
+                 wid < P ? (P - 1 - wid) / SPLIT_WARPS + 1 : 0, 0u, stage_floats * 4 != SPLIT_STAGE_BYTES,
+                 CLUSTER ? pass_tab + pt0 : nullptr};
     if (threadIdx.x < SPLIT_NBUF * SPLIT_WARPS) mbar_init(&mbar[threadIdx.x], 1);
     fence_proxy_async();
     __syncthreads();
@@ -1266,7 +1304,7 @@ __global__ void __launch_bounds__(SPLIT_WARPS * 32, SPLIT_CTAS_PER_SM) k_pcg_spl
             const int lr = u / 6, c = u - 6 * lr, i = rb + lr;
             const int rs = s_row[lr], rend = s_row[lr + 1];
             const float *r6 = hx + HX * (ob + lr);
-            const float wc = split_combine(lr, c, rs, rend, eb, ee, slot, rowacc) + split_diag(i, c, r6, Shd, diag_ident);
+            const float wc = split_combine(pp, s_src, lr, c, rs, rend, slot, rowacc) + split_diag(i, c, r6, Shd, diag_ident);
             rec0[(int64_t)SREC * i + 6 + c] = wc;
             float hr = 0.f;
 #pragma unroll
@@ -1325,7 +1363,7 @@ __global__ void __launch_bounds__(SPLIT_WARPS * 32, SPLIT_CTAS_PER_SM) k_pcg_spl
             const bool first = u == u0;
             const int rs = s_row[lr], rend = s_row[lr + 1];
             const float *rnew = hx + HX * (ob + lr);  // this row's new residual (all six components)
-            const float w_e = split_combine(lr, c, rs, rend, eb, ee, slot, rowacc) + split_diag(i, c, rnew, Shd, diag_ident);
+            const float w_e = split_combine(pp, s_src, lr, c, rs, rend, slot, rowacc) + split_diag(i, c, rnew, Shd, diag_ident);
             const float *o6 = own + 20 * lr;
             const float r_e = rnew[c], rold = o6[c], wold = o6[6 + c], sold = o6[12 + c];
             const float pval = __fmaf_rn(b, first ? p0 : __ldcg(p + e), rold);
@@ -1713,12 +1751,13 @@ static cudaLaunchConfig_t split_cluster_config(int grid, size_t smem, cudaStream
 
 // Work partition of the split CG, made once per problem on the host: the
 // grid size; each CTA's row range (contiguous rows, about equal entries + a
-// fixed cost per row); its halo (the sorted distinct columns of its entries;
+// fixed cost per row; in a cluster, several such ranges, each cut into passes by
+// itself); its halo (the sorted distinct columns of its entries;
 // its own rows are one contiguous stretch of it, starting at own_base); the
 // packed metadata of every entry (local row | halo index << 16), laid out
 // per CTA from a 16-byte aligned offset; and the dynamic shared memory of
 // the busiest CTA (copy buffers, pass slots and row sums, halo vectors, own
-// records).  Problems that need more than 200 KB in a CTA keep the standard
+// records, row starts).  Problems that need more than 226 KB in a CTA keep the standard
 // recurrence (split_grid < 0).
 static cudaError_t split_partition(ba_problem *p) {
     if (p->split_grid != 0) return cudaSuccess;
@@ -1763,29 +1802,24 @@ static cudaError_t split_partition(ba_problem *p) {
         p->split_grid = -1;
         return cudaSuccess;
     };
-    std::vector<int32_t> rows, hptr, hcol, obase;
+    std::vector<int32_t> parts, cut, rows, tab, hptr, hcol, obase;
     size_t smem = SPLIT_STAGE_BYTES;
-    int slot_floats = 0, stage_bytes = SPLIT_STAGE_BYTES, G = 0;
+    int slot_floats = 0, stage_bytes = SPLIT_STAGE_BYTES, GP = 0, G = 0;
     for (int attempt = 0; attempt < 4; ++attempt) {
         if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_pcg_split<false>, SPLIT_WARPS * 32, smem)) != cudaSuccess) return e;
         bps = std::min(bps, SPLIT_CTAS_PER_SM);
         if (bps < 1) return unavailable();
-        int g = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)bps * n_sm, (E + 255) / 256));
-        if (cluster) {  // the power of two below, at most CL_MAX, no more CTAs than rows
-            int c = 1;
-            while (2 * c <= std::min(std::min(g, CL_MAX), n)) c *= 2;
-            g = c;
-        }
-        if (g == G) break;
-        G = g;
-        rows.assign(G + 1, n);
-        rows[0] = 0;
+        const int g = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)bps * n_sm, (E + 255) / 256));
+        if (g == GP) break;
+        GP = g;
+        parts.assign(GP + 1, n);
+        parts[0] = 0;
         const double total = (double)E + (double)ROW_COST * n;
         int c = 1;
         double acc = 0.0;
-        for (int i = 0; i < n && c < G; ++i) {
+        for (int i = 0; i < n && c < GP; ++i) {
             acc += (double)(twp[i + 1] - twp[i]) + ROW_COST;
-            while (c < G && acc >= total * c / G) rows[c++] = i + 1;
+            while (c < GP && acc >= total * c / GP) parts[c++] = i + 1;
         }
         // A CTA's passes are shared round-robin by its warps, so the slowest
         // warp of a CTA with 16k + 1 passes takes k + 1: cap every CTA at the
@@ -1805,25 +1839,57 @@ static cudaError_t split_partition(ba_problem *p) {
                     }
                     cur += r;
                 }
-                return cnt <= G;
+                return cnt <= GP;
             };
-            int64_t cap = std::max<int64_t>(1, (E + round * G - 1) / (round * G)) * round;
+            int64_t cap = std::max<int64_t>(1, (E + round * GP - 1) / (round * GP)) * round;
             while (cap < E && !fits(cap)) cap += round;
-            auto ent = [&](int k) { return (int64_t)twp[rows[k + 1]] - twp[rows[k]]; };
+            auto ent = [&](int k) { return (int64_t)twp[parts[k + 1]] - twp[parts[k]]; };
             for (int sweep = 0; sweep < 4; ++sweep) {
                 bool over = false;
-                for (int k = 0; k + 1 < G; ++k)  // forward: last rows to the next CTA
-                    while (ent(k) > cap && rows[k + 1] > rows[k] + 1) --rows[k + 1];
-                for (int k = G - 1; k > 0; --k)  // backward: first rows to the previous CTA
-                    while (ent(k) > cap && rows[k] < rows[k + 1] - 1) ++rows[k];
-                for (int k = 0; k < G; ++k) over = over || ent(k) > cap;
+                for (int k = 0; k + 1 < GP; ++k)  // forward: last rows to the next CTA
+                    while (ent(k) > cap && parts[k + 1] > parts[k] + 1) --parts[k + 1];
+                for (int k = GP - 1; k > 0; --k)  // backward: first rows to the previous CTA
+                    while (ent(k) > cap && parts[k] < parts[k + 1] - 1) ++parts[k];
+                for (int k = 0; k < GP; ++k) over = over || ent(k) > cap;
                 if (!over) break;
             }
+        }
+        // A CTA of the grid takes one part.  A CTA of the cluster takes a run of
+        // rows and cuts them where the parts' passes do, so that every row's sum
+        // is made of the same segments and has the same bits either way (a
+        // segment's own sum depends on its length only): the fewest passes
+        // that runs of rows allow.
+        rows = parts;
+        G = GP;
+        cut.clear();
+        if (cluster) {
+            for (int k = 0; k < GP; ++k)
+                for (int32_t t = twp[parts[k]]; t < twp[parts[k + 1]]; t += 32) cut.push_back(t);
+            cut.push_back((int32_t)E);
+            G = 1;  // the power of two below, at most CL_MAX, no more CTAs than rows
+            while (2 * G <= std::min(std::min(GP, CL_MAX), n)) G *= 2;
+            auto deal = [&](int cap) {  // false if G CTAs of at most cap passes are too few
+                rows.assign(G + 1, n);
+                rows[0] = 0;
+                // a: first pass of the CTA's rows; e: past the last pass of the rows up to i
+                for (int i = 0, c = 0, a = 0, e = 0; i < n; ++i) {
+                    while (cut[e] < twp[i + 1]) ++e;
+                    if (e - a <= cap) continue;
+                    if (i == rows[c] || ++c == G) return false;
+                    rows[c] = i;
+                    while (cut[a + 1] <= twp[i]) ++a;
+                    if (e - a > cap) return false;
+                }
+                return true;
+            };
+            int cap = 1;
+            while (!deal(cap)) ++cap;
         }
         // halos
         hptr.assign(G + 1, 0);
         hcol.clear();
         obase.assign(G, 0);
+        tab.assign(cluster ? G + 1 : 1, 0);
         int Hmax = 0, Rmax = 0, Pmax = 1;
         slot_floats = 0;
         std::vector<int32_t> cols;
@@ -1837,35 +1903,43 @@ static cudaError_t split_partition(ba_problem *p) {
             hcol.insert(hcol.end(), cols.begin(), cols.end());
             hptr[k + 1] = (int32_t)hcol.size();
             const int R = rows[k + 1] - rows[k];
-            const int64_t P = ((int64_t)twp[rows[k + 1]] - twp[rows[k]] + 31) / 32;
+            int64_t P = ((int64_t)twp[rows[k + 1]] - twp[rows[k]] + 31) / 32;
+            if (cluster) {
+                tab[k] = (int32_t)tab.size();
+                int32_t t = twp[rows[k]];
+                const int32_t end = twp[rows[k + 1]];
+                for (auto q = std::upper_bound(cut.begin(), cut.end(), t); t < end; t = *q++) tab.push_back(t);
+                P = (int64_t)tab.size() - tab[k];
+                tab.push_back(end);
+                tab[k + 1] = (int32_t)tab.size();
+            }
             Hmax = std::max(Hmax, (int)cols.size());
             Rmax = std::max(Rmax, R);
             Pmax = std::max(Pmax, (int)P);
             slot_floats = std::max(slot_floats, (int)(12 * P + 6 * R + 3) & ~3);
         }
-        const size_t rest = ((size_t)slot_floats + (size_t)HX * Hmax + 21 * (size_t)Rmax + 1) * sizeof(float);
+        const size_t rest = ((size_t)slot_floats + (size_t)HX * Hmax + 21 * (size_t)Rmax + 1 +
+                             (cluster ? Rmax : 0)) * sizeof(float);
         // a buffer for every pass where they fit (one more where their number
         // is that of the streaming buffers: the kernel tells the modes by it)
         const size_t own = (size_t)PASS_BYTES * (Pmax == SPLIT_WARPS * SPLIT_NBUF ? Pmax + 1 : Pmax);
         stage_bytes = own + rest <= (size_t)(cluster ? SMEM_CLUSTER : SMEM_MAX) ? (int)own : SPLIT_STAGE_BYTES;
         smem = stage_bytes + rest;
-        if (cluster && smem > (size_t)SMEM_CLUSTER) {  // start over as a grid over all SMs
-            cluster = false;
-            smem = SPLIT_STAGE_BYTES;
-            G = 0;
-            attempt = -1;
-            continue;
+        if (cluster) {
+            cudaLaunchAttribute at;
+            const cudaLaunchConfig_t cfg = split_cluster_config(G, smem, p->st, &at);
+            int clusters = 0;
+            if (smem > (size_t)SMEM_CLUSTER || Hmax > (int)CL_NONE || Rmax >= (int)CL_NONE ||
+                cudaOccupancyMaxActiveClusters(&clusters, k_pcg_split<true>, &cfg) != cudaSuccess || clusters < 1) {
+                cudaGetLastError();
+                cluster = false;  // no room for such a cluster: start over as a grid over all SMs
+                smem = SPLIT_STAGE_BYTES;
+                GP = 0;
+                attempt = -1;
+                continue;
+            }
         }
         if (smem > (size_t)SMEM_MAX || Hmax > 0xFFFF || Rmax > 0xFFFE) return unavailable();
-    }
-    if (cluster) {
-        cudaLaunchAttribute at;
-        const cudaLaunchConfig_t cfg = split_cluster_config(G, smem, p->st, &at);
-        int clusters = 0;
-        if (cudaOccupancyMaxActiveClusters(&clusters, k_pcg_split<true>, &cfg) != cudaSuccess || clusters < 1) {
-            cudaGetLastError();
-            cluster = false;  // no room for such a cluster: the same partition as a grid
-        }
     }
     // the occupancy at the final shared-memory size must keep the grid resident
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_pcg_split<false>, SPLIT_WARPS * 32, smem)) != cudaSuccess) return e;
@@ -1876,19 +1950,31 @@ static cudaError_t split_partition(ba_problem *p) {
     int64_t mtotal = 0;
     for (int k = 0; k < G; ++k) {
         moff[k] = (int32_t)mtotal;
-        mtotal += ((int64_t)twp[rows[k + 1]] - twp[rows[k]] + 3) & ~3;
+        mtotal += cluster ? 32LL * (tab[k + 1] - tab[k] - 1) : ((int64_t)twp[rows[k + 1]] - twp[rows[k]] + 3) & ~3;
     }
     mtotal += 4;
-    std::vector<uint32_t> meta(mtotal, 0u);
+    std::vector<uint32_t> meta(mtotal, cluster ? CL_NONE : 0u);
+    std::vector<uint32_t> src(n, ROW_EMPTY);
     for (int k = 0; k < G; ++k) {
         const int32_t *hc = hcol.data() + hptr[k];
-        const int H = hptr[k + 1] - hptr[k];
+        const int H = hptr[k + 1] - hptr[k], P = cluster ? tab[k + 1] - tab[k] - 1 : 0;
+        int32_t q = 0;  // cluster: the entry's pass
         for (int i = rows[k]; i < rows[k + 1]; ++i)
-            for (int64_t t = twp[i]; t < twp[i + 1]; ++t) {
-                const uint32_t h = (uint32_t)(std::lower_bound(hc, hc + H, twe[t].y) - hc);
-                meta[moff[k] + (t - twp[rows[k]])] = (uint32_t)(i - rows[k]) | (h << 16);
+            for (int32_t t = twp[i]; t < twp[i + 1]; ++t) {
+                const uint32_t h = (uint32_t)(std::lower_bound(hc, hc + H, twe[t].y) - hc), lr = (uint32_t)(i - rows[k]);
+                if (!cluster) {
+                    meta[moff[k] + (t - twp[rows[k]])] = lr | (h << 16);
+                    continue;
+                }
+                const int32_t *ps = tab.data() + tab[k];
+                while (t >= ps[q + 1]) ++q;
+                const bool opens = twp[i] <= ps[q], closes = twp[i + 1] >= ps[q + 1];
+                meta[moff[k] + 32 * q + (t - ps[q])] = lr | (h << 16) | (opens ? 0u : (closes ? 0x8000u : 0x80000000u));
+                if (t == twp[i]) src[i] = (uint32_t)(opens ? 12 * q : (closes ? 12 * q + 6 : 12 * P + 6 * (int)lr));
+                else if (t == ps[q]) src[i] += 1u << 16;
             }
     }
+    if (cluster) tab.insert(tab.end(), src.begin(), src.end());
     std::vector<std::pair<void **, std::pair<const void *, size_t>>> up = {
         {(void **)&p->tws_ptr, {twp.data(), twp.size() * sizeof(int32_t)}},
         {(void **)&p->tws_ent, {twe.data(), twe.size() * sizeof(int2)}},
@@ -1897,7 +1983,8 @@ static cudaError_t split_partition(ba_problem *p) {
         {(void **)&p->meta_off, {moff.data(), moff.size() * sizeof(int32_t)}},
         {(void **)&p->halo_ptr, {hptr.data(), hptr.size() * sizeof(int32_t)}},
         {(void **)&p->halo_col, {hcol.data(), std::max<size_t>(hcol.size(), 1) * sizeof(int32_t)}},
-        {(void **)&p->own_base, {obase.data(), obase.size() * sizeof(int32_t)}}};
+        {(void **)&p->own_base, {obase.data(), obase.size() * sizeof(int32_t)}},
+        {(void **)&p->pass_tab, {tab.data(), tab.size() * sizeof(int32_t)}}};
     for (auto &u : up) {
         void *d = nullptr;
         if ((e = cudaMalloc(&d, u.second.second)) != cudaSuccess) return e;
@@ -1957,7 +2044,7 @@ cudaError_t launch_pcg_split(ba_problem *p) {
     p->test_wait_limit = 0;
     {
         const int *cr = p->cta_rows, *twp = p->tws_ptr, *mo = p->meta_off, *hp = p->halo_ptr, *hc = p->halo_col,
-                  *ob = p->own_base;
+                  *ob = p->own_base, *pt = p->pass_tab;
         const uint32_t *meta = p->tw_meta;
         int sf = p->split_slot_floats, stf = p->split_stage_floats;
         const float *Sh = p->Sh, *H = p->Hs, *Shd = p->Shd;
@@ -1970,7 +2057,7 @@ cudaError_t launch_pcg_split(ba_problem *p) {
         unsigned *bar = p->ar_bar;
         long long limit = test_limit > 0 ? test_limit : 4000000000LL;  // ~2 s of SM clock per wait
         int short_by = test_limit > 0 ? 1 : 0;
-        void *args[] = {&cr, &twp, &meta, &mo, &hp, &hc, &ob, &sf, &stf, &Sh, &H, &Shd, &ident, &x, &pp, &rec0, &rec1, &sc,
+        void *args[] = {&cr, &twp, &meta, &mo, &hp, &hc, &ob, &pt, &sf, &stf, &Sh, &H, &Shd, &ident, &x, &pp, &rec0, &rec1, &sc,
                         &red, &bar, &limit, &short_by};
         if (p->split_cluster) {
             cudaLaunchAttribute at;

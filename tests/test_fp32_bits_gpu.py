@@ -14,6 +14,7 @@ import numpy as np
 import pytest
 
 import scenes
+from test_pcg_sizes_gpu import banded_pattern
 
 pytestmark = pytest.mark.gpu
 
@@ -63,3 +64,72 @@ def formed(B, kind, size, seed):
 @pytest.mark.parametrize("kind,size,seed", list(FORMED))
 def test_formed_system(B, kind, size, seed):
     assert formed(B, kind, size, seed) == FORMED[kind, size, seed]
+
+
+SOLVED = {
+    (1, 1): "6b60bac415ca7841",
+    (2, 1): "81bce8132a56b548",
+    (24, 23): "9b64ab87d92c6a6b",
+    (60, 59): "0f582ece9e37bb23",
+    (128, 58): "c9216e937f2322e1",
+    (160, 75): "f11d1d32d91d7a0f",
+    (200, 33): "e2d9e2800fe43be4"}
+
+
+def integer_system(row_ptr, col, cdim, seed):
+    """Values and right-hand side of few bits: off-diagonal entries k / 16, |k| <= 8,
+    diagonal blocks symmetric with a diagonal above the sums of their rows."""
+    rng = np.random.default_rng(seed)
+    row = np.repeat(np.arange(len(cdim)), np.diff(row_ptr))
+    blocks, total = [], np.zeros(len(cdim), np.int64)
+    for i, j in zip(row, col):
+        k = rng.integers(-8, 9, (cdim[i], cdim[j]))
+        blocks.append(np.tril(k) + np.tril(k, -1).T if i == j else k)
+        total[i] += np.abs(k).sum(1).max()
+        if i != j:
+            total[j] += np.abs(k).sum(0).max()
+    for i in range(len(cdim)):
+        k = row_ptr[i]
+        d = blocks[k] - np.diag(np.diag(blocks[k]))
+        blocks[k] = d + np.diag(total[i] + np.abs(d).sum(1) + rng.integers(1, 40, cdim[i]))
+    val = np.concatenate([k.reshape(-1) for k in blocks]) / 16.0
+    return val, rng.integers(-200, 201, int(np.sum(cdim))) / 16.0
+
+
+def solved(B, n, half):
+    row_ptr, col = banded_pattern(n, half)
+    val, b = integer_system(row_ptr, col, np.full(n, 6, np.int32), 9600 + n)
+    g = B.Problem.from_rcs(row_ptr, col, val.reshape(-1, 6, 6), b.reshape(n, 6), precision=B.BA_FP32, pcg_rel_tol=1e-6)
+    out = [g.solve_rcs()[0]["pcg_iters"], g.step()[0]]
+    g.close()
+    return digest(*out)
+
+
+@pytest.mark.parametrize("n,half", list(SOLVED))
+def test_solved_system(B, n, half):
+    assert solved(B, n, half) == SOLVED[n, half]
+
+
+STEPPED = {
+    ("ring", 8, 1, 1e-2): "0565fe2ffdcc72e1",
+    ("ring", 16, 2, 1e-2): "5f09f9b988710b05",
+    ("ring", 40, 5, 1e-2): "0feb3c9e1128c962",
+    ("aerial", 8, 3, 0.1): "35d00e0f43339726",
+    ("aerial", 12, 6, 0.1): "328506db7bfe5236",
+    ("aerial", 20, 7, 0.1): "61170a5853468066",
+    ("aerial", 30, 8, 0.1): "d23b1b022fb034cf"}
+
+
+def stepped(B, kind, size, seed, tol):
+    g = adjustment(B, kind, size, seed, pcg_rel_tol=tol)
+    out = []
+    for _ in range(3):
+        info = g.lm_step()
+        out += [info["pcg_iters"], info["accepted"], info["cost_after"], *g.step()]
+    g.close()
+    return digest(*out)
+
+
+@pytest.mark.parametrize("kind,size,seed,tol", list(STEPPED))
+def test_lm_steps(B, kind, size, seed, tol):
+    assert stepped(B, kind, size, seed, tol) == STEPPED[kind, size, seed, tol]
