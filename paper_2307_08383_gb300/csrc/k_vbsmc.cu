@@ -23,20 +23,28 @@
 
 namespace ba {
 
-// One part of a row's product.  The warp's lanes form G = min(32 / c_i, 5)
-// groups of c_i lanes; group g takes entries e0 + g, e0 + g + step, ... below
+// One part of a row's product.  The warp's lanes form G groups of c_i lanes
+// (at most min(32 / c_i, 5)); group g takes entries e0 + g, e0 + g + step, ... below
 // e1, its lane a component a of the row.  The group stages the entry's c_j
 // values of x (each formed once, gx(index)) in the warp's shared memory sx and
 // holds the lane's row (or column) of the block in registers, so an entry
 // costs c_j multiply-adds per lane and one evaluation of x per value.  An
 // entry's record rec[e] is (value offset lo / hi, vector offset of j,
-// c_j << 1 | transposed).  PACKED: every block lies in shared memory stored by
-// columns of this row's form (element (a, c) at offset + c c_i + a).
-// Lanes 0 .. c_i - 1 return the part's sum.
+// c_j << 1 | transposed).  Lanes 0 .. c_i - 1 return the part's sum.
 // (The first version gave every entry 16 lanes, evaluated x in each of them
 // and ran 16 columns whatever c_j: in FP64, where a warp instruction takes 16
 // cycles of its SM, 32 per pair of entries instead of 12 at c = 11.)
 constexpr int VB_GROUPS = 5;
+// The PCG's row products: FP32 always in two groups (every c_i <= 16 allows
+// them), so that the order of a row's additions does not depend on c_i and an
+// FP32 system with six-unknown cameras keeps the bits of its iterates, on which
+// an LM trajectory rests (1,984 cameras, half of them c = 6: 24.1 us per iteration,
+// 22.8 with as many groups as fit; nothing to lose at c = 11); FP64 in as many as
+// fit (its issue rate is the limit).
+template <typename T>
+__host__ __device__ constexpr int vb_pcg_groups(int ci) {
+    return 32 / ci < (sizeof(T) == 4 ? 2 : VB_GROUPS) ? 32 / ci : (sizeof(T) == 4 ? 2 : VB_GROUPS);
+}
 // One entry's row (or column) of values in registers, zero beyond c_j.
 template <typename T>
 __device__ __forceinline__ void vb_load(int ci, int a, const int4 in, const T *__restrict__ val, T (&bv)[BA_VB_CMAX]) {
@@ -57,10 +65,10 @@ __device__ __forceinline__ T vb_join(T acc, int ci, int G, int a) {
     return tot;
 }
 template <typename T, class GX>
-__device__ __forceinline__ T vb_part(int ci, int e0, int e1, int step, const int4 *__restrict__ rec,
+__device__ __forceinline__ T vb_part(int ci, int G, int e0, int e1, int step, const int4 *__restrict__ rec,
                                      const T *__restrict__ val, T *sx, GX gx) {
     const int lane = threadIdx.x & 31;
-    const int G = min(32 / ci, VB_GROUPS), g = lane / ci, a = lane - g * ci;
+    const int g = lane / ci, a = lane - g * ci;
     T acc = T(0);
     for (int t = e0; t < e1; t += step) {
         const int e = t + g;
@@ -89,7 +97,7 @@ template <typename T, bool PACKED>
 __device__ __forceinline__ T vb_own_part(int ci, int e0, int e1, int step, const int4 *rec, const T *val,
                                          const T *sx) {
     const int lane = threadIdx.x & 31;
-    const int G = min(32 / ci, VB_GROUPS), g = lane / ci, a = lane - g * ci;
+    const int G = vb_pcg_groups<T>(ci), g = lane / ci, a = lane - g * ci;
     T acc = T(0);
     // all of a pass's loads are issued before its multiply-adds (columns beyond
     // c_j read as zeros; FP32 multiplies them, FP64 stops at the warp's
@@ -175,7 +183,7 @@ __global__ void __launch_bounds__(256) k_vb_spmv(int n, int wpr, const int *__re
         if (i < n) {
             ci = __ldg(cdim + i);
             const int G = min(32 / ci, VB_GROUPS), e0 = __ldg(tw_ptr + i), e1 = __ldg(tw_ptr + i + 1);
-            const T t = vb_part<T>(ci, e0 + part * G, e1, wpr * G, tw_info, val, s_x[w],
+            const T t = vb_part<T>(ci, G, e0 + part * G, e1, wpr * G, tw_info, val, s_x[w],
                                           [&](int k) { return __ldg(x + k); });
             if (wpr == 1) {
                 if (lane < ci) y[__ldg(off + i) + lane] = t;
@@ -447,7 +455,7 @@ __global__ void __launch_bounds__(vb_own_threads<T>(), 1)
         }
         __syncthreads();
         for (int u = w; u < units; u += W) {
-            const int lr = u / pl.wpr, ci = s_c[lr], G = min(32 / ci, VB_GROUPS);
+            const int lr = u / pl.wpr, ci = s_c[lr], G = vb_pcg_groups<T>(ci);
             const T t = vb_own_part<T, PACKED>(ci, s_e[lr] + (u - lr * pl.wpr) * G, s_e[lr + 1], pl.wpr * G, s_rec,
                                                PACKED ? s_val : val, s_x);
             if (lane < ci) s_part[u * BA_VB_CMAX + lane] = t;
@@ -576,8 +584,8 @@ __global__ void __launch_bounds__(256) k_vb_pcg(int n, int N, const int *__restr
         T pap_t = T(0);
         for (int i = tid >> 5; i < n; i += nw) {
             const int ci = __ldg(cdim + i), lane = threadIdx.x & 31;
-            const T v = vb_part<T>(ci, __ldg(tw_ptr + i), __ldg(tw_ptr + i + 1), min(32 / ci, VB_GROUPS),
-                                          tw_info, val, s_x[threadIdx.x >> 5], dir);
+            const int G = vb_pcg_groups<T>(ci);
+            const T v = vb_part<T>(ci, G, __ldg(tw_ptr + i), __ldg(tw_ptr + i + 1), G, tw_info, val, s_x[threadIdx.x >> 5], dir);
             if (lane < ci) {
                 const int idx = __ldg(off + i) + lane;
                 const T dv = dir(idx);
@@ -705,7 +713,7 @@ bool vb_own_plan(const ba_vbsmc *h, int n_sm, VbPlan *pl, int *grid, int *thread
     }
     const int nt = vb_own_threads<T>(), W = nt / 32;
     if (max_vec > nt) return false;
-    const int G = std::max(1, std::min(32 / std::max(1, h->max_dim), VB_GROUPS));
+    const int G = vb_pcg_groups<T>(std::max(1, h->max_dim));
     // FP32: one warp per row (a row's sum keeps its order, and more warps gained
     // 3 us of 10 at 120 cameras, nothing from 990 on); FP64: the split with the
     // fewest passes (18.3, 13.5, 11.2, 10.9 us per iteration with 1, 2, 4, 8

@@ -15,6 +15,7 @@ import pytest
 
 import scenes
 from test_pcg_sizes_gpu import banded_pattern
+from test_vb_sizes_gpu import sizes
 
 pytestmark = pytest.mark.gpu
 
@@ -133,3 +134,53 @@ def stepped(B, kind, size, seed, tol):
 @pytest.mark.parametrize("kind,size,seed,tol", list(STEPPED))
 def test_lm_steps(B, kind, size, seed, tol):
     assert stepped(B, kind, size, seed, tol) == STEPPED[kind, size, seed, tol]
+
+
+VARIABLE = {
+    (40, 30, "any"): "3bab62ea3c32c13e",
+    (90, 12, "6"): "c089feef167bdc76",
+    (330, 9, "mixed"): "00b12007f81d0148",
+    (700, 22, "mixed"): "a964c4219b711fb8",
+    (400, 5, "any"): "5b93de694b78c5ed",
+    (60, 20, "16"): "7435aab8a39ddd9d",
+    (3000, 4, "1"): "aadc50e04a404946",
+    (5200, 1, "any"): "d6fd02df987c0560"}
+
+
+def variable(B, n, half, kind):
+    row_ptr, col = banded_pattern(n, half)
+    cdim = sizes(kind, n, 77 + n)
+    val, b = integer_system(row_ptr, col, cdim, 9700 + n)
+    g = B.VBSMC(cdim, row_ptr, col, val, b, precision=B.BA_FP32)
+    x, its = g.solve(1e-5)[:2]
+    g.close()
+    return digest(its, x)
+
+
+@pytest.mark.parametrize("n,half,kind", list(VARIABLE))
+def test_variable_size_system(B, n, half, kind):
+    assert variable(B, n, half, kind) == VARIABLE[n, half, kind]
+
+
+INTERIORS = {
+    (5, 4, 0.5, 1): "cd94822313b22174",
+    (8, 5, 0.1, 2): "7a12002e595f49d3",
+    (12, 6, 1.0, 3): "63c87248ade01d32"}
+
+
+def interiors(B, along, across, frac, seed):
+    s = scenes.aerial_small(along, across, pts_per_cam=60, seed=9800 + seed)
+    intr = rounded(scenes.interiors0(s.n_cams, seed=seed), 20)
+    g = B.VBIProblem(rounded(s.cams0, 20), intr, scenes.block_sizes(s.n_cams, frac, seed), rounded(s.pts0, 20), s.obs_cam,
+                     s.obs_pt, rounded(s.obs_uv, 10), precision=B.BA_FP32, pcg_rel_tol=0.1)
+    out = []
+    for _ in range(2):
+        info = g.lm_step()
+        out += [info["pcg_iters"], info["accepted"], info["cost_after"], *g.step()]
+    g.close()
+    return digest(*out)
+
+
+@pytest.mark.parametrize("along,across,frac,seed", list(INTERIORS))
+def test_lm_steps_with_interiors(B, along, across, frac, seed):
+    assert interiors(B, along, across, frac, seed) == INTERIORS[along, across, frac, seed]
