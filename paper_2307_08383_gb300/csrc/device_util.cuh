@@ -108,6 +108,17 @@ __device__ __forceinline__ double widen(float f) {
 }
 __device__ __forceinline__ double widen(double d) { return d; }
 
+// a / b in two steps after the reciprocal inv = 1 / b (correctly rounded, formed
+// before a is known or for several a): the quotient's remainder is exact and the
+// correction leaves it correctly rounded (Markstein, IBM J. Res. Dev. 34, 1990).
+// Where the reciprocal or the remainder leaves the normal range, the division.
+__device__ __forceinline__ double quotient(double a, double b, double inv) {
+    const double q = a * inv, r = fma(-q, b, a);
+    const double m = fabs(b);
+    if (!(m > 1e-150 && m < 1e150 && fabs(q) > 1e-100 && fabs(q) < 1e100)) return a / b;
+    return fma(r, inv, q);
+}
+
 // Cholesky of symmetric 6x6 matrices, eight lanes each (lane r < 6 of a group
 // holds row r in a; lanes 6 and 7 hold zeros): on return a holds row r of L
 // (columns k <= r), x column r of L^-1 (rows k >= r, zeros above), and the
@@ -127,9 +138,10 @@ __device__ __forceinline__ bool chol6_lanes(T (&a)[6], T (&x)[6]) {
             ok = false;
             p = T(1);
         }
-        const T s = sqrt(p), inv = T(1) / s;
-        if (r == q) invd = inv;
-        a[q] = r == q ? s : a[q] * inv;
+        // one division for the column and for the pivot's reciprocal
+        const T s = sqrt(p), v = (r == q ? T(1) : a[q]) / s;
+        if (r == q) invd = v;
+        a[q] = r == q ? s : v;
 #pragma unroll
         for (int k = q + 1; k < 6; ++k) a[k] -= a[q] * __shfl_sync(FULL, a[q], k, 8);  // rows r >= k are meant
     }

@@ -550,7 +550,7 @@ __global__ void __launch_bounds__(32 * RES64_WARPS, 1)
                     sc->done = 1;
                 }
             }
-            beta = v2[0] * inv_rz;
+            beta = quotient(v2[0], rz, inv_rz);
             rz = v2[0];
             if (lane == 0) {
                 s_ctl = ctl;

@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(64) k_vb_minv(int n, const int *__restrict__ c
         }
         const double d = sqrt(p), inv = 1.0 / d;
         if (r == q) invd = inv;
-        A[q] = r == q ? d : A[q] * inv;
+        A[q] = r == q ? d : quotient(A[q], d, inv);
 #pragma unroll
         for (int k = q + 1; k < CM; ++k) {
             if (k >= cm) break;
@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(64) k_vb_minv(int n, const int *__restrict__ c
             double s = r == q ? 1.0 : 0.0;
 #pragma unroll
             for (int k = 0; k < q; ++k) s -= __shfl_sync(FULL, A[k], q, 16) * x[k];
-            x[q] = s * __shfl_sync(FULL, invd, q, 16);
+            x[q] = quotient(s, __shfl_sync(FULL, A[q], q, 16), __shfl_sync(FULL, invd, q, 16));
         }
     }
 #pragma unroll
@@ -261,7 +261,7 @@ __global__ void __launch_bounds__(64) k_vb_minv(int n, const int *__restrict__ c
 #pragma unroll
             for (int k = q + 1; k < CM; ++k)
                 if (k < cm) s -= __shfl_sync(FULL, A[q], k, 16) * x[k];
-            x[q] = s * __shfl_sync(FULL, invd, q, 16);
+            x[q] = quotient(s, __shfl_sync(FULL, A[q], q, 16), __shfl_sync(FULL, invd, q, 16));
         }
     }
     if (!ok && r == 0) atomicExch(err, (int)BA_ERR_NOT_SPD);
