@@ -35,12 +35,14 @@ namespace ba {
 // and ran 16 columns whatever c_j: in FP64, where a warp instruction takes 16
 // cycles of its SM, 32 per pair of entries instead of 12 at c = 11.)
 constexpr int VB_GROUPS = 5;
-// The PCG's row products: FP32 always in two groups (every c_i <= 16 allows
+// The row products of the owning PCG (k_vb_pcg_own): FP32 always in two groups (every c_i <= 16 allows
 // them), so that the order of a row's additions does not depend on c_i and an
 // FP32 system with six-unknown cameras keeps the bits of its iterates, on which
 // an LM trajectory rests (1,984 cameras, half of them c = 6: 24.1 us per iteration,
 // 22.8 with as many groups as fit; nothing to lose at c = 11); FP64 in as many as
-// fit (its issue rate is the limit).
+// fit (its issue rate is the limit).  k_vb_pcg, for larger systems, takes as many
+// as fit in both (20,000 cameras of c = 6, FP32: 460 us for four iterations, 884
+// with two).
 template <typename T>
 __host__ __device__ constexpr int vb_pcg_groups(int ci) {
     return 32 / ci < (sizeof(T) == 4 ? 2 : VB_GROUPS) ? 32 / ci : (sizeof(T) == 4 ? 2 : VB_GROUPS);
@@ -584,7 +586,7 @@ __global__ void __launch_bounds__(256) k_vb_pcg(int n, int N, const int *__restr
         T pap_t = T(0);
         for (int i = tid >> 5; i < n; i += nw) {
             const int ci = __ldg(cdim + i), lane = threadIdx.x & 31;
-            const int G = vb_pcg_groups<T>(ci);
+            const int G = min(32 / ci, VB_GROUPS);
             const T v = vb_part<T>(ci, G, __ldg(tw_ptr + i), __ldg(tw_ptr + i + 1), G, tw_info, val, s_x[threadIdx.x >> 5], dir);
             if (lane < ci) {
                 const int idx = __ldg(off + i) + lane;
