@@ -291,10 +291,6 @@ __global__ void __launch_bounds__(64) k_vb_minv(int n, const int *__restrict__ c
 // 115 -> 50 at 1,984 (values in L2); FP32 32 -> 10.3 at 120, 33.4 -> 13.7 at
 // 990 (22 with the neighbours' values gathered pass by pass), 38.7 -> 22.5 at
 // 1,984 (values in L2).
-struct VbPlan {
-    int rows, wpr, max_ent;  // rows per CTA; warps per row; longest entry list of a CTA
-    int64_t max_val;         // PACKED: largest value count of a CTA
-};
 template <typename T>
 __host__ __device__ constexpr size_t vb_own_smem(int rows, int wpr, int max_ent, int64_t max_val, int threads) {
     return (size_t)max_ent * sizeof(int4) +
@@ -692,30 +688,35 @@ cudaError_t vb_spmv_T(ba_vbsmc *h, const T *x, T *y) {
 
 // The owning kernel's launch shape: rows spread over every SM; 8 warps per CTA
 // in FP64 (its FP64 issue is the limit), 16 in FP32.
-// False when a CTA would own more entries than threads or its records and
-// vectors do not fit in shared memory.
+// Not taken (grid 0) when a CTA would own more entries than threads or its
+// records and vectors do not fit in shared memory.
 constexpr size_t VB_SMEM_MAX = 225 * 1024;
 template <typename T>
-bool vb_own_plan(const ba_vbsmc *h, int n_sm, VbPlan *pl, int *grid, int *threads, size_t *smem, bool *packed) {
-    const int n = h->n, R = (n + n_sm - 1) / n_sm;
-    int max_ent = 0, max_vec = 0, row_ent = 0;
+VbPlan vb_own_plan(int n, int n_sm, const int32_t *cdim, const std::vector<int32_t> &tw_ptr,
+                   const std::vector<int4> &tw_info) {
+    const int R = (n + n_sm - 1) / n_sm;
+    int max_ent = 0, max_vec = 0, row_ent = 0, max_dim = 1;
     int64_t max_val = 0;
     for (int r0 = 0; r0 < n; r0 += R) {
         int ent = 0, vec = 0;
         int64_t val = 0;
         for (int i = r0; i < std::min(n, r0 + R); ++i) {
-            ent += h->row_ent[i];
-            val += h->row_val[i];
-            vec += h->row_dim[i];
-            row_ent = std::max(row_ent, h->row_ent[i]);
+            int64_t cols = 0;
+            for (int32_t t = tw_ptr[i]; t < tw_ptr[i + 1]; ++t) cols += tw_info[t].w >> 1;
+            ent += tw_ptr[i + 1] - tw_ptr[i];
+            val += cols * cdim[i];
+            vec += cdim[i];
+            row_ent = std::max(row_ent, tw_ptr[i + 1] - tw_ptr[i]);
+            max_dim = std::max(max_dim, cdim[i]);
         }
         max_ent = std::max(max_ent, ent);
         max_vec = std::max(max_vec, vec);
         max_val = std::max(max_val, val);
     }
     const int nt = vb_own_threads<T>(), W = nt / 32;
-    if (max_vec > nt) return false;
-    const int G = vb_pcg_groups<T>(std::max(1, h->max_dim));
+    VbPlan pl;
+    if (max_vec > nt) return pl;
+    const int G = vb_pcg_groups<T>(max_dim);
     // FP32: one warp per row (a row's sum keeps its order, and more warps gained
     // 3 us of 10 at 120 cameras, nothing from 990 on); FP64: the split with the
     // fewest passes (18.3, 13.5, 11.2, 10.9 us per iteration with 1, 2, 4, 8
@@ -728,18 +729,22 @@ bool vb_own_plan(const ba_vbsmc *h, int n_sm, VbPlan *pl, int *grid, int *thread
             best_cost = cost;
         }
     }
-    *packed = max_val < (1 << 22) && vb_own_smem<T>(R, best, max_ent, max_val, nt) <= VB_SMEM_MAX;
-    *smem = vb_own_smem<T>(R, best, max_ent, *packed ? max_val : 0, nt);
-    if (*smem > VB_SMEM_MAX) return false;
-    *pl = VbPlan{R, best, max_ent, *packed ? max_val : 0};
-    *grid = (n + R - 1) / R;
-    *threads = nt;
-    return true;
+    pl.packed = max_val < (1 << 22) && vb_own_smem<T>(R, best, max_ent, max_val, nt) <= VB_SMEM_MAX;
+    pl.smem = vb_own_smem<T>(R, best, max_ent, pl.packed ? max_val : 0, nt);
+    if (pl.smem > VB_SMEM_MAX) return pl;
+    pl.rows = R;
+    pl.wpr = best;
+    pl.max_ent = max_ent;
+    pl.max_val = pl.packed ? max_val : 0;
+    pl.grid = (n + R - 1) / R;
+    pl.threads = nt;
+    return pl;
 }
 
 template <typename T>
-cudaError_t vb_pcg_own(ba_vbsmc *h, VbPlan pl, int grid, int threads, size_t smem, bool packed, long long limit) {
-    const void *k = packed ? (const void *)k_vb_pcg_own<T, true> : (const void *)k_vb_pcg_own<T, false>;
+cudaError_t vb_pcg_own(ba_vbsmc *h, long long limit) {
+    VbPlan pl = h->plan;
+    const void *k = pl.packed ? (const void *)k_vb_pcg_own<T, true> : (const void *)k_vb_pcg_own<T, false>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)VB_SMEM_MAX);
     if (e != cudaSuccess) return e;
     int n = h->n;
@@ -752,7 +757,7 @@ cudaError_t vb_pcg_own(ba_vbsmc *h, VbPlan pl, int grid, int threads, size_t sme
     double *red = h->red;
     unsigned *bar = h->bar;
     void *args[] = {&n, &pl, &cd, &of, &ec, &twp, &twi, &val, &mo, &Mi, &b, &y, &z, &d0, &d1, &sc, &red, &bar, &limit};
-    return cudaLaunchCooperativeKernel(k, dim3(grid), dim3(threads), args, smem, h->st);
+    return cudaLaunchCooperativeKernel(k, dim3(pl.grid), dim3(pl.threads), args, pl.smem, h->st);
 }
 
 template <typename T>
@@ -762,14 +767,7 @@ cudaError_t vb_pcg_T(ba_vbsmc *h) {
     if (e != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(h->bar, 0, AR_SUB * 32 * sizeof(unsigned), h->st)) != cudaSuccess) return e;
     long long limit = 4000000000LL;  // ~2 s of SM clock per grid wait
-    {
-        VbPlan pl;
-        int grid = 0, threads = 0;
-        size_t smem = 0;
-        bool packed = false;
-        if (vb_own_plan<T>(h, n_sm, &pl, &grid, &threads, &smem, &packed))
-            return vb_pcg_own<T>(h, pl, grid, threads, smem, packed, limit);
-    }
+    if (h->plan.grid > 0) return vb_pcg_own<T>(h, limit);
     if (per_sm > 2) per_sm = 2;
     if (per_sm < 1) return cudaErrorCooperativeLaunchTooLarge;
     const int64_t want = std::max<int64_t>(((int64_t)h->n * 32 + 255) / 256, (h->N + 255) / 256);
@@ -862,16 +860,6 @@ ba_status vb_build(const ba_options &o, int32_t n, const int32_t *cdim, int64_t 
     h->esz = h->fp32 ? 4 : 8;
     h->st = (cudaStream_t)o.cuda_stream;
     h->cap = o.device_mem_cap;
-    h->row_ent.resize(n);
-    h->row_val.resize(n);
-    h->row_dim.assign(cdim, cdim + n);
-    for (int32_t i = 0; i < n; ++i) {
-        h->row_ent[i] = tw_ptr[i + 1] - tw_ptr[i];
-        h->max_dim = std::max(h->max_dim, cdim[i]);
-        int64_t v = 0;
-        for (int32_t t = tw_ptr[i]; t < tw_ptr[i + 1]; ++t) v += tw_info[t].w >> 1;
-        h->row_val[i] = v * cdim[i];
-    }
     auto up = [&](void **d, const void *src, size_t bytes) -> ba_status {
         ba_status r = vb_alloc(h, d, bytes);
         if (r) return r;
@@ -880,6 +868,12 @@ ba_status vb_build(const ba_options &o, int32_t n, const int32_t *cdim, int64_t 
     std::vector<int32_t> brow(nnzb);
     for (int32_t i = 0; i < n; ++i)
         for (int32_t k = row_ptr[i]; k < row_ptr[i + 1]; ++k) brow[k] = i;
+    int dev = 0, n_sm = 0;
+    if (!s) s = vb_cuda(h, cudaGetDevice(&dev), "device");
+    if (!s) s = vb_cuda(h, cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev), "device");
+    if (!s)
+        h->plan = h->fp32 ? vb_own_plan<float>(n, n_sm, cdim, tw_ptr, tw_info)
+                          : vb_own_plan<double>(n, n_sm, cdim, tw_ptr, tw_info);
     if (!s) s = up((void **)&h->cdim, cdim, n * sizeof(int32_t));
     if (!s) s = up((void **)&h->off, off.data(), (n + 1) * sizeof(int32_t));
     if (!s) s = up((void **)&h->row_ptr, row_ptr, (n + 1) * sizeof(int32_t));

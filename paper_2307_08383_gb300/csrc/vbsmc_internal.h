@@ -18,6 +18,15 @@ struct VbScalars {
     int iters, done, max_iters, err;
 };
 
+// Launch shape of the PCG whose CTAs own their rows (grid 0: not taken).
+struct VbPlan {
+    int rows = 0, wpr = 1, max_ent = 0;  // rows per CTA; warps per row; longest entry list of a CTA
+    int64_t max_val = 0;                 // values in shared memory: largest value count of a CTA, else 0
+    int grid = 0, threads = 0;
+    size_t smem = 0;
+    bool packed = false;
+};
+
 }  // namespace ba
 
 struct ba_vbsmc {
@@ -36,10 +45,7 @@ struct ba_vbsmc {
     double *red = nullptr;
     unsigned *bar = nullptr;
     int *err = nullptr;
-    // per block row: two-sided entries, their values, unknowns (launch shapes)
-    std::vector<int32_t> row_ent, row_dim;
-    std::vector<int64_t> row_val;
-    int max_dim = 0;
+    ba::VbPlan plan;  // of the PCG, made with the layout
     std::vector<void *> allocs;
     cudaEvent_t ev[2] = {nullptr, nullptr};
 };
