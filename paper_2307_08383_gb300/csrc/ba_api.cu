@@ -294,7 +294,13 @@ ba_status ba_problem_create(const ba_options *opt, int32_t n_cams, const double 
     // error of an LM step's cost grew by 1.7).
     int target = p->obs_max;
     if (o.group_max_obs <= 0 && !p->fp32) {
-        const int64_t slots = 152, rounds = (m + slots * p->obs_max - 1) / (slots * p->obs_max);
+        int dev = 0, n_sm = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n_sm < 1) {
+            cudaGetLastError();  // (no device: the allocations below say so)
+            n_sm = 152;
+        }
+        const int64_t slots = n_sm, rounds = (m + slots * p->obs_max - 1) / (slots * p->obs_max);
         target = (int)std::min<int64_t>(p->obs_max, std::max<int64_t>(40, (m + slots * rounds - 1) / (slots * rounds) + 8));
     }
     const size_t camc_w = p->fp32 ? CAMC32_W * 4 : 12 * 8;
