@@ -220,6 +220,7 @@ struct ba_problem {
     int32_t *pass_tab = nullptr;   // cluster: the CTAs' passes (offsets, then first entries)
     int split_grid = 0;            // 0: not partitioned yet, < 0: unavailable
     bool split_cluster = false;    // the grid runs as one thread-block cluster
+    bool split_row_starts = true;  // the rows' starts fit in shared memory
     int split_slot_floats = 0, split_stage_floats = 0;
     size_t split_smem = 0;
     double ph_sum[4] = {};  // split CG phase totals over solves (profile >= 2)

@@ -946,7 +946,8 @@ __device__ __forceinline__ void split_drain(const SplitPipe &pp, long long limit
 // One sweep of the warp's passes over the halo vectors hx.  False on an
 // mbarrier timeout (then the warp stops; callers agree CTA-wide with
 // __syncthreads_and and leave).
-__device__ __forceinline__ bool split_passes(SplitPipe &pp, const int *row_ent, const float *hx,
+template <class RE>
+__device__ __forceinline__ bool split_passes(SplitPipe &pp, RE row_ent, const float *hx,
                                              float *slot, float *rowacc, int *err, long long limit) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     for (int k = 0; k < pp.m; ++k) {
@@ -1004,7 +1005,7 @@ __device__ __forceinline__ bool split_passes(SplitPipe &pp, const int *row_ent, 
             if (table) {
                 dst = md >> 31 ? rowacc + 6 * lr : slot + 12 * q + ((md & 0x8000u) ? 6 : 0);
             } else {
-                const int rs = row_ent[lr], rend = row_ent[lr + 1];
+                const int rs = row_ent(lr), rend = row_ent(lr + 1);
                 dst = rs <= ps ? slot + 12 * q : (rend >= pe ? slot + 12 * q + 6 : rowacc + 6 * lr);
             }
 #pragma unroll
@@ -1165,7 +1166,8 @@ __device__ __forceinline__ bool cluster_allreduce_df(df32 (&v)[NV], ClusterSlots
 // residual norm ||H r^|| (block-Jacobi: ||L r^||).  One grid all-reduce of
 // (gamma, delta, ||H r||^2) ends each phase; with CLUSTER the grid is one
 // thread-block cluster and the all-reduce stays in its shared memory.
-template <bool CLUSTER>
+// ROWS: the rows' starts in shared memory (the grid's, where they fit).
+template <bool CLUSTER, bool ROWS>
 __global__ void __launch_bounds__(SPLIT_WARPS * 32, SPLIT_CTAS_PER_SM) k_pcg_split(const int *__restrict__ cta_rows, const int *__restrict__ tw_ptr,
                                                       const uint32_t *__restrict__ tw_meta,
                                                       const int *__restrict__ meta_off,
@@ -1198,13 +1200,15 @@ __global__ void __launch_bounds__(SPLIT_WARPS * 32, SPLIT_CTAS_PER_SM) k_pcg_spl
     const int pt0 = CLUSTER ? __ldg(pass_tab + blockIdx.x) : 0;
     const int R = re - rb, wid = threadIdx.x >> 5;
     const int P = CLUSTER ? __ldg(pass_tab + blockIdx.x + 1) - pt0 - 1 : (ee - eb + 31) >> 5;
-    // dynamic shared memory: copy buffers | slots + row sums | halo | own records | row starts |
-    // (CLUSTER) rows' sums (split_combine)
+    // dynamic shared memory: copy buffers | slots + row sums | halo | own records | row
+    // starts (ROWS) or, CLUSTER, rows' sums (split_combine)
     float *slot = sdyn + stage_floats, *rowacc = slot + 12 * P;
     float *hx = slot + slot_floats, *own = hx + HX * NH;
     int *s_row = reinterpret_cast<int *>(own + 20 * R);  // first entry of each of the CTA's rows, and the end
-    uint32_t *s_src = reinterpret_cast<uint32_t *>(s_row + R + 1);
-    for (int q = threadIdx.x; q <= R; q += blockDim.x) s_row[q] = __ldg(tw_ptr + rb + q);
+    uint32_t *s_src = reinterpret_cast<uint32_t *>(own + 20 * R);
+    if (ROWS)
+        for (int q = threadIdx.x; q <= R; q += blockDim.x) s_row[q] = __ldg(tw_ptr + rb + q);
+    auto row_ent = [&](int lr) { return ROWS ? s_row[lr] : __ldg(tw_ptr + rb + lr); };
     if (CLUSTER) {
         const int *src = pass_tab + __ldg(pass_tab + gridDim.x) + rb;  // behind the lists
         for (int q = threadIdx.x; q < R; q += blockDim.x) s_src[q] = (uint32_t)__ldg(src + q);
@@ -1294,7 +1298,7 @@ __global__ void __launch_bounds__(SPLIT_WARPS * 32, SPLIT_CTAS_PER_SM) k_pcg_spl
         split_halo_fetch(halo_col, hb, NH, hj0, rec0, hx);
         split_halo_apply(NH, ob, R, true, 0.f, 0.f, hx, own);
         __syncthreads();
-        const bool ok = __syncthreads_and(split_passes(pp, s_row, hx, slot, rowacc, &sc->err, limit_cycles));
+        const bool ok = __syncthreads_and(split_passes(pp, row_ent, hx, slot, rowacc, &sc->err, limit_cycles));
         if (!ok) {
             leave();
             return;
@@ -1302,7 +1306,7 @@ __global__ void __launch_bounds__(SPLIT_WARPS * 32, SPLIT_CTAS_PER_SM) k_pcg_spl
         RunSum<float> gp, dp, rp;
         for (int u = threadIdx.x; u < 6 * R; u += blockDim.x) {
             const int lr = u / 6, c = u - 6 * lr, i = rb + lr;
-            const int rs = s_row[lr], rend = s_row[lr + 1];
+            const int rs = CLUSTER ? 0 : row_ent(lr), rend = CLUSTER ? 0 : row_ent(lr + 1);
             const float *r6 = hx + HX * (ob + lr);
             const float wc = split_combine(pp, s_src, lr, c, rs, rend, slot, rowacc) + split_diag(i, c, r6, Shd, diag_ident);
             rec0[(int64_t)SREC * i + 6 + c] = wc;
@@ -1351,7 +1355,7 @@ __global__ void __launch_bounds__(SPLIT_WARPS * 32, SPLIT_CTAS_PER_SM) k_pcg_spl
         if (prof) t0 = global_ns();
         split_halo_apply(NH, ob, R, false, a, b, hx, own);
         __syncthreads();
-        const bool ok = __syncthreads_and(split_passes(pp, s_row, hx, slot, rowacc, &sc->err, limit_cycles));
+        const bool ok = __syncthreads_and(split_passes(pp, row_ent, hx, slot, rowacc, &sc->err, limit_cycles));
         if (!ok) {
             leave();
             return;
@@ -1361,7 +1365,7 @@ __global__ void __launch_bounds__(SPLIT_WARPS * 32, SPLIT_CTAS_PER_SM) k_pcg_spl
         for (int u = threadIdx.x; u < 6 * R; u += blockDim.x) {
             const int lr = u / 6, c = u - 6 * lr, i = rb + lr, e = 6 * i + c;
             const bool first = u == u0;
-            const int rs = s_row[lr], rend = s_row[lr + 1];
+            const int rs = CLUSTER ? 0 : row_ent(lr), rend = CLUSTER ? 0 : row_ent(lr + 1);
             const float *rnew = hx + HX * (ob + lr);  // this row's new residual (all six components)
             const float w_e = split_combine(pp, s_src, lr, c, rs, rend, slot, rowacc) + split_diag(i, c, rnew, Shd, diag_ident);
             const float *o6 = own + 20 * lr;
@@ -1735,6 +1739,10 @@ cudaError_t launch_split_prepare(ba_problem *p, bool from_minv) {
 // cameras 3.4 / 4.4 us, 128 (7,700 entries) 3.6 / 4.8, 200 (12,000) 4.3 / 4.7,
 // 288 (17,500) 4.7 / 4.7, 392 5.5 / 4.7
 constexpr int64_t SPLIT_CLUSTER_ENTRIES = 14 * 1024;
+static const void *split_kernel(bool cluster, bool row_starts) {
+    return cluster ? (const void *)k_pcg_split<true, false>
+                   : (row_starts ? (const void *)k_pcg_split<false, true> : (const void *)k_pcg_split<false, false>);
+}
 static cudaLaunchConfig_t split_cluster_config(int grid, size_t smem, cudaStream_t st, cudaLaunchAttribute *at) {
     at->id = cudaLaunchAttributeClusterDimension;
     at->val.clusterDim.x = (unsigned)grid;
@@ -1787,15 +1795,16 @@ static cudaError_t split_partition(ba_problem *p) {
     if ((e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
     constexpr int ROW_COST = 8;
     constexpr int SMEM_MAX = 226 * 1024, SMEM_CLUSTER = 224 * 1024;  // 227 KB per CTA less the static part
-    for (const void *k : {(const void *)k_pcg_split<false>, (const void *)k_pcg_split<true>}) {
+    const void *const k_cluster = split_kernel(true, false);
+    for (const void *k : {k_cluster, split_kernel(false, true), split_kernel(false, false)}) {
         if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      k == (const void *)k_pcg_split<true> ? SMEM_CLUSTER : SMEM_MAX)) != cudaSuccess)
+                                      k == k_cluster ? SMEM_CLUSTER : SMEM_MAX)) != cudaSuccess)
             return e;
         if ((e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
                                       (int)cudaSharedmemCarveoutMaxShared)) != cudaSuccess)
             return e;
     }
-    if ((e = cudaFuncSetAttribute(k_pcg_split<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess)
+    if ((e = cudaFuncSetAttribute(k_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess)
         return e;
     bool cluster = E <= SPLIT_CLUSTER_ENTRIES;
     auto unavailable = [&]() {
@@ -1805,8 +1814,9 @@ static cudaError_t split_partition(ba_problem *p) {
     std::vector<int32_t> parts, cut, rows, tab, hptr, hcol, obase;
     size_t smem = SPLIT_STAGE_BYTES;
     int slot_floats = 0, stage_bytes = SPLIT_STAGE_BYTES, GP = 0, G = 0;
+    bool row_starts = true;
     for (int attempt = 0; attempt < 4; ++attempt) {
-        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_pcg_split<false>, SPLIT_WARPS * 32, smem)) != cudaSuccess) return e;
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, split_kernel(false, row_starts), SPLIT_WARPS * 32, smem)) != cudaSuccess) return e;
         bps = std::min(bps, SPLIT_CTAS_PER_SM);
         if (bps < 1) return unavailable();
         const int g = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)bps * n_sm, (E + 255) / 256));
@@ -1918,11 +1928,15 @@ static cudaError_t split_partition(ba_problem *p) {
             Pmax = std::max(Pmax, (int)P);
             slot_floats = std::max(slot_floats, (int)(12 * P + 6 * R + 3) & ~3);
         }
-        const size_t rest = ((size_t)slot_floats + (size_t)HX * Hmax + 21 * (size_t)Rmax + 1 +
-                             (cluster ? Rmax : 0)) * sizeof(float);
+        size_t rest = ((size_t)slot_floats + (size_t)HX * Hmax + 20 * (size_t)Rmax) * sizeof(float);
         // a buffer for every pass where they fit (one more where their number
         // is that of the streaming buffers: the kernel tells the modes by it)
         const size_t own = (size_t)PASS_BYTES * (Pmax == SPLIT_WARPS * SPLIT_NBUF ? Pmax + 1 : Pmax);
+        // a word for each row besides: its start (its sums' place in a cluster),
+        // unless that is more than fits (the starts are read from memory then)
+        const size_t words = ((size_t)Rmax + 1) * sizeof(float);
+        row_starts = !cluster && std::min(own, (size_t)SPLIT_STAGE_BYTES) + rest + words <= (size_t)SMEM_MAX;
+        if (cluster || row_starts) rest += words;
         stage_bytes = own + rest <= (size_t)(cluster ? SMEM_CLUSTER : SMEM_MAX) ? (int)own : SPLIT_STAGE_BYTES;
         smem = stage_bytes + rest;
         if (cluster) {
@@ -1930,7 +1944,7 @@ static cudaError_t split_partition(ba_problem *p) {
             const cudaLaunchConfig_t cfg = split_cluster_config(G, smem, p->st, &at);
             int clusters = 0;
             if (smem > (size_t)SMEM_CLUSTER || Hmax > (int)CL_NONE || Rmax >= (int)CL_NONE ||
-                cudaOccupancyMaxActiveClusters(&clusters, k_pcg_split<true>, &cfg) != cudaSuccess || clusters < 1) {
+                cudaOccupancyMaxActiveClusters(&clusters, k_cluster, &cfg) != cudaSuccess || clusters < 1) {
                 cudaGetLastError();
                 cluster = false;  // no room for such a cluster: start over as a grid over all SMs
                 smem = SPLIT_STAGE_BYTES;
@@ -1942,7 +1956,7 @@ static cudaError_t split_partition(ba_problem *p) {
         if (smem > (size_t)SMEM_MAX || Hmax > 0xFFFF || Rmax > 0xFFFE) return unavailable();
     }
     // the occupancy at the final shared-memory size must keep the grid resident
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, k_pcg_split<false>, SPLIT_WARPS * 32, smem)) != cudaSuccess) return e;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, split_kernel(false, row_starts), SPLIT_WARPS * 32, smem)) != cudaSuccess) return e;
     if (G < 1 || (int64_t)bps * n_sm < G) return unavailable();
     // packed entry metadata, per CTA from a 16-byte aligned offset (+ padding
     // for the rounded-up copy of a CTA's last pass)
@@ -1998,6 +2012,7 @@ static cudaError_t split_partition(ba_problem *p) {
     p->split_smem = smem;
     p->split_grid = G;
     p->split_cluster = cluster;
+    p->split_row_starts = row_starts;
     return cudaSuccess;
 }
 
@@ -2062,9 +2077,9 @@ cudaError_t launch_pcg_split(ba_problem *p) {
         if (p->split_cluster) {
             cudaLaunchAttribute at;
             const cudaLaunchConfig_t cfg = split_cluster_config(p->split_grid, p->split_smem, p->st, &at);
-            e = cudaLaunchKernelExC(&cfg, (const void *)k_pcg_split<true>, args);
+            e = cudaLaunchKernelExC(&cfg, split_kernel(true, false), args);
         } else {
-            e = cudaLaunchCooperativeKernel((const void *)k_pcg_split<false>, dim3(p->split_grid),
+            e = cudaLaunchCooperativeKernel(split_kernel(false, p->split_row_starts), dim3(p->split_grid),
                                             dim3(SPLIT_WARPS * 32), args, p->split_smem, p->st);
         }
     }
