@@ -1968,27 +1968,35 @@ static cudaError_t split_partition(ba_problem *p) {
     }
     mtotal += 4;
     std::vector<uint32_t> meta(mtotal, cluster ? CL_NONE : 0u);
-    std::vector<uint32_t> src(n, ROW_EMPTY);
-    for (int k = 0; k < G; ++k) {
-        const int32_t *hc = hcol.data() + hptr[k];
-        const int H = hptr[k + 1] - hptr[k], P = cluster ? tab[k + 1] - tab[k] - 1 : 0;
-        int32_t q = 0;  // cluster: the entry's pass
-        for (int i = rows[k]; i < rows[k + 1]; ++i)
-            for (int32_t t = twp[i]; t < twp[i + 1]; ++t) {
-                const uint32_t h = (uint32_t)(std::lower_bound(hc, hc + H, twe[t].y) - hc), lr = (uint32_t)(i - rows[k]);
-                if (!cluster) {
-                    meta[moff[k] + (t - twp[rows[k]])] = lr | (h << 16);
-                    continue;
+    auto halo_index = [&](int k, int32_t t) {
+        const int32_t *const hc = hcol.data() + hptr[k], *const he = hcol.data() + hptr[k + 1];
+        return (uint32_t)(std::lower_bound(hc, he, twe[t].y) - hc);
+    };
+    if (!cluster) {
+        for (int k = 0; k < G; ++k) {
+            uint32_t *m = meta.data() + moff[k];
+            for (int i = rows[k]; i < rows[k + 1]; ++i)
+                for (int32_t t = twp[i]; t < twp[i + 1]; ++t) *m++ = (uint32_t)(i - rows[k]) | (halo_index(k, t) << 16);
+        }
+    } else {
+        std::vector<uint32_t> src(n, ROW_EMPTY);
+        for (int k = 0; k < G; ++k) {
+            const int32_t *ps = tab.data() + tab[k];
+            const int P = tab[k + 1] - tab[k] - 1;
+            int32_t q = 0;  // the entry's pass
+            for (int i = rows[k]; i < rows[k + 1]; ++i)
+                for (int32_t t = twp[i]; t < twp[i + 1]; ++t) {
+                    const uint32_t lr = (uint32_t)(i - rows[k]);
+                    while (t >= ps[q + 1]) ++q;
+                    const bool opens = twp[i] <= ps[q], closes = twp[i + 1] >= ps[q + 1];
+                    meta[moff[k] + 32 * q + (t - ps[q])] =
+                        lr | (halo_index(k, t) << 16) | (opens ? 0u : (closes ? 0x8000u : 0x80000000u));
+                    if (t == twp[i]) src[i] = (uint32_t)(opens ? 12 * q : (closes ? 12 * q + 6 : 12 * P + 6 * (int)lr));
+                    else if (t == ps[q]) src[i] += 1u << 16;
                 }
-                const int32_t *ps = tab.data() + tab[k];
-                while (t >= ps[q + 1]) ++q;
-                const bool opens = twp[i] <= ps[q], closes = twp[i + 1] >= ps[q + 1];
-                meta[moff[k] + 32 * q + (t - ps[q])] = lr | (h << 16) | (opens ? 0u : (closes ? 0x8000u : 0x80000000u));
-                if (t == twp[i]) src[i] = (uint32_t)(opens ? 12 * q : (closes ? 12 * q + 6 : 12 * P + 6 * (int)lr));
-                else if (t == ps[q]) src[i] += 1u << 16;
-            }
+        }
+        tab.insert(tab.end(), src.begin(), src.end());
     }
-    if (cluster) tab.insert(tab.end(), src.begin(), src.end());
     std::vector<std::pair<void **, std::pair<const void *, size_t>>> up = {
         {(void **)&p->tws_ptr, {twp.data(), twp.size() * sizeof(int32_t)}},
         {(void **)&p->tws_ent, {twe.data(), twe.size() * sizeof(int2)}},
@@ -1997,8 +2005,8 @@ static cudaError_t split_partition(ba_problem *p) {
         {(void **)&p->meta_off, {moff.data(), moff.size() * sizeof(int32_t)}},
         {(void **)&p->halo_ptr, {hptr.data(), hptr.size() * sizeof(int32_t)}},
         {(void **)&p->halo_col, {hcol.data(), std::max<size_t>(hcol.size(), 1) * sizeof(int32_t)}},
-        {(void **)&p->own_base, {obase.data(), obase.size() * sizeof(int32_t)}},
-        {(void **)&p->pass_tab, {tab.data(), tab.size() * sizeof(int32_t)}}};
+        {(void **)&p->own_base, {obase.data(), obase.size() * sizeof(int32_t)}}};
+    if (cluster) up.push_back({(void **)&p->pass_tab, {tab.data(), tab.size() * sizeof(int32_t)}});
     for (auto &u : up) {
         void *d = nullptr;
         if ((e = cudaMalloc(&d, u.second.second)) != cudaSuccess) return e;
