@@ -70,8 +70,6 @@ __device__ __forceinline__ void grid_sum(double (&v)[NV], double *part, unsigned
     }
 }
 
-template <typename T> __device__ __forceinline__ T dmax(T a, T b) { return a > b ? a : b; }
-template <typename T> __device__ __forceinline__ T dmin(T a, T b) { return a < b ? a : b; }
 
 __device__ __forceinline__ double clampd(double x) { return x < 1e-6 ? 1e-6 : (x > 1e32 ? 1e32 : x); }
 template <typename T> __device__ __forceinline__ T clampT(T x) { return x < T(1e-6) ? T(1e-6) : (x > T(1e32) ? T(1e32) : x); }
@@ -325,14 +323,13 @@ __device__ __forceinline__ double warp_fold(const double (&v)[NV]) {
 // launch: v holds the CTA's partials in lane 0; they are published, the CTA
 // announces itself (arrivals spread over AR_SUB counters on lines of their own
 // as in grid_allreduce_df, the wait bounded), and the warp adds all CTAs'
-// partials, each lane's loads issued together.  after_wait() runs once every
-// CTA has arrived, behind those loads.  Totals in every lane, the same bits in
-// every CTA; false on timeout (the error word is set).  `bar` holds
+// partials, each lane's loads issued together.  Totals in every lane, the same
+// bits in every CTA; false on timeout (the error word is set).  `bar` holds
 // AR_SUB * 32 words, zero at launch; `gen` numbers the launch's calls.
 constexpr int AR_SUB = 16;
-template <int NV, class F>
+template <int NV>
 __device__ __forceinline__ bool grid_exchange(double (&v)[NV], double *part, unsigned gen, unsigned *bar, int *err,
-                                              long long limit_cycles, F &&after_wait) {
+                                              long long limit_cycles) {
     const int lane = threadIdx.x & 31;
     double2 *half = reinterpret_cast<double2 *>(part + (size_t)(gen & 1u) * gridDim.x * AR_NV_MAX);
     if (lane == 0) {
@@ -361,7 +358,6 @@ __device__ __forceinline__ bool grid_exchange(double (&v)[NV], double *part, uns
 #pragma unroll
         for (int q = 0; q < 5; ++q)
             u[q] = lane + 32 * q < (int)gridDim.x ? __ldcg(half + lane + 32 * q) : make_double2(0.0, 0.0);
-        after_wait();
 #pragma unroll
         for (int q = 0; q < 5; ++q) {
             acc[0] += u[q].x;
@@ -523,7 +519,7 @@ __device__ __forceinline__ bool grid_allreduce_w0(double (&v)[NV], double *part,
         double x[NV];
         x[NV - 1] = __shfl_sync(0xffffffffu, t, 16);
         x[0] = __shfl_sync(0xffffffffu, t, 0);
-        const bool ok = grid_exchange<NV>(x, part, gen, bar, err, limit_cycles, []() {});
+        const bool ok = grid_exchange<NV>(x, part, gen, bar, err, limit_cycles);
         fin(x, ok);
         if (lane == 0) {
 #pragma unroll

@@ -766,15 +766,6 @@ __global__ void __launch_bounds__(128) k_split_scale(int n, const int *__restric
 // so a gather of a neighbour's three vectors is five float4 loads.
 constexpr int SREC = 20;
 
-__device__ __forceinline__ void load_rec(const float *rec, int j, float (&v)[20]) {
-    const float4 *q = reinterpret_cast<const float4 *>(rec + (int64_t)SREC * j);
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-        const float4 t = __ldcg(q + k);
-        v[4 * k] = t.x; v[4 * k + 1] = t.y; v[4 * k + 2] = t.z; v[4 * k + 3] = t.w;
-    }
-}
-
 // r^_0 = G^T rhs per camera (rhs rounded to FP32) into record 0, s = 0 in both
 // records, x^ = p = 0, the scalars of the solve, and its all-reduce's arrival
 // counters (bar0: 0, or -1 for the armed test of the timeout path).  first:
