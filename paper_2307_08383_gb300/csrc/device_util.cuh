@@ -113,7 +113,7 @@ __device__ __forceinline__ double widen(double d) { return d; }
 __device__ __forceinline__ double quotient(double a, double b, double inv) {
     const double q = a * inv, r = fma(-q, b, a);
     const double m = fabs(b);
-    if (!(m > 1e-150 && m < 1e150 && fabs(q) > 1e-100 && fabs(q) < 1e100)) return a / b;
+    if (!(m > 1e-150 && m < 1e150 && ((fabs(q) > 1e-100 && fabs(q) < 1e100) || a == 0.0))) return a / b;
     return fma(r, inv, q);
 }
 
