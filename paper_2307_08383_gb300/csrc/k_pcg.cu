@@ -1730,6 +1730,15 @@ cudaError_t launch_split_prepare(ba_problem *p, bool from_minv) {
 // cameras 3.4 / 4.4 us, 128 (7,700 entries) 3.6 / 4.8, 200 (12,000) 4.3 / 4.7,
 // 288 (17,500) 4.7 / 4.7, 392 5.5 / 4.7
 constexpr int64_t SPLIT_CLUSTER_ENTRIES = 14 * 1024;
+// With few entries a row the CTAs have many rows, and the update takes a round of
+// the threads for every 85: more than one round pays only beside a single round
+// of passes, and up to about 220 rows.  Per iteration, cluster against grid: chains
+// (two entries a row) of 2,500 cameras (157 rows a CTA, 10 passes) 5.0 / 5.9 us,
+// 3,000 (188) 5.8 / 5.9, 4,000 (250) 6.3 / 6.0, 7,000 9.6 / 6.2; eight entries a row:
+// 1,250 cameras (79 rows, 20 passes) 4.6 / 5.0, 1,500 (94 rows, 24 passes) 5.4 / 4.9.
+static bool split_cluster_pays(int rows, int passes) {
+    return 6 * rows <= SPLIT_WARPS * 32 || (passes <= SPLIT_WARPS && rows <= 220);
+}
 static const void *split_kernel(bool cluster, bool row_starts) {
     return cluster ? (const void *)k_pcg_split<true, false>
                    : (row_starts ? (const void *)k_pcg_split<false, true> : (const void *)k_pcg_split<false, false>);
@@ -1883,7 +1892,7 @@ static cudaError_t split_partition(ba_problem *p) {
                 }
                 return true;
             };
-            int cap = 1;
+            int cap = std::max(1, ((int)cut.size() - 2 + G) / G);
             while (!deal(cap)) ++cap;
         }
         // halos
@@ -1934,7 +1943,7 @@ static cudaError_t split_partition(ba_problem *p) {
             cudaLaunchAttribute at;
             const cudaLaunchConfig_t cfg = split_cluster_config(G, smem, p->st, &at);
             int clusters = 0;
-            if (smem > (size_t)SMEM_CLUSTER || Hmax > (int)CL_NONE || Rmax >= (int)CL_NONE ||
+            if (smem > (size_t)SMEM_CLUSTER || !split_cluster_pays(Rmax, Pmax) || Hmax > (int)CL_NONE || Rmax >= (int)CL_NONE ||
                 cudaOccupancyMaxActiveClusters(&clusters, k_cluster, &cfg) != cudaSuccess || clusters < 1) {
                 cudaGetLastError();
                 cluster = false;  // no room for such a cluster: start over as a grid over all SMs

@@ -74,7 +74,11 @@ SOLVED = {
     (60, 59): "0f582ece9e37bb23",
     (128, 58): "c9216e937f2322e1",
     (160, 75): "f11d1d32d91d7a0f",
-    (200, 33): "e2d9e2800fe43be4"}
+    (200, 33): "e2d9e2800fe43be4",
+    (1300, 5): "890af9b61d8e3c73",
+    (1700, 5): "86c8c95352b3c85e",
+    (2400, 2): "adba1a73e1fa99a8",
+    (4000, 2): "cf6f9ce1e7e9fff3"}
 
 
 def integer_system(row_ptr, col, cdim, seed):
