@@ -229,7 +229,6 @@ struct ba_problem {
     float2 *xs = nullptr;  // x64 split in FP32 pairs (refinement residual of FP32 problems)
     unsigned char *mail = nullptr;  // mailboxes of the register-resident FP64 PCG
     unsigned mail_epoch = 0;        // its launches
-    unsigned *ar_bar = nullptr;  // arrival counters of the split CG's all-reduce (one per line)
     // > 0: the next PCG launch (split or standard recurrence) starts its
     // all-reduce counters one arrival short and waits at most this many SM
     // cycles (ba_debug_arm_wait_timeout; a test of the timeout path)

@@ -1457,17 +1457,11 @@ cudaError_t launch_pcg_init(ba_problem *p, const void *rhs, double tol, int max_
 // two-sided product, whose second read hits L2.
 constexpr int64_t ONCE_MIN_BYTES = 64ll << 20;
 
-// arrival counters of the PCG kernels' all-reduces, one per 128-byte line
-static cudaError_t ensure_ar_bar(ba_problem *p) {
-    if (p->ar_bar) return cudaSuccess;
-    void *v = nullptr;
-    const cudaError_t e = cudaMalloc(&v, AR_SUB * 32 * sizeof(unsigned));
-    if (e != cudaSuccess) return e;
-    p->ar_bar = (unsigned *)v;
-    p->allocs.push_back(v);
-    p->dev_bytes += AR_SUB * 32 * sizeof(unsigned);
-    return cudaSuccess;
-}
+// Arrival counters of the PCG kernels' all-reduces, one per 128-byte line: behind
+// the partials, of which the largest grid writes 2 x 608 x 4 (nothing to allocate in
+// a first solve).
+static_assert(AR_SUB * 32 * sizeof(unsigned) <= RED_SLOTS / 2 * sizeof(double), "counters fit behind the partials");
+static unsigned *ar_counters(const ba_problem *p) { return reinterpret_cast<unsigned *>(p->red + RED_SLOTS / 2); }
 
 // The register-resident FP64 loop, where its CTAs cover the system: at most
 // RES64_ROWS rows per SM, one lane per entry of the longest row.
@@ -1533,8 +1527,8 @@ static cudaError_t pcg_loop_T(ba_problem *p) {
     p->test_wait_limit = 0;
     const long long limit_cycles = test_limit > 0 ? test_limit : 4000000000LL;  // ~2 s of SM clock per wait
     if (sizeof(T) == 8 && p->mail && res64_fits(p, n_sm)) return launch_res64(p, n_sm, test_limit > 0 ? 1u : 0u, limit_cycles);
-    if ((e = ensure_ar_bar(p)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(p->ar_bar, test_limit > 0 ? 0xFF : 0, AR_SUB * 32 * sizeof(unsigned), p->st)) !=
+    unsigned *bar = ar_counters(p);
+    if ((e = cudaMemsetAsync(bar, test_limit > 0 ? 0xFF : 0, AR_SUB * 32 * sizeof(unsigned), p->st)) !=
         cudaSuccess)
         return e;
     int n = p->n;
@@ -1545,7 +1539,6 @@ static cudaError_t pcg_loop_T(ba_problem *p) {
     T *q = (T *)p->sv.pv[5], *r1 = (T *)p->sv.pv[6], *q1 = (T *)p->sv.pv[7];
     DevScalars *sc = p->sc;
     double *red = p->red;
-    unsigned *bar = p->ar_bar;
     long long limit = limit_cycles;
     void *args[] = {&n, &twp, &twe, &rp, &cl, &S, &Mi, &y, &r, &r1, &z, &d0, &d1, &q, &q1, &sc, &red, &bar, &limit};
     return cudaLaunchCooperativeKernel((const void *)k_pcg_persist<T, ONCE>, dim3(grid), dim3(32 * warps), args, 0, p->st);
@@ -2035,8 +2028,6 @@ bool split_available(ba_problem *p) {
 // vectors: pv[0] x^, pv[2] p of the active FP32 view; records in p->srec.
 // first: the sweep's right-hand side is b, else the residual r64
 cudaError_t launch_split_init(ba_problem *p, bool first, double tol, int max_iters) {
-    const cudaError_t e = ensure_ar_bar(p);
-    if (e != cudaSuccess) return e;
     cudaEvent_t ev;
     ktimer_begin(p, K_PCG_INIT, &ev);
     float **v = (float **)p->sv.pv;
@@ -2045,11 +2036,11 @@ cudaError_t launch_split_init(ba_problem *p, bool first, double tol, int max_ite
     const unsigned bar0 = p->test_wait_limit > 0 ? ~0u : 0u;
     if (first && p->fp32)
         k_split_init<float><<<g, 64, 0, p->st>>>(p->n, (const float *)p->b, p->Gs, rec0, rec1, v[0], v[2], p->sc,
-                                                 tol * tol, max_iters, prof, p->ar_bar, bar0, 1, p->red,
+                                                 tol * tol, max_iters, prof, ar_counters(p), bar0, 1, p->red,
                                                  p->counters + 6);
     else
         k_split_init<double><<<g, 64, 0, p->st>>>(p->n, first ? (const double *)p->b : p->r64, p->Gs, rec0, rec1, v[0],
-                                                  v[2], p->sc, tol * tol, max_iters, prof, p->ar_bar, bar0,
+                                                  v[2], p->sc, tol * tol, max_iters, prof, ar_counters(p), bar0,
                                                   first ? 1 : 0, p->red, p->counters + 6);
     ktimer_end(p, K_PCG_INIT, ev);
     p->launches += 1;
@@ -2077,7 +2068,7 @@ cudaError_t launch_pcg_split(ba_problem *p) {
         float *rec0 = p->srec, *rec1 = p->srec + (size_t)SREC * p->n;
         DevScalars *sc = p->sc;
         double *red = p->red;
-        unsigned *bar = p->ar_bar;
+        unsigned *bar = ar_counters(p);
         long long limit = test_limit > 0 ? test_limit : 4000000000LL;  // ~2 s of SM clock per wait
         int short_by = test_limit > 0 ? 1 : 0;
         void *args[] = {&cr, &twp, &meta, &mo, &hp, &hc, &ob, &pt, &sf, &stf, &Sh, &H, &Shd, &ident, &x, &pp, &rec0, &rec1, &sc,
