@@ -282,14 +282,15 @@ ba_status symbolic_setup(int32_t n, int64_t P, int64_t m, const int32_t *obs_cam
         // keeps the order, and with it the bits, of its sums)
         std::vector<int32_t> ord(nlb);
         std::iota(ord.begin(), ord.end(), 0);
-        auto item_size = [&](int32_t b) {
+        // one key per block: diagonal, item size, product count
+        std::vector<int64_t> key(nlb);
+        for (int32_t b = 0; b < nlb; ++b) {
             const int32_t k = (cnt[b] + ITEM_MAX - 1) / ITEM_MAX;
-            return (cnt[b] + k - 1) / k;
-        };
+            const int64_t size = even_items ? (cnt[b] + k - 1) / k : 0;
+            key[b] = ((int64_t)is_diag[b] << 40) | (size << 32) | cnt[b];
+        }
         std::sort(ord.begin(), ord.end(), [&](int32_t x, int32_t y) {
-            if (is_diag[x] != is_diag[y]) return is_diag[x] > is_diag[y];
-            if (even_items && item_size(x) != item_size(y)) return item_size(x) > item_size(y);
-            if (cnt[x] != cnt[y]) return cnt[x] > cnt[y];
+            if (key[x] != key[y]) return key[x] > key[y];
             return g_gblk[x] < g_gblk[y];
         });
         std::vector<int32_t> pos(nlb), start(nlb + 1, 0);
