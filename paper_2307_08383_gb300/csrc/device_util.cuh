@@ -412,7 +412,12 @@ __device__ __forceinline__ bool poll_over(long long t0, long long limit_cycles, 
 // bytes; `epoch` numbers the launches that use it from 1 on, `gen` the launch's
 // calls (two sets in turn: a set is written again only two calls later, by a
 // CTA that has every CTA's partials of call gen + 1, sent after reading call
-// gen).  miss: 0 (set, the tag waited for is one that nobody posts).
+// gen).  All accesses are relaxed; what orders that reuse is dependence: a post
+// of call gen + 1 is computed from the totals of call gen, so after the reads of
+// that call, and a post of gen + 2 from those of every gen + 1.  A slot written
+// too early would carry a tag that its reader does not take: the wait would end
+// by its limit, never with another call's value.
+// miss: 0 (set, the tag waited for is one that nobody posts).
 // Against grid_exchange: a store and a poll instead of a store, its
 // acknowledged release, an atomic, a poll and a read.  One slot per CTA that
 // all the others poll was slower than either at 100 CTAs and more (its few

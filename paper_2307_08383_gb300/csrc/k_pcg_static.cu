@@ -126,6 +126,12 @@ __global__ void k_static_init(int n, const float *__restrict__ b, float *x, floa
 }
 
 // d_new = z + beta d_old (row owner stores it), q += S d_new, d^T S d.
+// Two launches per iteration, the host reading the stop flag after every eight:
+// 30 us per iteration at 1,250 cameras, launches and read-backs.  The whole solve
+// in one cooperative launch took 11, but added the terms of q in another order;
+// near the stop, where the residual moves by a few percent per iteration both
+// ways, that order decides at which iteration the solve ends, and some systems
+// got another iterate (up to 4e-3 apart, 5e-4 between runs of one version).
 __global__ void __launch_bounds__(256) k_static_spmv(int n, const int *__restrict__ row_ptr, const int *__restrict__ col,
                                                      const float *__restrict__ S, const float *__restrict__ z,
                                                      const float *__restrict__ dold, float *__restrict__ dnew,
