@@ -263,37 +263,44 @@ ba_status symbolic_setup(int32_t n, int64_t P, int64_t m, const int32_t *obs_cam
     hs.max_nc = 0;
     GroupDesc g{};
     int32_t gid = 0;
+    // a block is diagonal iff it is the first block of its row
+    std::vector<char> first_of_row(nnzb, 0);
+    for (int32_t i = 0; i < n; ++i) first_of_row[hs.row_ptr[i]] = 1;
+    // a group's lists, kept between groups (FP64 problems have many small ones)
+    struct BlockKey {
+        int64_t key;
+        int32_t gblk, b;
+    };
+    std::vector<int32_t> cnt, ord, pos, start, fill;
+    std::vector<char> is_diag;
+    std::vector<BlockKey> keys;
+    std::vector<WorkItem> its;
     auto close_group = [&]() {
         if (g.npts == 0) return;
         const int32_t nlb = (int32_t)g_gblk.size();
-        std::vector<int32_t> cnt(nlb, 0);
-        std::vector<char> is_diag(nlb, 0);
+        cnt.assign(nlb, 0);
+        is_diag.resize(nlb);
         for (auto &c : g_c) cnt[c.first]++;
-        for (int32_t b = 0; b < nlb; ++b) {
-            // a block is diagonal iff it is the first block of its row
-            auto it = std::upper_bound(hs.row_ptr.begin(), hs.row_ptr.end(), g_gblk[b]);
-            is_diag[b] = hs.row_ptr[(it - hs.row_ptr.begin()) - 1] == g_gblk[b];
-        }
+        for (int32_t b = 0; b < nlb; ++b) is_diag[b] = first_of_row[g_gblk[b]];
         // diagonal blocks first (one code path per warp), then by product count
         // (descending) so that full items share warps; ties by global id.
         // even_items: by the size of their items before that (9 products make
         // items of 5 and 4, 8 one of 8), since a warp runs its longest item's
         // length (FP64, bound by those products: 450 cameras 316 -> 304 us; FP32
         // keeps the order, and with it the bits, of its sums)
-        std::vector<int32_t> ord(nlb);
-        std::iota(ord.begin(), ord.end(), 0);
-        // one key per block: diagonal, item size, product count
-        std::vector<int64_t> key(nlb);
+        keys.resize(nlb);
         for (int32_t b = 0; b < nlb; ++b) {
             const int32_t k = (cnt[b] + ITEM_MAX - 1) / ITEM_MAX;
             const int64_t size = even_items ? (cnt[b] + k - 1) / k : 0;
-            key[b] = ((int64_t)is_diag[b] << 40) | (size << 32) | cnt[b];
+            keys[b] = {((int64_t)is_diag[b] << 40) | (size << 32) | cnt[b], g_gblk[b], b};
         }
-        std::sort(ord.begin(), ord.end(), [&](int32_t x, int32_t y) {
-            if (key[x] != key[y]) return key[x] > key[y];
-            return g_gblk[x] < g_gblk[y];
+        std::sort(keys.begin(), keys.end(), [](const BlockKey &x, const BlockKey &y) {
+            return x.key != y.key ? x.key > y.key : x.gblk < y.gblk;
         });
-        std::vector<int32_t> pos(nlb), start(nlb + 1, 0);
+        ord.resize(nlb);
+        for (int32_t r = 0; r < nlb; ++r) ord[r] = keys[r].b;
+        pos.resize(nlb);
+        start.assign(nlb + 1, 0);
         for (int32_t r = 0; r < nlb; ++r) pos[ord[r]] = r;
         for (int32_t r = 0; r < nlb; ++r) start[r + 1] = start[r] + cnt[ord[r]];
         g.c_begin = (int64_t)hs.contrib.size();
@@ -302,10 +309,10 @@ ba_status symbolic_setup(int32_t n, int64_t P, int64_t m, const int32_t *obs_cam
         g.nc = (int32_t)g_c.size();
         // each group's list starts on a 16-byte boundary and spans a multiple of 16 bytes (bulk copies)
         hs.contrib.resize(hs.contrib.size() + ((g_c.size() + 3) & ~(size_t)3), 0u);
-        std::vector<int32_t> fill(start.begin(), start.end() - 1);
+        fill.assign(start.begin(), start.end() - 1);
         for (auto &c : g_c) hs.contrib[g.c_begin + fill[pos[c.first]]++] = c.second;  // stable: point order
         // work items of <= ITEM_MAX products, sizes balanced within a block
-        std::vector<WorkItem> its;
+        its.clear();
         for (int32_t r = 0; r < nlb; ++r) {
             const int32_t c = cnt[ord[r]];
             const int32_t k = (c + ITEM_MAX - 1) / ITEM_MAX;
