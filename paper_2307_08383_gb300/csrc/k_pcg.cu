@@ -652,7 +652,7 @@ __global__ void __launch_bounds__(32) k_split_factor(int n, const int *__restric
     double a[6], x[6];
 #pragma unroll
     for (int k = 0; k < 6; ++k) a[k] = on ? (double)src[6 * r + k] : (i < n ? 0.0 : 1.0);
-    const bool ok = chol6_lanes<double>(a, x);
+    const bool ok = chol6_lanes<double, false>(a, x);
     float *g = G + 36 * (int64_t)i + 6 * r, *h = H + 36 * (int64_t)i + 6 * r;
     float fl[6], fx[6];  // row r of L, row r of L^-T
 #pragma unroll

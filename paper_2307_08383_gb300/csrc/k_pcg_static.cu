@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(32) k_static_minv(int n, int64_t nnzb, const i
     const float *d = val + (int64_t)(ok ? rs : 0) * BW;
 #pragma unroll
     for (int c = 0; c < 6; ++c) a[c] = ok && r < 6 ? (double)d[6 * r + c] : 0.0;
-    const bool spd = chol6_lanes<double>(a, x);
+    const bool spd = chol6_lanes<double, false>(a, x);
     inv6_row<double>(x, out);
     if (i >= n || r >= 6) return;
     if (r == 0) {
