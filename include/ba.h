@@ -247,9 +247,10 @@ ba_status ba_set_profile(ba_problem *p, int32_t level);
  * (about 2 s), sets an error word the host reads, and leaves its kernel, so
  * that a stalled wait ends as a status instead of a hung GPU.  This call arms
  * the next PCG launch of p (the split CG of FP32 solves or the Sec. 3.2
- * recurrence) to start its all-reduce arrival counters one arrival short of
- * their targets and to wait at most limit_cycles (1 .. 4e9) cycles: the first
- * all-reduce then runs out on every CTA, the kernel leaves after its copies
+ * recurrence) to wait for what never comes (its arrival counters start one
+ * arrival short of their targets, its cluster's barriers expect one arrival too
+ * many, or its mailboxes are read for a tag that nobody posts) and at most
+ * limit_cycles (1 .. 4e9) cycles: the first all-reduce then runs out on every CTA, the kernel leaves after its copies
  * in flight have landed, and the solve returns BA_ERR_TIMEOUT.  As after any
  * BA_ERR_TIMEOUT, p is then unusable (later calls on it return BA_ERR_STATE;
  * ba_problem_destroy still frees it) while the CUDA context and other
