@@ -250,8 +250,9 @@ ba_status ba_set_profile(ba_problem *p, int32_t level);
  * recurrence) to wait for what never comes (its arrival counters start one
  * arrival short of their targets, its cluster's barriers expect one arrival too
  * many, or its mailboxes are read for a tag that nobody posts) and at most
- * limit_cycles (1 .. 4e9) cycles: the first all-reduce then runs out on every CTA, the kernel leaves after its copies
- * in flight have landed, and the solve returns BA_ERR_TIMEOUT.  As after any
+ * limit_cycles (1 .. 4e9) cycles: the first all-reduce then runs out on every
+ * CTA, the kernel leaves after its copies in flight have landed, and the solve
+ * returns BA_ERR_TIMEOUT.  As after any
  * BA_ERR_TIMEOUT, p is then unusable (later calls on it return BA_ERR_STATE;
  * ba_problem_destroy still frees it) while the CUDA context and other
  * problems are unaffected.  The arming is used up by that one launch. */
